@@ -35,6 +35,7 @@ struct qs_ctx {
     int block_level_n = 16;
     int tile_x = 0, tile_y = 0;
     size_t tile_offset = 0, block_offset = 0;
+    FftArgs fft = {};  // sine transforms of the direct solves
     double *hist = nullptr, *jzb = nullptr;
     // laser driver: |A|^2 and grad(|A|^2/4) of the current slice; |A|^2 and
     // chi of every base slice for the laser-driven step (allocated on use)
@@ -223,6 +224,66 @@ int validate(const qs_config *cfg, char *why, size_t nwhy) {
     return QS_OK;
 }
 
+// Tables and scratch grids of the sine transforms.
+int create_fft(qs_ctx *c) {
+    const int n = c->N, half = n / 2 + 1;
+    std::vector<double2> tw(n), dct(half);
+    std::vector<double> lam(n);
+    std::vector<float2> tw32(n), dct32(half);
+    std::vector<float> lam32(n);
+    const double pi = 3.14159265358979323846;
+    for (int k = 0; k < n; ++k) {
+        // angles reduced to [0, pi/4] so that the tables are exact to rounding
+        // and symmetric
+        auto unit = [&](int num, int den) {  // e^{-2 pi i num / den}, 0 <= num < den
+            const int oct = (int)((long long)num * 8 / den);
+            const int a = oct & 1 ? (oct + 1) * den - 8 * num : 8 * num - oct * den;
+            const double t = pi * a / (4.0 * den);
+            const double co = std::cos(t), si = std::sin(t);
+            double2 v{co, si};
+            switch (oct) {
+            case 1: v = {si, co}; break;
+            case 2: v = {-si, co}; break;
+            case 3: v = {-co, si}; break;
+            case 4: v = {-co, -si}; break;
+            case 5: v = {-si, -co}; break;
+            case 6: v = {si, -co}; break;
+            case 7: v = {co, -si}; break;
+            default: break;
+            }
+            return double2{v.x, -v.y};
+        };
+        tw[k] = unit(k, n);
+        if (k < half) dct[k] = unit(k, 4 * n);
+        const double cs = std::cos(0.5 * pi * k / n);  // 2 + 2 cos(t) = 4 cos^2(t/2)
+        lam[k] = -4.0 * cs * cs / (c->h * c->h);
+        tw32[k] = make_float2((float)tw[k].x, (float)tw[k].y);
+        if (k < half) dct32[k] = make_float2((float)dct[k].x, (float)dct[k].y);
+        lam32[k] = (float)lam[k];
+    }
+    auto &L = c->allocs;
+    FftArgs &f = c->fft;
+    AL(L, f.tw64, n);
+    AL(L, f.dct64, half);
+    AL(L, f.lam64, n);
+    AL(L, f.tw32, n);
+    AL(L, f.dct32, half);
+    AL(L, f.lam32, n);
+    AL(L, f.t1, (size_t)n * n);
+    AL(L, f.t2, (size_t)n * n);
+    auto up = [](void *d, const void *h, size_t b) {
+        return cudaMemcpy(d, h, b, cudaMemcpyHostToDevice);
+    };
+    CK(up(f.tw64, tw.data(), n * sizeof(double2)), "tables");
+    CK(up(f.dct64, dct.data(), half * sizeof(double2)), "tables");
+    CK(up(f.lam64, lam.data(), n * sizeof(double)), "tables");
+    CK(up(f.tw32, tw32.data(), n * sizeof(float2)), "tables");
+    CK(up(f.dct32, dct32.data(), half * sizeof(float2)), "tables");
+    CK(up(f.lam32, lam32.data(), n * sizeof(float)), "tables");
+    f.on = 1;
+    return QS_OK;
+}
+
 int create_impl(qs_ctx *c) {
     const qs_config &g = c->cfg;
     CK(cudaGetDevice(&c->dev), "cudaGetDevice");
@@ -314,13 +375,9 @@ int create_impl(qs_ctx *c) {
     c->engine_smem = qs_engine_smem_bytes(c->lev_n, c->nlev, c->block_level_n, g.precision,
                                           c->tile_x, c->tile_y, nu, g.post_sweeps,
                                           &c->block_offset, &c->tile_offset);
-    int cs = g.cluster_size;
-    if (cs == 0) {
-        if (!ref)  // float64: small grids, 16 blocks where the strips keep >= 2 rows
-            cs = (c->N <= 64 && c->N % 32 == 0) ? 16 : (c->N <= 64 && c->N % 16 == 0) ? 8 : 1;
-        else  // refined: the grid-wide cycles were faster at every size measured
-            cs = 1;
-    }
+    // thread-block clusters only on request: they were slower than the
+    // grid-wide cycles in the refined form, and slower than direct solves
+    const int cs = g.cluster_size == 0 ? 1 : g.cluster_size;
     if (cs > 1) {
         // the cluster arrays follow the coarsest inverses; they overlap the
         // shared-memory coarse part and tiles of the grid-wide cycle, which
@@ -344,6 +401,26 @@ int create_impl(qs_ctx *c) {
         const size_t cap_m = rm < lim ? rm : lim, cap_n = rn < lim ? rn : lim;
         c->band_rows = g.deposit_band_rows != 0 && cap_m >= 3 ? (int)cap_m : 0;
         c->band_rows_n = g.deposit_band_rows != 0 && cap_n >= 3 ? (int)cap_n : 0;
+    }
+    // Direct solves take even sides whose lines fit the block's buffers; a
+    // clustered launch keeps its multigrid cycles.
+    if (cs == 1 && c->N % 2 == 0 && c->N >= 8 && c->N <= 4096) {
+        const int r = create_fft(c);
+        if (r != QS_OK) return r;
+        // two buffers of gmax complex lines (at most 64 KB, at least one
+        // line each) over the multigrid's tiles, which a direct solve does
+        // not use, then the tables
+        FftArgs &f = c->fft;
+        f.gmax = 1;
+        while (f.gmax < 8 && (size_t)4 * f.gmax * c->N * sizeof(double2) <= 64 * 1024) f.gmax *= 2;
+        const size_t lines = c->block_offset + (size_t)2 * f.gmax * c->N * sizeof(double2);
+        if (lines + 256 > c->engine_smem) c->engine_smem = lines + 256;
+        const size_t tabs = (size_t)c->N * 24 + (size_t)(c->N / 2 + 1) * 16 + 256;
+        const size_t at = (c->engine_smem + 255) & ~(size_t)255;
+        if (c->N <= 1024 && at + tabs <= 200 * 1024) {
+            f.tab_off = (int)at;
+            c->engine_smem = at + tabs;
+        }
     }
     if (c->engine_smem > 220 * 1024)
         return fail(c, QS_ERR_ARG,
@@ -660,6 +737,7 @@ static int step_prepare(qs_ctx *c, const qs_beam *beams, int n_beams, const int3
         a.hist2[f] = c->hist2[f];
     }
     a.ws_order = g.warm_start_order;
+    a.fft = c->fft;
     a.nlev = c->nlev;
     for (int l = 0; l < c->nlev; ++l) {
         a.lev_n[l] = c->lev_n[l];

@@ -733,6 +733,7 @@ __device__ bool run_step(const EngineArgs &A, int bid, int nblk, const Sync &S, 
     DevScalars *sc = A.sc;
     const Thr T = grid_thr(bid, nblk);
     const bool lead = (bid == 0 && threadIdx.x == 0);
+    fft_load_tables(A, smem);
 
     using P = typename std::conditional<REF, float, double>::type;
     PS<P> Q;
@@ -802,13 +803,15 @@ __device__ bool run_step(const EngineArgs &A, int bid, int nblk, const Sync &S, 
             }
             __syncthreads();
             const Guess g = s_ctl.g;
+            Guess gp = g;  // direct solves take no guess
+            if (A.fft.on) gp.active = false;
             const double frac = s_ctl.frac;
-            phase_psi_rhs<P>(A, Q, ncur, nnext, base, j, q, frac, T, g);
+            phase_psi_rhs<P>(A, Q, ncur, nnext, base, j, q, frac, T, gp);
             if (!S(2)) return false;
             if (!mg_solve<REF>(A, S, Vpsi, slot, bid, nblk, smem, s_inv_ready)) return false;
             phase_moments<P>(A, Q, T, bid, nblk, smem);
             if (!S(3)) return false;
-            phase_assemble1<P>(A, Q, ncur, j, q, frac, T, g);
+            phase_assemble1<P>(A, Q, ncur, j, q, frac, T, gp);
             if (!S(4)) return false;
             if (!mg_solve<REF>(A, S, Veb, slot, bid, nblk, smem, s_inv_ready)) return false;
             phase_assemble2<P>(A, Q, ncur, T, g);

@@ -60,6 +60,19 @@ struct LevelArrays32 {
     float *d;
 };
 
+// Sine transforms of the direct solves (qs_fft.cuh): the tables in global
+// memory, per storage type, and two complex scratch grids.
+struct FftArgs {
+    int on;       // the uniform-grid Poisson problems are solved directly
+    int gmax;     // lines that fit a block's buffers
+    int tab_off;  // byte offset of the tables' copy in shared memory (0: none)
+    double2 *tw64, *dct64;
+    double *lam64;
+    float2 *tw32, *dct32;
+    float *lam32;
+    double2 *t1, *t2;
+};
+
 // Everything the slice engine reads or writes (passed by value).
 struct EngineArgs {
     // geometry (Sec. 3 normalised units)
@@ -91,6 +104,7 @@ struct EngineArgs {
     // warm start: solutions one and two slices back (psi, Ez, Bz, Bx, By)
     double *hist1[5], *hist2[5];
     int ws_order;
+    FftArgs fft;
     // coarse levels 1..nlev-1 (scratch shared by the three solves)
     int nlev;
     int lev_n[QS_MAX_LEV];

@@ -10,6 +10,7 @@
 #include <type_traits>
 
 #include "qs_cluster.cuh"
+#include "qs_fft.cuh"
 #include "qs_tile.cuh"
 
 namespace {
@@ -873,6 +874,70 @@ __device__ __noinline__ bool mg_solve_ref_cluster(const EngineArgs &A, const Syn
     return true;
 }
 
+// ---------------------------------------------------------------------------
+// direct solves by sine transforms (qs_fft.cuh)
+// ---------------------------------------------------------------------------
+
+// Copies the transform tables to shared memory, once per launch or instance.
+__device__ void fft_load_tables(const EngineArgs &A, void *smem_base) {
+    if (!A.fft.on || !A.fft.tab_off) return;
+    const int N = A.N, H = N / 2 + 1;
+    double2 *tw = (double2 *)((char *)smem_base + A.fft.tab_off);
+    double *lam = (double *)(tw + N + H);
+    for (int k = threadIdx.x; k < N; k += blockDim.x) {
+        tw[k] = A.fft.tw64[k];
+        if (k < H) tw[N + k] = A.fft.dct64[k];
+        lam[k] = A.fft.lam64[k];
+    }
+    __syncthreads();
+}
+
+__device__ __forceinline__ qsfft::Lines<double> fft_lines64(const EngineArgs &A,
+                                                            void *smem_base) {
+    qsfft::Lines<double> P;
+    P.N = A.N;
+    P.gmax = A.fft.gmax;
+    P.tw = A.fft.tw64;
+    P.dct = A.fft.dct64;
+    P.lam = A.fft.lam64;
+    if (A.fft.tab_off) {
+        P.tw = (const double2 *)((char *)smem_base + A.fft.tab_off);
+        P.dct = P.tw + P.N;
+        P.lam = (const double *)(P.dct + P.N / 2 + 1);
+    }
+    P.a = (double2 *)((char *)smem_base + A.block_smem_offset);
+    P.b = P.a + P.gmax * P.N;
+    return P;
+}
+
+// lap_h u = f for one field, or two at once as the parts of a complex one: three
+// grid phases in float64 whatever the right-hand side, against four to five
+// V-cycles of four phases each.
+template <int NC>
+__device__ bool direct_poisson(const EngineArgs &A, const Sync &S, const SolveSpec &V, int bid,
+                               int nblk, void *smem_base) {
+    const qsfft::Lines<double> P = fft_lines64(A, smem_base);
+    const int N = A.N;
+    const double *const f0 = V.f[0], *const f1 = NC == 2 ? V.f[1] : V.f[0] + N;
+    double *const u0 = V.u[0], *const u1 = NC == 2 ? V.u[1] : V.u[0] + N;
+    const int ld = NC == 2 ? N : 2 * N;
+    qsfft::rows_forward<double, NC>(P, bid, nblk, A.fft.t1, [&](int l, int x) {
+        const size_t i = (size_t)l * ld + x;
+        return make_double2(f0[i], f1[i]);
+    });
+    SYNC(26);
+    qsfft::columns<double, NC>(P, bid, nblk, A.fft.t1, A.fft.t2, 0.0);
+    SYNC(27);
+    qsfft::rows_inverse<double, NC>(P, bid, nblk, A.fft.t2, [&](int l, int x, double2 v) {
+        const size_t i = (size_t)l * ld + x;
+        u0[i] = v.x;
+        u1[i] = v.y;
+    });
+    if (bid == 0 && threadIdx.x == 0) A.sc->vcycles[V.kind] += 1;
+    SYNC(28);
+    return true;
+}
+
 // Iterate until, for every component,
 //   ||f - A u|| <= max(tol ||f||, 1e-13 ||u|| / h^2, atol)
 // (the second bound is a small multiple of the rounding level of the
@@ -883,6 +948,9 @@ template <bool REF>
 __device__ bool mg_solve(const EngineArgs &A, const Sync &S, const SolveSpec &V, int &slot,
                          int bid, int nblk, void *smem_base, int *inv_ready) {
     DevScalars *sc = A.sc;
+    if (A.fft.on && !V.screened)
+        return V.nc == 1 ? direct_poisson<1>(A, S, V, bid, nblk, smem_base)
+                         : direct_poisson<2>(A, S, V, bid, nblk, smem_base);
     // shared memory: [coarsest inverses][coarse levels + work][staged tile]
     void *smem = (char *)smem_base + A.block_smem_offset;
     const int mc = A.lev_n[A.nlev - 1] * A.lev_n[A.nlev - 1];
