@@ -145,18 +145,20 @@ __device__ void adj_prepare(const EngineArgs &A, const AdjArgs &D, const Slice &
     const bool base = (S.q == 0);
     const size_t fs = (size_t)A.n_xi * nn;
     const double *dh = (base && D.d_hist) ? D.d_hist + (size_t)S.j * nn : nullptr;
+    double sk = 0.0;
     for (int i = T.t0; i < nn; i += T.nt) {
         const int iy = i / n, ix = i - iy * n;
         double a = 1.0 + S.psi[i];
         if (a < A.psi_floor) a = A.psi_floor;
         const double kap = S.n[i] * (1.0 / a);
         A.kap[i] = kap;
+        sk += kap;
         const int nw = qsmg::walls(ix, iy, n);
         if (A.precision == QS_FP32_REFINED) {
             const float k32 = (float)kap;
             A.k32[i] = k32;
-            A.d32[i] = 1.f / ((float)(4 + nw) + A.lev_h2f[0] * k32);
-        } else {
+            if (!A.fft.on) A.d32[i] = 1.f / ((float)(4 + nw) + A.lev_h2f[0] * k32);
+        } else if (!A.fft.on) {
             A.invd0[i] = 1.0 / ((double)(4 + nw) + A.lev_h2[0] * kap);
         }
         A.dpx[i] = cdxo(S.psi, n, ix, i) * inv2h;
@@ -169,6 +171,8 @@ __device__ void adj_prepare(const EngineArgs &A, const AdjArgs &D, const Slice &
         D.g_dpx[i] = 0.0;
         D.g_dpy[i] = 0.0;
     }
+    sk = block_sum(sk);
+    if (threadIdx.x == 0) atomicAdd(&A.sc->ksum, sk);
 }
 
 // P1: reverse of the plasma push of this slice (Eqs. EoM_112_A, EoM_111 with
@@ -459,7 +463,7 @@ __device__ bool run_adjoint(const EngineArgs &A, const AdjArgs &D, int bid, int 
     DevScalars *sc = A.sc;
     const Thr T = grid_thr(bid, nblk);
     const bool lead = (bid == 0 && threadIdx.x == 0);
-    fft_load_tables(A, smem);
+    fft_load_tables<REF>(A, smem);
     const SolveSpec Vbp{2, 2, {D.mu_x, D.mu_y}, {D.g_bx, D.g_by}, true};
     const SolveSpec Veb{2, 1, {D.nu_ez, D.nu_bz}, {D.g_ez, D.g_bz}, false};
     const SolveSpec Vpsi{1, 0, {D.nu_psi, nullptr}, {D.f_nu_psi, nullptr}, false};
@@ -495,6 +499,7 @@ __device__ bool run_adjoint(const EngineArgs &A, const AdjArgs &D, int bid, int 
             sc->fnorm[0][0] = sc->fnorm[0][1] = 0.0;
             sc->fnorm[1][0] = sc->fnorm[1][1] = 0.0;
             sc->fnorm[2][0] = sc->fnorm[2][1] = 0.0;
+            sc->ksum = 0.0;
         }
         SYNC(108);
         // previous slice in forward order

@@ -261,25 +261,43 @@ int create_fft(qs_ctx *c) {
         if (k < half) dct32[k] = make_float2((float)dct[k].x, (float)dct[k].y);
         lam32[k] = (float)lam[k];
     }
-    auto &L = c->allocs;
+    // one allocation and one copy (a context is made per instance of a scan):
+    // [float64 tables][float32 tables][scratch and iteration grids]
+    const bool ref = c->cfg.precision == QS_FP32_REFINED;
+    const size_t nn = (size_t)n * n, cplx = ref ? sizeof(float2) : sizeof(double2);
+    const size_t tab64 = (size_t)n * 24 + (size_t)half * 16, tab32 = tab64 / 2;
+    const size_t tabs = (tab64 + tab32 + 255) & ~(size_t)255;
+    const size_t grids = nn * (2 * sizeof(double2) + 5 * cplx) + (ref ? 0 : 2 * nn * sizeof(double));
+    char *base = nullptr;
+    AL(c->allocs, base, tabs + grids);
+    std::vector<char> host(tabs);
     FftArgs &f = c->fft;
-    AL(L, f.tw64, n);
-    AL(L, f.dct64, half);
-    AL(L, f.lam64, n);
-    AL(L, f.tw32, n);
-    AL(L, f.dct32, half);
-    AL(L, f.lam32, n);
-    AL(L, f.t1, (size_t)n * n);
-    AL(L, f.t2, (size_t)n * n);
-    auto up = [](void *d, const void *h, size_t b) {
-        return cudaMemcpy(d, h, b, cudaMemcpyHostToDevice);
+    char *at = base;
+    auto put = [&](auto &ptr, const auto &v) {
+        const size_t bytes = v.size() * sizeof(v[0]);
+        std::memcpy(host.data() + (at - base), v.data(), bytes);
+        ptr = (decltype(+ptr))at;
+        at += bytes;
     };
-    CK(up(f.tw64, tw.data(), n * sizeof(double2)), "tables");
-    CK(up(f.dct64, dct.data(), half * sizeof(double2)), "tables");
-    CK(up(f.lam64, lam.data(), n * sizeof(double)), "tables");
-    CK(up(f.tw32, tw32.data(), n * sizeof(float2)), "tables");
-    CK(up(f.dct32, dct32.data(), half * sizeof(float2)), "tables");
-    CK(up(f.lam32, lam32.data(), n * sizeof(float)), "tables");
+    put(f.tw64, tw);
+    put(f.dct64, dct);
+    put(f.lam64, lam);
+    put(f.tw32, tw32);
+    put(f.dct32, dct32);
+    put(f.lam32, lam32);
+    at = base + tabs;
+    auto grid = [&](auto &ptr, size_t item) {
+        ptr = (decltype(+ptr))at;
+        at += nn * item;
+    };
+    grid(f.t1, sizeof(double2));
+    grid(f.t2, sizeof(double2));
+    for (void **q : {&f.cz, &f.cr, &f.cp, &f.cs, &f.ce}) grid(*q, cplx);
+    if (!ref) {
+        grid(c->r64[0], sizeof(double));
+        grid(c->r64[1], sizeof(double));
+    }
+    CK(cudaMemcpy(base, host.data(), tabs, cudaMemcpyHostToDevice), "tables");
     f.on = 1;
     return QS_OK;
 }
@@ -415,7 +433,7 @@ int create_impl(qs_ctx *c) {
         while (f.gmax < 8 && (size_t)4 * f.gmax * c->N * sizeof(double2) <= 64 * 1024) f.gmax *= 2;
         const size_t lines = c->block_offset + (size_t)2 * f.gmax * c->N * sizeof(double2);
         if (lines + 256 > c->engine_smem) c->engine_smem = lines + 256;
-        const size_t tabs = (size_t)c->N * 24 + (size_t)(c->N / 2 + 1) * 16 + 256;
+        const size_t tabs = (size_t)c->N * 36 + (size_t)(c->N / 2 + 1) * 24 + 256;
         const size_t at = (c->engine_smem + 255) & ~(size_t)255;
         if (c->N <= 1024 && at + tabs <= 200 * 1024) {
             f.tab_off = (int)at;

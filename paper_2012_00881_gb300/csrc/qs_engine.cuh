@@ -354,7 +354,7 @@ __device__ void phase_assemble1(const EngineArgs &A, const PS<P> &Q, const doubl
     const double *J0 = A.jzb + (size_t)j * nn;
     const double *J1 = (j + 1 < A.n_xi) ? A.jzb + (size_t)(j + 1) * nn : nullptr;
     unsigned hits = 0;
-    double sez = 0.0, sbz = 0.0;
+    double sez = 0.0, sbz = 0.0, sk = 0.0;
     for (int i = T.t0; i < nn; i += T.nt) {
         const int iy = i / n, ix = i - iy * n;
         if (g.active) {
@@ -374,12 +374,13 @@ __device__ void phase_assemble1(const EngineArgs &A, const PS<P> &Q, const doubl
         A.jz[i] = g_total(Q.G, ncur, i) * ia - nv + jzb;
         const double kap = nv * ia;
         A.kap[i] = kap;
+        sk += kap;
         const int nw = qsmg::walls(ix, iy, n);
         if (A.precision == QS_FP32_REFINED) {
             const float k32 = (float)kap;
             A.k32[i] = k32;
-            A.d32[i] = 1.f / ((float)(4 + nw) + A.lev_h2f[0] * k32);
-        } else {
+            if (!A.fft.on) A.d32[i] = 1.f / ((float)(4 + nw) + A.lev_h2f[0] * k32);
+        } else if (!A.fft.on) {
             A.invd0[i] = 1.0 / ((double)(4 + nw) + A.lev_h2[0] * kap);
         }
         A.dpx[i] = dxo(A.psi, n, ix, i, inv2h);
@@ -404,6 +405,8 @@ __device__ void phase_assemble1(const EngineArgs &A, const PS<P> &Q, const doubl
     if (threadIdx.x == 0) atomicAdd(&A.sc->fnorm[1][0], sez);
     sbz = block_sum(sbz);
     if (threadIdx.x == 0) atomicAdd(&A.sc->fnorm[1][1], sbz);
+    sk = block_sum(sk);
+    if (threadIdx.x == 0) atomicAdd(&A.sc->ksum, sk);
     add_hits(A.sc, hits);
 }
 
@@ -733,7 +736,7 @@ __device__ bool run_step(const EngineArgs &A, int bid, int nblk, const Sync &S, 
     DevScalars *sc = A.sc;
     const Thr T = grid_thr(bid, nblk);
     const bool lead = (bid == 0 && threadIdx.x == 0);
-    fft_load_tables(A, smem);
+    fft_load_tables<REF>(A, smem);
 
     using P = typename std::conditional<REF, float, double>::type;
     PS<P> Q;
@@ -798,20 +801,19 @@ __device__ bool run_step(const EngineArgs &A, int bid, int nblk, const Sync &S, 
             // (float64 divides repeated by every thread cost microseconds)
             __syncthreads();
             if (threadIdx.x == 0) {
-                s_ctl.g = make_guess(A.ws_order, have, xs, gx0, gx1, gx2);
+                if (!A.fft.on) s_ctl.g = make_guess(A.ws_order, have, xs, gx0, gx1, gx2);
                 s_ctl.frac = (double)q / (double)m;
             }
             __syncthreads();
-            const Guess g = s_ctl.g;
-            Guess gp = g;  // direct solves take no guess
-            if (A.fft.on) gp.active = false;
+            Guess g = s_ctl.g;
+            if (A.fft.on) g.active = false;  // the solves start from zero
             const double frac = s_ctl.frac;
-            phase_psi_rhs<P>(A, Q, ncur, nnext, base, j, q, frac, T, gp);
+            phase_psi_rhs<P>(A, Q, ncur, nnext, base, j, q, frac, T, g);
             if (!S(2)) return false;
             if (!mg_solve<REF>(A, S, Vpsi, slot, bid, nblk, smem, s_inv_ready)) return false;
             phase_moments<P>(A, Q, T, bid, nblk, smem);
             if (!S(3)) return false;
-            phase_assemble1<P>(A, Q, ncur, j, q, frac, T, gp);
+            phase_assemble1<P>(A, Q, ncur, j, q, frac, T, g);
             if (!S(4)) return false;
             if (!mg_solve<REF>(A, S, Veb, slot, bid, nblk, smem, s_inv_ready)) return false;
             phase_assemble2<P>(A, Q, ncur, T, g);
@@ -828,6 +830,7 @@ __device__ bool run_step(const EngineArgs &A, int bid, int nblk, const Sync &S, 
                 sc->fnorm[0][0] = sc->fnorm[0][1] = 0.0;
                 sc->fnorm[1][0] = sc->fnorm[1][1] = 0.0;
                 sc->fnorm[2][0] = sc->fnorm[2][1] = 0.0;
+                sc->ksum = 0.0;
             }
             if (!S(6)) return false;
             gx2 = gx1;

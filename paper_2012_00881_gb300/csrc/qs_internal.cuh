@@ -20,6 +20,8 @@ struct DevScalars {
     int err_where;                 // phase id of a timeout; -1: no clusters
     double rnorm[4][4];            // ||r||^2 (comps 0,1) and ||u||^2 (2,3), ring of 4
     double fnorm[3][2];            // ||f||^2 of the psi / (Ez,Bz) / (Bx,By) solves
+    double cgd[4][4];              // conjugate gradients: (r,z), (z,Az) per component, ring of 4
+    double ksum;                   // sum of kappa over the cells of this slice
     unsigned long long vmax_bits[2];  // V_max of a push (bits of a double >= 0)
     unsigned long long guard_hits;
     long long vcycles[3];
@@ -71,6 +73,9 @@ struct FftArgs {
     float2 *tw32, *dct32;
     float *lam32;
     double2 *t1, *t2;
+    // conjugate gradients of the screened solve, complex grids in the storage
+    // type of its inner iterations: z, r, p, A p, the correction e
+    void *cz, *cr, *cp, *cs, *ce;
 };
 
 // Everything the slice engine reads or writes (passed by value).
@@ -136,7 +141,7 @@ struct EngineArgs {
     // refined form: float32 copies of the push's fields (grad psi, B), so
     // that its gathers need no float64 conversions
     float *dpx32, *dpy32, *bx32, *by32, *bz32;
-    double *r64[2];  // float64 residual of the refined iteration
+    double *r64[2];  // float64 residual of the refined iterations
     LevelArrays32 lev32[QS_MAX_LEV];
     // cell sort of the plasma inside the slice loop: every sort_every base
     // slices (0: never) the particle arrays are reordered by (cell, id) into

@@ -879,33 +879,51 @@ __device__ __noinline__ bool mg_solve_ref_cluster(const EngineArgs &A, const Syn
 // ---------------------------------------------------------------------------
 
 // Copies the transform tables to shared memory, once per launch or instance.
+template <bool REF>
 __device__ void fft_load_tables(const EngineArgs &A, void *smem_base) {
     if (!A.fft.on || !A.fft.tab_off) return;
     const int N = A.N, H = N / 2 + 1;
     double2 *tw = (double2 *)((char *)smem_base + A.fft.tab_off);
     double *lam = (double *)(tw + N + H);
+    float2 *tw32 = (float2 *)(lam + N);
+    float *lam32 = (float *)(tw32 + N + H);
     for (int k = threadIdx.x; k < N; k += blockDim.x) {
         tw[k] = A.fft.tw64[k];
         if (k < H) tw[N + k] = A.fft.dct64[k];
         lam[k] = A.fft.lam64[k];
+        if (REF) {
+            tw32[k] = A.fft.tw32[k];
+            if (k < H) tw32[N + k] = A.fft.dct32[k];
+            lam32[k] = A.fft.lam32[k];
+        }
     }
     __syncthreads();
 }
 
-__device__ __forceinline__ qsfft::Lines<double> fft_lines64(const EngineArgs &A,
-                                                            void *smem_base) {
-    qsfft::Lines<double> P;
+template <typename T>
+__device__ __forceinline__ qsfft::Lines<T> fft_lines(const EngineArgs &A, void *smem_base) {
+    using V = qsfft::V2<T>;
+    qsfft::Lines<T> P;
     P.N = A.N;
     P.gmax = A.fft.gmax;
-    P.tw = A.fft.tw64;
-    P.dct = A.fft.dct64;
-    P.lam = A.fft.lam64;
-    if (A.fft.tab_off) {
-        P.tw = (const double2 *)((char *)smem_base + A.fft.tab_off);
-        P.dct = P.tw + P.N;
-        P.lam = (const double *)(P.dct + P.N / 2 + 1);
+    const size_t n = (size_t)P.N, h = n / 2 + 1;
+    const char *tab = (const char *)smem_base + A.fft.tab_off;
+    if constexpr (sizeof(T) == 8) {
+        P.tw = A.fft.tw64;
+        P.dct = A.fft.dct64;
+        P.lam = A.fft.lam64;
+    } else {
+        P.tw = A.fft.tw32;
+        P.dct = A.fft.dct32;
+        P.lam = A.fft.lam32;
+        tab += (n + h) * sizeof(double2) + n * sizeof(double);
     }
-    P.a = (double2 *)((char *)smem_base + A.block_smem_offset);
+    if (A.fft.tab_off) {
+        P.tw = (const V *)tab;
+        P.dct = P.tw + n;
+        P.lam = (const T *)(P.dct + h);
+    }
+    P.a = (V *)((char *)smem_base + A.block_smem_offset);
     P.b = P.a + P.gmax * P.N;
     return P;
 }
@@ -916,7 +934,7 @@ __device__ __forceinline__ qsfft::Lines<double> fft_lines64(const EngineArgs &A,
 template <int NC>
 __device__ bool direct_poisson(const EngineArgs &A, const Sync &S, const SolveSpec &V, int bid,
                                int nblk, void *smem_base) {
-    const qsfft::Lines<double> P = fft_lines64(A, smem_base);
+    const qsfft::Lines<double> P = fft_lines<double>(A, smem_base);
     const int N = A.N;
     const double *const f0 = V.f[0], *const f1 = NC == 2 ? V.f[1] : V.f[0] + N;
     double *const u0 = V.u[0], *const u1 = NC == 2 ? V.u[1] : V.u[0] + N;
@@ -938,6 +956,284 @@ __device__ bool direct_poisson(const EngineArgs &A, const Sync &S, const SolveSp
     return true;
 }
 
+// e at a cell and its five-point sum times h^2: sum of the neighbours minus
+// (4 + walls) e, exact to rounding of a float64 for float32 values (error-free
+// sums and an FMA product) without float64 arithmetic on the five values.
+__device__ __forceinline__ double five_point(float c, float w, float e, float n, float s,
+                                             float k) {
+    float hi = 0.f, lo = 0.f;
+    qstile::two_sum_acc(hi, lo, w);
+    qstile::two_sum_acc(hi, lo, e);
+    qstile::two_sum_acc(hi, lo, n);
+    qstile::two_sum_acc(hi, lo, s);
+    const float pc = __fmul_rn(k, c);
+    const float pe = __fmaf_rn(k, c, -pc);  // k c = pc + pe exactly
+    qstile::two_sum_acc(hi, lo, -pc);
+    lo = __fsub_rn(lo, pe);
+    return (double)hi + (double)lo;
+}
+__device__ __forceinline__ double five_point(double c, double w, double e, double n, double s,
+                                             double k) {
+    return (w + e) + (n + s) - k * c;
+}
+
+// The block's share of four sums into out[4]; clears the slots two uses ahead.
+__device__ void cg_reduce(DevScalars *sc, float v[4], double *out, int slot, int bid) {
+    block_sum4f(v);
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (v[k] != 0.f) atomicAdd(out + k, (double)v[k]);
+        if (bid == 0)
+            for (int k = 0; k < 4; ++k) sc->rnorm[(slot + 2) & 3][k] = sc->cgd[(slot + 2) & 3][k] = 0.0;
+    }
+}
+
+// (lap_h - kappa) u = f for the two components of B_perp by conjugate
+// gradients preconditioned with M = lap_h - kbar, kbar the mean of kappa, whose
+// inverse is a direct solve by sine transforms.  A z = M z + (kbar - kappa) z =
+// r + (kbar - kappa) z, so the operator costs one product a cell and every
+// vector update stays in the rows that the block transforms: an iteration is
+// three grid phases (columns; rows inverse with the dot products; update with
+// rows forward).  M^-1 A is a compact perturbation of the identity, so the
+// iteration converges superlinearly: 5 to 8 steps to 1e-10 on the 256^2
+// blowout (kappa 0 ... 18), 18 to 25 in a channel with kappa 1 ... 11, from a
+// zero guess (the extrapolated guess carries the macroparticle noise of three
+// slices: its residual is above the source's at the window's head).
+//
+// Refined form: the iteration runs in float32 on the residual equation, to
+// 1e-5 of the residual it starts from; then u += e, r <- r - A e in float64
+// and again.  Float64 form: in float64 to the tolerance; the same step then
+// checks it.  Both stop on the float64 residual.  The residual is scaled by a
+// power of two near 1 / ||f|| so that float32 cannot underflow.
+// Returns 1 (converged), 0 (not within its cap: u holds the last iterate and
+// the V-cycles take over), -1 (a barrier failed).
+template <bool REF>
+__device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &V, int &slot,
+                           int bid, int nblk, void *smem_base) {
+    using T = typename std::conditional<REF, float, double>::type;
+    using C = qsfft::V2<T>;
+    DevScalars *sc = A.sc;
+    const qsfft::Lines<T> P = fft_lines<T>(A, smem_base);
+    const int N = A.N;
+    C *const t1 = (C *)A.fft.t1, *const t2 = (C *)A.fft.t2;
+    C *const cz = (C *)A.fft.cz, *const cr = (C *)A.fft.cr, *const cp = (C *)A.fft.cp,
+             *const cs = (C *)A.fft.cs, *const ce = (C *)A.fft.ce;
+    __shared__ double s_scale[2], s_inv[2], s_thr[2], s_r0[2], s_ig[2], s_ia[2];
+    __shared__ T s_al[2], s_be[2], s_kbar;
+    __shared__ int s_go;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int any = 0;
+        for (int c = 0; c < 2; ++c) {
+            const double fn = vload(&sc->fnorm[V.kind][c]);
+            // 2^-k with k about half the exponent of ||f||^2 (a NaN or
+            // infinite source keeps 1: it fails the stopping test below)
+            const int ex = (int)((__double_as_longlong(fn) >> 52) & 0x7ff);
+            const int k = ex == 0 || ex == 0x7ff ? 0 : (ex - 1023) / 2;
+            s_scale[c] = __longlong_as_double((long long)(1023 - k) << 52);
+            s_inv[c] = __longlong_as_double((long long)(1023 + k) << 52);
+            const double s2 = s_scale[c] * s_scale[c];
+            s_thr[c] = fmax(A.mg_tol * A.mg_tol * fn, A.mg_atol * A.mg_atol) * s2;
+            s_r0[c] = fn * s2;
+            if (!(s_r0[c] <= s_thr[c])) any = 1;
+        }
+        s_kbar = (T)(vload(&sc->ksum) / ((double)N * (double)N));
+        s_go = any;
+    }
+    __syncthreads();
+    const T kbar = s_kbar;
+    const double sc0 = s_scale[0], sc1 = s_scale[1], is0 = s_inv[0], is1 = s_inv[1];
+    const bool any = s_go != 0;
+    if (!any) {  // both sources are rounding noise or zero
+        const Thr T0 = grid_thr(bid, nblk);
+        for (int c = 0; c < 2; ++c)
+            for (int i = T0.t0; i < N * N; i += T0.nt) {
+                V.u[c][i] = 0.0;
+                if (V.u32[c]) V.u32[c][i] = 0.f;
+            }
+        return S(50) ? 1 : -1;
+    }
+    auto dk = [&](size_t i) {  // kbar - kappa
+        if constexpr (REF) return kbar - A.k32[i];
+        else return kbar - A.kap[i];
+    };
+    qsfft::rows_forward<T, 2>(P, bid, nblk, t1, [&](int y, int x) {
+        const size_t i = (size_t)y * N + x;
+        const double f0 = V.f[0][i], f1 = V.f[1][i];
+        A.r64[0][i] = f0;
+        A.r64[1][i] = f1;
+        const C r = qsfft::mk<T>((T)(f0 * sc0), (T)(f1 * sc1));
+        cr[i] = r;
+        return r;
+    });
+    if (!S(51)) return -1;
+    const int cap = min(A.mg_max_vcycles, 48);
+    const double red = REF ? 1e-10 : 1e-26;  // inner reduction, squared
+    const double fl = 1e-13 * A.lev_inv_h2[0];
+    int it = 0, result = -2;
+    for (int outer = 0; result == -2; ++outer) {
+        for (int inner = 0;; ++inner) {
+            qsfft::columns<T, 2>(P, bid, nblk, t1, t2, kbar);
+            if (!S(52)) return -1;
+            float d[4] = {0.f, 0.f, 0.f, 0.f};
+            qsfft::rows_inverse<T, 2>(P, bid, nblk, t2, [&](int y, int x, C z) {
+                const size_t i = (size_t)y * N + x;
+                const C r = cr[i];
+                const T k = dk(i);
+                cz[i] = z;
+                d[0] += (float)(r.x * z.x);
+                d[1] += (float)(r.y * z.y);
+                d[2] += (float)(z.x * (r.x + k * z.x));
+                d[3] += (float)(z.y * (r.y + k * z.y));
+            });
+            cg_reduce(sc, d, sc->cgd[slot & 3], slot, bid);
+            if (!S(53)) return -1;
+            if (threadIdx.x < 2) {  // one thread a component: two float64 divides
+                const int c = threadIdx.x;
+                const double ga = vload(&sc->cgd[slot & 3][c]);
+                const double de = vload(&sc->cgd[slot & 3][2 + c]);
+                double be = 0.0, al = 0.0, ia = 0.0, ig = 0.0;
+                if (ga != 0.0) {
+                    ig = 1.0 / ga;
+                    be = inner > 0 ? ga * s_ig[c] : 0.0;
+                    ia = de * ig - be * (inner > 0 ? s_ia[c] : 0.0);
+                    al = ia != 0.0 ? 1.0 / ia : 0.0;
+                }
+                s_ig[c] = ig;
+                s_ia[c] = ia;
+                s_al[c] = (T)al;
+                s_be[c] = (T)be;
+            }
+            ++slot;
+            __syncthreads();
+            const T al0 = s_al[0], al1 = s_al[1], be0 = s_be[0], be1 = s_be[1];
+            const bool first = inner == 0;
+            float n[4] = {0.f, 0.f, 0.f, 0.f};
+            qsfft::rows_forward<T, 2>(P, bid, nblk, t1, [&](int y, int x) {
+                const size_t i = (size_t)y * N + x;
+                const C z = cz[i];
+                C r = cr[i];
+                const T k = dk(i);
+                C p = z, s = qsfft::mk<T>(r.x + k * z.x, r.y + k * z.y);
+                C e = qsfft::mk<T>(T(0), T(0));
+                if (!first) {
+                    const C po = cp[i], so = cs[i];
+                    e = ce[i];
+                    p.x += be0 * po.x;
+                    p.y += be1 * po.y;
+                    s.x += be0 * so.x;
+                    s.y += be1 * so.y;
+                }
+                e.x += al0 * p.x;
+                e.y += al1 * p.y;
+                r.x -= al0 * s.x;
+                r.y -= al1 * s.y;
+                cp[i] = p;
+                cs[i] = s;
+                ce[i] = e;
+                cr[i] = r;
+                n[0] += (float)(r.x * r.x);
+                n[1] += (float)(r.y * r.y);
+                return r;
+            });
+            cg_reduce(sc, n, sc->rnorm[slot & 3], slot, bid);
+            if (!S(54)) return -1;
+            ++it;
+            if (threadIdx.x == 0) {
+                int go = 0;
+                for (int c = 0; c < 2; ++c) {
+                    const double rn = vload(&sc->rnorm[slot & 3][c]);
+                    if (!(rn <= fmax(red * s_r0[c], 0.09 * s_thr[c]))) go = 1;
+                }
+                s_go = go;
+            }
+            ++slot;
+            __syncthreads();
+            const bool go = s_go != 0;
+            __syncthreads();  // s_go is rewritten by the next test
+            if (!go || it >= cap || inner >= 23) break;
+        }
+        // u += e, r <- r - A e in float64 with the norms of the stopping test;
+        // the new right-hand side goes through its row transform on the way
+        float n[4] = {0.f, 0.f, 0.f, 0.f};
+        const double ih2 = A.lev_inv_h2[0];
+        const bool fresh = outer == 0;
+        qsfft::rows_forward<T, 2>(P, bid, nblk, t1, [&](int y, int x) {
+            const size_t i = (size_t)y * N + x;
+            const C zero = qsfft::mk<T>(T(0), T(0));
+            const C e = ce[i];
+            const C ew = x > 0 ? ce[i - 1] : zero, ee = x < N - 1 ? ce[i + 1] : zero;
+            const C en = y > 0 ? ce[i - N] : zero, es = y < N - 1 ? ce[i + N] : zero;
+            const T cw = (T)(4 + qsmg::walls(x, y, N));
+            const double kap = A.kap[i];
+            const double a0 = five_point(e.x, ew.x, ee.x, en.x, es.x, cw) * ih2 - kap * (double)e.x;
+            const double a1 = five_point(e.y, ew.y, ee.y, en.y, es.y, cw) * ih2 - kap * (double)e.y;
+            const double r0 = A.r64[0][i] - a0 * is0, r1 = A.r64[1][i] - a1 * is1;
+            double u0 = (double)e.x * is0, u1 = (double)e.y * is1;
+            if (!fresh) {
+                u0 += V.u[0][i];
+                u1 += V.u[1][i];
+            }
+            V.u[0][i] = u0;
+            V.u[1][i] = u1;
+            if (V.u32[0]) {
+                V.u32[0][i] = (float)u0;
+                V.u32[1][i] = (float)u1;
+            }
+            A.r64[0][i] = r0;
+            A.r64[1][i] = r1;
+            const C r = qsfft::mk<T>((T)(r0 * sc0), (T)(r1 * sc1));
+            cr[i] = r;
+            const float v0 = (float)(u0 * sc0), v1 = (float)(u1 * sc1);
+            n[0] += (float)r.x * (float)r.x;
+            n[1] += (float)r.y * (float)r.y;
+            n[2] += v0 * v0;
+            n[3] += v1 * v1;
+            return r;
+        });
+        cg_reduce(sc, n, sc->rnorm[slot & 3], slot, bid);
+        if (!S(55)) return -1;
+        if (threadIdx.x == 0) {
+            int conv = 1, slow = 0;
+            for (int c = 0; c < 2; ++c) {
+                const double rn = vload(&sc->rnorm[slot & 3][c]);
+                const double un = vload(&sc->rnorm[slot & 3][2 + c]);
+                if (!(rn <= fmax(s_thr[c], fl * fl * un))) {
+                    conv = 0;
+                    if (!(rn <= 0.0625 * s_r0[c])) slow = 1;
+                }
+                s_r0[c] = rn;
+                if (bid == 0) {
+                    const double fn = vload(&sc->fnorm[V.kind][c]);
+                    const double rel = fn > 0.0 ? sqrt(rn / fn) * s_inv[c] : 0.0;
+                    if (conv && rel > sc->max_relres) sc->max_relres = rel;
+                }
+            }
+            s_go = conv ? 1 : (slow || it >= cap) ? 0 : -2;
+        }
+        ++slot;
+        __syncthreads();
+        result = s_go;
+        __syncthreads();
+    }
+    if (bid == 0 && threadIdx.x == 0) sc->vcycles[V.kind] += it;
+    return result;
+}
+
+// The screened smoother's inverse diagonal, needed only when the V-cycles
+// take over from the conjugate gradients.
+__device__ void screened_diagonal(const EngineArgs &A, Thr T) {
+    const int n = A.N;
+    for (qsmg::Walk w(T.t0, T.nt, n); w.q < n * n; w.next()) {
+        const int nw = qsmg::walls(w.col, w.row, n);
+        if (A.precision == QS_FP32_REFINED)
+            A.d32[w.q] = 1.f / ((float)(4 + nw) + A.lev_h2f[0] * A.k32[w.q]);
+        else
+            A.invd0[w.q] = 1.0 / ((double)(4 + nw) + A.lev_h2[0] * A.kap[w.q]);
+    }
+}
+
 // Iterate until, for every component,
 //   ||f - A u|| <= max(tol ||f||, 1e-13 ||u|| / h^2, atol)
 // (the second bound is a small multiple of the rounding level of the
@@ -951,6 +1247,12 @@ __device__ bool mg_solve(const EngineArgs &A, const Sync &S, const SolveSpec &V,
     if (A.fft.on && !V.screened)
         return V.nc == 1 ? direct_poisson<1>(A, S, V, bid, nblk, smem_base)
                          : direct_poisson<2>(A, S, V, bid, nblk, smem_base);
+    if (A.fft.on) {
+        const int r = cg_screened<REF>(A, S, V, slot, bid, nblk, smem_base);
+        if (r != 0) return r > 0;
+        screened_diagonal(A, grid_thr(bid, nblk));
+        SYNC(56);
+    }
     // shared memory: [coarsest inverses][coarse levels + work][staged tile]
     void *smem = (char *)smem_base + A.block_smem_offset;
     const int mc = A.lev_n[A.nlev - 1] * A.lev_n[A.nlev - 1];
