@@ -463,7 +463,7 @@ __device__ bool run_adjoint(const EngineArgs &A, const AdjArgs &D, int bid, int 
     DevScalars *sc = A.sc;
     const Thr T = grid_thr(bid, nblk);
     const bool lead = (bid == 0 && threadIdx.x == 0);
-    fft_load_tables<REF>(A, smem);
+    fft_load_tables<REF>(A);
     const SolveSpec Vbp{2, 2, {D.mu_x, D.mu_y}, {D.g_bx, D.g_by}, true};
     const SolveSpec Veb{2, 1, {D.nu_ez, D.nu_bz}, {D.g_ez, D.g_bz}, false};
     const SolveSpec Vpsi{1, 0, {D.nu_psi, nullptr}, {D.f_nu_psi, nullptr}, false};

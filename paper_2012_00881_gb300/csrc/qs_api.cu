@@ -267,7 +267,7 @@ int create_fft(qs_ctx *c) {
     const size_t nn = (size_t)n * n, cplx = ref ? sizeof(float2) : sizeof(double2);
     const size_t tab64 = (size_t)n * 24 + (size_t)half * 16, tab32 = tab64 / 2;
     const size_t tabs = (tab64 + tab32 + 255) & ~(size_t)255;
-    const size_t grids = nn * (2 * sizeof(double2) + 5 * cplx) + (ref ? 0 : 2 * nn * sizeof(double));
+    const size_t grids = nn * (2 * sizeof(double2) + 7 * cplx) + (ref ? 0 : 2 * nn * sizeof(double));
     char *base = nullptr;
     AL(c->allocs, base, tabs + grids);
     std::vector<char> host(tabs);
@@ -292,7 +292,7 @@ int create_fft(qs_ctx *c) {
     };
     grid(f.t1, sizeof(double2));
     grid(f.t2, sizeof(double2));
-    for (void **q : {&f.cz, &f.cr, &f.cp, &f.cs, &f.ce}) grid(*q, cplx);
+    for (void **q : {&f.cz, &f.cr, &f.cp, &f.cs, &f.ce, &f.tz, &f.tp}) grid(*q, cplx);
     if (!ref) {
         grid(c->r64[0], sizeof(double));
         grid(c->r64[1], sizeof(double));
@@ -420,24 +420,24 @@ int create_impl(qs_ctx *c) {
         c->band_rows = g.deposit_band_rows != 0 && cap_m >= 3 ? (int)cap_m : 0;
         c->band_rows_n = g.deposit_band_rows != 0 && cap_n >= 3 ? (int)cap_n : 0;
     }
-    // Direct solves take even sides whose lines fit the block's buffers; a
-    // clustered launch keeps its multigrid cycles.
-    if (cs == 1 && c->N % 2 == 0 && c->N >= 8 && c->N <= 4096) {
-        const int r = create_fft(c);
-        if (r != QS_OK) return r;
-        // two buffers of gmax complex lines (at most 64 KB, at least one
-        // line each) over the multigrid's tiles, which a direct solve does
-        // not use, then the tables
+    // Direct solves take even sides whose lines and tables fit in shared memory;
+    // a clustered launch keeps its multigrid cycles.
+    if (cs == 1 && c->N % 2 == 0 && c->N >= 8 && c->N <= 2048) {
+        // two buffers of gmax complex lines (64 KB, or one line each) over the
+        // multigrid's tiles, which a direct solve does not use, then the tables
         FftArgs &f = c->fft;
+        const size_t line = (size_t)(c->N + c->N / 8 + 1) * sizeof(double2);  // padded
         f.gmax = 1;
-        while (f.gmax < 8 && (size_t)4 * f.gmax * c->N * sizeof(double2) <= 64 * 1024) f.gmax *= 2;
-        const size_t lines = c->block_offset + (size_t)2 * f.gmax * c->N * sizeof(double2);
-        if (lines + 256 > c->engine_smem) c->engine_smem = lines + 256;
-        const size_t tabs = (size_t)c->N * 36 + (size_t)(c->N / 2 + 1) * 24 + 256;
-        const size_t at = (c->engine_smem + 255) & ~(size_t)255;
-        if (c->N <= 1024 && at + tabs <= 200 * 1024) {
-            f.tab_off = (int)at;
-            c->engine_smem = at + tabs;
+        while (f.gmax < 8 && 4 * f.gmax * line <= 76 * 1024) f.gmax *= 2;
+        size_t need = c->block_offset + 2 * f.gmax * line;
+        if (need < c->engine_smem) need = c->engine_smem;
+        need = (need + 255) & ~(size_t)255;
+        const size_t tabs = (size_t)c->N * (ref ? 36 : 24) + (size_t)(c->N / 2 + 1) * (ref ? 24 : 16);
+        if (need + tabs <= 220 * 1024) {
+            f.tab_off = (int)need;
+            c->engine_smem = need + tabs;
+            const int r = create_fft(c);
+            if (r != QS_OK) return r;
         }
     }
     if (c->engine_smem > 220 * 1024)

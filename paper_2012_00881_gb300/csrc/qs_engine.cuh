@@ -736,7 +736,7 @@ __device__ bool run_step(const EngineArgs &A, int bid, int nblk, const Sync &S, 
     DevScalars *sc = A.sc;
     const Thr T = grid_thr(bid, nblk);
     const bool lead = (bid == 0 && threadIdx.x == 0);
-    fft_load_tables<REF>(A, smem);
+    fft_load_tables<REF>(A);
 
     using P = typename std::conditional<REF, float, double>::type;
     PS<P> Q;

@@ -25,10 +25,30 @@
 
 #include <type_traits>
 
+#include "qs_ff.cuh"
+
 namespace qsfft {
 
+using qsff::Ff;
+
+// complex numbers of a storage type
+struct __align__(16) Ff2 {
+    Ff x, y;
+};
 template <typename T>
-using V2 = typename std::conditional<sizeof(T) == 8, double2, float2>::type;
+struct Cplx {
+    using type = float2;
+};
+template <>
+struct Cplx<double> {
+    using type = double2;
+};
+template <>
+struct Cplx<Ff> {
+    using type = Ff2;
+};
+template <typename T>
+using V2 = typename Cplx<T>::type;
 
 template <typename T>
 __device__ __forceinline__ V2<T> mk(T x, T y) {
@@ -63,178 +83,295 @@ __device__ __forceinline__ V cmul(V a, V w) {
     return r;
 }
 
-// Tables and line buffers of a block.  tw[k] = e^{-2 pi i k / N}, k < N;
-// dct[j] = e^{-i pi j / 2N}, j <= N/2; lam[j] = -(2 + 2 cos(pi j / N)) / h^2,
-// the eigenvalue of cosine index j.  a, b: G lines of N complex values each.
+// The block's dynamic shared memory (every kernel's extern array is this one):
+// buffers and tables are passed as byte offsets into it, so that all accesses
+// compile to shared-memory instructions across calls.
+__device__ __forceinline__ char *dyn_smem() {
+    extern __shared__ double smem[];
+    return (char *)smem;
+}
 template <typename T>
+__device__ __forceinline__ V2<T> *cplx_at(int off) {
+    return (V2<T> *)(dyn_smem() + off);
+}
+
+// Line buffers and tables of a block, all in shared memory: a, b hold gmax
+// lines of N complex values each; at tab: tw[k] = e^{-2 pi i k / N}, k < N;
+// dct[j] = e^{-i pi j / 2N}, j <= N/2; lam[j] = -(2 + 2 cos(pi j / N)) / h^2, the
+// eigenvalue of cosine index j.
 struct Lines {
-    int N, gmax;
-    const V2<T> *tw, *dct;
-    const T *lam;
-    V2<T> *a, *b;
+    int N, gmax, a, tab;
+};
+template <typename T>
+__device__ __forceinline__ const V2<T> *dct_table(int tab, int N) {
+    return cplx_at<T>(tab) + N;
+}
+template <typename T>
+__device__ __forceinline__ const T *lam_table(int tab, int N) {
+    return (const T *)(cplx_at<T>(tab) + N + N / 2 + 1);
+}
+
+// Where point i of a line sits in its buffer: one free element after every 128
+// bytes, so that the strided writes of a radix-8 pass fall into different
+// banks (512 points, four lines: 1,150 -> 350 cycles a pass).
+template <typename T>
+__host__ __device__ __forceinline__ constexpr int pad(int i) {
+    return i + (i >> (sizeof(T) == 8 ? 3 : 4));
+}
+// elements of a padded line of N points
+template <typename T>
+__host__ __device__ __forceinline__ constexpr int line_len(int N) {
+    return pad<T>(N - 1) + 1;
+}
+
+template <typename T>
+__device__ __forceinline__ int buf_b(const Lines &P) {
+    return P.a + P.gmax * line_len<T>(P.N) * (int)sizeof(V2<T>);
+}
+// A thread's items of a line-wise loop: the block's warps are dealt to G (a power
+// of two) lines in turn, so that a loop with few items still uses all four
+// schedulers (and FP64 units) of the SM; an index computed by division or by a
+// loop costs 250 cycles a pass, this one a few.
+struct Deal {
+    int g, j0, stride;
+    __device__ __forceinline__ explicit Deal(int lgG) {
+        const int w = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
+        g = w & ((1 << lgG) - 1);
+        j0 = ((w >> lgG) << 5) + lane;
+        stride = (int)blockDim.x >> lgG;
+    }
 };
 
-// index t over lines of n items: (line, item); few lines per block, so a
-// subtraction loop is cheaper than a division
-struct Split {
-    int g, j, n;
-    __device__ Split(int n_) : g(0), j((int)threadIdx.x), n(n_) { wrap(); }
-    __device__ void wrap() {
-        while (j >= n) {
-            j -= n;
-            ++g;
-        }
-    }
-    __device__ void next() {
-        j += (int)blockDim.x;
-        wrap();
-    }
-};
+// -i v forward, +i v inverse
+template <bool INV, typename V>
+__device__ __forceinline__ V mul_i(V v) {
+    V r;
+    r.x = INV ? -v.y : v.y;
+    r.y = INV ? v.x : -v.x;
+    return r;
+}
 
-// One Stockham pass of radix R over gl lines: the sub-transforms done so far
-// have length Ns (a power of two).
+template <typename T, bool INV, typename V>
+__device__ __forceinline__ void dft4(V &a, V &b, V &c, V &d) {
+    const V s02 = cadd(a, c), d02 = csub(a, c);
+    const V s13 = cadd(b, d), q = mul_i<INV>(csub(b, d));
+    a = cadd(s02, s13);
+    b = cadd(d02, q);
+    c = csub(s02, s13);
+    d = csub(d02, q);
+}
+
+// One Stockham pass of radix R over gl lines of N points: the sub-transforms
+// done so far have length Ns = N / n (a power of two).
 template <typename T, int R, bool INV>
-__device__ __forceinline__ void pass(const Lines<T> &P, const V2<T> *src, V2<T> *dst, int Ns,
-                                     int gl) {
+__device__ __forceinline__ void pass(const V2<T> *src, V2<T> *dst, const V2<T> *tw, int N, int n,
+                                     int Ns, const Deal &D, int gl) {
     using V = V2<T>;
-    const int nb = P.N / R, step = nb / Ns;
-    for (Split s(nb); s.g < gl; s.next()) {
-        const int j = s.j, k = j & (Ns - 1);
-        const V *x = src + s.g * P.N;
-        V *y = dst + s.g * P.N + (j - k) * R + k;
+    const int nb = (unsigned)N / R, step = (unsigned)n / R, line = D.g * line_len<T>(N);
+    for (int j = D.g < gl ? D.j0 : nb; j < nb; j += D.stride) {
+        const int k = j & (Ns - 1), ks = k * step, o = (j - k) * R + k;
+        const V *x = src + line;
+        V *y = dst + line;
         V v[R];
-        v[0] = x[j];
 #pragma unroll
-        for (int r = 1; r < R; ++r) {
-            v[r] = x[j + r * nb];
-            if (Ns > 1) v[r] = cmul<INV>(v[r], P.tw[k * r * step]);
+        for (int r = 0; r < R; ++r) v[r] = x[pad<T>(j + r * nb)];
+        if (Ns > 1) {
+            if constexpr (std::is_same<T, float>::value && (R == 4 || R == 8)) {
+                // powers of one twiddle: its multiples' table entries lie in
+                // few banks (512 points, four lines: 1,400 cycles a pass)
+                const V w1 = tw[ks], w2 = cmul<false>(w1, w1), w3 = cmul<false>(w2, w1);
+                v[1] = cmul<INV>(v[1], w1);
+                v[2] = cmul<INV>(v[2], w2);
+                v[3] = cmul<INV>(v[3], w3);
+                if constexpr (R == 8) {
+                    const V w4 = cmul<false>(w2, w2);
+                    v[4] = cmul<INV>(v[4], w4);
+                    v[5] = cmul<INV>(v[5], cmul<false>(w4, w1));
+                    v[6] = cmul<INV>(v[6], cmul<false>(w4, w2));
+                    v[7] = cmul<INV>(v[7], cmul<false>(w4, w3));
+                }
+            } else {
+#pragma unroll
+                for (int r = 1; r < R; ++r) v[r] = cmul<INV>(v[r], tw[r * ks]);
+            }
         }
+        auto put = [&](int r, V q) { y[pad<T>(o + r * Ns)] = q; };
         if constexpr (R == 2) {
-            y[0] = cadd(v[0], v[1]);
-            y[Ns] = csub(v[0], v[1]);
+            put(0, cadd(v[0], v[1]));
+            put(1, csub(v[0], v[1]));
         } else if constexpr (R == 4) {
-            const V s02 = cadd(v[0], v[2]), d02 = csub(v[0], v[2]);
-            const V s13 = cadd(v[1], v[3]), d13 = csub(v[1], v[3]);
-            // -i d13 forward, +i d13 inverse
-            const V q = INV ? mk<T>(-d13.y, d13.x) : mk<T>(d13.y, -d13.x);
-            y[0] = cadd(s02, s13);
-            y[Ns] = cadd(d02, q);
-            y[2 * Ns] = csub(s02, s13);
-            y[3 * Ns] = csub(d02, q);
+            dft4<T, INV>(v[0], v[1], v[2], v[3]);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) put(r, v[r]);
+        } else if constexpr (R == 8) {
+            // even and odd halves, the odd one turned by multiples of pi / 4
+            dft4<T, INV>(v[0], v[2], v[4], v[6]);
+            dft4<T, INV>(v[1], v[3], v[5], v[7]);
+            const T h = T(0.70710678118654752440);
+            const V q1 = mul_i<INV>(v[3]), q3 = mul_i<INV>(v[7]);
+            const V o1 = mk<T>(h * (v[3].x + q1.x), h * (v[3].y + q1.y));
+            const V o2 = mul_i<INV>(v[5]);
+            const V o3 = mk<T>(h * (q3.x - v[7].x), h * (q3.y - v[7].y));
+            put(0, cadd(v[0], v[1]));
+            put(1, cadd(v[2], o1));
+            put(2, cadd(v[4], o2));
+            put(3, cadd(v[6], o3));
+            put(4, csub(v[0], v[1]));
+            put(5, csub(v[2], o1));
+            put(6, csub(v[4], o2));
+            put(7, csub(v[6], o3));
         } else {
 #pragma unroll
-            for (int o = 0; o < R; ++o) {
+            for (int q = 0; q < R; ++q) {
                 V t = v[0];
 #pragma unroll
-                for (int r = 1; r < R; ++r) t = cadd(t, cmul<INV>(v[r], P.tw[((o * r) % R) * nb]));
-                y[o * Ns] = t;
+                for (int r = 1; r < R; ++r) t = cadd(t, cmul<INV>(v[r], tw[((q * r) % R) * nb]));
+                put(q, t);
             }
         }
     }
+    __syncthreads();
 }
 
-// The transform of the gl lines in P.a; returns the buffer that holds the
-// result (the other one is free).  Every thread of the block; the caller has
-// synchronised the block after filling P.a.
+// Powers of two with every size a constant.  float32: radix 8 while more than 4
+// or 16 is left, then 4.  Pairs: radix 4, whose 300 instructions on two warps a
+// 256-point line finish sooner than radix 8's 900 on one (4,400 -> 2,340
+// cycles a transform).  LGS: log2 of the sub-transforms done.
+template <typename T, bool INV, int LG, int LGS>
+__device__ __forceinline__ bool pow2(V2<T> *a, V2<T> *b, const V2<T> *tw, const Deal &D, int gl) {
+    constexpr int left = LG - LGS;
+    if constexpr (left == 0) {
+        return false;
+    } else {
+        constexpr bool four = !std::is_same<T, float>::value || left == 2 || left == 4;
+        constexpr int lr = left == 1 ? 1 : four ? 2 : 3;
+        pass<T, 1 << lr, INV>(a, b, tw, 1 << LG, 1 << left, 1 << LGS, D, gl);
+        return !pow2<T, INV, LG, LGS + lr>(b, a, tw, D, gl);
+    }
+}
+
+// The transform of the gl lines at offset `a`; returns the offset of the buffer
+// that holds the result, a or b.  Every thread of the block; the caller has
+// synchronised the block after filling the lines.  Out of line: the slice
+// engine's phases would otherwise hold a dozen copies and run from a cold
+// instruction cache.
+//
+// float32 is bound by the passes' latency (shared memory, block barrier): few
+// passes of a high radix with constant sizes (256 points, two lines: 1,780 ->
+// 950 cycles).  float64 is bound by the FP64 pipe: a warp-wide
+// instruction occupies one of the SM's four units for 64 cycles however many
+// lanes are active, and a radix-4 pass on fewer than 128 butterflies leaves
+// units idle; radix 2 has twice as many, each less than half the work.
 template <typename T, bool INV>
-__device__ V2<T> *fft(const Lines<T> &P, int gl) {
-    V2<T> *src = P.a, *dst = P.b;
-    int Ns = 1, n = P.N;
-    // float64: a pass on fewer than 128 radix-4 butterflies would leave some of
-    // the SM's four FP64 units idle; radix 2 has twice as many, each less than
-    // half the work (256 points, one line: 4.1k against 7.2k pipe cycles)
-    const bool r4 = sizeof(T) == 4 || gl * P.N >= 512;
-    auto done = [&](int R) {
-        V2<T> *t = src;
-        src = dst;
-        dst = t;
+__device__ __noinline__ int fft(int a, int b, int tab, int N, int lgG, int gl) {
+    const V2<T> *tw = cplx_at<T>(tab);
+    const Deal D(lgG);
+    constexpr bool fp64 = std::is_same<T, double>::value;
+    if constexpr (!fp64) {
+        V2<T> *const pa = cplx_at<T>(a), *const pb = cplx_at<T>(b);
+        switch (N) {
+        case 32: return pow2<T, INV, 5, 0>(pa, pb, tw, D, gl) ? b : a;
+        case 64: return pow2<T, INV, 6, 0>(pa, pb, tw, D, gl) ? b : a;
+        case 128: return pow2<T, INV, 7, 0>(pa, pb, tw, D, gl) ? b : a;
+        case 256: return pow2<T, INV, 8, 0>(pa, pb, tw, D, gl) ? b : a;
+        case 512: return pow2<T, INV, 9, 0>(pa, pb, tw, D, gl) ? b : a;
+        case 1024: return pow2<T, INV, 10, 0>(pa, pb, tw, D, gl) ? b : a;
+        default: break;
+        }
+    }
+    int Ns = 1, n = N;
+    auto run = [&](auto radix) {
+        constexpr int R = decltype(radix)::value;
+        pass<T, R, INV>(cplx_at<T>(a), cplx_at<T>(b), tw, N, n, Ns, D, gl);
+        const int t = a;
+        a = b;
+        b = t;
         Ns *= R;
-        n /= R;
-        __syncthreads();
+        n = (unsigned)n / R;
     };
-    while (r4 && (n & 3) == 0) {
-        pass<T, 4, INV>(P, src, dst, Ns, gl);
-        done(4);
-    }
-    while ((n & 1) == 0) {
-        pass<T, 2, INV>(P, src, dst, Ns, gl);
-        done(2);
-    }
-    if (n == 3) {
-        pass<T, 3, INV>(P, src, dst, Ns, gl);
-        done(3);
-    } else if (n == 5) {
-        pass<T, 5, INV>(P, src, dst, Ns, gl);
-        done(5);
-    } else if (n == 7) {
-        pass<T, 7, INV>(P, src, dst, Ns, gl);
-        done(7);
-    }
-    return src;
+    while ((!fp64 || gl * N >= 512) && (n & 3) == 0) run(std::integral_constant<int, 4>());
+    while ((n & 1) == 0) run(std::integral_constant<int, 2>());
+    if (n == 3) run(std::integral_constant<int, 3>());
+    else if (n == 5) run(std::integral_constant<int, 5>());
+    else if (n == 7) run(std::integral_constant<int, 7>());
+    return a;
 }
 
-// Lines a block takes at a time: as few as spread nl lines over nblk blocks in
-// one round (a power of two), at most gmax.
+// log2 of the lines a block takes at a time: as few as spread nl lines over nblk
+// blocks in one round, at most gmax.
 __device__ __forceinline__ int lines_at_once(int nl, int nblk, int gmax) {
-    int g = 1;
-    while (g < gmax && g * nblk < nl) g <<= 1;
-    return g;
+    int lg = 0;
+    while ((1 << lg) < gmax && (nblk << lg) < nl) ++lg;
+    return lg;
 }
 
 // Where sample i of a line sits in the FFT input; odd samples change sign.
 __device__ __forceinline__ int slot_of(int i, int N) { return (i & 1) ? N - 1 - (i >> 1) : i >> 1; }
 
+// The second half of rows_forward: transform of the filled lines l0 ... and
+// the coefficients (times 2) to `out`.
+template <typename T, int NC>
+__device__ __noinline__ void rows_forward_rest(int a, int b, int tab, int N, int l0, int lgG, int gl,
+                                               V2<T> *out) {
+    using V = V2<T>;
+    const Deal D(lgG);
+    __syncthreads();
+    const V *r = cplx_at<T>(fft<T, false>(a, b, tab, N, lgG, gl));
+    const V *dct = dct_table<T>(tab, N);
+    for (int j = D.g < gl ? D.j0 : N; 2 * j <= N; j += D.stride) {
+        const V *x = r + D.g * line_len<T>(N);
+        V c, d;
+        if (j == 0) {
+            c = cadd(x[0], x[0]);
+            d = c;
+        } else {
+            const V w = dct[j];
+            const V A = cmul<false>(x[pad<T>(j)], w), B = cmul<true>(x[pad<T>(N - j)], w);
+            const V m = csub(A, B);
+            c = cadd(A, B);
+            d = mk<T>(-m.y, m.x);
+        }
+        const bool two = j > 0 && 2 * j < N;
+        if constexpr (NC == 2) {
+            V *o = out + (size_t)(l0 + D.g) * N;
+            o[j] = c;
+            if (two) o[N - j] = d;
+        } else {
+            T *o = (T *)out + (size_t)(2 * (l0 + D.g)) * N;
+            o[j] = c.x;
+            o[N + j] = c.y;
+            if (two) {
+                o[N - j] = d.x;
+                o[2 * N - j] = d.y;
+            }
+        }
+    }
+    __syncthreads();
+}
+
 // Rows forward.  Two components (NC = 2): line y is the complex row of both.
 // One component: line p is rows 2p (real part) and 2p + 1.  load(line, x) gives
-// the samples; the coefficients (times 2) go to `out`, complex [y][j] or real
-// [y][j].
+// the samples; the coefficients go to `out`, complex [y][j] or real [y][j].
 template <typename T, int NC, typename F>
-__device__ void rows_forward(const Lines<T> &P, int bid, int nblk, V2<T> *out, F load) {
+__device__ __forceinline__ void rows_forward(const Lines &P, int bid, int nblk, V2<T> *out,
+                                             F load) {
     using V = V2<T>;
     const int N = P.N, nl = NC == 2 ? N : N / 2;
-    const int G = lines_at_once(nl, nblk, P.gmax);
+    const int lgG = lines_at_once(nl, nblk, P.gmax), G = 1 << lgG;
+    const Deal D(lgG);
+    V *const a = cplx_at<T>(P.a);
     for (int l0 = bid * G; l0 < nl; l0 += nblk * G) {
         const int gl = min(G, nl - l0);
-        for (Split s(N); s.g < gl; s.next()) {
-            V v = load(l0 + s.g, s.j);
-            if (s.j & 1) v = mk<T>(-v.x, -v.y);
-            P.a[s.g * N + slot_of(s.j, N)] = v;
+        for (int x = D.g < gl ? D.j0 : N; x < N; x += D.stride) {
+            V v = load(l0 + D.g, x);
+            if (x & 1) v = mk<T>(-v.x, -v.y);
+            a[D.g * line_len<T>(N) + pad<T>(slot_of(x, N))] = v;
         }
-        __syncthreads();
-        const V *r = fft<T, false>(P, gl);
-        for (Split s(N / 2 + 1); s.g < gl; s.next()) {
-            const int j = s.j;
-            const V *x = r + s.g * N;
-            V c, d;
-            if (j == 0) {
-                c = cadd(x[0], x[0]);
-                d = c;
-            } else {
-                const V w = P.dct[j];
-                const V A = cmul<false>(x[j], w), B = cmul<true>(x[N - j], w);
-                const V m = csub(A, B);
-                c = cadd(A, B);
-                d = mk<T>(-m.y, m.x);
-            }
-            const bool two = j > 0 && 2 * j < N;
-            if constexpr (NC == 2) {
-                V *o = out + (size_t)(l0 + s.g) * N;
-                o[j] = c;
-                if (two) o[N - j] = d;
-            } else {
-                T *o = (T *)out + (size_t)(2 * (l0 + s.g)) * N;
-                o[j] = c.x;
-                o[N + j] = c.y;
-                if (two) {
-                    o[N - j] = d.x;
-                    o[2 * N - j] = d.y;
-                }
-            }
-        }
-        __syncthreads();
+        rows_forward_rest<T, NC>(P.a, buf_b<T>(P), P.tab, N, l0, lgG, gl, out);
     }
 }
 
+using qsff::recip;
 // 1 / d for d != 0: float32 directly, float64 by two Newton steps from the
 // float32 reciprocal (a float64 divide is a long sequence on the FP64 pipe)
 __device__ __forceinline__ float recip(float d) { return 1.f / d; }
@@ -245,104 +382,156 @@ __device__ __forceinline__ double recip(double d) {
     return r;
 }
 
-// Columns: forward, times 1 / (4 N^2 (lam_x + lam_y - kbar)), inverse.  The
-// one-component array seen as complex pairs puts columns 2p and 2p + 1 into
-// line p.  in and out may not overlap.
+// The rest of `columns` after its lines are filled: forward, times
+// 1 / (4 N^2 (lam_x + lam_y - kbar)), inverse, and the store.
 template <typename T, int NC>
-__device__ void columns(const Lines<T> &P, int bid, int nblk, const V2<T> *in, V2<T> *out,
-                        T kbar) {
+__device__ __noinline__ void columns_rest(int a, int b, int tab, int N, int l0, int lgG, int gl,
+                                          V2<T> *out, T kbar) {
+    using V = V2<T>;
+    const int nl = NC == 2 ? N : N / 2, G = 1 << lgG;
+    const Deal D(lgG);
+    const T c4 = recip(T(4 * N * N));
+    const V *const dct = dct_table<T>(tab, N);
+    const T *const lam = lam_table<T>(tab, N);
+    __syncthreads();
+    const int f = fft<T, false>(a, b, tab, N, lgG, gl);
+    for (int j = D.g < gl ? D.j0 : N; 2 * j <= N; j += D.stride) {
+        const int l = l0 + D.g;
+        const T lx0 = lam[NC == 2 ? l : 2 * l] - kbar;
+        const T lx1 = NC == 2 ? lx0 : lam[2 * l + 1] - kbar;
+        auto scaled = [&](V c, int jj) {
+            const T ly = lam[jj];
+            const T s0 = c4 * recip(lx0 + ly);
+            const T s1 = NC == 2 ? s0 : c4 * recip(lx1 + ly);
+            return mk<T>(c.x * s0, c.y * s1);
+        };
+        V *x = cplx_at<T>(f) + D.g * line_len<T>(N);
+        if (j == 0) {
+            x[0] = scaled(cadd(x[0], x[0]), 0);
+            continue;
+        }
+        const V w = dct[j];
+        const V A = cmul<false>(x[pad<T>(j)], w), B = cmul<true>(x[pad<T>(N - j)], w);
+        const V c = scaled(cadd(A, B), j), m = csub(A, B);
+        // -i C_{N-j} with C_{N-j} = i m scaled: the parts swap twice
+        V d = scaled(mk<T>(-m.y, m.x), N - j);
+        d = mk<T>(d.y, -d.x);
+        x[pad<T>(j)] = cmul<true>(cadd(c, d), w);
+        if (2 * j < N) x[pad<T>(N - j)] = cmul<false>(csub(c, d), w);
+    }
+    __syncthreads();
+    const V *r = cplx_at<T>(fft<T, true>(f, f == a ? b : a, tab, N, lgG, gl));
+    for (int t = threadIdx.x; t < (N << lgG); t += blockDim.x) {
+        const int y = t >> lgG, g = t & (G - 1);
+        if (g >= gl) continue;
+        V v = r[g * line_len<T>(N) + pad<T>(slot_of(y, N))];
+        if (y & 1) v = mk<T>(-v.x, -v.y);
+        out[(size_t)y * nl + l0 + g] = v;
+    }
+    __syncthreads();
+}
+
+// Columns: load(y, line) gives the row coefficients; the solution's row
+// coefficients go to `out`.  The one-component array seen as complex pairs puts
+// columns 2p and 2p + 1 into line p.
+template <typename T, int NC, typename F>
+__device__ __forceinline__ void columns(const Lines &P, int bid, int nblk, V2<T> *out, T kbar,
+                                        F load) {
     using V = V2<T>;
     const int N = P.N, nl = NC == 2 ? N : N / 2;
-    const int G = lines_at_once(nl, nblk, P.gmax);
-    const int sh = 31 - __clz(G);
-    const T c4 = T(0.25) / ((T)N * (T)N);
+    const int lgG = lines_at_once(nl, nblk, P.gmax), G = 1 << lgG;
+    V *const a = cplx_at<T>(P.a);
     for (int l0 = bid * G; l0 < nl; l0 += nblk * G) {
         const int gl = min(G, nl - l0);
-        for (int t = threadIdx.x; t < (N << sh); t += blockDim.x) {
-            const int y = t >> sh, g = t & (G - 1);
+        for (int t = threadIdx.x; t < (N << lgG); t += blockDim.x) {
+            const int y = t >> lgG, g = t & (G - 1);
             if (g >= gl) continue;
-            V v = in[(size_t)y * nl + l0 + g];
+            V v = load(y, l0 + g);
             if (y & 1) v = mk<T>(-v.x, -v.y);
-            P.a[g * N + slot_of(y, N)] = v;
+            a[g * line_len<T>(N) + pad<T>(slot_of(y, N))] = v;
         }
-        __syncthreads();
-        Lines<T> Q = P;
-        Q.a = fft<T, false>(P, gl);
-        Q.b = Q.a == P.a ? P.b : P.a;
-        for (Split s(N / 2 + 1); s.g < gl; s.next()) {
-            const int j = s.j, l = l0 + s.g;
-            const T lx0 = P.lam[NC == 2 ? l : 2 * l] - kbar;
-            const T lx1 = NC == 2 ? lx0 : P.lam[2 * l + 1] - kbar;
-            auto scaled = [&](V c, int jj) {
-                const T ly = P.lam[jj];
-                const T s0 = c4 * recip(lx0 + ly);
-                const T s1 = NC == 2 ? s0 : c4 * recip(lx1 + ly);
-                return mk<T>(c.x * s0, c.y * s1);
-            };
-            V *x = Q.a + s.g * N;
-            if (j == 0) {
-                x[0] = scaled(cadd(x[0], x[0]), 0);
-                continue;
+        columns_rest<T, NC>(P.a, buf_b<T>(P), P.tab, N, l0, lgG, gl, out, kbar);
+    }
+}
+
+// The first half of rows_inverse: coefficients of lines l0 ... to samples;
+// returns the offset of the buffer that holds them.
+template <typename T, int NC>
+__device__ __noinline__ int rows_inverse_first(int a, int b, int tab, int N, int l0, int lgG, int gl,
+                                               const V2<T> *in) {
+    using V = V2<T>;
+    const V *const dct = dct_table<T>(tab, N);
+    const Deal D(lgG);
+    for (int j = D.g < gl ? D.j0 : N; 2 * j <= N; j += D.stride) {
+        const int l = l0 + D.g;
+        auto coef = [&](int jj) {
+            if constexpr (NC == 2) {
+                return in[(size_t)l * N + jj];
+            } else {
+                const T *o = (const T *)in + (size_t)(2 * l) * N;
+                return mk<T>(o[jj], o[N + jj]);
             }
-            const V w = P.dct[j];
-            const V A = cmul<false>(x[j], w), B = cmul<true>(x[N - j], w);
-            const V c = scaled(cadd(A, B), j), m = csub(A, B);
-            // -i C_{N-j} with C_{N-j} = i m scaled: the parts swap twice
-            V d = scaled(mk<T>(-m.y, m.x), N - j);
-            d = mk<T>(d.y, -d.x);
-            x[j] = cmul<true>(cadd(c, d), w);
-            if (2 * j < N) x[N - j] = cmul<false>(csub(c, d), w);
+        };
+        V *x = cplx_at<T>(a) + D.g * line_len<T>(N);
+        const V c = coef(j);
+        if (j == 0) {
+            x[0] = c;
+            continue;
         }
-        __syncthreads();
-        const V *r = fft<T, true>(Q, gl);
-        for (int t = threadIdx.x; t < (N << sh); t += blockDim.x) {
-            const int y = t >> sh, g = t & (G - 1);
-            if (g >= gl) continue;
-            V v = r[g * N + slot_of(y, N)];
-            if (y & 1) v = mk<T>(-v.x, -v.y);
-            out[(size_t)y * nl + l0 + g] = v;
+        const V w = dct[j], e = coef(N - j);
+        const V d = mk<T>(e.y, -e.x);  // -i C_{N-j}
+        x[pad<T>(j)] = cmul<true>(cadd(c, d), w);
+        if (2 * j < N) x[pad<T>(N - j)] = cmul<false>(csub(c, d), w);
+    }
+    __syncthreads();
+    return fft<T, true>(a, b, tab, N, lgG, gl);
+}
+
+// Rows inverse: store(line, x, value) takes the solution's samples.
+template <typename T, int NC, typename F>
+__device__ __forceinline__ void rows_inverse(const Lines &P, int bid, int nblk, const V2<T> *in,
+                                             F store) {
+    using V = V2<T>;
+    const int N = P.N, nl = NC == 2 ? N : N / 2;
+    const int lgG = lines_at_once(nl, nblk, P.gmax), G = 1 << lgG;
+    const Deal D(lgG);
+    for (int l0 = bid * G; l0 < nl; l0 += nblk * G) {
+        const int gl = min(G, nl - l0);
+        const V *r = cplx_at<T>(
+            rows_inverse_first<T, NC>(P.a, buf_b<T>(P), P.tab, N, l0, lgG, gl, in));
+        for (int x = D.g < gl ? D.j0 : N; x < N; x += D.stride) {
+            V v = r[D.g * line_len<T>(N) + pad<T>(slot_of(x, N))];
+            if (x & 1) v = mk<T>(-v.x, -v.y);
+            store(l0 + D.g, x, v);
         }
         __syncthreads();
     }
 }
 
-// Rows inverse: store(line, x, value) takes the solution's samples.
+// Rows inverse and, of what next(line, x, value) makes of the samples, rows
+// forward again.
 template <typename T, int NC, typename F>
-__device__ void rows_inverse(const Lines<T> &P, int bid, int nblk, const V2<T> *in, F store) {
+__device__ __forceinline__ void rows_inverse_forward(const Lines &P, int bid, int nblk,
+                                                     const V2<T> *in, V2<T> *out, F next) {
     using V = V2<T>;
-    const int N = P.N, nl = NC == 2 ? N : N / 2;
-    const int G = lines_at_once(nl, nblk, P.gmax);
+    const int N = P.N, nl = NC == 2 ? N : N / 2, b = buf_b<T>(P);
+    const int lgG = lines_at_once(nl, nblk, P.gmax), G = 1 << lgG;
+    const Deal D(lgG);
     for (int l0 = bid * G; l0 < nl; l0 += nblk * G) {
         const int gl = min(G, nl - l0);
-        for (Split s(N / 2 + 1); s.g < gl; s.next()) {
-            const int j = s.j, l = l0 + s.g;
-            auto coef = [&](int jj) {
-                if constexpr (NC == 2) {
-                    return in[(size_t)l * N + jj];
-                } else {
-                    const T *o = (const T *)in + (size_t)(2 * l) * N;
-                    return mk<T>(o[jj], o[N + jj]);
-                }
-            };
-            V *x = P.a + s.g * N;
-            const V c = coef(j);
-            if (j == 0) {
-                x[0] = c;
-                continue;
-            }
-            const V w = P.dct[j], e = coef(N - j);
-            const V d = mk<T>(e.y, -e.x);  // -i C_{N-j}
-            x[j] = cmul<true>(cadd(c, d), w);
-            if (2 * j < N) x[N - j] = cmul<false>(csub(c, d), w);
+        const int f = rows_inverse_first<T, NC>(P.a, b, P.tab, N, l0, lgG, gl, in);
+        const int o = f == P.a ? b : P.a;
+        const V *r = cplx_at<T>(f) + D.g * line_len<T>(N);
+        V *q = cplx_at<T>(o) + D.g * line_len<T>(N);
+        for (int x = D.g < gl ? D.j0 : N; x < N; x += D.stride) {
+            const int at = pad<T>(slot_of(x, N));
+            V v = r[at];
+            if (x & 1) v = mk<T>(-v.x, -v.y);
+            v = next(l0 + D.g, x, v);
+            if (x & 1) v = mk<T>(-v.x, -v.y);
+            q[at] = v;
         }
-        __syncthreads();
-        const V *r = fft<T, true>(P, gl);
-        for (Split s(N); s.g < gl; s.next()) {
-            V v = r[s.g * N + slot_of(s.j, N)];
-            if (s.j & 1) v = mk<T>(-v.x, -v.y);
-            store(l0 + s.g, s.j, v);
-        }
-        __syncthreads();
+        rows_forward_rest<T, NC>(o, f, P.tab, N, l0, lgG, gl, out);
     }
 }
 

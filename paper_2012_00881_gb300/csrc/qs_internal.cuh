@@ -20,7 +20,7 @@ struct DevScalars {
     int err_where;                 // phase id of a timeout; -1: no clusters
     double rnorm[4][4];            // ||r||^2 (comps 0,1) and ||u||^2 (2,3), ring of 4
     double fnorm[3][2];            // ||f||^2 of the psi / (Ez,Bz) / (Bx,By) solves
-    double cgd[4][4];              // conjugate gradients: (r,z), (z,Az) per component, ring of 4
+    double cgd[4][16];             // conjugate gradients: dot products per component, ring of 4
     double ksum;                   // sum of kappa over the cells of this slice
     unsigned long long vmax_bits[2];  // V_max of a push (bits of a double >= 0)
     unsigned long long guard_hits;
@@ -67,15 +67,16 @@ struct LevelArrays32 {
 struct FftArgs {
     int on;       // the uniform-grid Poisson problems are solved directly
     int gmax;     // lines that fit a block's buffers
-    int tab_off;  // byte offset of the tables' copy in shared memory (0: none)
+    int tab_off;  // byte offset of the tables' copy in shared memory
     double2 *tw64, *dct64;
     double *lam64;
     float2 *tw32, *dct32;
     float *lam32;
     double2 *t1, *t2;
     // conjugate gradients of the screened solve, complex grids in the storage
-    // type of its inner iterations: z, r, p, A p, the correction e
-    void *cz, *cr, *cp, *cs, *ce;
+    // type of its inner iterations: z, r, p, A p, the correction e; the row
+    // transforms of A z and A p
+    void *cz, *cr, *cp, *cs, *ce, *tz, *tp;
 };
 
 // Everything the slice engine reads or writes (passed by value).

@@ -878,19 +878,23 @@ __device__ __noinline__ bool mg_solve_ref_cluster(const EngineArgs &A, const Syn
 // direct solves by sine transforms (qs_fft.cuh)
 // ---------------------------------------------------------------------------
 
-// Copies the transform tables to shared memory, once per launch or instance.
+// Copies the transform tables to shared memory, once per launch or instance
+// (the refined form keeps the float64 ones as float pairs).
 template <bool REF>
-__device__ void fft_load_tables(const EngineArgs &A, void *smem_base) {
-    if (!A.fft.on || !A.fft.tab_off) return;
+__device__ void fft_load_tables(const EngineArgs &A) {
+    if (!A.fft.on) return;
     const int N = A.N, H = N / 2 + 1;
-    double2 *tw = (double2 *)((char *)smem_base + A.fft.tab_off);
-    double *lam = (double *)(tw + N + H);
+    using D = typename std::conditional<REF, qsff::Ff, double>::type;
+    using D2 = qsfft::V2<D>;
+    D2 *tw = (D2 *)(qsfft::dyn_smem() + A.fft.tab_off);
+    D *lam = (D *)(tw + N + H);
     float2 *tw32 = (float2 *)(lam + N);
     float *lam32 = (float *)(tw32 + N + H);
+    auto conv = [](double2 v) { return qsfft::mk<D>(D(v.x), D(v.y)); };
     for (int k = threadIdx.x; k < N; k += blockDim.x) {
-        tw[k] = A.fft.tw64[k];
-        if (k < H) tw[N + k] = A.fft.dct64[k];
-        lam[k] = A.fft.lam64[k];
+        tw[k] = conv(A.fft.tw64[k]);
+        if (k < H) tw[N + k] = conv(A.fft.dct64[k]);
+        lam[k] = D(A.fft.lam64[k]);
         if (REF) {
             tw32[k] = A.fft.tw32[k];
             if (k < H) tw32[N + k] = A.fft.dct32[k];
@@ -901,64 +905,16 @@ __device__ void fft_load_tables(const EngineArgs &A, void *smem_base) {
 }
 
 template <typename T>
-__device__ __forceinline__ qsfft::Lines<T> fft_lines(const EngineArgs &A, void *smem_base) {
-    using V = qsfft::V2<T>;
-    qsfft::Lines<T> P;
-    P.N = A.N;
-    P.gmax = A.fft.gmax;
-    const size_t n = (size_t)P.N, h = n / 2 + 1;
-    const char *tab = (const char *)smem_base + A.fft.tab_off;
-    if constexpr (sizeof(T) == 8) {
-        P.tw = A.fft.tw64;
-        P.dct = A.fft.dct64;
-        P.lam = A.fft.lam64;
-    } else {
-        P.tw = A.fft.tw32;
-        P.dct = A.fft.dct32;
-        P.lam = A.fft.lam32;
-        tab += (n + h) * sizeof(double2) + n * sizeof(double);
-    }
-    if (A.fft.tab_off) {
-        P.tw = (const V *)tab;
-        P.dct = P.tw + n;
-        P.lam = (const T *)(P.dct + h);
-    }
-    P.a = (V *)((char *)smem_base + A.block_smem_offset);
-    P.b = P.a + P.gmax * P.N;
-    return P;
+__device__ __forceinline__ qsfft::Lines fft_lines(const EngineArgs &A) {
+    const int n = A.N, h = n / 2 + 1;
+    const int tab = A.fft.tab_off +
+                    (sizeof(T) == 4 ? (n + h) * (int)sizeof(double2) + n * (int)sizeof(double) : 0);
+    return qsfft::Lines{n, A.fft.gmax, A.block_smem_offset, tab};
 }
 
-// lap_h u = f for one field, or two at once as the parts of a complex one: three
-// grid phases in float64 whatever the right-hand side, against four to five
-// V-cycles of four phases each.
-template <int NC>
-__device__ bool direct_poisson(const EngineArgs &A, const Sync &S, const SolveSpec &V, int bid,
-                               int nblk, void *smem_base) {
-    const qsfft::Lines<double> P = fft_lines<double>(A, smem_base);
-    const int N = A.N;
-    const double *const f0 = V.f[0], *const f1 = NC == 2 ? V.f[1] : V.f[0] + N;
-    double *const u0 = V.u[0], *const u1 = NC == 2 ? V.u[1] : V.u[0] + N;
-    const int ld = NC == 2 ? N : 2 * N;
-    qsfft::rows_forward<double, NC>(P, bid, nblk, A.fft.t1, [&](int l, int x) {
-        const size_t i = (size_t)l * ld + x;
-        return make_double2(f0[i], f1[i]);
-    });
-    SYNC(26);
-    qsfft::columns<double, NC>(P, bid, nblk, A.fft.t1, A.fft.t2, 0.0);
-    SYNC(27);
-    qsfft::rows_inverse<double, NC>(P, bid, nblk, A.fft.t2, [&](int l, int x, double2 v) {
-        const size_t i = (size_t)l * ld + x;
-        u0[i] = v.x;
-        u1[i] = v.y;
-    });
-    if (bid == 0 && threadIdx.x == 0) A.sc->vcycles[V.kind] += 1;
-    SYNC(28);
-    return true;
-}
-
-// e at a cell and its five-point sum times h^2: sum of the neighbours minus
-// (4 + walls) e, exact to rounding of a float64 for float32 values (error-free
-// sums and an FMA product) without float64 arithmetic on the five values.
+// The five-point sum of e times h^2, neighbours minus (4 + walls) e.  float32
+// values: exact to the rounding of a float64, by error-free float32 sums and
+// an FMA product, without float64 arithmetic on the five values.
 __device__ __forceinline__ double five_point(float c, float w, float e, float n, float s,
                                              float k) {
     float hi = 0.f, lo = 0.f;
@@ -977,204 +933,375 @@ __device__ __forceinline__ double five_point(double c, double w, double e, doubl
     return (w + e) + (n + s) - k * c;
 }
 
-// The block's share of four sums into out[4]; clears the slots two uses ahead.
-__device__ void cg_reduce(DevScalars *sc, float v[4], double *out, int slot, int bid) {
-    block_sum4f(v);
-    if (threadIdx.x == 0) {
+// Sums of 16 values over the block, into out[0 .. 15] (global); clears the slots
+// of the ring two uses ahead.  Each shuffle halves the values a lane holds: 16
+// shuffles instead of 80.
+__device__ void reduce16(DevScalars *sc, float v[16], double *out, int slot, int bid) {
+    __shared__ float red[32][17];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (int)blockDim.x >> 5;
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-            if (v[k] != 0.f) atomicAdd(out + k, (double)v[k]);
-        if (bid == 0)
-            for (int k = 0; k < 4; ++k) sc->rnorm[(slot + 2) & 3][k] = sc->cgd[(slot + 2) & 3][k] = 0.0;
+    for (int o = 16; o >= 2; o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int k = 0; k < o / 2; ++k) {
+            const float give = up ? v[k] : v[k + o / 2];
+            const float keep = up ? v[k + o / 2] : v[k];
+            v[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
     }
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+    // lane bits 4..1 select the value: bit 4 its half, and so on
+    if ((lane & 1) == 0) red[wid][lane >> 1] = v[0];
+    __syncthreads();
+    if (threadIdx.x < 16) {
+        float t = 0.f;
+        for (int w = 0; w < nw; ++w) t += red[w][threadIdx.x];
+        if (t != 0.f) atomicAdd(out + threadIdx.x, (double)t);
+        if (bid == 0) {
+            sc->cgd[(slot + 2) & 3][threadIdx.x] = 0.0;
+            if (threadIdx.x < 4) sc->rnorm[(slot + 2) & 3][threadIdx.x] = 0.0;
+        }
+    }
+    __syncthreads();  // red is reused by the next call
+}
+
+// Scalars of an iterative solve, one copy per block (thread 0, or thread c for
+// component c, writes them between block barriers).
+struct IterScalars {
+    double scale[2], inv[2];  // powers of two near 1 / ||f|| and their inverses
+    double thr[2], r0[2];     // stopping bound, residual a round starts from (squared, scaled)
+    double ig[2], ia[2];      // 1 / (r, z) and 1 / alpha of the last iteration
+    float rr[2], ss[2];       // ||r||^2 after the last step, ||A p||^2 (scaled)
+    double al[2], be[2];
+    double kbar;
+    int go;
+};
+
+// Source scales and stopping bounds; go: whether any component needs work.  A
+// NaN or infinite source keeps scale 1 and fails every stopping test.
+__device__ void iter_begin(const EngineArgs &A, const SolveSpec &V, IterScalars &I) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int any = 0;
+        for (int c = 0; c < 2; ++c) {
+            const double fn = c < V.nc ? vload(&A.sc->fnorm[V.kind][c]) : 0.0;
+            const int ex = (int)((__double_as_longlong(fn) >> 52) & 0x7ff);
+            const int k = ex == 0 || ex == 0x7ff ? 0 : (ex - 1023) / 2;
+            I.scale[c] = __longlong_as_double((long long)(1023 - k) << 52);
+            I.inv[c] = __longlong_as_double((long long)(1023 + k) << 52);
+            const double s2 = I.scale[c] * I.scale[c];
+            I.thr[c] = fmax(A.mg_tol * A.mg_tol * fn, A.mg_atol * A.mg_atol) * s2;
+            I.r0[c] = fn * s2;
+            if (!(I.r0[c] <= I.thr[c])) any = 1;
+        }
+        I.kbar = V.screened ? vload(&A.sc->ksum) / ((double)A.N * (double)A.N) : 0.0;
+        I.go = any;
+    }
+    __syncthreads();
+}
+
+// After u += e and the new residual's norms (rnorm[slot]): converged (1), too
+// slow or out of iterations (0), or another round (-2).
+__device__ int iter_check(const EngineArgs &A, const SolveSpec &V, IterScalars &I, int slot,
+                          int bid, bool last) {
+    DevScalars *sc = A.sc;
+    if (threadIdx.x == 0) {
+        const double fl = 1e-13 * A.lev_inv_h2[0];
+        int conv = 1, slow = 0;
+        double rel = 0.0;
+        for (int c = 0; c < V.nc; ++c) {
+            const double rn = vload(&sc->rnorm[slot & 3][c]);
+            const double un = vload(&sc->rnorm[slot & 3][2 + c]);
+            if (!(rn <= fmax(I.thr[c], fl * fl * un))) {
+                conv = 0;
+                if (!(rn <= 0.0625 * I.r0[c])) slow = 1;
+            }
+            I.r0[c] = rn;
+            if (bid == 0) {
+                const double fn = vload(&sc->fnorm[V.kind][c]);
+                if (fn > 0.0) rel = fmax(rel, sqrt(rn / fn) * I.inv[c]);
+            }
+        }
+        if (bid == 0 && conv && rel > sc->max_relres) sc->max_relres = rel;
+        I.go = conv ? 1 : (slow || last) ? 0 : -2;
+    }
+    __syncthreads();
+    const int r = I.go;
+    __syncthreads();  // rewritten by the next test
+    return r;
+}
+
+__device__ void zero_solution(const EngineArgs &A, const SolveSpec &V, int bid, int nblk) {
+    const Thr T0 = grid_thr(bid, nblk);
+    for (int c = 0; c < V.nc; ++c)
+        for (int i = T0.t0; i < A.N * A.N; i += T0.nt) {
+            V.u[c][i] = 0.0;
+            if (V.u32[c]) V.u32[c][i] = 0.f;
+        }
+}
+
+// lap_h u = f for one field, or two at once as the parts of a complex one, in
+// three grid phases.  Float64 form: in float64, bound by the FP64 pipe (two
+// fields at 256^2: 37 us).  Refined form: in pairs of floats, whose 47 bits
+// leave a residual of 1e-13 (two fields at 256^2: 28 us; 512^2: 57, against 96); the source
+// is scaled by a power of two near 1 / ||f|| to keep the pairs' low parts in
+// range.
+template <bool REF, int NC>
+__device__ bool direct_poisson(const EngineArgs &A, const Sync &S, const SolveSpec &V, int bid,
+                               int nblk) {
+    using T = typename std::conditional<REF, qsff::Ff, double>::type;
+    using C = qsfft::V2<T>;
+    const qsfft::Lines P = fft_lines<T>(A);
+    const int N = A.N, nl = NC == 2 ? N : N / 2;
+    const double *const f0 = V.f[0], *const f1 = NC == 2 ? V.f[1] : V.f[0] + N;
+    double *const u0 = V.u[0], *const u1 = NC == 2 ? V.u[1] : V.u[0] + N;
+    const int ld = NC == 2 ? N : 2 * N;
+    C *const t1 = (C *)A.fft.t1, *const t2 = (C *)A.fft.t2;
+    __shared__ IterScalars I;
+    double sc0 = 1.0, sc1 = 1.0, is0 = 1.0, is1 = 1.0;
+    if constexpr (REF) {
+        iter_begin(A, V, I);
+        sc0 = I.scale[0];
+        sc1 = I.scale[NC - 1];
+        is0 = I.inv[0];
+        is1 = I.inv[NC - 1];
+    }
+    qsfft::rows_forward<T, NC>(P, bid, nblk, t1, [&](int l, int x) {
+        const size_t i = (size_t)l * ld + x;
+        if constexpr (REF) return qsfft::mk<T>(qsff::split(f0[i] * sc0), qsff::split(f1[i] * sc1));
+        else return make_double2(f0[i], f1[i]);
+    });
+    SYNC(26);
+    qsfft::columns<T, NC>(P, bid, nblk, t2, T(0.0),
+                          [&](int y, int l) { return t1[(size_t)y * nl + l]; });
+    SYNC(27);
+    qsfft::rows_inverse<T, NC>(P, bid, nblk, t2, [&](int l, int x, C v) {
+        const size_t i = (size_t)l * ld + x;
+        if constexpr (REF) {
+            u0[i] = qsff::join(v.x) * is0;
+            u1[i] = qsff::join(v.y) * is1;
+        } else {
+            u0[i] = v.x;
+            u1[i] = v.y;
+        }
+    });
+    if (bid == 0 && threadIdx.x == 0) A.sc->vcycles[V.kind] += 1;
+    SYNC(28);
+    return true;
 }
 
 // (lap_h - kappa) u = f for the two components of B_perp by conjugate
 // gradients preconditioned with M = lap_h - kbar, kbar the mean of kappa, whose
 // inverse is a direct solve by sine transforms.  A z = M z + (kbar - kappa) z =
-// r + (kbar - kappa) z, so the operator costs one product a cell and every
-// vector update stays in the rows that the block transforms: an iteration is
-// three grid phases (columns; rows inverse with the dot products; update with
-// rows forward).  M^-1 A is a compact perturbation of the identity, so the
-// iteration converges superlinearly: 5 to 8 steps to 1e-10 on the 256^2
-// blowout (kappa 0 ... 18), 18 to 25 in a channel with kappa 1 ... 11, from a
-// zero guess (the extrapolated guess carries the macroparticle noise of three
-// slices: its residual is above the source's at the window's head).
+// r + (kbar - kappa) z, so the operator costs one product a cell.  M^-1 A is a
+// compact perturbation of the identity, so the iteration converges
+// superlinearly: 4 to 8 steps to 1e-10 on the 256^2 blowout (kappa 0 ... 18),
+// 18 to 25 in a channel with kappa 1 ... 11, from a zero guess (the guess
+// extrapolated from three slices carries their macroparticle noise: its
+// residual is above the source's at the window's head).
 //
-// Refined form: the iteration runs in float32 on the residual equation, to
-// 1e-5 of the residual it starts from; then u += e, r <- r - A e in float64
-// and again.  Float64 form: in float64 to the tolerance; the same step then
-// checks it.  Both stop on the float64 residual.  The residual is scaled by a
-// power of two near 1 / ||f|| so that float32 cannot underflow.
+// An iteration is two grid phases.  Rows: the last update of p, A p, e and r
+// (with the step sizes that the previous barrier brought), z = M^-1 r from its
+// row coefficients, A z, the dot products, and the row transform of A z at
+// once, before the step sizes are known: the row transforms of r and A p
+// follow the same recurrences, which the column phase applies to its own
+// elements.  (With the update and the forward transform behind the dot
+// products' barrier an iteration was three phases.)  ||r||^2 follows from the
+// dot products too, so that the end of a round costs no phase.
+//
+// Refined form: float32 iterations on the residual equation, to 1e-5 of the
+// residual they start from; then u += e, r <- r - A e in float64 and again.
+// Float64 form: in float64 to the tolerance; the same step then checks it.
+// Both stop on the float64 residual.  The residual is scaled by a power of two
+// near 1 / ||f|| so that float32 cannot underflow.
 // Returns 1 (converged), 0 (not within its cap: u holds the last iterate and
 // the V-cycles take over), -1 (a barrier failed).
 template <bool REF>
 __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &V, int &slot,
-                           int bid, int nblk, void *smem_base) {
+                           int bid, int nblk) {
     using T = typename std::conditional<REF, float, double>::type;
     using C = qsfft::V2<T>;
     DevScalars *sc = A.sc;
-    const qsfft::Lines<T> P = fft_lines<T>(A, smem_base);
+    const qsfft::Lines P = fft_lines<T>(A);
     const int N = A.N;
-    C *const t1 = (C *)A.fft.t1, *const t2 = (C *)A.fft.t2;
+    C *const tr = (C *)A.fft.t1, *const t2 = (C *)A.fft.t2, *const tz = (C *)A.fft.tz,
+             *const tp = (C *)A.fft.tp;
     C *const cz = (C *)A.fft.cz, *const cr = (C *)A.fft.cr, *const cp = (C *)A.fft.cp,
              *const cs = (C *)A.fft.cs, *const ce = (C *)A.fft.ce;
-    __shared__ double s_scale[2], s_inv[2], s_thr[2], s_r0[2], s_ig[2], s_ia[2];
-    __shared__ T s_al[2], s_be[2], s_kbar;
-    __shared__ int s_go;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int any = 0;
-        for (int c = 0; c < 2; ++c) {
-            const double fn = vload(&sc->fnorm[V.kind][c]);
-            // 2^-k with k about half the exponent of ||f||^2 (a NaN or
-            // infinite source keeps 1: it fails the stopping test below)
-            const int ex = (int)((__double_as_longlong(fn) >> 52) & 0x7ff);
-            const int k = ex == 0 || ex == 0x7ff ? 0 : (ex - 1023) / 2;
-            s_scale[c] = __longlong_as_double((long long)(1023 - k) << 52);
-            s_inv[c] = __longlong_as_double((long long)(1023 + k) << 52);
-            const double s2 = s_scale[c] * s_scale[c];
-            s_thr[c] = fmax(A.mg_tol * A.mg_tol * fn, A.mg_atol * A.mg_atol) * s2;
-            s_r0[c] = fn * s2;
-            if (!(s_r0[c] <= s_thr[c])) any = 1;
-        }
-        s_kbar = (T)(vload(&sc->ksum) / ((double)N * (double)N));
-        s_go = any;
-    }
-    __syncthreads();
-    const T kbar = s_kbar;
-    const double sc0 = s_scale[0], sc1 = s_scale[1], is0 = s_inv[0], is1 = s_inv[1];
-    const bool any = s_go != 0;
-    if (!any) {  // both sources are rounding noise or zero
-        const Thr T0 = grid_thr(bid, nblk);
-        for (int c = 0; c < 2; ++c)
-            for (int i = T0.t0; i < N * N; i += T0.nt) {
-                V.u[c][i] = 0.0;
-                if (V.u32[c]) V.u32[c][i] = 0.f;
-            }
+    __shared__ IterScalars I;
+    iter_begin(A, V, I);
+    if (!I.go) {  // both sources are rounding noise or zero
+        zero_solution(A, V, bid, nblk);
         return S(50) ? 1 : -1;
     }
+    const T kbar = (T)I.kbar;
+    const double sc0 = I.scale[0], sc1 = I.scale[1], is0 = I.inv[0], is1 = I.inv[1];
     auto dk = [&](size_t i) {  // kbar - kappa
         if constexpr (REF) return kbar - A.k32[i];
         else return kbar - A.kap[i];
     };
-    qsfft::rows_forward<T, 2>(P, bid, nblk, t1, [&](int y, int x) {
+    qsfft::rows_forward<T, 2>(P, bid, nblk, tr, [&](int y, int x) {
         const size_t i = (size_t)y * N + x;
-        const double f0 = V.f[0][i], f1 = V.f[1][i];
-        A.r64[0][i] = f0;
-        A.r64[1][i] = f1;
-        const C r = qsfft::mk<T>((T)(f0 * sc0), (T)(f1 * sc1));
+        const C r = qsfft::mk<T>((T)(V.f[0][i] * sc0), (T)(V.f[1][i] * sc1));
         cr[i] = r;
         return r;
     });
     if (!S(51)) return -1;
     const int cap = min(A.mg_max_vcycles, 48);
-    const double red = REF ? 1e-10 : 1e-26;  // inner reduction, squared
-    const double fl = 1e-13 * A.lev_inv_h2[0];
+    const double red = REF ? 1e-10 : 1e-26;  // a round's reduction, squared
     int it = 0, result = -2;
-    for (int outer = 0; result == -2; ++outer) {
-        for (int inner = 0;; ++inner) {
-            qsfft::columns<T, 2>(P, bid, nblk, t1, t2, kbar);
-            if (!S(52)) return -1;
-            float d[4] = {0.f, 0.f, 0.f, 0.f};
-            qsfft::rows_inverse<T, 2>(P, bid, nblk, t2, [&](int y, int x, C z) {
-                const size_t i = (size_t)y * N + x;
-                const C r = cr[i];
-                const T k = dk(i);
-                cz[i] = z;
-                d[0] += (float)(r.x * z.x);
-                d[1] += (float)(r.y * z.y);
-                d[2] += (float)(z.x * (r.x + k * z.x));
-                d[3] += (float)(z.y * (r.y + k * z.y));
+    for (int round = 0; result == -2; ++round) {
+        T al0 = T(0), al1 = T(0), be0 = T(0), be1 = T(0);
+        int inner = 0;
+        for (;;) {
+            qsfft::columns<T, 2>(P, bid, nblk, t2, kbar, [&](int y, int l) {
+                const size_t i = (size_t)y * N + l;
+                C r = tr[i];
+                if (inner > 0) {
+                    C s = tz[i];
+                    if (inner > 1) {
+                        const C so = tp[i];
+                        s.x += be0 * so.x;
+                        s.y += be1 * so.y;
+                    }
+                    tp[i] = s;
+                    r.x -= al0 * s.x;
+                    r.y -= al1 * s.y;
+                    tr[i] = r;
+                }
+                return r;
             });
-            cg_reduce(sc, d, sc->cgd[slot & 3], slot, bid);
+            if (!S(52)) return -1;
+            float d[16] = {0.f};
+            qsfft::rows_inverse_forward<T, 2>(P, bid, nblk, t2, tz, [&](int y, int x, C z) {
+                const size_t i = (size_t)y * N + x;
+                const T k = dk(i);
+                C r = cr[i], s = qsfft::mk<T>(T(0), T(0));
+                if (inner > 0) {  // the update of the last iteration
+                    const C zo = cz[i];
+                    C p = zo, e;
+                    s = qsfft::mk<T>(r.x + k * zo.x, r.y + k * zo.y);
+                    if (inner > 1) {
+                        const C po = cp[i], so = cs[i];
+                        e = ce[i];
+                        p.x += be0 * po.x;
+                        p.y += be1 * po.y;
+                        s.x += be0 * so.x;
+                        s.y += be1 * so.y;
+                        e.x += al0 * p.x;
+                        e.y += al1 * p.y;
+                    } else {
+                        e = qsfft::mk<T>(al0 * p.x, al1 * p.y);
+                    }
+                    r.x -= al0 * s.x;
+                    r.y -= al1 * s.y;
+                    cp[i] = p;
+                    cs[i] = s;
+                    ce[i] = e;
+                    cr[i] = r;
+                }
+                cz[i] = z;
+                const C w = qsfft::mk<T>(r.x + k * z.x, r.y + k * z.y);
+                const float rx = (float)r.x, ry = (float)r.y, zx = (float)z.x, zy = (float)z.y,
+                            wx = (float)w.x, wy = (float)w.y, sx = (float)s.x, sy = (float)s.y;
+                d[0] += rx * zx;
+                d[1] += ry * zy;
+                d[2] += zx * wx;
+                d[3] += zy * wy;
+                d[4] += rx * wx;
+                d[5] += ry * wy;
+                d[6] += rx * sx;
+                d[7] += ry * sy;
+                d[8] += wx * wx;
+                d[9] += wy * wy;
+                d[10] += wx * sx;
+                d[11] += wy * sy;
+                d[12] += rx * rx;
+                d[13] += ry * ry;
+                return w;
+            });
+            reduce16(sc, d, sc->cgd[slot & 3], slot, bid);
             if (!S(53)) return -1;
-            if (threadIdx.x < 2) {  // one thread a component: two float64 divides
+            if (threadIdx.x < 2) {  // one thread a component
                 const int c = threadIdx.x;
-                const double ga = vload(&sc->cgd[slot & 3][c]);
-                const double de = vload(&sc->cgd[slot & 3][2 + c]);
+                const double *g = sc->cgd[slot & 3];
+                const double ga = vload(g + c), de = vload(g + 2 + c);
                 double be = 0.0, al = 0.0, ia = 0.0, ig = 0.0;
                 if (ga != 0.0) {
                     ig = 1.0 / ga;
-                    be = inner > 0 ? ga * s_ig[c] : 0.0;
-                    ia = de * ig - be * (inner > 0 ? s_ia[c] : 0.0);
+                    be = inner > 0 ? ga * I.ig[c] : 0.0;
+                    ia = de * ig - be * (inner > 0 ? I.ia[c] : 0.0);
                     al = ia != 0.0 ? 1.0 / ia : 0.0;
                 }
-                s_ig[c] = ig;
-                s_ia[c] = ia;
-                s_al[c] = (T)al;
-                s_be[c] = (T)be;
+                I.ig[c] = ig;
+                I.ia[c] = ia;
+                I.al[c] = al;
+                I.be[c] = be;
+                // ||r - al s||^2 with s = w + be s_old.  The sums are good to
+                // about 1e-7 of ||r||^2: no smaller value is believed.
+                const float a = (float)al, b = (float)be;
+                const float rw = (float)vload(g + 4 + c), rs = (float)vload(g + 6 + c),
+                            ww = (float)vload(g + 8 + c), ws = (float)vload(g + 10 + c);
+                const float so = inner > 0 ? I.ss[c] : 0.f;
+                const float ss = ww + b * (2.f * ws + b * so);
+                const float rr = (float)vload(g + 12 + c);
+                I.ss[c] = ss;
+                const float nr = rr - a * (2.f * (rw + b * rs) - a * ss);
+                I.rr[c] = nr < 2e-7f * rr ? 2e-7f * rr : nr;  // a NaN stays
             }
             ++slot;
             __syncthreads();
-            const T al0 = s_al[0], al1 = s_al[1], be0 = s_be[0], be1 = s_be[1];
-            const bool first = inner == 0;
-            float n[4] = {0.f, 0.f, 0.f, 0.f};
-            qsfft::rows_forward<T, 2>(P, bid, nblk, t1, [&](int y, int x) {
-                const size_t i = (size_t)y * N + x;
-                const C z = cz[i];
-                C r = cr[i];
-                const T k = dk(i);
-                C p = z, s = qsfft::mk<T>(r.x + k * z.x, r.y + k * z.y);
-                C e = qsfft::mk<T>(T(0), T(0));
-                if (!first) {
-                    const C po = cp[i], so = cs[i];
-                    e = ce[i];
-                    p.x += be0 * po.x;
-                    p.y += be1 * po.y;
-                    s.x += be0 * so.x;
-                    s.y += be1 * so.y;
-                }
-                e.x += al0 * p.x;
-                e.y += al1 * p.y;
-                r.x -= al0 * s.x;
-                r.y -= al1 * s.y;
-                cp[i] = p;
-                cs[i] = s;
-                ce[i] = e;
-                cr[i] = r;
-                n[0] += (float)(r.x * r.x);
-                n[1] += (float)(r.y * r.y);
-                return r;
-            });
-            cg_reduce(sc, n, sc->rnorm[slot & 3], slot, bid);
-            if (!S(54)) return -1;
-            ++it;
             if (threadIdx.x == 0) {
                 int go = 0;
-                for (int c = 0; c < 2; ++c) {
-                    const double rn = vload(&sc->rnorm[slot & 3][c]);
-                    if (!(rn <= fmax(red * s_r0[c], 0.09 * s_thr[c]))) go = 1;
-                }
-                s_go = go;
+                for (int c = 0; c < 2; ++c)
+                    if (!((double)I.rr[c] <= fmax(red * I.r0[c], 0.09 * I.thr[c]))) go = 1;
+                I.go = go;
             }
-            ++slot;
+            al0 = (T)I.al[0];
+            al1 = (T)I.al[1];
+            be0 = (T)I.be[0];
+            be1 = (T)I.be[1];
             __syncthreads();
-            const bool go = s_go != 0;
-            __syncthreads();  // s_go is rewritten by the next test
-            if (!go || it >= cap || inner >= 23) break;
+            const bool go = I.go != 0;
+            __syncthreads();  // rewritten by the next test
+            ++it;
+            ++inner;
+            if (!go || it >= cap || inner >= 24) break;
         }
         // u += e, r <- r - A e in float64 with the norms of the stopping test;
-        // the new right-hand side goes through its row transform on the way
-        float n[4] = {0.f, 0.f, 0.f, 0.f};
+        // the new right-hand side goes through its row transform on the way.
+        // e is e + al p with the last step, at the cell and its neighbours.
+        auto e_at = [&](size_t i) {
+            C p = cz[i];
+            if (inner == 1) return qsfft::mk<T>(al0 * p.x, al1 * p.y);
+            const C po = cp[i], eo = ce[i];
+            p.x += be0 * po.x;
+            p.y += be1 * po.y;
+            return qsfft::mk<T>(eo.x + al0 * p.x, eo.y + al1 * p.y);
+        };
+        float n[16] = {0.f};
         const double ih2 = A.lev_inv_h2[0];
-        const bool fresh = outer == 0;
-        qsfft::rows_forward<T, 2>(P, bid, nblk, t1, [&](int y, int x) {
+        qsfft::rows_forward<T, 2>(P, bid, nblk, tr, [&](int y, int x) {
             const size_t i = (size_t)y * N + x;
             const C zero = qsfft::mk<T>(T(0), T(0));
-            const C e = ce[i];
-            const C ew = x > 0 ? ce[i - 1] : zero, ee = x < N - 1 ? ce[i + 1] : zero;
-            const C en = y > 0 ? ce[i - N] : zero, es = y < N - 1 ? ce[i + N] : zero;
+            const C e = e_at(i);
+            const C ew = x > 0 ? e_at(i - 1) : zero, ee = x < N - 1 ? e_at(i + 1) : zero;
+            const C en = y > 0 ? e_at(i - N) : zero, es = y < N - 1 ? e_at(i + N) : zero;
             const T cw = (T)(4 + qsmg::walls(x, y, N));
             const double kap = A.kap[i];
             const double a0 = five_point(e.x, ew.x, ee.x, en.x, es.x, cw) * ih2 - kap * (double)e.x;
             const double a1 = five_point(e.y, ew.y, ee.y, en.y, es.y, cw) * ih2 - kap * (double)e.y;
-            const double r0 = A.r64[0][i] - a0 * is0, r1 = A.r64[1][i] - a1 * is1;
-            double u0 = (double)e.x * is0, u1 = (double)e.y * is1;
-            if (!fresh) {
+            double u0 = (double)e.x * is0, u1 = (double)e.y * is1, q0, q1;
+            if (round == 0) {
+                q0 = V.f[0][i];
+                q1 = V.f[1][i];
+            } else {
                 u0 += V.u[0][i];
                 u1 += V.u[1][i];
+                q0 = A.r64[0][i];
+                q1 = A.r64[1][i];
             }
+            const double r0 = q0 - a0 * is0, r1 = q1 - a1 * is1;
             V.u[0][i] = u0;
             V.u[1][i] = u1;
             if (V.u32[0]) {
@@ -1192,30 +1319,10 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
             n[3] += v1 * v1;
             return r;
         });
-        cg_reduce(sc, n, sc->rnorm[slot & 3], slot, bid);
+        reduce16(sc, n, A.sc->rnorm[slot & 3], slot, bid);
         if (!S(55)) return -1;
-        if (threadIdx.x == 0) {
-            int conv = 1, slow = 0;
-            for (int c = 0; c < 2; ++c) {
-                const double rn = vload(&sc->rnorm[slot & 3][c]);
-                const double un = vload(&sc->rnorm[slot & 3][2 + c]);
-                if (!(rn <= fmax(s_thr[c], fl * fl * un))) {
-                    conv = 0;
-                    if (!(rn <= 0.0625 * s_r0[c])) slow = 1;
-                }
-                s_r0[c] = rn;
-                if (bid == 0) {
-                    const double fn = vload(&sc->fnorm[V.kind][c]);
-                    const double rel = fn > 0.0 ? sqrt(rn / fn) * s_inv[c] : 0.0;
-                    if (conv && rel > sc->max_relres) sc->max_relres = rel;
-                }
-            }
-            s_go = conv ? 1 : (slow || it >= cap) ? 0 : -2;
-        }
+        result = iter_check(A, V, I, slot, bid, it >= cap);
         ++slot;
-        __syncthreads();
-        result = s_go;
-        __syncthreads();
     }
     if (bid == 0 && threadIdx.x == 0) sc->vcycles[V.kind] += it;
     return result;
@@ -1244,11 +1351,11 @@ template <bool REF>
 __device__ bool mg_solve(const EngineArgs &A, const Sync &S, const SolveSpec &V, int &slot,
                          int bid, int nblk, void *smem_base, int *inv_ready) {
     DevScalars *sc = A.sc;
-    if (A.fft.on && !V.screened)
-        return V.nc == 1 ? direct_poisson<1>(A, S, V, bid, nblk, smem_base)
-                         : direct_poisson<2>(A, S, V, bid, nblk, smem_base);
     if (A.fft.on) {
-        const int r = cg_screened<REF>(A, S, V, slot, bid, nblk, smem_base);
+        if (!V.screened)
+            return V.nc == 1 ? direct_poisson<REF, 1>(A, S, V, bid, nblk)
+                             : direct_poisson<REF, 2>(A, S, V, bid, nblk);
+        const int r = cg_screened<REF>(A, S, V, slot, bid, nblk);
         if (r != 0) return r > 0;
         screened_diagonal(A, grid_thr(bid, nblk));
         SYNC(56);
