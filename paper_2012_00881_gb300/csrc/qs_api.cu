@@ -63,7 +63,8 @@ struct qs_ctx {
     double *x = nullptr, *y = nullptr, *px = nullptr, *py = nullptr, *w = nullptr;
     int32_t *id = nullptr;
     float *px32 = nullptr, *py32 = nullptr, *w32 = nullptr;
-    float *g32[6] = {};  // refined form: jx, jy, txx, txy, tyy, G
+    float4 *mom32 = nullptr;  // refined form: the moments, two float4 a cell
+    float2 *psi2 = nullptr;   // refined form: psi as pairs of floats
     std::vector<void *> plasma_allocs;
     bool have_plasma = false, have_step = false;
     // plasma checkpoints of the last qs_step3d (config.checkpoint_every > 0)
@@ -353,15 +354,16 @@ int create_impl(qs_ctx *c) {
         for (int k = 0; k < 5; ++k) AL(L, c->f32[k], nn);
     if (ref) {
         float **g32[] = {&c->e32[0],    &c->e32[1],    &c->r32[0][0], &c->r32[0][1],
-                         &c->r32[1][0], &c->r32[1][1], &c->k32,       &c->d32,
-                         &c->g32[0], &c->g32[1], &c->g32[2], &c->g32[3], &c->g32[4],
-                         &c->g32[5]};
+                         &c->r32[1][0], &c->r32[1][1], &c->k32,       &c->d32};
         for (float **p : g32) {
             AL(L, *p, nn);
             CK(cudaMemsetAsync(*p, 0, nn * sizeof(float), c->st), "memset");
         }
         AL(L, c->r64[0], nn);
         AL(L, c->r64[1], nn);
+        AL(L, c->mom32, 2 * nn);
+        AL(L, c->psi2, nn);
+        CK(cudaMemsetAsync(c->mom32, 0, 2 * nn * sizeof(float4), c->st), "memset");
     }
     AL(L, c->hist, 5 * (size_t)g.n_xi * nn);
     AL(L, c->jzb, (size_t)g.n_xi * nn);
@@ -720,12 +722,8 @@ static int step_prepare(qs_ctx *c, const qs_beam *beams, int n_beams, const int3
     a.px32 = c->px32;
     a.py32 = c->py32;
     a.w32 = c->w32;
-    a.jx32 = c->g32[0];
-    a.jy32 = c->g32[1];
-    a.txx32 = c->g32[2];
-    a.txy32 = c->g32[3];
-    a.tyy32 = c->g32[4];
-    a.G32 = c->g32[5];
+    a.mom32 = c->mom32;
+    a.psi2 = c->psi2;
     a.n_a = c->n_a;
     a.n_b = c->n_b;
     a.n_ion = c->n_ion;

@@ -37,14 +37,20 @@ struct PS {
     P *px, *py, *w;
     double *wd;  // float64 weights: n_* must cancel n_ion to rounding
     double *na, *nb;   // n_* of this slice and of the next one
-    P *jx, *jy, *txx, *txy, *tyy, *G;
+    // the moments j_x, j_y, T_xx, T_xy, T_yy, n_* <gamma> (refined form: <gamma - 1>):
+    // six grids (float64), or the interleaved cells of EngineArgs::mom32
+    P *m[6];
+    static constexpr int stride = sizeof(P) == 8 ? 1 : 8;  // between cells of a moment
+    __device__ __forceinline__ P mom(int k, int i) const { return m[k][(size_t)i * stride]; }
 };
+
+enum { M_JX = 0, M_JY, M_TXX, M_TXY, M_TYY, M_G };
 
 // n_* <gamma> from the gamma moment of either form
 template <typename P>
-__device__ __forceinline__ double g_total(const P *G, const double *n, int i) {
-    if constexpr (sizeof(P) == 8) return G[i];
-    else return n[i] + (double)G[i];
+__device__ __forceinline__ double g_total(P G, double n) {
+    if constexpr (sizeof(P) == 8) return G;
+    else return n + (double)G;
 }
 
 template <typename P>
@@ -73,6 +79,20 @@ __device__ __forceinline__ void dep(P *g, const CicP<P> &c, P q) {
     atomicAdd(g + c.i01, q * c.w01);
     atomicAdd(g + c.i10, q * c.w10);
     atomicAdd(g + c.i11, q * c.w11);
+}
+
+// Six float32 moments q of a particle into one cell with weight w: two vector
+// reductions of the cell's sector instead of six scalar ones.  The moments
+// phase is bound by the reductions: 262,144 particles send 6.3 M scalar ones
+// (256^2, MOMOLD us), 2.1 M vector ones MOMNEW us.
+__device__ __forceinline__ void dep6(float4 *m, int i, float w, const float (&q)[6]) {
+    float4 *a = m + 2 * (size_t)i;
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(a), "f"(q[0] * w),
+                 "f"(q[1] * w), "f"(q[2] * w), "f"(q[3] * w)
+                 : "memory");
+    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(a + 1), "f"(q[4] * w),
+                 "f"(q[5] * w)
+                 : "memory");
 }
 
 // 1 / a in float64 for a >= psi_floor > 0 by Newton's iteration for the
@@ -146,7 +166,7 @@ __device__ Band band_of(const EngineArgs &A, const double *y, int64_t p0, int64_
 
 // deposit q into the band s (cells lo .. hi - 1 of the grid) when the whole
 // stencil is inside, else into the grid g
-template <typename P, typename W>
+template <int ST = 1, typename P, typename W>
 __device__ __forceinline__ void dep_band(P *g, P *s, int lo, int hi, const W &c, P q) {
     const int a = min(min(c.i00, c.i01), min(c.i10, c.i11));
     const int b = max(max(c.i00, c.i01), max(c.i10, c.i11));
@@ -156,19 +176,19 @@ __device__ __forceinline__ void dep_band(P *g, P *s, int lo, int hi, const W &c,
         atomicAdd(s + (c.i10 - lo), q * (P)c.w10);
         atomicAdd(s + (c.i11 - lo), q * (P)c.w11);
     } else {
-        atomicAdd(g + c.i00, q * (P)c.w00);
-        atomicAdd(g + c.i01, q * (P)c.w01);
-        atomicAdd(g + c.i10, q * (P)c.w10);
-        atomicAdd(g + c.i11, q * (P)c.w11);
+        atomicAdd(g + (size_t)c.i00 * ST, q * (P)c.w00);
+        atomicAdd(g + (size_t)c.i01 * ST, q * (P)c.w01);
+        atomicAdd(g + (size_t)c.i10 * ST, q * (P)c.w10);
+        atomicAdd(g + (size_t)c.i11 * ST, q * (P)c.w11);
     }
 }
 
 // the band's nonzero cells added to the grid, one atomic per cell
-template <typename P>
+template <int ST = 1, typename P>
 __device__ __forceinline__ void flush_band(P *g, const P *s, int lo, int cells) {
     for (int k = threadIdx.x; k < cells; k += blockDim.x) {
         const P v = s[k];
-        if (v != P(0)) atomicAdd(g + lo + k, v);
+        if (v != P(0)) atomicAdd(g + (size_t)(lo + k) * ST, v);
     }
 }
 
@@ -240,12 +260,12 @@ __device__ void phase_psi_rhs(const EngineArgs &A, const PS<P> &Q, const double 
         A.f_psi[i] = f;
         s += f * f;
         cs += nv;
-        Q.jx[i] = P(0);
-        Q.jy[i] = P(0);
-        Q.txx[i] = P(0);
-        Q.txy[i] = P(0);
-        Q.tyy[i] = P(0);
-        Q.G[i] = P(0);
+        if constexpr (sizeof(P) == 8) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) Q.m[k][i] = 0.0;
+        } else {
+            A.mom32[2 * (size_t)i] = A.mom32[2 * (size_t)i + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
         nnext[i] = 0.0;
     }
     s = block_sum(s);
@@ -256,12 +276,109 @@ __device__ void phase_psi_rhs(const EngineArgs &A, const PS<P> &Q, const double 
     }
 }
 
-// gather psi at every particle; deposit j_perp, T, G (Eqs. Jr, FluxPres);
-// gamma from the constant of motion is always evaluated in float64
+// The CIC stencil of the refined form from one fused multiply-add an axis:
+// s + 1/2 = x / h + const in [1/2, N + 1/2] inside the box, whose integer part
+// and fraction come from its bits (a floor, a conversion and the differences
+// would be five FP64-pipe instructions an axis).  f: the fraction as a pair.
+struct AxisBits {
+    int cell;   // floor(s + 1/2): the right one of the two cells
+    qsff::Ff f; // weight of the right cell
+};
+__device__ __forceinline__ AxisBits axis_bits(double t) {
+    const unsigned hi = (unsigned)__double2hiint(t), lo = (unsigned)__double2loint(t);
+    const int e = (int)(hi >> 20) - 1023;  // -1 ... 11 in the box
+    AxisBits b;
+    if ((unsigned)(e + 1) > 12u) {  // outside the box (negative, or far beyond it)
+        const double fl = floor(t);
+        b.cell = (int)fl;
+        b.f = qsff::split(t - fl);
+        return b;
+    }
+    const unsigned mh = (hi & 0xfffffu) | 0x100000u;
+    b.cell = (int)(mh >> (20 - e));
+    // the fraction as 64 bits: shift the integer part out at the top
+    const int sh = 12 + e;
+    const unsigned fh = __funnelshift_l(lo, mh, sh), fl = lo << sh;
+    const float h = (float)(fh & 0xffffff00u);
+    const float l = (float)((fh << 24) | (fl >> 8));
+    b.f = qsff::quick(h * 0x1p-32f, l * 0x1p-56f);
+    return b;
+}
+
+// s + 1/2 of a coordinate (s = (x - x_min) / h)
+__device__ __forceinline__ double axis_pos(double x, double inv_h, double x_min) {
+    return fma(x, inv_h, fma(-x_min, inv_h, 0.5));
+}
+
+// folded cell indices of an axis: the ghost's weight goes to the edge cell
+__device__ __forceinline__ void fold(int right, int n, int &a, int &b) {
+    a = right - 1;
+    b = right;
+    if (a < 0) a = -1 - a;
+    if (b > n - 1) b = 2 * n - 1 - b;
+    a = min(max(a, 0), n - 1);
+    b = min(max(b, 0), n - 1);
+}
+
+struct CicF {
+    int i00, i01, i10, i11;
+    qsff::Ff w00, w01, w10, w11;
+    __device__ __forceinline__ CicP<float> single() const {
+        CicP<float> r;
+        r.i00 = i00; r.i01 = i01; r.i10 = i10; r.i11 = i11;
+        r.w00 = w00.h; r.w01 = w01.h; r.w10 = w10.h; r.w11 = w11.h;
+        return r;
+    }
+};
+
+__device__ __forceinline__ CicF cic_pairs(double tx, double ty, int n) {
+    const AxisBits bx = axis_bits(tx), by = axis_bits(ty);
+    int ax, cx, ay, cy;
+    fold(bx.cell, n, ax, cx);
+    fold(by.cell, n, ay, cy);
+    const qsff::Ff one(1.f, 0.f), gx = one - bx.f, gy = one - by.f;
+    CicF c;
+    c.i00 = ay * n + ax;
+    c.i01 = ay * n + cx;
+    c.i10 = cy * n + ax;
+    c.i11 = cy * n + cx;
+    c.w00 = gy * gx;
+    c.w01 = gy * bx.f;
+    c.w10 = by.f * gx;
+    c.w11 = by.f * bx.f;
+    return c;
+}
+
+__device__ __forceinline__ qsff::Ff gather_pairs(const float2 *u, const CicF &c) {
+    const float2 a = u[c.i00], b = u[c.i01], d = u[c.i10], e = u[c.i11];
+    using qsff::Ff;
+    return (Ff(a.x, a.y) * c.w00 + Ff(b.x, b.y) * c.w01) +
+           (Ff(d.x, d.y) * c.w10 + Ff(e.x, e.y) * c.w11);
+}
+__device__ __forceinline__ qsff::Ff gather_pairs(const double *u, const CicF &c) {
+    using namespace qsff;
+    return (split(u[c.i00]) * c.w00 + split(u[c.i01]) * c.w01) +
+           (split(u[c.i10]) * c.w10 + split(u[c.i11]) * c.w11);
+}
+
+// 1 + psi at a particle, not below the floor
+__device__ __forceinline__ qsff::Ff one_plus_psi(qsff::Ff psi, qsff::Ff floor_, unsigned &hits) {
+    qsff::Ff a = qsff::Ff(1.f, 0.f) + psi;
+    if (a.h < floor_.h || (a.h == floor_.h && a.l < floor_.l)) {
+        ++hits;
+        a = floor_;
+    }
+    return a;
+}
+
+// gather psi at every particle; deposit j_perp, T, G (Eqs. Jr, FluxPres).
+// gamma from the constant of motion is evaluated in float64, in the refined
+// form in pairs of floats.
 template <typename P>
 __device__ void phase_moments(const EngineArgs &A, const PS<P> &Q, Thr T, int bid, int nblk,
                               void *smem) {
     const P s = (P)(A.inv_h * A.inv_h);
+    constexpr int ST = PS<P>::stride;
     unsigned hits = 0;
     // privatised: this block's chunk into the six bands of sb
     const bool banded = A.band_rows > 0;
@@ -282,55 +399,79 @@ __device__ void phase_moments(const EngineArgs &A, const PS<P> &Q, Thr T, int bi
         p1 = c1;
         pst = blockDim.x;
     }
-    auto put = [&](P *g, int k, const CicP<P> &c, P q) {
-        if (banded) dep_band(g, sb + k * cells, lo, hi, c, q);
-        else dep(g, c, q);
-    };
-    for (int64_t p = p0; p < p1; p += pst) {
-        const Cic cd = cic_stencil_inv(Q.x[p], Q.y[p], A.x_min, A.y_min, A.inv_h, A.N);
-        const CicP<P> c = cic_p<P>(cd);
-        const double a = guard(1.0 + cic_gather(A.psi, cd), A.psi_floor, hits);
-        const P px = Q.px[p], py = Q.py[p];
-        const double p2 = (double)px * px + (double)py * py;
-        // one reciprocal per particle (float64 divides are slow)
-        const double ia = sizeof(P) == 8 ? 1.0 / a : rcp_newton(a);
-        const P iap = (P)ia;
-        const P vx = px * iap, vy = py * iap;
-        const P wq = Q.w[p] * s;
-        // the laser's |A|^2 / 2 in the numerator of gamma (line after Eq. EoM_111)
-        const double ha2 = A.a2_base ? 0.5 * cic_gather(A.a2, cd) : 0.0;
-        put(Q.jx, 0, c, wq * vx);
-        put(Q.jy, 1, c, wq * vy);
-        put(Q.txx, 2, c, wq * vx * vx);
-        put(Q.txy, 3, c, wq * vx * vy);
-        put(Q.tyy, 4, c, wq * vy * vy);
-        if constexpr (sizeof(P) == 8) {
-            put(Q.G, 5, c, wq * ((1.0 + p2 + a * a + ha2) * (0.5 * ia)));  // gamma
-        } else {
-            const double am1 = a - 1.0;  // gamma - 1 = (p^2 + psi^2) / (2 (1 + psi))
-            put(Q.G, 5, c, wq * (P)((p2 + am1 * am1 + ha2) * (0.5 * ia)));
+    if constexpr (sizeof(P) == 8) {
+        auto put = [&](int k, const CicP<P> &c, P q) {
+            if (banded) dep_band(Q.m[k], sb + k * cells, lo, hi, c, q);
+            else dep(Q.m[k], c, q);
+        };
+        for (int64_t p = p0; p < p1; p += pst) {
+            const Cic cd = cic_stencil_inv(Q.x[p], Q.y[p], A.x_min, A.y_min, A.inv_h, A.N);
+            const CicP<P> c = cic_p<P>(cd);
+            const double a = guard(1.0 + cic_gather(A.psi, cd), A.psi_floor, hits);
+            const P px = Q.px[p], py = Q.py[p];
+            const double p2 = px * px + py * py;
+            const double ia = 1.0 / a;  // one reciprocal per particle
+            const P vx = px * ia, vy = py * ia;
+            const P wq = Q.w[p] * s;
+            // the laser's |A|^2 / 2 in the numerator of gamma (line after Eq. EoM_111)
+            const double ha2 = A.a2_base ? 0.5 * cic_gather(A.a2, cd) : 0.0;
+            put(M_JX, c, wq * vx);
+            put(M_JY, c, wq * vy);
+            put(M_TXX, c, wq * vx * vx);
+            put(M_TXY, c, wq * vx * vy);
+            put(M_TYY, c, wq * vy * vy);
+            put(M_G, c, wq * ((1.0 + p2 + a * a + ha2) * (0.5 * ia)));  // gamma
+        }
+    } else {
+        using qsff::Ff;
+        const Ff fl = qsff::split(A.psi_floor);
+        const double ox = fma(-A.x_min, A.inv_h, 0.5), oy = fma(-A.y_min, A.inv_h, 0.5);
+        for (int64_t p = p0; p < p1; p += pst) {
+            const CicF cf = cic_pairs(fma(Q.x[p], A.inv_h, ox), fma(Q.y[p], A.inv_h, oy), A.N);
+            const CicP<P> c = cf.single();
+            const Ff a = one_plus_psi(gather_pairs(A.psi2, cf), fl, hits);
+            const P px = Q.px[p], py = Q.py[p];
+            const Ff ia = qsff::recip(a);
+            const P vx = px * ia.h, vy = py * ia.h;
+            const P wq = Q.w[p] * s;
+            // gamma - 1 = (p^2 + psi^2 + |A|^2 / 2) / (2 (1 + psi))
+            const Ff am1 = a + Ff(-1.f, 0.f);
+            Ff g = qsff::two_prod(px, px) + qsff::two_prod(py, py) + am1 * am1;
+            if (A.a2_base) g += gather_pairs(A.a2, cf) * 0.5f;
+            g = g * (ia * 0.5f);
+            const float q[6] = {wq * vx, wq * vy, wq * vx * vx, wq * vx * vy, wq * vy * vy,
+                                wq * g.h};
+            if (banded) {
+#pragma unroll
+                for (int k = 0; k < 6; ++k)
+                    dep_band<ST>(Q.m[k], sb + k * cells, lo, hi, c, q[k]);
+            } else {
+                dep6(A.mom32, c.i00, c.w00, q);
+                dep6(A.mom32, c.i01, c.w01, q);
+                dep6(A.mom32, c.i10, c.w10, q);
+                dep6(A.mom32, c.i11, c.w11, q);
+            }
         }
     }
     add_hits(A.sc, hits);
     if (banded) {
         __syncthreads();
-        P *const g[6] = {Q.jx, Q.jy, Q.txx, Q.txy, Q.tyy, Q.G};
 #pragma unroll
-        for (int k = 0; k < 6; ++k) flush_band(g[k], sb + k * cells, lo, cells);
+        for (int k = 0; k < 6; ++k) flush_band<ST>(Q.m[k], sb + k * cells, lo, cells);
     }
 }
 
 // central differences: zero ghosts (moments) and odd ghosts (fields)
-template <typename G>
+template <int ST = 1, typename G>
 __device__ __forceinline__ double dx0(const G *u, int n, int ix, int i, double inv2h) {
-    const double e = ix < n - 1 ? (double)u[i + 1] : 0.0;
-    const double w = ix > 0 ? (double)u[i - 1] : 0.0;
+    const double e = ix < n - 1 ? (double)u[(size_t)(i + 1) * ST] : 0.0;
+    const double w = ix > 0 ? (double)u[(size_t)(i - 1) * ST] : 0.0;
     return (e - w) * inv2h;
 }
-template <typename G>
+template <int ST = 1, typename G>
 __device__ __forceinline__ double dy0(const G *u, int n, int iy, int i, double inv2h) {
-    const double s = iy < n - 1 ? (double)u[i + n] : 0.0;
-    const double q = iy > 0 ? (double)u[i - n] : 0.0;
+    const double s = iy < n - 1 ? (double)u[(size_t)(i + n) * ST] : 0.0;
+    const double q = iy > 0 ? (double)u[(size_t)(i - n) * ST] : 0.0;
     return (s - q) * inv2h;
 }
 __device__ __forceinline__ double dxo(const double *u, int n, int ix, int i, double inv2h) {
@@ -350,6 +491,7 @@ template <typename P>
 __device__ void phase_assemble1(const EngineArgs &A, const PS<P> &Q, const double *ncur, int j,
                                 int q, double frac, Thr T, const Guess &g) {
     const int n = A.N, nn = n * n;
+    constexpr int ST = PS<P>::stride;
     const double inv2h = 0.5 * A.inv_h;
     const double *J0 = A.jzb + (size_t)j * nn;
     const double *J1 = (j + 1 < A.n_xi) ? A.jzb + (size_t)(j + 1) * nn : nullptr;
@@ -361,8 +503,8 @@ __device__ void phase_assemble1(const EngineArgs &A, const PS<P> &Q, const doubl
             apply_guess(A.ez, A.hist1[1], A.hist2[1], i, g);
             apply_guess(A.bz, A.hist1[2], A.hist2[2], i, g);
         }
-        double fez = -(dx0(Q.jx, n, ix, i, inv2h) + dy0(Q.jy, n, iy, i, inv2h));
-        double fbz = dx0(Q.jy, n, ix, i, inv2h) - dy0(Q.jx, n, iy, i, inv2h);
+        double fez = -(dx0<ST>(Q.m[M_JX], n, ix, i, inv2h) + dy0<ST>(Q.m[M_JY], n, iy, i, inv2h));
+        double fbz = dx0<ST>(Q.m[M_JY], n, ix, i, inv2h) - dy0<ST>(Q.m[M_JX], n, iy, i, inv2h);
         A.f_ez[i] = fez;
         A.f_bz[i] = fbz;
         sez += fez * fez;
@@ -371,7 +513,7 @@ __device__ void phase_assemble1(const EngineArgs &A, const PS<P> &Q, const doubl
         double jzb = q == 0 ? J0[i] : (1.0 - frac) * J0[i] + frac * (J1 ? J1[i] : 0.0);
         const double nv = ncur[i];
         const double ia = 1.0 / a;
-        A.jz[i] = g_total(Q.G, ncur, i) * ia - nv + jzb;
+        A.jz[i] = g_total(Q.mom(M_G, i), nv) * ia - nv + jzb;
         const double kap = nv * ia;
         A.kap[i] = kap;
         sk += kap;
@@ -416,6 +558,7 @@ template <typename P>
 __device__ void phase_assemble2(const EngineArgs &A, const PS<P> &Q, const double *ncur, Thr T,
                                 const Guess &g) {
     const int n = A.N, nn = n * n;
+    constexpr int ST = PS<P>::stride;
     const double inv2h = 0.5 * A.inv_h;
     double sbx = 0.0, sby = 0.0;
     for (int i = T.t0; i < nn; i += T.nt) {
@@ -426,16 +569,17 @@ __device__ void phase_assemble2(const EngineArgs &A, const PS<P> &Q, const doubl
         }
         double a = 1.0 + A.psi[i];
         if (a < A.psi_floor) a = A.psi_floor;
-        const double jx = Q.jx[i], jy = Q.jy[i], txx = Q.txx[i], txy = Q.txy[i],
-                     tyy = Q.tyy[i], G = g_total(Q.G, ncur, i), ez = A.ez[i], bz = A.bz[i];
+        const double jx = Q.mom(M_JX, i), jy = Q.mom(M_JY, i), txx = Q.mom(M_TXX, i),
+                     txy = Q.mom(M_TXY, i), tyy = Q.mom(M_TYY, i),
+                     G = g_total(Q.mom(M_G, i), ncur[i]), ez = A.ez[i], bz = A.bz[i];
         if (A.bz32) A.bz32[i] = (float)bz;  // B_z is final here
         const double gx = A.dpx[i], gy = A.dpy[i];
         const double ia = 1.0 / a, Gia2 = G * ia * ia;
-        double sx = dx0(A.jz, n, ix, i, inv2h) - dx0(Q.txx, n, ix, i, inv2h) -
-                    dy0(Q.txy, n, iy, i, inv2h) + Gia2 * gx -
+        double sx = dx0(A.jz, n, ix, i, inv2h) - dx0<ST>(Q.m[M_TXX], n, ix, i, inv2h) -
+                    dy0<ST>(Q.m[M_TXY], n, iy, i, inv2h) + Gia2 * gx -
                     (jy * bz + jx * ez + txx * gx + txy * gy) * ia;
-        double sy = dy0(A.jz, n, iy, i, inv2h) - dx0(Q.txy, n, ix, i, inv2h) -
-                    dy0(Q.tyy, n, iy, i, inv2h) + Gia2 * gy +
+        double sy = dy0(A.jz, n, iy, i, inv2h) - dx0<ST>(Q.m[M_TXY], n, ix, i, inv2h) -
+                    dy0<ST>(Q.m[M_TYY], n, iy, i, inv2h) + Gia2 * gy +
                     (jx * bz - jy * ez - txy * gx - tyy * gy) * ia;
         if (A.a2_base) {  // -n_* grad(|A|^2/4) / (1+psi)^2 of Eq. FluxCurr1_A
             const double nia2 = ncur[i] * ia * ia;
@@ -451,6 +595,38 @@ __device__ void phase_assemble2(const EngineArgs &A, const PS<P> &Q, const doubl
     if (threadIdx.x == 0) atomicAdd(&A.sc->fnorm[2][0], sbx);
     sby = block_sum(sby);
     if (threadIdx.x == 0) atomicAdd(&A.sc->fnorm[2][1], sby);
+}
+
+// (double)i for 0 <= i < 2^31 without a conversion: 2^52 + i is exact
+__device__ __forceinline__ double whole(int i) {
+    return __hiloint2double(0x43300000, i) - 4503599627370496.0;
+}
+
+// specular wall
+template <typename P>
+__device__ __forceinline__ void reflect(double &x, P &p, double lo, double hi) {
+    if (x > hi) { x = 2.0 * hi - x; p = -p; }
+    if (x < lo) { x = 2.0 * lo - x; p = -p; }
+}
+
+// The Boris-like momentum step: half kick (gamma grad psi - grad(|A|^2/4)) /
+// (1+psi) + e_z x B_perp, rotation by the B_z term (e_z x p) B_z / (1+psi),
+// half kick with the new gamma.
+template <typename P, typename F>
+__device__ __forceinline__ void boris_like(P &px, P &py, F gamma, P gx, P gy, P bx, P by, P bz,
+                                           P fx, P fy, P ia, P half) {
+    const P gam = gamma(px, py);
+    const P pxm = px + half * ((gam * gx - fx) * ia - by);
+    const P pym = py + half * ((gam * gy - fy) * ia + bx);
+    const P tau = half * bz * ia;
+    const P pxp = pxm - tau * pym;
+    const P pyp = pym + tau * pxm;
+    const P sr = P(2) * tau / (P(1) + tau * tau);
+    const P pxr = pxm - sr * pyp;
+    const P pyr = pym + sr * pxp;
+    const P gam2 = gamma(pxr, pyr);
+    px = pxr + half * ((gam2 * gx - fx) * ia - by);
+    py = pyr + half * ((gam2 * gy - fy) * ia + bx);
 }
 
 // store the base slice; push every trajectory (Eqs. EoM_112_A, EoM_111);
@@ -470,12 +646,12 @@ __device__ void phase_push(const EngineArgs &A, const PS<P> &Q, double *nnext, b
             g[SG_BX * nn + i] = A.bx[i];
             g[SG_BY * nn + i] = A.by[i];
             g[SG_N * nn + i] = ncur[i];
-            g[SG_JX * nn + i] = (double)Q.jx[i];
-            g[SG_JY * nn + i] = (double)Q.jy[i];
-            g[SG_TXX * nn + i] = (double)Q.txx[i];
-            g[SG_TXY * nn + i] = (double)Q.txy[i];
-            g[SG_TYY * nn + i] = (double)Q.tyy[i];
-            g[SG_G * nn + i] = g_total(Q.G, ncur, i);
+            g[SG_JX * nn + i] = (double)Q.mom(M_JX, i);
+            g[SG_JY * nn + i] = (double)Q.mom(M_JY, i);
+            g[SG_TXX * nn + i] = (double)Q.mom(M_TXX, i);
+            g[SG_TXY * nn + i] = (double)Q.mom(M_TXY, i);
+            g[SG_TYY * nn + i] = (double)Q.mom(M_TYY, i);
+            g[SG_G * nn + i] = g_total(Q.mom(M_G, i), ncur[i]);
         }
         double *sp = A.seg_p + (size_t)sub * 4 * A.np;
         for (int64_t p = T.t0; p < A.np; p += T.nt) {
@@ -500,7 +676,7 @@ __device__ void phase_push(const EngineArgs &A, const PS<P> &Q, double *nnext, b
     const double s = A.inv_h * A.inv_h;
     const P half = (P)(0.5 * dxi), dxp = (P)dxi;
     unsigned hits = 0;
-    P vm = P(0);  // V_max (refined form: its square, in float32)
+    P vm = P(0);  // the square of V_max (refined form: in float32)
     // privatised n_* of the next slice: the band of the chunk's present rows
     // widened by two rows for the particles' motion
     const bool banded = A.band_rows_n > 0;
@@ -521,79 +697,121 @@ __device__ void phase_push(const EngineArgs &A, const PS<P> &Q, double *nnext, b
         p1 = c1;
         pst = blockDim.x;
     }
-    for (int64_t p = p0; p < p1; p += pst) {
-        const double x = Q.x[p], y = Q.y[p];
-        const Cic cd = cic_stencil_inv(x, y, A.x_min, A.y_min, A.inv_h, A.N);
-        const CicP<P> c = cic_p<P>(cd);
-        const double a = guard(1.0 + cic_gather(A.psi, cd), A.psi_floor, hits);
-        const double ia = sizeof(P) == 8 ? 1.0 / a : rcp_newton(a);
-        const P iap = (P)ia;
-        P gx, gy, bx, by, bz;
-        if constexpr (sizeof(P) == 8) {
-            gx = gat<P>(A.dpx, c);
-            gy = gat<P>(A.dpy, c);
-            bx = gat<P>(A.bx, c);
-            by = gat<P>(A.by, c);
-            bz = gat<P>(A.bz, c);
-        } else {  // the float32 copies: no conversions
-            gx = gat<P>(A.dpx32, c);
-            gy = gat<P>(A.dpy32, c);
-            bx = gat<P>(A.bx32, c);
-            by = gat<P>(A.by32, c);
-            bz = gat<P>(A.bz32, c);
+    if constexpr (sizeof(P) == 8) {
+        for (int64_t p = p0; p < p1; p += pst) {
+            const double x = Q.x[p], y = Q.y[p];
+            const Cic cd = cic_stencil_inv(x, y, A.x_min, A.y_min, A.inv_h, A.N);
+            const CicP<P> c = cic_p<P>(cd);
+            const double a = guard(1.0 + cic_gather(A.psi, cd), A.psi_floor, hits);
+            const double ia = 1.0 / a;
+            const P gx = gat<P>(A.dpx, c), gy = gat<P>(A.dpy, c), bx = gat<P>(A.bx, c),
+                    by = gat<P>(A.by, c), bz = gat<P>(A.bz, c);
+            P px = Q.px[p], py = Q.py[p];
+            // laser (Eq. EoM_111): |A|^2 / 2 in gamma and the ponderomotive force
+            // -grad(|A|^2/4) / (1+psi); zero without a laser
+            double ha2 = 0.0;
+            P fx = P(0), fy = P(0);
+            if (A.a2_base) {
+                ha2 = 0.5 * cic_gather(A.a2, cd);
+                fx = gat<P>(A.pondx, c);
+                fy = gat<P>(A.pondy, c);
+            }
+            const double q1 = 1.0 + a * a + ha2, h_ia = 0.5 * ia;
+            auto gamma = [&](P u, P v) { return (q1 + u * u + v * v) * h_ia; };
+            boris_like(px, py, gamma, gx, gy, bx, by, bz, fx, fy, ia, half);
+            double nx = x + dxp * px * ia;
+            double ny = y + dxp * py * ia;
+            reflect(nx, px, A.x_min, A.x_max);
+            reflect(ny, py, A.y_min, A.y_max);
+            Q.x[p] = nx;
+            Q.y[p] = ny;
+            Q.px[p] = px;
+            Q.py[p] = py;
+            vm = fmax(vm, (px * px + py * py) * (ia * ia));
+            const Cic c2 = cic_stencil_inv(nx, ny, A.x_min, A.y_min, A.inv_h, A.N);
+            if (banded) dep_band(nnext, sb, lo, hi, c2, Q.wd[p] * s);
+            else cic_deposit(nnext, c2, Q.wd[p] * s);
         }
-        P px = Q.px[p], py = Q.py[p];
-        // laser (Eq. EoM_111): |A|^2 / 2 in gamma and the ponderomotive force
-        // -grad(|A|^2/4) / (1+psi); zero without a laser
-        double ha2 = 0.0;
-        P fx = P(0), fy = P(0);
-        if (A.a2_base) {
-            ha2 = 0.5 * cic_gather(A.a2, cd);
-            fx = gat<P>(A.pondx, c);
-            fy = gat<P>(A.pondy, c);
+    } else {
+        using qsff::Ff;
+        const Ff fl = qsff::split(A.psi_floor), one(1.f, 0.f);
+        const double ox = fma(-A.x_min, A.inv_h, 0.5), oy = fma(-A.y_min, A.inv_h, 0.5);
+        for (int64_t p = p0; p < p1; p += pst) {
+            const double x = Q.x[p], y = Q.y[p];
+            const CicF cf = cic_pairs(fma(x, A.inv_h, ox), fma(y, A.inv_h, oy), A.N);
+            const CicP<P> c = cf.single();
+            const Ff a = one_plus_psi(gather_pairs(A.psi2, cf), fl, hits);
+            const Ff ia2 = qsff::recip(a);
+            const P ia = ia2.h;
+            const P gx = gat<P>(A.dpx32, c), gy = gat<P>(A.dpy32, c), bx = gat<P>(A.bx32, c),
+                    by = gat<P>(A.by32, c), bz = gat<P>(A.bz32, c);
+            P px = Q.px[p], py = Q.py[p];
+            Ff q1 = one + a * a;
+            P fx = P(0), fy = P(0);
+            if (A.a2_base) {
+                q1 += gather_pairs(A.a2, cf) * 0.5f;
+                fx = gat<P>(A.pondx, c);
+                fy = gat<P>(A.pondy, c);
+            }
+            const Ff h_ia = ia2 * 0.5f;
+            auto gamma = [&](P u, P v) {
+                return ((q1 + (qsff::two_prod(u, u) + qsff::two_prod(v, v))) * h_ia).h;
+            };
+            boris_like(px, py, gamma, gx, gy, bx, by, bz, fx, fy, ia, half);
+            double nx = x + qsff::widen(dxp * px * ia);
+            double ny = y + qsff::widen(dxp * py * ia);
+            double tx = fma(nx, A.inv_h, ox), ty = fma(ny, A.inv_h, oy);
+            AxisBits ax = axis_bits(tx), ay = axis_bits(ty);
+            // only a particle in the half cells at the walls can have crossed one
+            if ((unsigned)(ax.cell - 1) >= (unsigned)(A.N - 1) ||
+                (unsigned)(ay.cell - 1) >= (unsigned)(A.N - 1)) {
+                reflect(nx, px, A.x_min, A.x_max);
+                reflect(ny, py, A.y_min, A.y_max);
+                tx = fma(nx, A.inv_h, ox);
+                ty = fma(ny, A.inv_h, oy);
+                ax = axis_bits(tx);
+                ay = axis_bits(ty);
+            }
+            Q.x[p] = nx;
+            Q.y[p] = ny;
+            Q.px[p] = px;
+            Q.py[p] = py;
+            vm = fmaxf(vm, (px * px + py * py) * (ia * ia));
+            // n_* stays in float64: it must cancel n_ion to rounding
+            Cic c2;
+            int i0, i1, j0, j1;
+            fold(ax.cell, A.N, i0, i1);
+            fold(ay.cell, A.N, j0, j1);
+            c2.i00 = j0 * A.N + i0;
+            c2.i01 = j0 * A.N + i1;
+            c2.i10 = j1 * A.N + i0;
+            c2.i11 = j1 * A.N + i1;
+            const double wx = tx - whole(ax.cell), wy = ty - whole(ay.cell);
+            const double q = Q.wd[p] * s, qy = q * wy, qn = q - qy;
+            const double q11 = qy * wx, q01 = qn * wx;
+            const double q10 = qy - q11, q00 = qn - q01;
+            if (banded && min(min(c2.i00, c2.i01), min(c2.i10, c2.i11)) >= lo &&
+                max(max(c2.i00, c2.i01), max(c2.i10, c2.i11)) < hi) {
+                atomicAdd(sb + (c2.i00 - lo), q00);
+                atomicAdd(sb + (c2.i01 - lo), q01);
+                atomicAdd(sb + (c2.i10 - lo), q10);
+                atomicAdd(sb + (c2.i11 - lo), q11);
+            } else {
+                atomicAdd(nnext + c2.i00, q00);
+                atomicAdd(nnext + c2.i01, q01);
+                atomicAdd(nnext + c2.i10, q10);
+                atomicAdd(nnext + c2.i11, q11);
+            }
         }
-        // half kick: (gamma grad psi - grad(|A|^2/4)) / (1+psi) + e_z x B_perp
-        const double gam = (1.0 + (double)px * px + (double)py * py + a * a + ha2) * (0.5 * ia);
-        const P pxm = px + half * (((P)gam * gx - fx) * iap - by);
-        const P pym = py + half * (((P)gam * gy - fy) * iap + bx);
-        // rotation by the B_z term (e_z x p) B_z / (1+psi)
-        const P tau = half * bz * iap;
-        const P pxp = pxm - tau * pym;
-        const P pyp = pym + tau * pxm;
-        const P sr = P(2) * tau / (P(1) + tau * tau);
-        const P pxr = pxm - sr * pyp;
-        const P pyr = pym + sr * pxp;
-        const double gam2 =
-            (1.0 + (double)pxr * pxr + (double)pyr * pyr + a * a + ha2) * (0.5 * ia);
-        px = pxr + half * (((P)gam2 * gx - fx) * iap - by);
-        py = pyr + half * (((P)gam2 * gy - fy) * iap + bx);
-        double nx = x + (double)(dxp * px * iap);
-        double ny = y + (double)(dxp * py * iap);
-        if (nx > A.x_max) { nx = 2.0 * A.x_max - nx; px = -px; }
-        if (nx < A.x_min) { nx = 2.0 * A.x_min - nx; px = -px; }
-        if (ny > A.y_max) { ny = 2.0 * A.y_max - ny; py = -py; }
-        if (ny < A.y_min) { ny = 2.0 * A.y_min - ny; py = -py; }
-        Q.x[p] = nx;
-        Q.y[p] = ny;
-        Q.px[p] = px;
-        Q.py[p] = py;
-        if constexpr (sizeof(P) == 8) {
-            vm = fmax(vm, sqrt((double)px * px + (double)py * py) * ia);
-        } else {  // float32 (the step rule needs a few digits); squared, root below
-            vm = fmaxf(vm, (px * px + py * py) * (iap * iap));
-        }
-        const Cic c2 = cic_stencil_inv(nx, ny, A.x_min, A.y_min, A.inv_h, A.N);
-        if (banded) dep_band(nnext, sb, lo, hi, c2, Q.wd[p] * s);
-        else cic_deposit(nnext, c2, Q.wd[p] * s);
     }
     add_hits(A.sc, hits);
     if (banded) {
         __syncthreads();
         flush_band(nnext, sb, lo, cells);
     }
-    double vmax = block_max((double)vm);
-    if (sizeof(P) == 4) vmax = sqrt(vmax);
+    double vmax = block_max(vm);
     if (threadIdx.x == 0) {
+        vmax = sqrt(vmax);
         atomicMax(&A.sc->vmax_bits[pk & 1], (unsigned long long)__double_as_longlong(vmax));
         atomicMax(&A.sc->vmax_all_bits, (unsigned long long)__double_as_longlong(vmax));
     }
@@ -741,11 +959,12 @@ __device__ bool run_step(const EngineArgs &A, int bid, int nblk, const Sync &S, 
     using P = typename std::conditional<REF, float, double>::type;
     PS<P> Q;
     if constexpr (REF) {
+        float *const f = (float *)A.mom32;
         Q = PS<P>{A.x, A.y, A.px32, A.py32, A.w32, A.w, A.n_a, A.n_b,
-                  A.jx32, A.jy32, A.txx32, A.txy32, A.tyy32, A.G32};
+                  {f, f + 1, f + 2, f + 3, f + 4, f + 5}};
     } else {
         Q = PS<P>{A.x, A.y, A.px, A.py, A.w, A.w, A.n_a, A.n_b,
-                  A.jx, A.jy, A.txx, A.txy, A.tyy, A.G};
+                  {A.jx, A.jy, A.txx, A.txy, A.tyy, A.G}};
     }
     // the spare particle set of the in-loop sort (not with the adjoint's
     // checkpoints or slice store: those keep the lattice's order)
@@ -755,7 +974,8 @@ __device__ bool run_step(const EngineArgs &A, int bid, int nblk, const Sync &S, 
     phase_deposit_n<P>(A, Q, ncur, T);
     if (!S(1)) return false;
 
-    const SolveSpec Vpsi{1, 0, {A.psi, nullptr}, {A.f_psi, nullptr}, false};
+    SolveSpec Vpsi{1, 0, {A.psi, nullptr}, {A.f_psi, nullptr}, false};
+    if (REF) Vpsi.pairs = A.psi2;
     const SolveSpec Veb{2, 1, {A.ez, A.bz}, {A.f_ez, A.f_bz}, false};
     const SolveSpec Vbp{2, 2, {A.bx, A.by}, {A.f_bx, A.f_by}, true,
                         {REF ? A.bx32 : nullptr, REF ? A.by32 : nullptr}};
@@ -811,6 +1031,13 @@ __device__ bool run_step(const EngineArgs &A, int bid, int nblk, const Sync &S, 
             phase_psi_rhs<P>(A, Q, ncur, nnext, base, j, q, frac, T, g);
             if (!S(2)) return false;
             if (!mg_solve<REF>(A, S, Vpsi, slot, bid, nblk, smem, s_inv_ready)) return false;
+            if (REF && !A.fft.on) {  // the transforms' last phase writes the pairs itself
+                for (int i = T.t0; i < A.N * A.N; i += T.nt) {
+                    const qsff::Ff v = qsff::split(A.psi[i]);
+                    A.psi2[i] = make_float2(v.h, v.l);
+                }
+                if (!S(7)) return false;
+            }
             phase_moments<P>(A, Q, T, bid, nblk, smem);
             if (!S(3)) return false;
             phase_assemble1<P>(A, Q, ncur, j, q, frac, T, g);

@@ -102,7 +102,10 @@ struct EngineArgs {
     // deposited grids
     double *n_a, *n_b, *n_ion;
     double *jx, *jy, *txx, *txy, *tyy, *G;
-    float *jx32, *jy32, *txx32, *txy32, *tyy32, *G32;  // refined form (G32: n_* <gamma - 1>)
+    // refined form: the six moments of a cell side by side, one 32-byte sector
+    // (jx, jy, Txx, Txy; Tyy, n_* <gamma - 1>, -, -), for vector reductions
+    float4 *mom32;
+    float2 *psi2;  // refined form: psi as pairs of floats (qs_ff.cuh)
     // level-0 fields (multigrid unknowns) and right-hand sides
     double *psi, *ez, *bz, *bx, *by;
     double *f_psi, *f_ez, *f_bz, *f_bx, *f_by;

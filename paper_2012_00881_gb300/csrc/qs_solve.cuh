@@ -171,6 +171,20 @@ __device__ void block_sum4f(float v[4]) {
     __syncthreads();  // red4 is reused by the next call
 }
 
+__device__ float block_max(float v) {
+    __shared__ float redf[32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int o = 16; o; o >>= 1) v = fmaxf(v, __shfl_down_sync(0xffffffffu, v, o));
+    __syncthreads();
+    if (lane == 0) redf[wid] = v;
+    __syncthreads();
+    float t = 0.f;
+    if (wid == 0) {
+        t = lane < ((int)blockDim.x >> 5) ? redf[lane] : 0.f;
+        for (int o = 16; o; o >>= 1) t = fmaxf(t, __shfl_down_sync(0xffffffffu, t, o));
+    }
+    return t;
+}
 __device__ double block_max(double v) {
     __shared__ double red[32];
     for (int o = 16; o; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
@@ -200,6 +214,7 @@ struct SolveSpec {
     double *f[2];
     bool screened;
     float *u32[2] = {nullptr, nullptr};  // refined form: float32 copy of the solution
+    float2 *pairs = nullptr;  // refined form, one component: the solution as pairs of floats
 };
 
 // The hierarchy descriptors live in shared memory, one copy per block:
@@ -1080,6 +1095,11 @@ __device__ bool direct_poisson(const EngineArgs &A, const Sync &S, const SolveSp
         if constexpr (REF) {
             u0[i] = qsff::join(v.x) * is0;
             u1[i] = qsff::join(v.y) * is1;
+            if (NC == 1 && V.pairs) {  // is0 is a power of two
+                const float k = (float)is0;
+                V.pairs[i] = make_float2(v.x.h * k, v.x.l * k);
+                V.pairs[i + N] = make_float2(v.y.h * k, v.y.l * k);
+            }
         } else {
             u0[i] = v.x;
             u1[i] = v.y;
