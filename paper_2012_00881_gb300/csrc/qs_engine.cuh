@@ -83,8 +83,8 @@ __device__ __forceinline__ void dep(P *g, const CicP<P> &c, P q) {
 
 // Six float32 moments q of a particle into one cell with weight w: two vector
 // reductions of the cell's sector instead of six scalar ones.  The moments
-// phase is bound by the reductions: 262,144 particles send 6.3 M scalar ones
-// (256^2, MOMOLD us), 2.1 M vector ones MOMNEW us.
+// phase is bound by them (512^2, nine particles a cell: 247 us with 57 M scalar
+// ones and float64 arithmetic, 121 us with 19 M vector ones and pairs).
 __device__ __forceinline__ void dep6(float4 *m, int i, float w, const float (&q)[6]) {
     float4 *a = m + 2 * (size_t)i;
     asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(a), "f"(q[0] * w),
@@ -496,7 +496,7 @@ __device__ void phase_assemble1(const EngineArgs &A, const PS<P> &Q, const doubl
     const double *J0 = A.jzb + (size_t)j * nn;
     const double *J1 = (j + 1 < A.n_xi) ? A.jzb + (size_t)(j + 1) * nn : nullptr;
     unsigned hits = 0;
-    double sez = 0.0, sbz = 0.0, sk = 0.0;
+    double sez = 0.0, sbz = 0.0;
     for (int i = T.t0; i < nn; i += T.nt) {
         const int iy = i / n, ix = i - iy * n;
         if (g.active) {
@@ -516,13 +516,12 @@ __device__ void phase_assemble1(const EngineArgs &A, const PS<P> &Q, const doubl
         A.jz[i] = g_total(Q.mom(M_G, i), nv) * ia - nv + jzb;
         const double kap = nv * ia;
         A.kap[i] = kap;
-        sk += kap;
         const int nw = qsmg::walls(ix, iy, n);
         if (A.precision == QS_FP32_REFINED) {
             const float k32 = (float)kap;
             A.k32[i] = k32;
-            if (!A.fft.on) A.d32[i] = 1.f / ((float)(4 + nw) + A.lev_h2f[0] * k32);
-        } else if (!A.fft.on) {
+            A.d32[i] = 1.f / ((float)(4 + nw) + A.lev_h2f[0] * k32);
+        } else {
             A.invd0[i] = 1.0 / ((double)(4 + nw) + A.lev_h2[0] * kap);
         }
         A.dpx[i] = dxo(A.psi, n, ix, i, inv2h);
@@ -547,8 +546,6 @@ __device__ void phase_assemble1(const EngineArgs &A, const PS<P> &Q, const doubl
     if (threadIdx.x == 0) atomicAdd(&A.sc->fnorm[1][0], sez);
     sbz = block_sum(sbz);
     if (threadIdx.x == 0) atomicAdd(&A.sc->fnorm[1][1], sbz);
-    sk = block_sum(sk);
-    if (threadIdx.x == 0) atomicAdd(&A.sc->ksum, sk);
     add_hits(A.sc, hits);
 }
 
@@ -595,6 +592,249 @@ __device__ void phase_assemble2(const EngineArgs &A, const PS<P> &Q, const doubl
     if (threadIdx.x == 0) atomicAdd(&A.sc->fnorm[2][0], sbx);
     sby = block_sum(sby);
     if (threadIdx.x == 0) atomicAdd(&A.sc->fnorm[2][1], sby);
+}
+
+// ---------------------------------------------------------------------------
+// The same phases fused with the transforms of the direct solves: a source is
+// formed where its row transform reads it, and a solution goes on to the next
+// source where its inverse transform ends.  That saves three grid phases and
+// the trips of six grids through L2 a slice, and in the refined form the
+// sources are formed in pairs of floats, with no conversions to float64 (the
+// five separate phases' FP64-pipe instructions took 37 us a 256^2 slice).
+// ---------------------------------------------------------------------------
+using qsff::Ff;
+using qsfft::Ff2;
+
+// source of psi (f = n_* - n_ion); charge sum; cleared accumulators
+template <typename P>
+__device__ void rows_psi(const EngineArgs &A, const PS<P> &Q, const double *ncur, double *nnext,
+                         bool base, int j, int q, double frac, int bid, int nblk) {
+    const int N = A.N, nn = N * N;
+    double cs = 0.0;
+    const double *a0 = A.a2_base ? A.a2_base + (size_t)j * nn : nullptr;
+    const double *a1 = a0 && j + 1 < A.n_xi ? a0 + nn : nullptr;
+    const bool diag = base && A.diag_charge;
+    auto cell = [&](int i) {
+        if (a0) A.a2[i] = q == 0 ? a0[i] : (1.0 - frac) * a0[i] + frac * (a1 ? a1[i] : 0.0);
+        const double nv = ncur[i];
+        if (diag) cs += nv;
+        if constexpr (sizeof(P) == 8) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) Q.m[k][i] = 0.0;
+        } else {
+            A.mom32[2 * (size_t)i] = A.mom32[2 * (size_t)i + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        nnext[i] = 0.0;
+        return qsff::split(nv - A.n_ion[i]);
+    };
+    poisson_rows<1>(A, bid, nblk, [&](int l, int x) {
+        const int i = 2 * l * N + x;
+        const Ff f0 = cell(i), f1 = cell(i + N);
+        return qsfft::mk<Ff>(f0, f1);
+    });
+    if (diag) {
+        cs = block_sum(cs);
+        if (threadIdx.x == 0) atomicAdd(&A.diag_charge[j], cs * A.h * A.h);
+    }
+}
+
+template <typename P>
+__device__ void rows_psi_out(const EngineArgs &A, int bid, int nblk) {
+    const int N = A.N;
+    poisson_inverse<1>(A, bid, nblk, [&](int l, int x, Ff2 v) {
+        const int i = 2 * l * N + x;
+        A.psi[i] = qsff::join(v.x);
+        A.psi[i + N] = qsff::join(v.y);
+        if (sizeof(P) == 4) {
+            A.psi2[i] = make_float2(v.x.h, v.x.l);
+            A.psi2[i + N] = make_float2(v.y.h, v.y.l);
+        }
+    });
+}
+
+// grad(|A|^2 / 4) with even ghosts (the ghost repeats the edge cell)
+__device__ __forceinline__ void ponderomotive(const EngineArgs &A, int ix, int iy, int i,
+                                              double inv2h) {
+    const int n = A.N;
+    const double *a2 = A.a2;
+    const double e = ix < n - 1 ? a2[i + 1] : a2[i];
+    const double w = ix > 0 ? a2[i - 1] : a2[i];
+    const double so = iy < n - 1 ? a2[i + n] : a2[i];
+    const double no = iy > 0 ? a2[i - n] : a2[i];
+    A.pondx[i] = 0.25 * (e - w) * inv2h;
+    A.pondy[i] = 0.25 * (so - no) * inv2h;
+}
+
+// driver current at the cell, linear in xi between base slices
+__device__ __forceinline__ double driver_jz(const double *J0, const double *J1, int i, int q,
+                                            double frac) {
+    return q == 0 ? J0[i] : (1.0 - frac) * J0[i] + frac * (J1 ? J1[i] : 0.0);
+}
+
+// sources of E_z, B_z; j_z, kappa and its sum, grad psi.  The refined form
+// keeps j_z and grad psi as pairs of floats in the float64 grids' memory.
+template <typename P>
+__device__ void rows_eb(const EngineArgs &A, const PS<P> &Q, const double *ncur, int j, int q,
+                        double frac, int bid, int nblk) {
+    const int n = A.N, nn = n * n;
+    const double inv2h = 0.5 * A.inv_h;
+    const double *J0 = A.jzb + (size_t)j * nn;
+    const double *J1 = (j + 1 < A.n_xi) ? J0 + nn : nullptr;
+    unsigned hits = 0;
+    float sums[16] = {0.f};
+    const Ff fl = qsff::split(A.psi_floor), i2h = qsff::split(inv2h);
+    poisson_rows<2>(A, bid, nblk, [&](int iy, int ix) {
+        const int i = iy * n + ix;
+        const double nv = ncur[i];
+        double kap;
+        Ff2 f;
+        if constexpr (sizeof(P) == 8) {
+            f.x = qsff::split(-(dx0(Q.m[M_JX], n, ix, i, inv2h) + dy0(Q.m[M_JY], n, iy, i, inv2h)));
+            f.y = qsff::split(dx0(Q.m[M_JY], n, ix, i, inv2h) - dy0(Q.m[M_JX], n, iy, i, inv2h));
+            const double a = guard(1.0 + A.psi[i], A.psi_floor, hits), ia = 1.0 / a;
+            A.jz[i] = Q.m[M_G][i] * ia - nv + driver_jz(J0, J1, i, q, frac);
+            kap = nv * ia;
+            A.kap[i] = kap;
+            sums[0] += qsff::split(kap).h;
+            A.dpx[i] = dxo(A.psi, n, ix, i, inv2h);
+            A.dpy[i] = dyo(A.psi, n, iy, i, inv2h);
+        } else {
+            auto jj = [&](bool in, int k) {
+                const float2 *m = (const float2 *)(A.mom32 + 2 * (size_t)k);
+                return in ? *m : make_float2(0.f, 0.f);
+            };
+            const float2 e = jj(ix < n - 1, i + 1), w = jj(ix > 0, i - 1),
+                         s = jj(iy < n - 1, i + n), u = jj(iy > 0, i - n);
+            f.x = -((qsff::two_sum(e.x, -w.x) + qsff::two_sum(s.y, -u.y)) * i2h);
+            f.y = (qsff::two_sum(e.y, -w.y) - qsff::two_sum(s.x, -u.x)) * i2h;
+            auto psi = [&](int k) {
+                const float2 v = A.psi2[k];
+                return Ff(v.x, v.y);
+            };
+            const Ff pc = psi(i), nf = qsff::split(nv);
+            const Ff ia = qsff::recip(one_plus_psi(pc, fl, hits));
+            const Ff jz = (nf + Ff(Q.mom(M_G, i), 0.f)) * ia - nf +
+                          qsff::split(driver_jz(J0, J1, i, q, frac));
+            ((float2 *)A.jz)[i] = make_float2(jz.h, jz.l);
+            const Ff kf = nf * ia;
+            kap = qsff::join(kf);
+            A.kap[i] = kap;
+            A.k32[i] = kf.h;
+            sums[0] += kf.h;
+            // central differences of psi with odd ghosts
+            const Ff gx = ((ix < n - 1 ? psi(i + 1) : -pc) - (ix > 0 ? psi(i - 1) : -pc)) * i2h;
+            const Ff gy = ((iy < n - 1 ? psi(i + n) : -pc) - (iy > 0 ? psi(i - n) : -pc)) * i2h;
+            ((float2 *)A.dpx)[i] = make_float2(gx.h, gx.l);
+            ((float2 *)A.dpy)[i] = make_float2(gy.h, gy.l);
+            A.dpx32[i] = gx.h;
+            A.dpy32[i] = gy.h;
+        }
+        if (A.a2_base) {
+            ponderomotive(A, ix, iy, i, inv2h);
+            if (A.chi && q == 0) A.chi[(size_t)j * nn + i] = kap;  // Eq. laser_Enve
+        }
+        return f;
+    });
+    sums[1] = (float)hits;
+    const float t = block_sums16(sums);
+    if (threadIdx.x == 0) atomicAdd(&A.sc->ksum, (double)t);
+    if (threadIdx.x == 1 && t != 0.f) atomicAdd(&A.sc->guard_hits, (unsigned long long)t);
+}
+
+// E_z, B_z from their row coefficients; explicit source S of Eq. FluxCurr1_A
+// from them, the right-hand side -e_z x S = (S_y, -S_x) of Eq. Main_Eq_A with
+// its norms, and its row transform: what cg_screened starts from.
+template <typename P>
+__device__ void rows_eb_bp(const EngineArgs &A, const PS<P> &Q, const double *ncur, int bid,
+                           int nblk) {
+    using T = typename std::conditional<sizeof(P) == 4, float, Ff>::type;
+    using C = qsfft::V2<T>;
+    const int n = A.N;
+    const double inv2h = 0.5 * A.inv_h;
+    float sums[16] = {0.f};
+    const Ff fl = qsff::split(A.psi_floor), i2h = qsff::split(inv2h);
+    C *const cr = (C *)A.fft.cr;
+    qsfft::rows_inverse_forward<Ff, T, 2>(
+        fft_lines<Ff>(A), fft_lines<T>(A), bid, nblk, (const Ff2 *)A.fft.t2, (C *)A.fft.t1,
+        [&](int iy, int ix, Ff2 v) {
+            const int i = iy * n + ix;
+            const double ezd = qsff::join(v.x), bzd = qsff::join(v.y);
+            A.ez[i] = ezd;
+            A.bz[i] = bzd;
+            double fx, fy;  // S_y, -S_x
+            C r;
+            if constexpr (sizeof(P) == 8) {
+                double a = 1.0 + A.psi[i];
+                if (a < A.psi_floor) a = A.psi_floor;
+                const double jx = Q.m[M_JX][i], jy = Q.m[M_JY][i], txx = Q.m[M_TXX][i],
+                             txy = Q.m[M_TXY][i], tyy = Q.m[M_TYY][i], G = Q.m[M_G][i];
+                const double gx = A.dpx[i], gy = A.dpy[i];
+                const double ia = 1.0 / a, Gia2 = G * ia * ia;
+                double sx = dx0(A.jz, n, ix, i, inv2h) - dx0(Q.m[M_TXX], n, ix, i, inv2h) -
+                            dy0(Q.m[M_TXY], n, iy, i, inv2h) + Gia2 * gx -
+                            (jy * bzd + jx * ezd + txx * gx + txy * gy) * ia;
+                double sy = dy0(A.jz, n, iy, i, inv2h) - dx0(Q.m[M_TXY], n, ix, i, inv2h) -
+                            dy0(Q.m[M_TYY], n, iy, i, inv2h) + Gia2 * gy +
+                            (jx * bzd - jy * ezd - txy * gx - tyy * gy) * ia;
+                if (A.a2_base) {  // -n_* grad(|A|^2/4) / (1+psi)^2
+                    const double nia2 = ncur[i] * ia * ia;
+                    sx -= nia2 * A.pondx[i];
+                    sy -= nia2 * A.pondy[i];
+                }
+                fx = sy;
+                fy = -sx;
+                r = qsfft::mk<T>(qsff::split(fx), qsff::split(fy));
+            } else {
+                A.bz32[i] = v.y.h;  // B_z is final here
+                // T_xx, T_xy, T_yy of a neighbour
+                auto tt = [&](bool in, int k) {
+                    const float4 *m = A.mom32 + 2 * (size_t)k;
+                    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (!in) return z;
+                    const float2 d = *(const float2 *)m, b = *((const float2 *)m + 1);
+                    return make_float4(b.x, b.y, ((const float *)m)[4], d.x);
+                };
+                auto pair = [](const void *g, int k) {
+                    const float2 u = ((const float2 *)g)[k];
+                    return Ff(u.x, u.y);
+                };
+                const Ff zero(0.f, 0.f);
+                const float4 te = tt(ix < n - 1, i + 1), tw = tt(ix > 0, i - 1),
+                             ts = tt(iy < n - 1, i + n), tn = tt(iy > 0, i - n);
+                const Ff dx = (ix < n - 1 ? pair(A.jz, i + 1) : zero) -
+                              (ix > 0 ? pair(A.jz, i - 1) : zero) - qsff::two_sum(te.x, -tw.x) -
+                              qsff::two_sum(ts.y, -tn.y);
+                const Ff dy = (iy < n - 1 ? pair(A.jz, i + n) : zero) -
+                              (iy > 0 ? pair(A.jz, i - n) : zero) - qsff::two_sum(te.y, -tw.y) -
+                              qsff::two_sum(ts.z, -tn.z);
+                const float4 m0 = A.mom32[2 * (size_t)i], m1 = A.mom32[2 * (size_t)i + 1];
+                unsigned dummy = 0;
+                const Ff ia = qsff::recip(one_plus_psi(pair(A.psi2, i), fl, dummy));
+                const Ff nf = qsff::split(ncur[i]), gx = pair(A.dpx, i), gy = pair(A.dpy, i);
+                const Ff Gia = (nf + Ff(m1.y, 0.f)) * ia;
+                // the products with 1 / (1 + psi) taken out
+                Ff px = Gia * gx - (v.y * m0.y + v.x * m0.x + gx * m0.z + gy * m0.w);
+                Ff py = Gia * gy + (v.y * m0.x - v.x * m0.y - gx * m0.w - gy * m1.x);
+                if (A.a2_base) {
+                    const Ff nia = nf * ia;
+                    px -= nia * qsff::split(A.pondx[i]);
+                    py -= nia * qsff::split(A.pondy[i]);
+                }
+                const Ff sx = dx * i2h + px * ia, sy = dy * i2h + py * ia;
+                fx = qsff::join(sy);
+                fy = -qsff::join(sx);
+                r = make_float2(sy.h, -sx.h);
+            }
+            A.f_bx[i] = fx;
+            A.f_by[i] = fy;
+            cr[i] = r;
+            const float hx = head(r.x), hy = head(r.y);
+            sums[0] += hx * hx;
+            sums[1] += hy * hy;
+            return r;
+        });
+    const float t = block_sums16(sums);
+    if (threadIdx.x < 2) atomicAdd(&A.sc->fnorm[2][threadIdx.x], (double)t);
 }
 
 // (double)i for 0 <= i < 2^31 without a conversion: 2^52 + i is exact
@@ -974,8 +1214,7 @@ __device__ bool run_step(const EngineArgs &A, int bid, int nblk, const Sync &S, 
     phase_deposit_n<P>(A, Q, ncur, T);
     if (!S(1)) return false;
 
-    SolveSpec Vpsi{1, 0, {A.psi, nullptr}, {A.f_psi, nullptr}, false};
-    if (REF) Vpsi.pairs = A.psi2;
+    const SolveSpec Vpsi{1, 0, {A.psi, nullptr}, {A.f_psi, nullptr}, false};
     const SolveSpec Veb{2, 1, {A.ez, A.bz}, {A.f_ez, A.f_bz}, false};
     const SolveSpec Vbp{2, 2, {A.bx, A.by}, {A.f_bx, A.f_by}, true,
                         {REF ? A.bx32 : nullptr, REF ? A.by32 : nullptr}};
@@ -1025,27 +1264,45 @@ __device__ bool run_step(const EngineArgs &A, int bid, int nblk, const Sync &S, 
                 s_ctl.frac = (double)q / (double)m;
             }
             __syncthreads();
-            Guess g = s_ctl.g;
-            if (A.fft.on) g.active = false;  // the solves start from zero
+            const Guess g = s_ctl.g;
             const double frac = s_ctl.frac;
-            phase_psi_rhs<P>(A, Q, ncur, nnext, base, j, q, frac, T, g);
-            if (!S(2)) return false;
-            if (!mg_solve<REF>(A, S, Vpsi, slot, bid, nblk, smem, s_inv_ready)) return false;
-            if (REF && !A.fft.on) {  // the transforms' last phase writes the pairs itself
-                for (int i = T.t0; i < A.N * A.N; i += T.nt) {
-                    const qsff::Ff v = qsff::split(A.psi[i]);
-                    A.psi2[i] = make_float2(v.h, v.l);
+            if (A.fft.on) {
+                rows_psi<P>(A, Q, ncur, nnext, base, j, q, frac, bid, nblk);
+                SYNC(2);
+                poisson_columns<1>(A, bid, nblk);
+                SYNC(27);
+                rows_psi_out<P>(A, bid, nblk);
+                SYNC(28);
+                phase_moments<P>(A, Q, T, bid, nblk, smem);
+                SYNC(3);
+                rows_eb<P>(A, Q, ncur, j, q, frac, bid, nblk);
+                SYNC(4);
+                poisson_columns<2>(A, bid, nblk);
+                SYNC(29);
+                rows_eb_bp<P>(A, Q, ncur, bid, nblk);
+                SYNC(5);
+                if (!mg_solve<REF>(A, S, Vbp, slot, bid, nblk, smem, s_inv_ready, true))
+                    return false;
+            } else {
+                phase_psi_rhs<P>(A, Q, ncur, nnext, base, j, q, frac, T, g);
+                if (!S(2)) return false;
+                if (!mg_solve<REF>(A, S, Vpsi, slot, bid, nblk, smem, s_inv_ready)) return false;
+                if (REF) {  // psi as pairs, for the gathers
+                    for (int i = T.t0; i < A.N * A.N; i += T.nt) {
+                        const qsff::Ff v = qsff::split(A.psi[i]);
+                        A.psi2[i] = make_float2(v.h, v.l);
+                    }
+                    if (!S(7)) return false;
                 }
-                if (!S(7)) return false;
+                phase_moments<P>(A, Q, T, bid, nblk, smem);
+                if (!S(3)) return false;
+                phase_assemble1<P>(A, Q, ncur, j, q, frac, T, g);
+                if (!S(4)) return false;
+                if (!mg_solve<REF>(A, S, Veb, slot, bid, nblk, smem, s_inv_ready)) return false;
+                phase_assemble2<P>(A, Q, ncur, T, g);
+                if (!S(5)) return false;
+                if (!mg_solve<REF>(A, S, Vbp, slot, bid, nblk, smem, s_inv_ready)) return false;
             }
-            phase_moments<P>(A, Q, T, bid, nblk, smem);
-            if (!S(3)) return false;
-            phase_assemble1<P>(A, Q, ncur, j, q, frac, T, g);
-            if (!S(4)) return false;
-            if (!mg_solve<REF>(A, S, Veb, slot, bid, nblk, smem, s_inv_ready)) return false;
-            phase_assemble2<P>(A, Q, ncur, T, g);
-            if (!S(5)) return false;
-            if (!mg_solve<REF>(A, S, Vbp, slot, bid, nblk, smem, s_inv_ready)) return false;
             phase_push<P>(A, Q, nnext, base, last, j, dxi, pk, sub, T, bid, nblk, smem);
             ++sub;
             if (lead) {

@@ -509,10 +509,12 @@ __device__ __forceinline__ void rows_inverse(const Lines &P, int bid, int nblk, 
 }
 
 // Rows inverse and, of what next(line, x, value) makes of the samples, rows
-// forward again.
-template <typename T, int NC, typename F>
-__device__ __forceinline__ void rows_inverse_forward(const Lines &P, int bid, int nblk,
-                                                     const V2<T> *in, V2<T> *out, F next) {
+// forward again, in another storage type if asked.  Two components only when
+// the types differ.
+template <typename T, typename U, int NC, typename F>
+__device__ __forceinline__ void rows_inverse_forward(const Lines &P, const Lines &PU, int bid,
+                                                     int nblk, const V2<T> *in, V2<U> *out,
+                                                     F next) {
     using V = V2<T>;
     const int N = P.N, nl = NC == 2 ? N : N / 2, b = buf_b<T>(P);
     const int lgG = lines_at_once(nl, nblk, P.gmax), G = 1 << lgG;
@@ -520,18 +522,18 @@ __device__ __forceinline__ void rows_inverse_forward(const Lines &P, int bid, in
     for (int l0 = bid * G; l0 < nl; l0 += nblk * G) {
         const int gl = min(G, nl - l0);
         const int f = rows_inverse_first<T, NC>(P.a, b, P.tab, N, l0, lgG, gl, in);
-        const int o = f == P.a ? b : P.a;
+        const int o = f == P.a ? b : P.a;  // the free buffer: no smaller than U needs
         const V *r = cplx_at<T>(f) + D.g * line_len<T>(N);
-        V *q = cplx_at<T>(o) + D.g * line_len<T>(N);
+        V2<U> *q = cplx_at<U>(o) + D.g * line_len<U>(N);
         for (int x = D.g < gl ? D.j0 : N; x < N; x += D.stride) {
-            const int at = pad<T>(slot_of(x, N));
-            V v = r[at];
+            const int at = slot_of(x, N);
+            V v = r[pad<T>(at)];
             if (x & 1) v = mk<T>(-v.x, -v.y);
-            v = next(l0 + D.g, x, v);
-            if (x & 1) v = mk<T>(-v.x, -v.y);
-            q[at] = v;
+            V2<U> w = next(l0 + D.g, x, v);
+            if (x & 1) w = mk<U>(-w.x, -w.y);
+            q[pad<U>(at)] = w;
         }
-        rows_forward_rest<T, NC>(o, f, P.tab, N, l0, lgG, gl, out);
+        rows_forward_rest<U, NC>(o, f, PU.tab, N, l0, lgG, gl, out);
     }
 }
 

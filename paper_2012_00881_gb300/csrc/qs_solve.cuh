@@ -214,7 +214,6 @@ struct SolveSpec {
     double *f[2];
     bool screened;
     float *u32[2] = {nullptr, nullptr};  // refined form: float32 copy of the solution
-    float2 *pairs = nullptr;  // refined form, one component: the solution as pairs of floats
 };
 
 // The hierarchy descriptors live in shared memory, one copy per block:
@@ -893,23 +892,23 @@ __device__ __noinline__ bool mg_solve_ref_cluster(const EngineArgs &A, const Syn
 // direct solves by sine transforms (qs_fft.cuh)
 // ---------------------------------------------------------------------------
 
-// Copies the transform tables to shared memory, once per launch or instance
-// (the refined form keeps the float64 ones as float pairs).
+// Copies the transform tables to shared memory, once per launch or instance:
+// as pairs of floats for the Poisson solves (and the float64 form's iterations),
+// as float32 for the refined form's iterations.
 template <bool REF>
 __device__ void fft_load_tables(const EngineArgs &A) {
     if (!A.fft.on) return;
+    using qsff::Ff;
     const int N = A.N, H = N / 2 + 1;
-    using D = typename std::conditional<REF, qsff::Ff, double>::type;
-    using D2 = qsfft::V2<D>;
-    D2 *tw = (D2 *)(qsfft::dyn_smem() + A.fft.tab_off);
-    D *lam = (D *)(tw + N + H);
+    qsfft::Ff2 *tw = (qsfft::Ff2 *)(qsfft::dyn_smem() + A.fft.tab_off);
+    Ff *lam = (Ff *)(tw + N + H);
     float2 *tw32 = (float2 *)(lam + N);
     float *lam32 = (float *)(tw32 + N + H);
-    auto conv = [](double2 v) { return qsfft::mk<D>(D(v.x), D(v.y)); };
+    auto conv = [](double2 v) { return qsfft::mk<Ff>(qsff::split(v.x), qsff::split(v.y)); };
     for (int k = threadIdx.x; k < N; k += blockDim.x) {
         tw[k] = conv(A.fft.tw64[k]);
         if (k < H) tw[N + k] = conv(A.fft.dct64[k]);
-        lam[k] = D(A.fft.lam64[k]);
+        lam[k] = qsff::split(A.fft.lam64[k]);
         if (REF) {
             tw32[k] = A.fft.tw32[k];
             if (k < H) tw32[N + k] = A.fft.dct32[k];
@@ -922,8 +921,7 @@ __device__ void fft_load_tables(const EngineArgs &A) {
 template <typename T>
 __device__ __forceinline__ qsfft::Lines fft_lines(const EngineArgs &A) {
     const int n = A.N, h = n / 2 + 1;
-    const int tab = A.fft.tab_off +
-                    (sizeof(T) == 4 ? (n + h) * (int)sizeof(double2) + n * (int)sizeof(double) : 0);
+    const int tab = A.fft.tab_off + (sizeof(T) == 4 ? (n + h) * 16 + n * 8 : 0);
     return qsfft::Lines{n, A.fft.gmax, A.block_smem_offset, tab};
 }
 
@@ -941,17 +939,30 @@ __device__ __forceinline__ double five_point(float c, float w, float e, float n,
     const float pe = __fmaf_rn(k, c, -pc);  // k c = pc + pe exactly
     qstile::two_sum_acc(hi, lo, -pc);
     lo = __fsub_rn(lo, pe);
-    return (double)hi + (double)lo;
+    return qsff::join(qsff::quick(hi, lo));
 }
-__device__ __forceinline__ double five_point(double c, double w, double e, double n, double s,
-                                             double k) {
-    return (w + e) + (n + s) - k * c;
+// pairs: in float64 (the cancellation of the sum would show the pairs' last bits)
+__device__ __forceinline__ double five_point(qsff::Ff c, qsff::Ff w, qsff::Ff e, qsff::Ff n,
+                                             qsff::Ff s, float k) {
+    using qsff::join;
+    return (join(w) + join(e)) + (join(n) + join(s)) - qsff::widen(k) * join(c);
 }
 
-// Sums of 16 values over the block, into out[0 .. 15] (global); clears the slots
-// of the ring two uses ahead.  Each shuffle halves the values a lane holds: 16
-// shuffles instead of 80.
-__device__ void reduce16(DevScalars *sc, float v[16], double *out, int slot, int bid) {
+// float64 to and from the storage type of an iteration
+template <typename T>
+__device__ __forceinline__ T narrow(double v) {
+    const qsff::Ff p = qsff::split(v);
+    if constexpr (sizeof(T) == 4) return p.h;
+    else return p;
+}
+__device__ __forceinline__ double value(float v) { return qsff::widen(v); }
+__device__ __forceinline__ double value(qsff::Ff v) { return qsff::join(v); }
+__device__ __forceinline__ float head(float v) { return v; }
+__device__ __forceinline__ float head(qsff::Ff v) { return v.h; }
+
+// Sums of 16 values over the block: thread t < 16 returns the sum of v[t].  Each
+// shuffle halves the values a lane holds: 16 shuffles instead of 80.
+__device__ float block_sums16(float v[16]) {
     __shared__ float red[32][17];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (int)blockDim.x >> 5;
 #pragma unroll
@@ -968,22 +979,29 @@ __device__ void reduce16(DevScalars *sc, float v[16], double *out, int slot, int
     // lane bits 4..1 select the value: bit 4 its half, and so on
     if ((lane & 1) == 0) red[wid][lane >> 1] = v[0];
     __syncthreads();
-    if (threadIdx.x < 16) {
-        float t = 0.f;
+    float t = 0.f;
+    if (threadIdx.x < 16)
         for (int w = 0; w < nw; ++w) t += red[w][threadIdx.x];
+    __syncthreads();  // red is reused by the next call
+    return t;
+}
+
+// The same into out[0 .. 15] (global); clears the ring's slots two uses ahead.
+__device__ void reduce16(DevScalars *sc, float v[16], double *out, int slot, int bid) {
+    const float t = block_sums16(v);
+    if (threadIdx.x < 16) {
         if (t != 0.f) atomicAdd(out + threadIdx.x, (double)t);
         if (bid == 0) {
             sc->cgd[(slot + 2) & 3][threadIdx.x] = 0.0;
             if (threadIdx.x < 4) sc->rnorm[(slot + 2) & 3][threadIdx.x] = 0.0;
         }
     }
-    __syncthreads();  // red is reused by the next call
 }
 
 // Scalars of an iterative solve, one copy per block (thread 0, or thread c for
 // component c, writes them between block barriers).
 struct IterScalars {
-    double scale[2], inv[2];  // powers of two near 1 / ||f|| and their inverses
+    float scale[2];           // powers of two near 1 / ||f|| (sums are of scaled values)
     double thr[2], r0[2];     // stopping bound, residual a round starts from (squared, scaled)
     double ig[2], ia[2];      // 1 / (r, z) and 1 / alpha of the last iteration
     float rr[2], ss[2];       // ||r||^2 after the last step, ||A p||^2 (scaled)
@@ -1002,9 +1020,9 @@ __device__ void iter_begin(const EngineArgs &A, const SolveSpec &V, IterScalars 
             const double fn = c < V.nc ? vload(&A.sc->fnorm[V.kind][c]) : 0.0;
             const int ex = (int)((__double_as_longlong(fn) >> 52) & 0x7ff);
             const int k = ex == 0 || ex == 0x7ff ? 0 : (ex - 1023) / 2;
-            I.scale[c] = __longlong_as_double((long long)(1023 - k) << 52);
-            I.inv[c] = __longlong_as_double((long long)(1023 + k) << 52);
-            const double s2 = I.scale[c] * I.scale[c];
+            const int kc = min(max(k, -120), 120);
+            I.scale[c] = __int_as_float((127 - kc) << 23);
+            const double s2 = (double)I.scale[c] * (double)I.scale[c];
             I.thr[c] = fmax(A.mg_tol * A.mg_tol * fn, A.mg_atol * A.mg_atol) * s2;
             I.r0[c] = fn * s2;
             if (!(I.r0[c] <= I.thr[c])) any = 1;
@@ -1034,7 +1052,7 @@ __device__ int iter_check(const EngineArgs &A, const SolveSpec &V, IterScalars &
             I.r0[c] = rn;
             if (bid == 0) {
                 const double fn = vload(&sc->fnorm[V.kind][c]);
-                if (fn > 0.0) rel = fmax(rel, sqrt(rn / fn) * I.inv[c]);
+                if (fn > 0.0) rel = fmax(rel, sqrt(rn / fn) / (double)I.scale[c]);
             }
         }
         if (bid == 0 && conv && rel > sc->max_relres) sc->max_relres = rel;
@@ -1056,56 +1074,49 @@ __device__ void zero_solution(const EngineArgs &A, const SolveSpec &V, int bid, 
 }
 
 // lap_h u = f for one field, or two at once as the parts of a complex one, in
-// three grid phases.  Float64 form: in float64, bound by the FP64 pipe (two
-// fields at 256^2: 37 us).  Refined form: in pairs of floats, whose 47 bits
-// leave a residual of 1e-13 (two fields at 256^2: 28 us; 512^2: 57, against 96); the source
-// is scaled by a power of two near 1 / ||f|| to keep the pairs' low parts in
-// range.
-template <bool REF, int NC>
+// three grid phases, in pairs of floats: their 47 bits leave a residual of
+// 1e-13.  (In float64 the phases are bound by the FP64 pipe: two fields at
+// 256^2 37 us, pairs 28; at 512^2 96 and 57.)  load(line, x) gives the source at
+// a line's point (two fields, or rows 2 line and 2 line + 1 of one field) and
+// store(line, x, value) takes the solution.
+template <int NC, typename L>
+__device__ __forceinline__ void poisson_rows(const EngineArgs &A, int bid, int nblk, L load) {
+    qsfft::rows_forward<qsff::Ff, NC>(fft_lines<qsff::Ff>(A), bid, nblk, (qsfft::Ff2 *)A.fft.t1,
+                                      load);
+}
+template <int NC>
+__device__ __noinline__ void poisson_columns(const EngineArgs &A, int bid, int nblk) {
+    const qsfft::Ff2 *const t1 = (const qsfft::Ff2 *)A.fft.t1;
+    const int nl = NC == 2 ? A.N : A.N / 2;
+    qsfft::columns<qsff::Ff, NC>(fft_lines<qsff::Ff>(A), bid, nblk, (qsfft::Ff2 *)A.fft.t2,
+                                 qsff::Ff(0.f, 0.f),
+                                 [&](int y, int l) { return t1[(size_t)y * nl + l]; });
+    if (bid == 0 && threadIdx.x == 0) A.sc->vcycles[NC - 1] += 1;
+}
+template <int NC, typename F>
+__device__ __forceinline__ void poisson_inverse(const EngineArgs &A, int bid, int nblk, F store) {
+    qsfft::rows_inverse<qsff::Ff, NC>(fft_lines<qsff::Ff>(A), bid, nblk,
+                                      (const qsfft::Ff2 *)A.fft.t2, store);
+}
+
+template <int NC>
 __device__ bool direct_poisson(const EngineArgs &A, const Sync &S, const SolveSpec &V, int bid,
                                int nblk) {
-    using T = typename std::conditional<REF, qsff::Ff, double>::type;
-    using C = qsfft::V2<T>;
-    const qsfft::Lines P = fft_lines<T>(A);
-    const int N = A.N, nl = NC == 2 ? N : N / 2;
+    const int N = A.N, ld = NC == 2 ? N : 2 * N;
     const double *const f0 = V.f[0], *const f1 = NC == 2 ? V.f[1] : V.f[0] + N;
     double *const u0 = V.u[0], *const u1 = NC == 2 ? V.u[1] : V.u[0] + N;
-    const int ld = NC == 2 ? N : 2 * N;
-    C *const t1 = (C *)A.fft.t1, *const t2 = (C *)A.fft.t2;
-    __shared__ IterScalars I;
-    double sc0 = 1.0, sc1 = 1.0, is0 = 1.0, is1 = 1.0;
-    if constexpr (REF) {
-        iter_begin(A, V, I);
-        sc0 = I.scale[0];
-        sc1 = I.scale[NC - 1];
-        is0 = I.inv[0];
-        is1 = I.inv[NC - 1];
-    }
-    qsfft::rows_forward<T, NC>(P, bid, nblk, t1, [&](int l, int x) {
+    poisson_rows<NC>(A, bid, nblk, [&](int l, int x) {
         const size_t i = (size_t)l * ld + x;
-        if constexpr (REF) return qsfft::mk<T>(qsff::split(f0[i] * sc0), qsff::split(f1[i] * sc1));
-        else return make_double2(f0[i], f1[i]);
+        return qsfft::mk<qsff::Ff>(qsff::split(f0[i]), qsff::split(f1[i]));
     });
     SYNC(26);
-    qsfft::columns<T, NC>(P, bid, nblk, t2, T(0.0),
-                          [&](int y, int l) { return t1[(size_t)y * nl + l]; });
+    poisson_columns<NC>(A, bid, nblk);
     SYNC(27);
-    qsfft::rows_inverse<T, NC>(P, bid, nblk, t2, [&](int l, int x, C v) {
+    poisson_inverse<NC>(A, bid, nblk, [&](int l, int x, qsfft::Ff2 v) {
         const size_t i = (size_t)l * ld + x;
-        if constexpr (REF) {
-            u0[i] = qsff::join(v.x) * is0;
-            u1[i] = qsff::join(v.y) * is1;
-            if (NC == 1 && V.pairs) {  // is0 is a power of two
-                const float k = (float)is0;
-                V.pairs[i] = make_float2(v.x.h * k, v.x.l * k);
-                V.pairs[i + N] = make_float2(v.y.h * k, v.y.l * k);
-            }
-        } else {
-            u0[i] = v.x;
-            u1[i] = v.y;
-        }
+        u0[i] = qsff::join(v.x);
+        u1[i] = qsff::join(v.y);
     });
-    if (bid == 0 && threadIdx.x == 0) A.sc->vcycles[V.kind] += 1;
     SYNC(28);
     return true;
 }
@@ -1131,15 +1142,18 @@ __device__ bool direct_poisson(const EngineArgs &A, const Sync &S, const SolveSp
 //
 // Refined form: float32 iterations on the residual equation, to 1e-5 of the
 // residual they start from; then u += e, r <- r - A e in float64 and again.
-// Float64 form: in float64 to the tolerance; the same step then checks it.
-// Both stop on the float64 residual.  The residual is scaled by a power of two
-// near 1 / ||f|| so that float32 cannot underflow.
+// Float64 form: in pairs of floats to the tolerance (in float64 the two phases
+// of an iteration took 21 and 20 us at 256^2, bound by the FP64 pipe; pairs:
+// CGFF us); the same step then checks it.  Both stop on the float64 residual.
+// The sums are of values scaled by a power of two near 1 / ||f||, so that
+// float32 cannot underflow in them.
+// prepared: the source's row transform and copy are in tr and cr already.
 // Returns 1 (converged), 0 (not within its cap: u holds the last iterate and
 // the V-cycles take over), -1 (a barrier failed).
 template <bool REF>
 __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &V, int &slot,
-                           int bid, int nblk) {
-    using T = typename std::conditional<REF, float, double>::type;
+                           int bid, int nblk, bool prepared) {
+    using T = typename std::conditional<REF, float, qsff::Ff>::type;
     using C = qsfft::V2<T>;
     DevScalars *sc = A.sc;
     const qsfft::Lines P = fft_lines<T>(A);
@@ -1154,24 +1168,26 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
         zero_solution(A, V, bid, nblk);
         return S(50) ? 1 : -1;
     }
-    const T kbar = (T)I.kbar;
-    const double sc0 = I.scale[0], sc1 = I.scale[1], is0 = I.inv[0], is1 = I.inv[1];
+    const T kbar = narrow<T>(I.kbar);
+    const float sc0 = I.scale[0], sc1 = I.scale[1];
     auto dk = [&](size_t i) {  // kbar - kappa
         if constexpr (REF) return kbar - A.k32[i];
-        else return kbar - A.kap[i];
+        else return kbar - qsff::split(A.kap[i]);
     };
-    qsfft::rows_forward<T, 2>(P, bid, nblk, tr, [&](int y, int x) {
-        const size_t i = (size_t)y * N + x;
-        const C r = qsfft::mk<T>((T)(V.f[0][i] * sc0), (T)(V.f[1][i] * sc1));
-        cr[i] = r;
-        return r;
-    });
-    if (!S(51)) return -1;
+    if (!prepared) {
+        qsfft::rows_forward<T, 2>(P, bid, nblk, tr, [&](int y, int x) {
+            const size_t i = (size_t)y * N + x;
+            const C r = qsfft::mk<T>(narrow<T>(V.f[0][i]), narrow<T>(V.f[1][i]));
+            cr[i] = r;
+            return r;
+        });
+        if (!S(51)) return -1;
+    }
     const int cap = min(A.mg_max_vcycles, 48);
     const double red = REF ? 1e-10 : 1e-26;  // a round's reduction, squared
     int it = 0, result = -2;
     for (int round = 0; result == -2; ++round) {
-        T al0 = T(0), al1 = T(0), be0 = T(0), be1 = T(0);
+        T al0 = T(0.f), al1 = T(0.f), be0 = T(0.f), be1 = T(0.f);
         int inner = 0;
         for (;;) {
             qsfft::columns<T, 2>(P, bid, nblk, t2, kbar, [&](int y, int l) {
@@ -1193,10 +1209,10 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
             });
             if (!S(52)) return -1;
             float d[16] = {0.f};
-            qsfft::rows_inverse_forward<T, 2>(P, bid, nblk, t2, tz, [&](int y, int x, C z) {
+            qsfft::rows_inverse_forward<T, T, 2>(P, P, bid, nblk, t2, tz, [&](int y, int x, C z) {
                 const size_t i = (size_t)y * N + x;
                 const T k = dk(i);
-                C r = cr[i], s = qsfft::mk<T>(T(0), T(0));
+                C r = cr[i], s = qsfft::mk<T>(T(0.f), T(0.f));
                 if (inner > 0) {  // the update of the last iteration
                     const C zo = cz[i];
                     C p = zo, e;
@@ -1222,8 +1238,9 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
                 }
                 cz[i] = z;
                 const C w = qsfft::mk<T>(r.x + k * z.x, r.y + k * z.y);
-                const float rx = (float)r.x, ry = (float)r.y, zx = (float)z.x, zy = (float)z.y,
-                            wx = (float)w.x, wy = (float)w.y, sx = (float)s.x, sy = (float)s.y;
+                const float rx = head(r.x) * sc0, ry = head(r.y) * sc1, zx = head(z.x) * sc0,
+                            zy = head(z.y) * sc1, wx = head(w.x) * sc0, wy = head(w.y) * sc1,
+                            sx = head(s.x) * sc0, sy = head(s.y) * sc1;
                 d[0] += rx * zx;
                 d[1] += ry * zy;
                 d[2] += zx * wx;
@@ -1277,10 +1294,10 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
                     if (!((double)I.rr[c] <= fmax(red * I.r0[c], 0.09 * I.thr[c]))) go = 1;
                 I.go = go;
             }
-            al0 = (T)I.al[0];
-            al1 = (T)I.al[1];
-            be0 = (T)I.be[0];
-            be1 = (T)I.be[1];
+            al0 = narrow<T>(I.al[0]);
+            al1 = narrow<T>(I.al[1]);
+            be0 = narrow<T>(I.be[0]);
+            be1 = narrow<T>(I.be[1]);
             __syncthreads();
             const bool go = I.go != 0;
             __syncthreads();  // rewritten by the next test
@@ -1303,15 +1320,15 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
         const double ih2 = A.lev_inv_h2[0];
         qsfft::rows_forward<T, 2>(P, bid, nblk, tr, [&](int y, int x) {
             const size_t i = (size_t)y * N + x;
-            const C zero = qsfft::mk<T>(T(0), T(0));
+            const C zero = qsfft::mk<T>(T(0.f), T(0.f));
             const C e = e_at(i);
             const C ew = x > 0 ? e_at(i - 1) : zero, ee = x < N - 1 ? e_at(i + 1) : zero;
             const C en = y > 0 ? e_at(i - N) : zero, es = y < N - 1 ? e_at(i + N) : zero;
-            const T cw = (T)(4 + qsmg::walls(x, y, N));
+            const float cw = (float)(4 + qsmg::walls(x, y, N));
             const double kap = A.kap[i];
-            const double a0 = five_point(e.x, ew.x, ee.x, en.x, es.x, cw) * ih2 - kap * (double)e.x;
-            const double a1 = five_point(e.y, ew.y, ee.y, en.y, es.y, cw) * ih2 - kap * (double)e.y;
-            double u0 = (double)e.x * is0, u1 = (double)e.y * is1, q0, q1;
+            double u0 = value(e.x), u1 = value(e.y), q0, q1;
+            const double a0 = five_point(e.x, ew.x, ee.x, en.x, es.x, cw) * ih2 - kap * u0;
+            const double a1 = five_point(e.y, ew.y, ee.y, en.y, es.y, cw) * ih2 - kap * u1;
             if (round == 0) {
                 q0 = V.f[0][i];
                 q1 = V.f[1][i];
@@ -1321,20 +1338,21 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
                 q0 = A.r64[0][i];
                 q1 = A.r64[1][i];
             }
-            const double r0 = q0 - a0 * is0, r1 = q1 - a1 * is1;
+            const double r0 = q0 - a0, r1 = q1 - a1;
             V.u[0][i] = u0;
             V.u[1][i] = u1;
+            const float h0 = narrow<float>(u0), h1 = narrow<float>(u1);
             if (V.u32[0]) {
-                V.u32[0][i] = (float)u0;
-                V.u32[1][i] = (float)u1;
+                V.u32[0][i] = h0;
+                V.u32[1][i] = h1;
             }
             A.r64[0][i] = r0;
             A.r64[1][i] = r1;
-            const C r = qsfft::mk<T>((T)(r0 * sc0), (T)(r1 * sc1));
+            const C r = qsfft::mk<T>(narrow<T>(r0), narrow<T>(r1));
             cr[i] = r;
-            const float v0 = (float)(u0 * sc0), v1 = (float)(u1 * sc1);
-            n[0] += (float)r.x * (float)r.x;
-            n[1] += (float)r.y * (float)r.y;
+            const float v0 = h0 * sc0, v1 = h1 * sc1, n0 = head(r.x) * sc0, n1 = head(r.y) * sc1;
+            n[0] += n0 * n0;
+            n[1] += n1 * n1;
             n[2] += v0 * v0;
             n[3] += v1 * v1;
             return r;
@@ -1369,13 +1387,14 @@ __device__ void screened_diagonal(const EngineArgs &A, Thr T) {
 // V-cycle on the correction, float64 update (iterative refinement).
 template <bool REF>
 __device__ bool mg_solve(const EngineArgs &A, const Sync &S, const SolveSpec &V, int &slot,
-                         int bid, int nblk, void *smem_base, int *inv_ready) {
+                         int bid, int nblk, void *smem_base, int *inv_ready,
+                         bool prepared = false) {
     DevScalars *sc = A.sc;
     if (A.fft.on) {
         if (!V.screened)
-            return V.nc == 1 ? direct_poisson<REF, 1>(A, S, V, bid, nblk)
-                             : direct_poisson<REF, 2>(A, S, V, bid, nblk);
-        const int r = cg_screened<REF>(A, S, V, slot, bid, nblk);
+            return V.nc == 1 ? direct_poisson<1>(A, S, V, bid, nblk)
+                             : direct_poisson<2>(A, S, V, bid, nblk);
+        const int r = cg_screened<REF>(A, S, V, slot, bid, nblk, prepared);
         if (r != 0) return r > 0;
         screened_diagonal(A, grid_thr(bid, nblk));
         SYNC(56);
