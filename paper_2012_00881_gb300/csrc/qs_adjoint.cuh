@@ -519,7 +519,7 @@ __device__ bool run_adjoint(const EngineArgs &A, const AdjArgs &D, int bid, int 
 template <bool REF>
 __global__ void __launch_bounds__(QS_ENGINE_THREADS, 1)
     adjoint_engine(const __grid_constant__ EngineArgs A0, const __grid_constant__ AdjArgs D0) {
-    extern __shared__ double smem[];
+    extern __shared__ __align__(16) double smem[];
     __shared__ unsigned long long s_epoch;
     __shared__ int s_inv_ready[2];
     __shared__ EngineArgs A;

@@ -8,6 +8,7 @@
 #include <cstring>
 #include <vector>
 
+#include "qs_fft.cuh"
 #include "qs_internal.cuh"
 
 struct qs_ctx {
@@ -232,32 +233,10 @@ int create_fft(qs_ctx *c) {
     std::vector<double> lam(n);
     std::vector<float2> tw32(n), dct32(half);
     std::vector<float> lam32(n);
-    const double pi = 3.14159265358979323846;
     for (int k = 0; k < n; ++k) {
-        // angles reduced to [0, pi/4] so that the tables are exact to rounding
-        // and symmetric
-        auto unit = [&](int num, int den) {  // e^{-2 pi i num / den}, 0 <= num < den
-            const int oct = (int)((long long)num * 8 / den);
-            const int a = oct & 1 ? (oct + 1) * den - 8 * num : 8 * num - oct * den;
-            const double t = pi * a / (4.0 * den);
-            const double co = std::cos(t), si = std::sin(t);
-            double2 v{co, si};
-            switch (oct) {
-            case 1: v = {si, co}; break;
-            case 2: v = {-si, co}; break;
-            case 3: v = {-co, si}; break;
-            case 4: v = {-co, -si}; break;
-            case 5: v = {-si, -co}; break;
-            case 6: v = {si, -co}; break;
-            case 7: v = {co, -si}; break;
-            default: break;
-            }
-            return double2{v.x, -v.y};
-        };
-        tw[k] = unit(k, n);
-        if (k < half) dct[k] = unit(k, 4 * n);
-        const double cs = std::cos(0.5 * pi * k / n);  // 2 + 2 cos(t) = 4 cos^2(t/2)
-        lam[k] = -4.0 * cs * cs / (c->h * c->h);
+        tw[k] = qsfft::host_unit(k, n);
+        if (k < half) dct[k] = qsfft::host_unit(k, 4LL * n);
+        lam[k] = qsfft::host_lam(k, n, c->h);
         tw32[k] = make_float2((float)tw[k].x, (float)tw[k].y);
         if (k < half) dct32[k] = make_float2((float)dct[k].x, (float)dct[k].y);
         lam32[k] = (float)lam[k];

@@ -736,7 +736,7 @@ __device__ void rows_eb(const EngineArgs &A, const PS<P> &Q, const double *ncur,
         return f;
     });
     sums[1] = (float)hits;
-    const float t = block_sums16(sums);
+    const float t = qsfft::block_sums16(sums);
     if (threadIdx.x == 0) atomicAdd(&A.sc->ksum, (double)t);
     if (threadIdx.x == 1 && t != 0.f) atomicAdd(&A.sc->guard_hits, (unsigned long long)t);
 }
@@ -833,7 +833,7 @@ __device__ void rows_eb_bp(const EngineArgs &A, const PS<P> &Q, const double *nc
             sums[1] += hy * hy;
             return r;
         });
-    const float t = block_sums16(sums);
+    const float t = qsfft::block_sums16(sums);
     if (threadIdx.x < 2) atomicAdd(&A.sc->fnorm[2][threadIdx.x], (double)t);
 }
 
@@ -1261,7 +1261,7 @@ __device__ bool run_step(const EngineArgs &A, int bid, int nblk, const Sync &S, 
             __syncthreads();
             if (threadIdx.x == 0) {
                 if (!A.fft.on) s_ctl.g = make_guess(A.ws_order, have, xs, gx0, gx1, gx2);
-                s_ctl.frac = (double)q / (double)m;
+                s_ctl.frac = q == 0 ? 0.0 : (double)q / (double)m;
             }
             __syncthreads();
             const Guess g = s_ctl.g;
@@ -1358,7 +1358,7 @@ __device__ bool run_step(const EngineArgs &A, int bid, int nblk, const Sync &S, 
 // per-thread copy in local memory.
 template <bool REF>
 __global__ void __launch_bounds__(QS_ENGINE_THREADS, 1) slice_engine(const __grid_constant__ EngineArgs A0) {
-    extern __shared__ double smem[];
+    extern __shared__ __align__(16) double smem[];
     __shared__ unsigned long long s_epoch;
     __shared__ int s_inv_ready[2];
     __shared__ EngineArgs A;
@@ -1390,7 +1390,7 @@ __global__ void __launch_bounds__(QS_ENGINE_THREADS, 1) slice_engine(const __gri
 template <bool REF>
 __global__ void __launch_bounds__(QS_ENGINE_THREADS, 1)
     slice_engine_batched(const EngineArgs *list, int n_inst, int team, BatchState *bs) {
-    extern __shared__ double smem[];
+    extern __shared__ __align__(16) double smem[];
     __shared__ unsigned long long s_epoch;
     __shared__ int s_inv_ready[2];
     __shared__ EngineArgs sA;

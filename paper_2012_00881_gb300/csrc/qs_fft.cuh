@@ -23,7 +23,9 @@
 
 #include <cuda_runtime.h>
 
+#include <cmath>
 #include <type_traits>
+#include <vector>
 
 #include "qs_ff.cuh"
 
@@ -87,12 +89,40 @@ __device__ __forceinline__ V cmul(V a, V w) {
 // buffers and tables are passed as byte offsets into it, so that all accesses
 // compile to shared-memory instructions across calls.
 __device__ __forceinline__ char *dyn_smem() {
-    extern __shared__ double smem[];
+    extern __shared__ __align__(16) double smem[];
     return (char *)smem;
 }
 template <typename T>
 __device__ __forceinline__ V2<T> *cplx_at(int off) {
     return (V2<T> *)(dyn_smem() + off);
+}
+
+// e^{-2 pi i num / den}, 0 <= num < den, on the host: the angle reduced to
+// [0, pi / 4], so that the tables are exact to rounding and symmetric.
+inline double2 host_unit(long long num, long long den) {
+    const int oct = (int)(num * 8 / den);
+    const long long a = oct & 1 ? (oct + 1) * den - 8 * num : 8 * num - oct * den;
+    const double t = 3.14159265358979323846 * (double)a / (4.0 * (double)den);
+    const double c = std::cos(t), s = std::sin(t);
+    const double re[8] = {c, s, -s, -c, -c, -s, s, c}, im[8] = {s, c, c, s, -s, -c, -c, -s};
+    return double2{re[oct], -im[oct]};
+}
+// eigenvalue of cosine index j: -(2 + 2 cos(pi j / n)) / h^2
+inline double host_lam(int j, int n, double h) {
+    const double c = std::cos(0.5 * 3.14159265358979323846 * j / n);
+    return -4.0 * c * c / (h * h);
+}
+// [tw][dct][lam] of a side, as pairs (two a complex number)
+inline std::vector<Ff> host_tables(int n, double h) {
+    std::vector<Ff> t;
+    auto put = [&](double2 v) {
+        t.push_back(Ff(v.x));
+        t.push_back(Ff(v.y));
+    };
+    for (int k = 0; k < n; ++k) put(host_unit(k, n));
+    for (int k = 0; 2 * k <= n; ++k) put(host_unit(k, 4LL * n));
+    for (int k = 0; k < n; ++k) t.push_back(Ff(host_lam(k, n, h)));
+    return t;
 }
 
 // Line buffers and tables of a block, all in shared memory: a, b hold gmax
@@ -383,10 +413,13 @@ __device__ __forceinline__ double recip(double d) {
 }
 
 // The rest of `columns` after its lines are filled: forward, times
-// 1 / (4 N^2 (lam_x + lam_y - kbar)), inverse, and the store.
-template <typename T, int NC>
+// 1 / (4 N^2 (lam_x + lam_y - kbar)), inverse, and the store.  kbar: a real
+// number, or a complex one (two components as one complex field).
+template <typename T, int NC, typename K>
 __device__ __noinline__ void columns_rest(int a, int b, int tab, int N, int l0, int lgG, int gl,
-                                          V2<T> *out, T kbar) {
+                                          V2<T> *out, K kbar) {
+    constexpr bool cplx = !std::is_same<K, T>::value;
+    static_assert(!cplx || NC == 2, "a complex shift needs a complex field");
     using V = V2<T>;
     const int nl = NC == 2 ? N : N / 2, G = 1 << lgG;
     const Deal D(lgG);
@@ -397,10 +430,17 @@ __device__ __noinline__ void columns_rest(int a, int b, int tab, int N, int l0, 
     const int f = fft<T, false>(a, b, tab, N, lgG, gl);
     for (int j = D.g < gl ? D.j0 : N; 2 * j <= N; j += D.stride) {
         const int l = l0 + D.g;
-        const T lx0 = lam[NC == 2 ? l : 2 * l] - kbar;
-        const T lx1 = NC == 2 ? lx0 : lam[2 * l + 1] - kbar;
+        T kr;
+        if constexpr (cplx) kr = kbar.x;
+        else kr = kbar;
+        const T lx0 = lam[NC == 2 ? l : 2 * l] - kr;
+        const T lx1 = NC == 2 ? lx0 : lam[2 * l + 1] - kr;
         auto scaled = [&](V c, int jj) {
             const T ly = lam[jj];
+            if constexpr (cplx) {  // 1 / (d - i k) = (d + i k) / (d^2 + k^2)
+                const T d = lx0 + ly, g = c4 * recip(d * d + kbar.y * kbar.y);
+                return cmul<false>(c, mk<T>(d * g, kbar.y * g));
+            }
             const T s0 = c4 * recip(lx0 + ly);
             const T s1 = NC == 2 ? s0 : c4 * recip(lx1 + ly);
             return mk<T>(c.x * s0, c.y * s1);
@@ -434,8 +474,8 @@ __device__ __noinline__ void columns_rest(int a, int b, int tab, int N, int l0, 
 // Columns: load(y, line) gives the row coefficients; the solution's row
 // coefficients go to `out`.  The one-component array seen as complex pairs puts
 // columns 2p and 2p + 1 into line p.
-template <typename T, int NC, typename F>
-__device__ __forceinline__ void columns(const Lines &P, int bid, int nblk, V2<T> *out, T kbar,
+template <typename T, int NC, typename K, typename F>
+__device__ __forceinline__ void columns(const Lines &P, int bid, int nblk, V2<T> *out, K kbar,
                                         F load) {
     using V = V2<T>;
     const int N = P.N, nl = NC == 2 ? N : N / 2;
@@ -450,7 +490,7 @@ __device__ __forceinline__ void columns(const Lines &P, int bid, int nblk, V2<T>
             if (y & 1) v = mk<T>(-v.x, -v.y);
             a[g * line_len<T>(N) + pad<T>(slot_of(y, N))] = v;
         }
-        columns_rest<T, NC>(P.a, buf_b<T>(P), P.tab, N, l0, lgG, gl, out, kbar);
+        columns_rest<T, NC, K>(P.a, buf_b<T>(P), P.tab, N, l0, lgG, gl, out, kbar);
     }
 }
 
@@ -535,6 +575,32 @@ __device__ __forceinline__ void rows_inverse_forward(const Lines &P, const Lines
         }
         rows_forward_rest<U, NC>(o, f, PU.tab, N, l0, lgG, gl, out);
     }
+}
+
+// Sums of 16 values over the block: thread t < 16 returns the sum of v[t].  Each
+// shuffle halves the values a lane holds: 16 shuffles instead of 80.
+static __device__ float block_sums16(float v[16]) {
+    __shared__ float red[32][17];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (int)blockDim.x >> 5;
+#pragma unroll
+    for (int o = 16; o >= 2; o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int k = 0; k < o / 2; ++k) {
+            const float give = up ? v[k] : v[k + o / 2];
+            const float keep = up ? v[k + o / 2] : v[k];
+            v[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+    // lane bits 4..1 select the value: bit 4 its half, and so on
+    if ((lane & 1) == 0) red[wid][lane >> 1] = v[0];
+    __syncthreads();
+    float t = 0.f;
+    if (threadIdx.x < 16)
+        for (int w = 0; w < nw; ++w) t += red[w][threadIdx.x];
+    __syncthreads();  // red is reused by the next call
+    return t;
 }
 
 }  // namespace qsfft

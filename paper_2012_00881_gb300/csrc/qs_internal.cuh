@@ -20,7 +20,7 @@ struct DevScalars {
     int err_where;                 // phase id of a timeout; -1: no clusters
     double rnorm[4][4];            // ||r||^2 (comps 0,1) and ||u||^2 (2,3), ring of 4
     double fnorm[3][2];            // ||f||^2 of the psi / (Ez,Bz) / (Bx,By) solves
-    double cgd[4][16];             // conjugate gradients: dot products per component, ring of 4
+    float cgd[4][16];              // conjugate gradients: dot products per component, ring of 4
     double ksum;                   // sum of kappa over the cells of this slice
     unsigned long long vmax_bits[2];  // V_max of a push (bits of a double >= 0)
     unsigned long long guard_hits;

@@ -12,7 +12,18 @@
 // 5-point Laplacian).  The paper solves it with the same multigrid as the
 // wake, warm-started from the previous time step (Sec. 7.1).
 //
-// Solver: complex multigrid V(2,2) on the cell-centred grid, red-black
+// Solver: where the side has an odd factor of at most 7 (and max_cycles is not a
+// tight cap), conjugate gradients for the complex symmetric operator
+// (COCG, van der Vorst and Melissen, IEEE Trans. Magn. 26 (1990) 706) on the
+// change of the slice's envelope, preconditioned with M = lap - chibar + c by
+// sine transforms (qs_fft.cuh, which see for the phases and the recurrences
+// in transformed rows): A z = r + (chibar - chi) z.  |c| is large, so few
+// iterations are needed (256^2 blowout: 5), each two grid phases, against
+// seven V-cycles of nine phases.  The iteration is in pairs of floats; its end
+// forms the float64 residual and, if that is above the bound, starts again
+// on it.  Otherwise, or when that does not converge:
+//
+// complex multigrid V(2,2) on the cell-centred grid, red-black
 // Gauss-Seidel (the 5-point operator decouples the colours), 4-cell average
 // restriction of the residual and of kappa, bilinear prolongation with odd
 // ghosts, rediscretised coarse operators, 20 red-black sweeps on the
@@ -33,7 +44,10 @@
 #include <cmath>
 #include <new>
 
+#include <vector>
+
 #include "qs.h"
+#include "qs_fft.cuh"
 #include "qs_grid_sync.cuh"
 
 namespace {
@@ -47,6 +61,7 @@ constexpr int kLocalN = 8;             // levels this small run in block 0
 constexpr int kNu = 2;                 // pre- and post-sweeps, V(2, 2)
 constexpr int kTileX = 32, kTileY = 16;  // largest staged output tile
 constexpr int kCoarseSweeps = 20;
+constexpr size_t kScalarBytes = 1024;     // room for LzScalars ahead of the grids
 constexpr long long kBarrierLimit = 4000000000LL;  // clock cycles, ~2 s
 
 struct LzScalars {
@@ -59,7 +74,11 @@ struct LzScalars {
     double max_relres;        // largest final relative residual of a slice
     double norm[3];           // rotating residual-norm slots
     double fnorm[3];          // |f|^2 of the slices (rotating by slice count)
+    double start[3][2];       // |r|^2 and sum of chi of a slice's start (likewise)
+    float dots[4][16];        // dot products of the iterations (ring of 4 uses)
 };
+
+static_assert(sizeof(LzScalars) <= kScalarBytes, "scalars");
 
 struct LzLevel {
     int n;
@@ -76,8 +95,14 @@ struct LzArgs {
     double2 c;
     const double *chi;        // caller: [n_xi][n][n]
     double2 *a;               // caller: [n_xi][n][n], A^n in, A^{n+steps} out
-    double2 *ubuf[2];         // level-0 solutions of consecutive slices
-    double2 *old[2];          // A^n of consecutive slices
+    double2 *u;               // level-0 iterate of the V-cycles
+    double2 *dlt;             // A^{n+1} - A^n of the last slice done
+    // direct-solve preconditioner: on, lines per block, byte offset of the
+    // tables in shared memory and their source; complex scratch grids
+    int fft, gmax, tab_off;
+    const qsfft::Ff *tables;
+    qsfft::Ff2 *tr, *t2, *tz, *tp, *cz, *cr, *cp, *cs, *ce;
+    double2 *r64;
     LzScalars *sc;
 };
 
@@ -498,8 +523,267 @@ __device__ bool up(const LzLevel *H, int from, int to, Team tm, const Sync &sync
     return true;
 }
 
+// ---------------------------------------------------------------------------
+// Direct-solve preconditioned iterations
+// ---------------------------------------------------------------------------
+using qsff::Ff;
+using qsfft::Ff2;
+
+__device__ __forceinline__ Ff2 split2(double2 v) {
+    return qsfft::mk<Ff>(qsff::split(v.x), qsff::split(v.y));
+}
+__device__ __forceinline__ double2 join2(Ff2 v) {
+    return make_double2(qsff::join(v.x), qsff::join(v.y));
+}
+// a + b s for a complex float s
+__device__ __forceinline__ Ff2 axpy(Ff2 a, float2 s, Ff2 b) {
+    return qsfft::mk<Ff>(a.x + (b.x * s.x + b.y * -s.y), a.y + (b.y * s.x + b.x * s.y));
+}
+__device__ __forceinline__ float2 fmul(float2 a, float2 b) {
+    return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+}
+// 1 / a, scaled: late in an iteration |a|^2 is below float32's range
+__device__ __forceinline__ float2 finv(float2 a) {
+    const float m = 1.f / fmaxf(fabsf(a.x), fabsf(a.y)), x = a.x * m, y = a.y * m;
+    const float d = m / (x * x + y * y);
+    return make_float2(x * d, -y * d);
+}
+
+// Adds the block's 16 sums to dots[use & 3] and clears the slots two uses ahead.
+__device__ void lz_reduce(LzScalars *sc, float v[16], int use) {
+    const float t = qsfft::block_sums16(v);
+    if (threadIdx.x < 16) {
+        if (t != 0.f) atomicAdd(&sc->dots[use & 3][threadIdx.x], t);
+        if (blockIdx.x == 0) sc->dots[(use + 2) & 3][threadIdx.x] = 0.f;
+    }
+}
+
+// The change of slice j's envelope into A.dlt.  On entry A.dlt is the previous
+// slice's change (added to the caller's array here).  Returns 1 (converged),
+// 0 (not: A.u = A^n + the change so far, for the V-cycles), -1 (a barrier
+// failed).  its: iterations; relres: the final relative residual (thread 0).
+__device__ int slice_direct(const LzArgs &A, const qsync::GridBarrier<LzScalars> &gsync, int j,
+                            long long g, long long &kglob, int &use, int &its, double &relres) {
+    LzScalars *sc = A.sc;
+    const int n = A.n, nn = n * n;
+    const qsfft::Lines P{n, A.gmax, 0, A.tab_off};
+    const LzLevel &L0 = A.lv[0];
+    const double2 *aj = A.a + (size_t)j * nn;
+    const double *chij = A.chi + (size_t)j * nn;
+    __shared__ float2 s_al, s_be, s_ig, s_ia;
+    __shared__ float s_ss;
+    __shared__ double s_r0, s_thr;
+    __shared__ int s_go;
+    its = 0;
+    // source f (its norm sets the bound) and the residual of A^n, in which the
+    // large c A^n cancels: r = 2 chi A^n - 2 lap A^n - q (change of slice j - 1)
+    double st[3] = {0.0, 0.0, 0.0};
+    qsfft::rows_forward<Ff, 2>(P, blockIdx.x, gridDim.x, A.tr, [&](int y, int x) {
+        const int p = y * n + x;
+        const double2 ao = aj[p], lap = lap_at(aj, n, L0.ih2, x, y);
+        const double chi = chij[p];
+        double2 h = csub(cscale(chi, ao), lap);
+        double2 f = cadd(cmul(A.c, ao), h);
+        double2 r = cadd(h, h);
+        if (j > 0) {
+            const double2 d = A.dlt[p], gq = cscale(A.q, d);
+            f = csub(f, gq);
+            r = csub(r, gq);
+            double2 *prev = A.a + (size_t)(j - 1) * nn + p;
+            *prev = cadd(*prev, d);
+        }
+        L0.f[p] = f;
+        A.r64[p] = r;
+        st[0] += cabs2(f);
+        st[1] += cabs2(r);
+        st[2] += chi;
+        const Ff2 rf = split2(r);
+        A.cr[p] = rf;
+        return rf;
+    });
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        sc->fnorm[(g + 1) % 3] = 0.0;
+        sc->start[(g + 1) % 3][0] = sc->start[(g + 1) % 3][1] = 0.0;
+    }
+    qsync::block_sum_add<kThreads>(st, 1, &sc->fnorm[g % 3]);
+    qsync::block_sum_add<kThreads>(st + 1, 2, sc->start[g % 3]);
+    if (!gsync(1)) return -1;
+    if (threadIdx.x == 0) {
+        const double f2 = qsync::vload(&sc->fnorm[g % 3]);
+        s_r0 = qsync::vload(&sc->start[g % 3][0]);
+        s_thr = A.tol * A.tol * f2;
+        s_go = s_r0 <= s_thr;
+        relres = f2 > 0.0 ? sqrt(s_r0 / f2) : 0.0;
+    }
+    __syncthreads();
+    const bool done = s_go != 0;
+    const double chibar = qsync::vload(&sc->start[g % 3][1]) / (double)nn;
+    const Ff cb = qsff::split(chibar);
+    // M = lap - chibar + c = lap - (chibar - c)
+    const Ff2 shift = qsfft::mk<Ff>(qsff::split(chibar - A.c.x), qsff::split(-A.c.y));
+    auto dk = [&](int p) { return cb - qsff::split(chij[p]); };
+    // power of two near 1 / |r|: the sums are of scaled values
+    const int ex = (int)((__double_as_longlong(s_r0) >> 52) & 0x7ff);
+    const int k2 = ex == 0 || ex == 0x7ff ? 0 : min(max((ex - 1023) / 2, -120), 120);
+    const float scale = __int_as_float((127 - k2) << 23);
+    const double scale2 = (double)scale * (double)scale;
+    if (done) {
+        const qsync::Team grid = qsync::spread_team();
+        for (int p = grid.t; p < nn; p += grid.nt) A.dlt[p] = make_double2(0.0, 0.0);
+        return gsync(2) ? 1 : -1;
+    }
+    const int cap = min(4 * A.max_cycles, 48);
+    for (int round = 0;; ++round) {
+        float2 al = make_float2(0.f, 0.f), be = al;
+        int inner = 0;
+        for (;;) {
+            qsfft::columns<Ff, 2>(P, blockIdx.x, gridDim.x, A.t2, shift, [&](int y, int l) {
+                const int p = y * n + l;
+                Ff2 r = A.tr[p];
+                if (inner > 0) {
+                    Ff2 s = A.tz[p];
+                    if (inner > 1) s = axpy(s, be, A.tp[p]);
+                    A.tp[p] = s;
+                    r = axpy(r, make_float2(-al.x, -al.y), s);
+                    A.tr[p] = r;
+                }
+                return r;
+            });
+            if (!gsync(7)) return -1;
+            float d[16] = {0.f};
+            qsfft::rows_inverse_forward<Ff, Ff, 2>(
+                P, P, blockIdx.x, gridDim.x, A.t2, A.tz, [&](int y, int x, Ff2 z) {
+                    const int p = y * n + x;
+                    const Ff k = dk(p);
+                    Ff2 r = A.cr[p], s = qsfft::mk<Ff>(Ff(0.f, 0.f), Ff(0.f, 0.f));
+                    if (inner > 0) {  // the update of the last iteration
+                        const Ff2 zo = A.cz[p];
+                        Ff2 q = zo, e = s;
+                        s = qsfft::mk<Ff>(r.x + k * zo.x, r.y + k * zo.y);
+                        if (inner > 1) {
+                            q = axpy(q, be, A.cp[p]);
+                            s = axpy(s, be, A.cs[p]);
+                            e = A.ce[p];
+                        }
+                        e = axpy(e, al, q);
+                        r = axpy(r, make_float2(-al.x, -al.y), s);
+                        A.cp[p] = q;
+                        A.cs[p] = s;
+                        A.ce[p] = e;
+                        A.cr[p] = r;
+                    }
+                    A.cz[p] = z;
+                    const Ff2 w = qsfft::mk<Ff>(r.x + k * z.x, r.y + k * z.y);
+                    const float rx = r.x.h * scale, ry = r.y.h * scale, zx = z.x.h * scale,
+                                zy = z.y.h * scale, wx = w.x.h * scale, wy = w.y.h * scale,
+                                sx = s.x.h * scale, sy = s.y.h * scale;
+                    d[0] += rx * zx - ry * zy;  // r z
+                    d[1] += rx * zy + ry * zx;
+                    d[2] += zx * wx - zy * wy;  // z A z
+                    d[3] += zx * wy + zy * wx;
+                    d[4] += wx * rx + wy * ry;  // A z conj(r)
+                    d[5] += wy * rx - wx * ry;
+                    d[6] += sx * rx + sy * ry;  // A p conj(r), the last p
+                    d[7] += sy * rx - sx * ry;
+                    d[8] += sx * wx + sy * wy;  // A p conj(A z)
+                    d[9] += sy * wx - sx * wy;
+                    d[10] += wx * wx + wy * wy;
+                    d[11] += rx * rx + ry * ry;
+                    return w;
+                });
+            lz_reduce(sc, d, use);
+            if (!gsync(8)) return -1;
+            if (threadIdx.x == 0) {
+                const volatile float *v = sc->dots[use & 3];
+                const float2 ga = make_float2(v[0], v[1]), de = make_float2(v[2], v[3]);
+                const float2 zero = make_float2(0.f, 0.f);
+                float2 b = zero, a = zero, ia = zero, ig = zero;
+                if (ga.x != 0.f || ga.y != 0.f) {
+                    ig = finv(ga);
+                    if (inner > 0) b = fmul(ga, s_ig);
+                    ia = fmul(de, ig);
+                    if (inner > 0) {
+                        const float2 t = fmul(b, s_ia);
+                        ia = make_float2(ia.x - t.x, ia.y - t.y);
+                    }
+                    if (ia.x != 0.f || ia.y != 0.f) a = finv(ia);
+                }
+                s_ig = ig;
+                s_ia = ia;
+                s_al = a;
+                s_be = b;
+                // |r - a s|^2 with s = w + b s_old; the sums are good to about
+                // 1e-7 of |r|^2: no smaller value is believed
+                const float so = inner > 0 ? s_ss : 0.f;
+                const float2 ws = fmul(b, make_float2(v[8], v[9]));
+                const float2 rs = fmul(b, make_float2(v[6], v[7]));
+                const float ss = v[10] + 2.f * ws.x + (b.x * b.x + b.y * b.y) * so;
+                const float2 ars = fmul(a, make_float2(v[4] + rs.x, v[5] + rs.y));
+                const float rr = v[11];
+                float nr = rr - 2.f * ars.x + (a.x * a.x + a.y * a.y) * ss;
+                nr = nr < 2e-7f * rr ? 2e-7f * rr : nr;
+                s_ss = ss;
+                s_go = !((double)nr <= fmax(1e-24 * s_r0, 0.09 * s_thr) * scale2);
+            }
+            ++use;
+            __syncthreads();
+            al = s_al;
+            be = s_be;
+            const bool go = s_go != 0;
+            __syncthreads();  // rewritten by the next test
+            ++its;
+            ++inner;
+            if (!go || its >= cap || inner >= 24) break;
+        }
+        // change += e, r <- r - A e in float64, with its norm
+        auto e_at = [&](int p) {
+            Ff2 q = A.cz[p], e = qsfft::mk<Ff>(Ff(0.f, 0.f), Ff(0.f, 0.f));
+            if (inner > 1) {
+                q = axpy(q, be, A.cp[p]);
+                e = A.ce[p];
+            }
+            return join2(axpy(e, al, q));
+        };
+        double rn = 0.0;
+        if (blockIdx.x == 0 && threadIdx.x == 0) sc->norm[(kglob + 1) % 3] = 0.0;
+        qsfft::rows_forward<Ff, 2>(P, blockIdx.x, gridDim.x, A.tr, [&](int y, int x) {
+            const int p = y * n + x;
+            const double2 e = e_at(p), zero = make_double2(0.0, 0.0);
+            const double2 s = cadd(cadd(x > 0 ? e_at(p - 1) : zero, x < n - 1 ? e_at(p + 1) : zero),
+                                   cadd(y > 0 ? e_at(p - n) : zero, y < n - 1 ? e_at(p + n) : zero));
+            const int w = 4 + (x == 0) + (x == n - 1) + (y == 0) + (y == n - 1);
+            const double2 lap = cscale(L0.ih2, csub(s, cscale((double)w, e)));
+            const double2 le = cadd(lap, cmul(make_double2(A.c.x - chij[p], A.c.y), e));
+            const double2 r = csub(A.r64[p], le);
+            A.r64[p] = r;
+            const double2 dn = round > 0 ? cadd(A.dlt[p], e) : e;
+            A.dlt[p] = dn;
+            A.u[p] = cadd(aj[p], dn);
+            rn += cabs2(r);
+            const Ff2 rf = split2(r);
+            A.cr[p] = rf;
+            return rf;
+        });
+        qsync::block_sum_add<kThreads>(&rn, 1, &sc->norm[kglob % 3]);
+        if (!gsync(9)) return -1;
+        if (threadIdx.x == 0) {
+            const double r2 = qsync::vload(&sc->norm[kglob % 3]);
+            const double f2 = qsync::vload(&sc->fnorm[g % 3]);
+            const bool slow = !(r2 <= 0.0625 * s_r0);
+            s_go = r2 <= s_thr ? 1 : (slow || its >= cap) ? 0 : 2;
+            s_r0 = r2;
+            relres = f2 > 0.0 ? sqrt(r2 / f2) : 0.0;
+        }
+        ++kglob;
+        __syncthreads();
+        const int r = s_go;
+        __syncthreads();
+        if (r != 2) return r;
+    }
+}
+
 __global__ void __launch_bounds__(kThreads, 1) laser_kernel(const __grid_constant__ LzArgs P) {
-    extern __shared__ double2 lz_dyn[];  // the staged regions
+    double2 *const lz_dyn = (double2 *)qsfft::dyn_smem();  // the staged regions
     __shared__ LzArgs A;
     __shared__ unsigned long long epoch;
     if (threadIdx.x == 0) {
@@ -528,37 +812,63 @@ __global__ void __launch_bounds__(kThreads, 1) laser_kernel(const __grid_constan
     long long kglob = 0;  // residual-norm computations so far (slot kglob % 3)
     long long g = 0;      // slices so far
 
+    if (A.fft) {
+        const int words = 6 * n + 4 * (n / 2 + 1);  // floats of [tw][dct][lam], as pairs
+        float *const t = (float *)((char *)lz_dyn + A.tab_off);
+        for (int k = threadIdx.x; k < words; k += blockDim.x) t[k] = ((const float *)A.tables)[k];
+        if (threadIdx.x == 0) A.lv[0].u = A.u;
+        __syncthreads();
+    }
+    int use = 0;  // uses of the dot products' ring
     for (int step = 0; step < A.steps; ++step) {
         for (int j = 0; j < A.n_xi; ++j, ++g) {
-            double2 *U = A.ubuf[j & 1], *O = A.old[j & 1];
-            const double2 *Up = A.ubuf[(j + 1) & 1], *Op = A.old[(j + 1) & 1];
+            double2 *U = A.u;
             if (threadIdx.x == 0) A.lv[0].u = U;
             __syncthreads();
             const LzLevel &L0 = A.lv[0];
-            // right-hand side, warm start, kappa and 1/diag of level 0; the
-            // previous slice's new envelope goes back to the caller's array
-            double fn = 0.0;
             const double2 *aj = A.a + (size_t)j * nn;
             const double *chij = A.chi + (size_t)j * nn;
-            // slot (g + 1) % 3 was last read two slices ago, before a barrier
-            if (blockIdx.x == 0 && threadIdx.x == 0) sc->fnorm[(g + 1) % 3] = 0.0;
-            for (int p = grid.t; p < nn; p += grid.nt) {
-                const int jj = p / n, i = p - jj * n;
-                const double2 ao = aj[p];
-                const double chi = chij[p];
-                double2 f = csub(cmul(make_double2(A.c.x + chi, A.c.y), ao),
-                                 lap_at(aj, n, L0.ih2, i, jj));
-                if (j > 0) {
-                    f = csub(f, cscale(A.q, csub(Up[p], Op[p])));
-                    A.a[(size_t)(j - 1) * nn + p] = Up[p];
+            const bool direct = A.fft != 0;
+            if (direct) {
+                int its = 0;
+                double rel = 0.0;
+                const int r = slice_direct(A, gsync, j, g, kglob, use, its, rel);
+                if (r < 0) return;
+                if (r > 0) {
+                    if (blockIdx.x == 0 && threadIdx.x == 0) {
+                        sc->cycles += (its + 3) / 4;  // the work of a V-cycle, at least
+                        if (rel > sc->max_relres) sc->max_relres = rel;
+                    }
+                    continue;
                 }
-                L0.f[p] = f;
-                U[p] = ao;
-                O[p] = ao;
-                L0.kap[p] = make_double2(chi - A.c.x, -A.c.y);
-                fn += cabs2(f);
+                // the V-cycles go on from its iterate
+                for (int p = grid.t; p < nn; p += grid.nt)
+                    L0.kap[p] = make_double2(chij[p] - A.c.x, -A.c.y);
+            } else {
+                // right-hand side, warm start, kappa and 1/diag of level 0; the
+                // previous slice's new envelope goes to the caller's array
+                double fn = 0.0;
+                // slot (g + 1) % 3 was last read two slices ago, before a barrier
+                if (blockIdx.x == 0 && threadIdx.x == 0) sc->fnorm[(g + 1) % 3] = 0.0;
+                for (int p = grid.t; p < nn; p += grid.nt) {
+                    const int jj = p / n, i = p - jj * n;
+                    const double2 ao = aj[p];
+                    const double chi = chij[p];
+                    double2 f = csub(cmul(make_double2(A.c.x + chi, A.c.y), ao),
+                                     lap_at(aj, n, L0.ih2, i, jj));
+                    if (j > 0) {
+                        const double2 d = A.dlt[p];
+                        f = csub(f, cscale(A.q, d));
+                        double2 *prev = A.a + (size_t)(j - 1) * nn + p;
+                        *prev = cadd(*prev, d);
+                    }
+                    L0.f[p] = f;
+                    U[p] = ao;
+                    L0.kap[p] = make_double2(chi - A.c.x, -A.c.y);
+                    fn += cabs2(f);
+                }
+                qsync::block_sum_add<kThreads>(&fn, 1, &sc->fnorm[g % 3]);
             }
-            qsync::block_sum_add<kThreads>(&fn, 1, &sc->fnorm[g % 3]);
             set_idiag(L0, grid);
             if (!gsync(1)) return;
             for (int l = 1; l <= Lc; ++l) {
@@ -675,10 +985,12 @@ __global__ void __launch_bounds__(kThreads, 1) laser_kernel(const __grid_constan
                 qsync::block_sum_add<kThreads>(&rn, 1, &sc->norm[kglob % 3]);
                 if (!gsync(4)) return;
             }
+            for (int p = grid.t; p < nn; p += grid.nt) A.dlt[p] = csub(U[p], aj[p]);
+            if (!gsync(5)) return;
         }
         // the last slice's new envelope
-        const double2 *Ul = A.ubuf[(A.n_xi - 1) & 1];
-        for (int p = grid.t; p < nn; p += grid.nt) A.a[(size_t)(A.n_xi - 1) * nn + p] = Ul[p];
+        double2 *const last = A.a + (size_t)(A.n_xi - 1) * nn;
+        for (int p = grid.t; p < nn; p += grid.nt) last[p] = cadd(last[p], A.dlt[p]);
         if (!gsync(6)) return;
     }
 }
@@ -696,6 +1008,7 @@ struct qs_laser {
     double width = 0.0, dxi = 0.0;
     cudaStream_t stream = nullptr;
     int grid_blocks = 0;
+    size_t smem = 0;
     LzArgs args{};
     void *dev = nullptr;
     void *pinned = nullptr;
@@ -730,9 +1043,15 @@ extern "C" int qs_laser_create(int n, double width, int n_xi, double k0, double 
         m /= 2;
     }
     A.levels = levels;
-    size_t elems = 4 * (size_t)n * n;  // ubuf[2], old[2]
+    int odd = n;
+    while (odd % 2 == 0) odd /= 2;
+    const size_t line = (size_t)(n + n / 8 + 1) * sizeof(qsfft::Ff2);  // padded
+    const bool fft = n % 2 == 0 && n >= 8 && n <= 2048 && odd <= 7;
+    size_t elems = 2 * (size_t)n * n;  // u, dlt
+    const size_t tab_pairs = 3 * (size_t)n + 2 * (size_t)(n / 2 + 1);
+    if (fft) elems += 10 * (size_t)n * n + (tab_pairs + 1) / 2;
     for (int l = 0; l < levels; ++l) elems += 5 * (size_t)sides[l] * sides[l];
-    const size_t bytes = 256 + elems * sizeof(double2);
+    const size_t bytes = kScalarBytes + elems * sizeof(double2);
     int st = cuda_status(cudaMalloc(&s->dev, bytes));
     if (st == QS_OK) st = cuda_status(cudaMallocHost(&s->pinned, sizeof(LzScalars)));
     if (st != QS_OK) {
@@ -741,12 +1060,33 @@ extern "C" int qs_laser_create(int n, double width, int n_xi, double k0, double 
     }
     char *base = static_cast<char *>(s->dev);
     A.sc = reinterpret_cast<LzScalars *>(base);
-    double2 *p = reinterpret_cast<double2 *>(base + 256);
-    for (int k = 0; k < 2; ++k) {
-        A.ubuf[k] = p;
+    double2 *p = reinterpret_cast<double2 *>(base + kScalarBytes);
+    A.u = p;
+    p += (size_t)n * n;
+    A.dlt = p;
+    p += (size_t)n * n;
+    s->smem = lz_smem_bytes() + kCoarseBytes;
+    if (fft) {
+        A.r64 = p;
         p += (size_t)n * n;
-        A.old[k] = p;
-        p += (size_t)n * n;
+        for (qsfft::Ff2 **q : {&A.tr, &A.t2, &A.tz, &A.tp, &A.cz, &A.cr, &A.cp, &A.cs, &A.ce}) {
+            *q = reinterpret_cast<qsfft::Ff2 *>(p);
+            p += (size_t)n * n;
+        }
+        A.tables = reinterpret_cast<const qsfft::Ff *>(p);
+        std::vector<qsfft::Ff> tab = qsfft::host_tables(n, width / n);
+        st = cuda_status(cudaMemcpy(p, tab.data(), tab.size() * sizeof(qsfft::Ff),
+                                    cudaMemcpyHostToDevice));
+        p += (tab_pairs + 1) / 2;
+        A.gmax = 1;
+        while (A.gmax < 8 && 4 * A.gmax * line <= 76 * 1024) A.gmax *= 2;
+        // the lines lie over the staged regions, the tables after everything
+        if (2 * A.gmax * line > s->smem) s->smem = 2 * A.gmax * line;
+        s->smem = (s->smem + 255) & ~(size_t)255;
+        A.tab_off = (int)s->smem;
+        s->smem += tab_pairs * sizeof(qsfft::Ff);
+        A.fft = s->smem <= 220 * 1024;
+        if (!A.fft) s->smem = lz_smem_bytes() + kCoarseBytes;
     }
     for (int l = 0; l < levels; ++l) {
         LzLevel &L = A.lv[l];
@@ -754,7 +1094,7 @@ extern "C" int qs_laser_create(int n, double width, int n_xi, double k0, double 
         const double h = width / sides[l];
         L.n = sides[l];
         L.ih2 = 1.0 / (h * h);
-        L.u = p;  // level 0's u is replaced by a ping-pong buffer per slice
+        L.u = p;  // level 0's u is replaced by A.u
         p += m;
         L.f = p;
         p += m;
@@ -771,10 +1111,10 @@ extern "C" int qs_laser_create(int n, double width, int n_xi, double k0, double 
     if (st == QS_OK)
         st = cuda_status(cudaFuncSetAttribute((const void *)laser_kernel,
                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)(lz_smem_bytes() + kCoarseBytes)));
+                                              (int)s->smem));
     if (st == QS_OK)
         st = cuda_status(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, laser_kernel, kThreads,
-                                                                       lz_smem_bytes() + kCoarseBytes));
+                                                                       s->smem));
     if (st == QS_OK && per_sm < 1) st = QS_ERR_CUDA;
     if (st != QS_OK) {
         qs_laser_destroy(s);
@@ -799,12 +1139,19 @@ extern "C" int qs_laser_advance(qs_laser *s, const double *d_chi, double *d_a, i
     A.steps = steps;
     A.tol = tol;
     A.max_cycles = max_cycles;
+    // a cap of a few V-cycles keeps its meaning: V-cycles
+    if (max_cycles < 4) A.fft = 0;
     int st = cuda_status(cudaMemsetAsync(A.sc, 0, sizeof(LzScalars), s->stream));
     if (st != QS_OK) return st;
     void *params[] = {&A};
+    // the limit belongs to the kernel, which every envelope object shares
+    if (st == QS_OK)
+        st = cuda_status(cudaFuncSetAttribute((const void *)laser_kernel,
+                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)s->smem));
+    if (st != QS_OK) return st;
     st = cuda_status(cudaLaunchCooperativeKernel((const void *)laser_kernel, dim3(s->grid_blocks),
-                                                 dim3(kThreads), params,
-                                                 lz_smem_bytes() + kCoarseBytes, s->stream));
+                                                 dim3(kThreads), params, s->smem, s->stream));
     if (st != QS_OK) return st;
     st = cuda_status(cudaMemcpyAsync(s->pinned, A.sc, sizeof(LzScalars), cudaMemcpyDeviceToHost,
                                      s->stream));

@@ -21,6 +21,7 @@ namespace {
     } while (0)
 
 __device__ __forceinline__ int vload(const int *p) { return *(const volatile int *)p; }
+__device__ __forceinline__ float vload(const float *p) { return *(const volatile float *)p; }
 __device__ __forceinline__ double vload(const double *p) { return *(const volatile double *)p; }
 __device__ __forceinline__ unsigned long long vload(const unsigned long long *p) {
     return *(const volatile unsigned long long *)p;
@@ -960,39 +961,14 @@ __device__ __forceinline__ double value(qsff::Ff v) { return qsff::join(v); }
 __device__ __forceinline__ float head(float v) { return v; }
 __device__ __forceinline__ float head(qsff::Ff v) { return v.h; }
 
-// Sums of 16 values over the block: thread t < 16 returns the sum of v[t].  Each
-// shuffle halves the values a lane holds: 16 shuffles instead of 80.
-__device__ float block_sums16(float v[16]) {
-    __shared__ float red[32][17];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (int)blockDim.x >> 5;
-#pragma unroll
-    for (int o = 16; o >= 2; o >>= 1) {
-        const bool up = (lane & o) != 0;
-#pragma unroll
-        for (int k = 0; k < o / 2; ++k) {
-            const float give = up ? v[k] : v[k + o / 2];
-            const float keep = up ? v[k + o / 2] : v[k];
-            v[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
-        }
-    }
-    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
-    // lane bits 4..1 select the value: bit 4 its half, and so on
-    if ((lane & 1) == 0) red[wid][lane >> 1] = v[0];
-    __syncthreads();
-    float t = 0.f;
-    if (threadIdx.x < 16)
-        for (int w = 0; w < nw; ++w) t += red[w][threadIdx.x];
-    __syncthreads();  // red is reused by the next call
-    return t;
-}
-
-// The same into out[0 .. 15] (global); clears the ring's slots two uses ahead.
-__device__ void reduce16(DevScalars *sc, float v[16], double *out, int slot, int bid) {
-    const float t = block_sums16(v);
+// Sums of 16 values over the block into out[0 .. 15] (global); clears the ring's slots two uses ahead.
+template <typename O>
+__device__ void reduce16(DevScalars *sc, float v[16], O *out, int slot, int bid) {
+    const float t = qsfft::block_sums16(v);
     if (threadIdx.x < 16) {
-        if (t != 0.f) atomicAdd(out + threadIdx.x, (double)t);
+        if (t != 0.f) atomicAdd(out + threadIdx.x, (O)t);
         if (bid == 0) {
-            sc->cgd[(slot + 2) & 3][threadIdx.x] = 0.0;
+            sc->cgd[(slot + 2) & 3][threadIdx.x] = 0.f;
             if (threadIdx.x < 4) sc->rnorm[(slot + 2) & 3][threadIdx.x] = 0.0;
         }
     }
@@ -1003,9 +979,10 @@ __device__ void reduce16(DevScalars *sc, float v[16], double *out, int slot, int
 struct IterScalars {
     float scale[2];           // powers of two near 1 / ||f|| (sums are of scaled values)
     double thr[2], r0[2];     // stopping bound, residual a round starts from (squared, scaled)
-    double ig[2], ia[2];      // 1 / (r, z) and 1 / alpha of the last iteration
-    float rr[2], ss[2];       // ||r||^2 after the last step, ||A p||^2 (scaled)
-    double al[2], be[2];
+    // of the last iteration: 1 / (r, z), 1 / alpha, step sizes; ||r||^2 after it,
+    // ||A p||^2 (scaled).  float32: a step size only has to be the same for all
+    // vectors, and a float64 division takes thread 0 a third of a microsecond.
+    float ig[2], ia[2], al[2], be[2], rr[2], ss[2];
     double kbar;
     int go;
 };
@@ -1187,7 +1164,7 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
     const double red = REF ? 1e-10 : 1e-26;  // a round's reduction, squared
     int it = 0, result = -2;
     for (int round = 0; result == -2; ++round) {
-        T al0 = T(0.f), al1 = T(0.f), be0 = T(0.f), be1 = T(0.f);
+        float al0 = 0.f, al1 = 0.f, be0 = 0.f, be1 = 0.f;
         int inner = 0;
         for (;;) {
             qsfft::columns<T, 2>(P, bid, nblk, t2, kbar, [&](int y, int l) {
@@ -1197,12 +1174,12 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
                     C s = tz[i];
                     if (inner > 1) {
                         const C so = tp[i];
-                        s.x += be0 * so.x;
-                        s.y += be1 * so.y;
+                        s.x += so.x * be0;
+                        s.y += so.y * be1;
                     }
                     tp[i] = s;
-                    r.x -= al0 * s.x;
-                    r.y -= al1 * s.y;
+                    r.x -= s.x * al0;
+                    r.y -= s.y * al1;
                     tr[i] = r;
                 }
                 return r;
@@ -1220,17 +1197,17 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
                     if (inner > 1) {
                         const C po = cp[i], so = cs[i];
                         e = ce[i];
-                        p.x += be0 * po.x;
-                        p.y += be1 * po.y;
-                        s.x += be0 * so.x;
-                        s.y += be1 * so.y;
-                        e.x += al0 * p.x;
-                        e.y += al1 * p.y;
+                        p.x += po.x * be0;
+                        p.y += po.y * be1;
+                        s.x += so.x * be0;
+                        s.y += so.y * be1;
+                        e.x += p.x * al0;
+                        e.y += p.y * al1;
                     } else {
-                        e = qsfft::mk<T>(al0 * p.x, al1 * p.y);
+                        e = qsfft::mk<T>(p.x * al0, p.y * al1);
                     }
-                    r.x -= al0 * s.x;
-                    r.y -= al1 * s.y;
+                    r.x -= s.x * al0;
+                    r.y -= s.y * al1;
                     cp[i] = p;
                     cs[i] = s;
                     ce[i] = e;
@@ -1261,14 +1238,14 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
             if (!S(53)) return -1;
             if (threadIdx.x < 2) {  // one thread a component
                 const int c = threadIdx.x;
-                const double *g = sc->cgd[slot & 3];
-                const double ga = vload(g + c), de = vload(g + 2 + c);
-                double be = 0.0, al = 0.0, ia = 0.0, ig = 0.0;
-                if (ga != 0.0) {
-                    ig = 1.0 / ga;
-                    be = inner > 0 ? ga * I.ig[c] : 0.0;
-                    ia = de * ig - be * (inner > 0 ? I.ia[c] : 0.0);
-                    al = ia != 0.0 ? 1.0 / ia : 0.0;
+                const float *g = sc->cgd[slot & 3];
+                const float ga = vload(g + c), de = vload(g + 2 + c);
+                float be = 0.f, al = 0.f, ia = 0.f, ig = 0.f;
+                if (ga != 0.f) {
+                    ig = 1.f / ga;
+                    be = inner > 0 ? ga * I.ig[c] : 0.f;
+                    ia = de * ig - be * (inner > 0 ? I.ia[c] : 0.f);
+                    al = ia != 0.f ? 1.f / ia : 0.f;
                 }
                 I.ig[c] = ig;
                 I.ia[c] = ia;
@@ -1276,12 +1253,12 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
                 I.be[c] = be;
                 // ||r - al s||^2 with s = w + be s_old.  The sums are good to
                 // about 1e-7 of ||r||^2: no smaller value is believed.
-                const float a = (float)al, b = (float)be;
-                const float rw = (float)vload(g + 4 + c), rs = (float)vload(g + 6 + c),
-                            ww = (float)vload(g + 8 + c), ws = (float)vload(g + 10 + c);
+                const float a = al, b = be;
+                const float rw = vload(g + 4 + c), rs = vload(g + 6 + c), ww = vload(g + 8 + c),
+                            ws = vload(g + 10 + c);
                 const float so = inner > 0 ? I.ss[c] : 0.f;
                 const float ss = ww + b * (2.f * ws + b * so);
-                const float rr = (float)vload(g + 12 + c);
+                const float rr = vload(g + 12 + c);
                 I.ss[c] = ss;
                 const float nr = rr - a * (2.f * (rw + b * rs) - a * ss);
                 I.rr[c] = nr < 2e-7f * rr ? 2e-7f * rr : nr;  // a NaN stays
@@ -1294,10 +1271,10 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
                     if (!((double)I.rr[c] <= fmax(red * I.r0[c], 0.09 * I.thr[c]))) go = 1;
                 I.go = go;
             }
-            al0 = narrow<T>(I.al[0]);
-            al1 = narrow<T>(I.al[1]);
-            be0 = narrow<T>(I.be[0]);
-            be1 = narrow<T>(I.be[1]);
+            al0 = I.al[0];
+            al1 = I.al[1];
+            be0 = I.be[0];
+            be1 = I.be[1];
             __syncthreads();
             const bool go = I.go != 0;
             __syncthreads();  // rewritten by the next test
@@ -1310,11 +1287,11 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
         // e is e + al p with the last step, at the cell and its neighbours.
         auto e_at = [&](size_t i) {
             C p = cz[i];
-            if (inner == 1) return qsfft::mk<T>(al0 * p.x, al1 * p.y);
+            if (inner == 1) return qsfft::mk<T>(p.x * al0, p.y * al1);
             const C po = cp[i], eo = ce[i];
-            p.x += be0 * po.x;
-            p.y += be1 * po.y;
-            return qsfft::mk<T>(eo.x + al0 * p.x, eo.y + al1 * p.y);
+            p.x += po.x * be0;
+            p.y += po.y * be1;
+            return qsfft::mk<T>(eo.x + p.x * al0, eo.y + p.y * al1);
         };
         float n[16] = {0.f};
         const double ih2 = A.lev_inv_h2[0];
