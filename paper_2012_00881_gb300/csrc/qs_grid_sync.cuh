@@ -16,6 +16,7 @@
 namespace qsync {
 
 __device__ __forceinline__ int vload(const int *p) { return *(const volatile int *)p; }
+__device__ __forceinline__ float vload(const float *p) { return *(const volatile float *)p; }
 __device__ __forceinline__ double vload(const double *p) { return *(const volatile double *)p; }
 
 __device__ __forceinline__ unsigned long long acquire_u64(const unsigned long long *p) {
