@@ -3,6 +3,7 @@
 // and the stable counting sort of particles by cell.
 #include <cuda_runtime.h>
 
+#include "qs_ff.cuh"
 #include "qs_internal.cuh"
 
 namespace {
@@ -130,37 +131,158 @@ __device__ void wake_at(const double *hist, int n, int n_xi, double x_min, doubl
     }
 }
 
+// The same gather in pairs of floats for a particle whose cells and their
+// neighbours, and both slices, are inside (`ok`; others take wake_at).  The
+// float64 gather and push issue about 300 FP64-pipe instructions a particle
+// (64 cycles a warp each): 500,000 particles 260 us.  In pairs, with float64 for
+// the position and momentum sums, 120 us, bound by the latency of the gathers (56 loads of
+// a particle's own sectors).
+using qsff::Ff;
+
+// the particle's cells: left cell i = iy n + ix, slice j, weights of the corners
+// (00, 01, 10, 11) at slice j and at slice j + 1
+struct Where {
+    int i, j;
+    Ff w[2][4];
+    bool ok;
+};
+// positions as fused multiply-adds: cells + 1/2, slices + 1
+struct Scale {
+    double inv_h, ox, oy, inv_xi, oxi;
+    Ff inv2h;
+};
+__device__ __forceinline__ Scale scale_of(double x_min, double y_min, double h, double xi_min,
+                                          double dxi0) {
+    Scale s;
+    s.inv_h = 1.0 / h;
+    s.ox = fma(-x_min, s.inv_h, 0.5);
+    s.oy = fma(-y_min, s.inv_h, 0.5);
+    s.inv_xi = 1.0 / dxi0;
+    s.oxi = fma(-xi_min, s.inv_xi, 1.0);
+    s.inv2h = qsff::split(0.5 * s.inv_h);
+    return s;
+}
+// margin: slices needed before and after the two around the particle
+__device__ __forceinline__ Where where_of(const Scale &S, double x, double y, double xi, int n,
+                                          int n_xi, int margin) {
+    using namespace qsff;
+    const double tx = fma(x, S.inv_h, S.ox), ty = fma(y, S.inv_h, S.oy),
+                 tz = fma(xi, S.inv_xi, S.oxi);
+    Where r;
+    // the bits of 2 <= t < 4096; anything else (walls, window ends, NaN) is not ok
+    auto in = [](double t) {
+        const unsigned e = ((unsigned)__double2hiint(t) >> 20) - 1024u;
+        return e <= 10u;
+    };
+    r.ok = false;
+    r.i = r.j = 0;
+    if (!(in(tx) && in(ty) && ((unsigned)__double2hiint(tz) >> 20) - 1023u <= 30u)) return r;
+    const AxisBits bx = axis_bits(tx), by = axis_bits(ty), bz = axis_bits(tz);
+    r.j = bz.cell - 1;
+    if (bx.cell > n - 2 || by.cell > n - 2 || r.j < margin || r.j + 1 + margin > n_xi - 1) return r;
+    r.ok = true;
+    r.i = (by.cell - 1) * n + bx.cell - 1;
+    const Ff one(1.f, 0.f), gx = one - bx.f, gy = one - by.f, gz = one - bz.f;
+    const Ff w00 = gy * gx, w01 = gy * bx.f, w10 = by.f * gx, w11 = by.f * bx.f;
+    r.w[0][0] = w00 * gz;
+    r.w[0][1] = w01 * gz;
+    r.w[0][2] = w10 * gz;
+    r.w[0][3] = w11 * gz;
+    r.w[1][0] = w00 * bz.f;
+    r.w[1][1] = w01 * bz.f;
+    r.w[1][2] = w10 * bz.f;
+    r.w[1][3] = w11 * bz.f;
+    return r;
+}
+
+__device__ __forceinline__ Ff dot4(const Ff (&w)[4], Ff a, Ff b, Ff c, Ff d) {
+    return (w[0] * a + w[1] * b) + (w[2] * c + w[3] * d);
+}
+
+// out as wake_at's: E_z, B_z, B_x, B_y, d_x psi, d_y psi
+__device__ __forceinline__ void wake_pairs(const double *hist, int n, int n_xi, const Scale &S,
+                                           const Where &r, Ff out[6]) {
+    using qsff::split;
+    const size_t nn = (size_t)n * n, fs = (size_t)n_xi * nn;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) out[k] = Ff(0.f, 0.f);
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+        const double *ps = hist + (size_t)(r.j + side) * nn + r.i;
+        const Ff(&w)[4] = r.w[side];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const double *f = ps + (size_t)(k + 1) * fs;
+            out[k] += dot4(w, split(f[0]), split(f[1]), split(f[n]), split(f[n + 1]));
+        }
+        // psi on the 4 x 4 patch without its corners
+        auto at = [&](int dx, int dy) { return split(ps[dy * n + dx]); };
+        const Ff a0 = at(-1, 0), a1 = at(0, 0), a2 = at(1, 0), a3 = at(2, 0);
+        const Ff b0 = at(-1, 1), b1 = at(0, 1), b2 = at(1, 1), b3 = at(2, 1);
+        out[4] += dot4(w, a2 - a0, a3 - a1, b2 - b0, b3 - b1);
+        out[5] += dot4(w, b1 - at(0, -1), b2 - at(1, -1), at(0, 2) - a1, at(1, 2) - a2);
+    }
+    out[4] = out[4] * S.inv2h;
+    out[5] = out[5] * S.inv2h;
+}
+
+// One relativistic Boris step: half kick, rotation, half kick, drift; the
+// changes are formed in pairs and added in float64.  xi advances by
+// dt (1 - v_z), with 1 - v_z = (1 + p_perp^2) / (gamma (gamma + p_z)) where p_z > 0
+// so that nothing cancels.
+__device__ __forceinline__ void boris_pairs(double &x, double &y, double &xi, double &px,
+                                            double &py, double &pz, Ff ex, Ff ey, Ff ez, Ff bx,
+                                            Ff by, Ff bz, Ff hq, Ff dt) {
+    using namespace qsff;
+    const Ff one(1.f, 0.f);
+    const Ff kx = hq * ex, ky = hq * ey, kz = hq * ez;
+    const Ff ux = split(px) + kx, uy = split(py) + ky, uz = split(pz) + kz;
+    const Ff s = hq * recip(sqrt_pair(one + (ux * ux + uy * uy) + uz * uz));
+    const Ff tx = s * bx, ty = s * by, tz = s * bz;
+    const Ff vx = ux + (uy * tz - uz * ty), vy = uy + (uz * tx - ux * tz),
+             vz = uz + (ux * ty - uy * tx);
+    const Ff ss = recip(one + (tx * tx + ty * ty) + tz * tz) * 2.f;
+    px += join(kx * 2.f + ss * (vy * tz - vz * ty));
+    py += join(ky * 2.f + ss * (vz * tx - vx * tz));
+    pz += join(kz * 2.f + ss * (vx * ty - vy * tx));
+    const Ff qx = split(px), qy = split(py), qz = split(pz);
+    const Ff p2 = one + (qx * qx + qy * qy), g = sqrt_pair(p2 + qz * qz);
+    const Ff v = dt * recip(g);
+    x += join(v * qx);
+    y += join(v * qy);
+    xi += join(qz.h > 0.f ? v * (p2 * recip(g + qz)) : dt - v * qz);
+}
+
 // Push_Driver: relativistic Boris step in E = (-d_x psi + B_y, -d_y psi - B_x,
 // E_z), B = (B_x, B_y, B_z); xi advances by dt (1 - v_z).
-__global__ void k_beam_push(double *x, double *y, double *xi, double *px, double *py,
+__device__ __noinline__ void wake_at_edge(const double *hist, int n, int n_xi, double x_min,
+                                          double x_max, double y_min, double y_max, double h,
+                                          double xi_min, double dxi0, double x, double y,
+                                          double xi, Ff out[6]) {
+    double wk[6];
+    wake_at(hist, n, n_xi, x_min, x_max, y_min, y_max, h, xi_min, dxi0, x, y, xi, wk);
+    for (int k = 0; k < 6; ++k) out[k] = qsff::split(wk[k]);
+}
+
+__global__ void __launch_bounds__(kThreads, 4) k_beam_push(double *x, double *y, double *xi, double *px, double *py,
                             double *pz, int64_t nb, double qm, int n, double x_min,
                             double x_max, double y_min, double y_max, double h, int n_xi,
                             double xi_min, double dxi0, const double *hist, double dt) {
+    const Scale S = scale_of(x_min, y_min, h, xi_min, dxi0);
+    const Ff hq = qsff::split(0.5 * dt * qm), dtf = qsff::split(dt);
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < nb;
          p += (int64_t)gridDim.x * blockDim.x) {
-        double wk[6];
-        wake_at(hist, n, n_xi, x_min, x_max, y_min, y_max, h, xi_min, dxi0, x[p], y[p], xi[p],
-                wk);
-        const double ez = wk[0], bz = wk[1], bx = wk[2], by = wk[3];
-        const double ex = -wk[4] + by, ey = -wk[5] - bx;
-        const double hq = 0.5 * dt * qm;
-        double ux = px[p] + hq * ex, uy = py[p] + hq * ey, uz = pz[p] + hq * ez;
-        double gam = sqrt(1.0 + ux * ux + uy * uy + uz * uz);
-        const double tx = hq * bx / gam, ty = hq * by / gam, tz = hq * bz / gam;
-        const double ss = 2.0 / (1.0 + tx * tx + ty * ty + tz * tz);
-        const double upx = ux + (uy * tz - uz * ty);
-        const double upy = uy + (uz * tx - ux * tz);
-        const double upz = uz + (ux * ty - uy * tx);
-        ux = ux + ss * (upy * tz - upz * ty);
-        uy = uy + ss * (upz * tx - upx * tz);
-        uz = uz + ss * (upx * ty - upy * tx);
-        ux += hq * ex;
-        uy += hq * ey;
-        uz += hq * ez;
-        gam = sqrt(1.0 + ux * ux + uy * uy + uz * uz);
-        x[p] += dt * ux / gam;
-        y[p] += dt * uy / gam;
-        xi[p] += dt * (1.0 - uz / gam);
+        double X = x[p], Y = y[p], Z = xi[p], ux = px[p], uy = py[p], uz = pz[p];
+        const Where r = where_of(S, X, Y, Z, n, n_xi, 0);
+        Ff wk[6];
+        if (r.ok) wake_pairs(hist, n, n_xi, S, r, wk);
+        else
+            wake_at_edge(hist, n, n_xi, x_min, x_max, y_min, y_max, h, xi_min, dxi0, X, Y, Z, wk);
+        boris_pairs(X, Y, Z, ux, uy, uz, wk[3] - wk[4], -(wk[5] + wk[2]), wk[0], wk[2], wk[3],
+                    wk[1], hq, dtf);
+        x[p] = X;
+        y[p] = Y;
+        xi[p] = Z;
         px[p] = ux;
         py[p] = uy;
         pz[p] = uz;
@@ -220,6 +342,84 @@ __device__ void envelope_at(const double2 *env, int n, int n_xi, double x_min, d
     }
 }
 
+// The envelope's terms at time fraction fr = 1 - fo in pairs of floats, for a
+// particle well inside (wake_pairs): A, d_t A, d_xi A, d_x A, d_y A.
+__device__ __forceinline__ void envelope_pairs(const double2 *en, const double2 *ep, int n,
+                                               const Scale &S, const Where &r, Ff fo, Ff fr,
+                                               Ff inv2xi, Ff inv_dt, Ff a[2], Ff t[2], Ff axi[2],
+                                               Ff ax[2], Ff ay[2]) {
+    using qsff::split;
+    const size_t nn = (size_t)n * n;
+    const Ff zero(0.f, 0.f);
+#pragma unroll
+    for (int c = 0; c < 2; ++c) a[c] = t[c] = axi[c] = ax[c] = ay[c] = zero;
+    struct Cx {
+        Ff re, im;
+    };
+#pragma unroll 1
+    for (int side = 0; side < 2; ++side) {
+        const size_t base = (size_t)(r.j + side) * nn + r.i;
+        const Ff(&w)[4] = r.w[side];
+        auto mix = [&](size_t i) {  // the envelope at the sub-step's time
+            const double2 u = en[i], v = ep[i];
+            return Cx{fo * split(u.x) + fr * split(v.x), fo * split(u.y) + fr * split(v.y)};
+        };
+        const int corner[4] = {0, 1, n, n + 1};
+        Cx m[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const size_t i = base + corner[k];
+            const double2 u = en[i], v = ep[i];
+            const Ff ur = split(u.x), ui = split(u.y), vr = split(v.x), vi = split(v.y);
+            m[k] = Cx{fo * ur + fr * vr, fo * ui + fr * vi};
+            a[0] += w[k] * m[k].re;
+            a[1] += w[k] * m[k].im;
+            t[0] += w[k] * (vr - ur);
+            t[1] += w[k] * (vi - ui);
+            const Cx nx = mix(i + nn), pv = mix(i - nn);
+            axi[0] += w[k] * (nx.re - pv.re);
+            axi[1] += w[k] * (nx.im - pv.im);
+        }
+        const Cx w0 = mix(base - 1), w1 = mix(base + n - 1), e0 = mix(base + 2),
+                 e1 = mix(base + n + 2);
+        ax[0] += dot4(w, m[1].re - w0.re, e0.re - m[0].re, m[3].re - w1.re, e1.re - m[2].re);
+        ax[1] += dot4(w, m[1].im - w0.im, e0.im - m[0].im, m[3].im - w1.im, e1.im - m[2].im);
+        const Cx s0 = mix(base - n), s1 = mix(base - n + 1), n0 = mix(base + 2 * n),
+                 n1 = mix(base + 2 * n + 1);
+        ay[0] += dot4(w, m[2].re - s0.re, m[3].re - s1.re, n0.re - m[0].re, n1.re - m[1].re);
+        ay[1] += dot4(w, m[2].im - s0.im, m[3].im - s1.im, n0.im - m[0].im, n1.im - m[1].im);
+    }
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        t[c] = t[c] * inv_dt;
+        axi[c] = axi[c] * inv2xi;
+        ax[c] = ax[c] * S.inv2h;
+        ay[c] = ay[c] * S.inv2h;
+    }
+}
+
+// wake and envelope terms of any particle, in float64
+__device__ __noinline__ void dla_at_edge(const double *hist, const double2 *env_n,
+                                         const double2 *env_np1, int n, int n_xi, double x_min,
+                                         double x_max, double y_min, double y_max, double h,
+                                         double xi_min, double dxi0, double x, double y,
+                                         double xi, double fr, double inv_dt, Ff wk[6], Ff a[2],
+                                         Ff t[2], Ff axi[2], Ff ax[2], Ff ay[2]) {
+    using qsff::split;
+    wake_at_edge(hist, n, n_xi, x_min, x_max, y_min, y_max, h, xi_min, dxi0, x, y, xi, wk);
+    double2 gn[4], gp[4];
+    envelope_at(env_n, n, n_xi, x_min, x_max, y_min, y_max, h, xi_min, dxi0, x, y, xi, gn);
+    envelope_at(env_np1, n, n_xi, x_min, x_max, y_min, y_max, h, xi_min, dxi0, x, y, xi, gp);
+    const double fo = 1.0 - fr;
+    Ff *const out[4] = {a, axi, ax, ay};
+    for (int k = 0; k < 4; ++k) {
+        out[k][0] = split(fo * gn[k].x + fr * gp[k].x);
+        out[k][1] = split(fo * gn[k].y + fr * gp[k].y);
+    }
+    t[0] = split((gp[0].x - gn[0].x) * inv_dt);
+    t[1] = split((gp[0].y - gn[0].y) * inv_dt);
+}
+
 // Push_Driver in the wake plus the laser's fields of Eq. E_B_Fields (the
 // real parts of the printed complex fields; x polarisation):
 //   E_x = Re[-((d_t A + d_xi A) - i k0 A) e^{-i k0 xi}],  B_y = Re[(-d_xi A + i k0 A) e^{-i k0 xi}],
@@ -228,57 +428,65 @@ __device__ void envelope_at(const double2 *env, int n, int n_xi, double x_min, d
 // sub-step s the envelope is taken linearly in time between env_n and
 // env_np1 at frac = s / n_sub, d_t A = (A^{n+1} - A^n) / dt; the carrier
 // phase is evaluated at the particle's own xi; the wake is frozen.
-__global__ void k_beam_push_dla(double *x, double *y, double *xi, double *px, double *py,
+__global__ void __launch_bounds__(kThreads, 3) k_beam_push_dla(double *x, double *y, double *xi, double *px, double *py,
                                 double *pz, int64_t nb, double qm, int n, double x_min,
                                 double x_max, double y_min, double y_max, double h, int n_xi,
                                 double xi_min, double dxi0, const double *hist,
                                 const double2 *env_n, const double2 *env_np1, double k0,
                                 double dt, int n_sub) {
-    const double hs = dt / n_sub, hq = 0.5 * hs * qm, inv_dt = 1.0 / dt;
+    const double hs = dt / n_sub, inv_dt = 1.0 / dt;
+    const Scale S = scale_of(x_min, y_min, h, xi_min, dxi0);
+    const Ff hq = qsff::split(0.5 * hs * qm), hsf = qsff::split(hs), k0f = qsff::split(k0);
+    const Ff inv2xi = qsff::split(0.5 * S.inv_xi), inv_dtf = qsff::split(inv_dt);
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < nb;
          p += (int64_t)gridDim.x * blockDim.x) {
         double X = x[p], Y = y[p], XI = xi[p];
         double ux = px[p], uy = py[p], uz = pz[p];
         for (int s = 0; s < n_sub; ++s) {
-            double wk[6];
-            wake_at(hist, n, n_xi, x_min, x_max, y_min, y_max, h, xi_min, dxi0, X, Y, XI, wk);
-            double2 gn[4], gp[4];
-            envelope_at(env_n, n, n_xi, x_min, x_max, y_min, y_max, h, xi_min, dxi0, X, Y, XI,
-                        gn);
-            envelope_at(env_np1, n, n_xi, x_min, x_max, y_min, y_max, h, xi_min, dxi0, X, Y,
-                        XI, gp);
-            const double fr = (double)s / (double)n_sub, fo = 1.0 - fr;
-            const double ar = fo * gn[0].x + fr * gp[0].x, ai = fo * gn[0].y + fr * gp[0].y;
-            const double tr = (gp[0].x - gn[0].x) * inv_dt, ti = (gp[0].y - gn[0].y) * inv_dt;
-            const double xr = fo * gn[1].x + fr * gp[1].x, xim = fo * gn[1].y + fr * gp[1].y;
-            const double dxr = fo * gn[2].x + fr * gp[2].x, dxim = fo * gn[2].y + fr * gp[2].y;
-            const double dyr = fo * gn[3].x + fr * gp[3].x, dyim = fo * gn[3].y + fr * gp[3].y;
-            double sn, cs;
-            sincos(k0 * XI, &sn, &cs);  // e^{-i k0 xi} = cs - i sn
+            const double fr = (double)s / (double)n_sub;
+            const Where r = where_of(S, X, Y, XI, n, n_xi, 1);
+            Ff wk[6], a[2], t[2], axi[2], ax[2], ay[2];  // complex envelope terms
+            if (r.ok) {
+                wake_pairs(hist, n, n_xi, S, r, wk);
+                envelope_pairs(env_n, env_np1, n, S, r, qsff::split(1.0 - fr), qsff::split(fr),
+                               inv2xi, inv_dtf, a, t, axi, ax, ay);
+            } else {
+                dla_at_edge(hist, env_n, env_np1, n, n_xi, x_min, x_max, y_min, y_max, h, xi_min,
+                            dxi0, X, Y, XI, fr, inv_dt, wk, a, t, axi, ax, ay);
+            }
+            // e^{-i k0 xi} = cs - i sn: the phase less a multiple of pi / 2, in
+            // float64 (2^52 + 2^51 added rounds to an integer), the rest in pairs
+            const double ph = k0 * XI;
+            const double m = fma(ph, 0.63661977236758134308, 6755399441055744.0);
+            const int quad = __double2loint(m);
+            const double q = m - 6755399441055744.0;
+            Ff sn, cs;
+            if (fabsf((float)q) < 1e6f) {
+                const double red = fma(q, -6.123233995736766036e-17, fma(q, -1.57079632679489661923, ph));
+                qsff::sincos_pair(qsff::split(red), sn, cs);
+                if (quad & 1) {
+                    const Ff o = sn;
+                    sn = cs;
+                    cs = -o;
+                }
+                if (quad & 2) {
+                    sn = -sn;
+                    cs = -cs;
+                }
+            } else {
+                double sd, cd;
+                sincos(ph, &sd, &cd);
+                sn = qsff::split(sd);
+                cs = qsff::split(cd);
+            }
             // Re[(u + i v)(cs - i sn)] = u cs + v sn
-            const double exl = -((tr + xr) + k0 * ai) * cs - ((ti + xim) - k0 * ar) * sn;
-            const double byl = (-xr - k0 * ai) * cs + (-xim + k0 * ar) * sn;
-            const double ezl = -dxr * cs - dxim * sn;
-            const double bzl = -dyr * cs - dyim * sn;
-            const double ez = wk[0] + ezl, bz = wk[1] + bzl, bx = wk[2], by = wk[3] + byl;
-            const double ex = -wk[4] + wk[3] + exl, ey = -wk[5] - wk[2];
-            double vx = ux + hq * ex, vy = uy + hq * ey, vz = uz + hq * ez;
-            double gam = sqrt(1.0 + vx * vx + vy * vy + vz * vz);
-            const double tx = hq * bx / gam, ty = hq * by / gam, tz = hq * bz / gam;
-            const double ss = 2.0 / (1.0 + tx * tx + ty * ty + tz * tz);
-            const double upx = vx + (vy * tz - vz * ty);
-            const double upy = vy + (vz * tx - vx * tz);
-            const double upz = vz + (vx * ty - vy * tx);
-            vx = vx + ss * (upy * tz - upz * ty);
-            vy = vy + ss * (upz * tx - upx * tz);
-            vz = vz + ss * (upx * ty - upy * tx);
-            ux = vx + hq * ex;
-            uy = vy + hq * ey;
-            uz = vz + hq * ez;
-            gam = sqrt(1.0 + ux * ux + uy * uy + uz * uz);
-            X += hs * ux / gam;
-            Y += hs * uy / gam;
-            XI += hs * (1.0 - uz / gam);
+            const Ff kr = k0f * a[0], ki = k0f * a[1];
+            const Ff exl = -((t[0] + axi[0] + ki) * cs + (t[1] + axi[1] - kr) * sn);
+            const Ff byl = (kr - axi[1]) * sn - (axi[0] + ki) * cs;
+            const Ff ezl = -(ax[0] * cs + ax[1] * sn);
+            const Ff bzl = -(ay[0] * cs + ay[1] * sn);
+            boris_pairs(X, Y, XI, ux, uy, uz, wk[3] - wk[4] + exl, -(wk[5] + wk[2]), wk[0] + ezl,
+                        wk[2], wk[3] + byl, wk[1] + bzl, hq, hsf);
         }
         x[p] = X;
         y[p] = Y;

@@ -276,40 +276,6 @@ __device__ void phase_psi_rhs(const EngineArgs &A, const PS<P> &Q, const double 
     }
 }
 
-// The CIC stencil of the refined form from one fused multiply-add an axis:
-// s + 1/2 = x / h + const in [1/2, N + 1/2] inside the box, whose integer part
-// and fraction come from its bits (a floor, a conversion and the differences
-// would be five FP64-pipe instructions an axis).  f: the fraction as a pair.
-struct AxisBits {
-    int cell;   // floor(s + 1/2): the right one of the two cells
-    qsff::Ff f; // weight of the right cell
-};
-__device__ __forceinline__ AxisBits axis_bits(double t) {
-    const unsigned hi = (unsigned)__double2hiint(t), lo = (unsigned)__double2loint(t);
-    const int e = (int)(hi >> 20) - 1023;  // -1 ... 11 in the box
-    AxisBits b;
-    if ((unsigned)(e + 1) > 12u) {  // outside the box (negative, or far beyond it)
-        const double fl = floor(t);
-        b.cell = (int)fl;
-        b.f = qsff::split(t - fl);
-        return b;
-    }
-    const unsigned mh = (hi & 0xfffffu) | 0x100000u;
-    b.cell = (int)(mh >> (20 - e));
-    // the fraction as 64 bits: shift the integer part out at the top
-    const int sh = 12 + e;
-    const unsigned fh = __funnelshift_l(lo, mh, sh), fl = lo << sh;
-    const float h = (float)(fh & 0xffffff00u);
-    const float l = (float)((fh << 24) | (fl >> 8));
-    b.f = qsff::quick(h * 0x1p-32f, l * 0x1p-56f);
-    return b;
-}
-
-// s + 1/2 of a coordinate (s = (x - x_min) / h)
-__device__ __forceinline__ double axis_pos(double x, double inv_h, double x_min) {
-    return fma(x, inv_h, fma(-x_min, inv_h, 0.5));
-}
-
 // folded cell indices of an axis: the ghost's weight goes to the edge cell
 __device__ __forceinline__ void fold(int right, int n, int &a, int &b) {
     a = right - 1;
@@ -332,7 +298,7 @@ struct CicF {
 };
 
 __device__ __forceinline__ CicF cic_pairs(double tx, double ty, int n) {
-    const AxisBits bx = axis_bits(tx), by = axis_bits(ty);
+    const qsff::AxisBits bx = qsff::axis_bits(tx), by = qsff::axis_bits(ty);
     int ax, cx, ay, cy;
     fold(bx.cell, n, ax, cx);
     fold(by.cell, n, ay, cy);
@@ -1001,7 +967,7 @@ __device__ void phase_push(const EngineArgs &A, const PS<P> &Q, double *nnext, b
             double nx = x + qsff::widen(dxp * px * ia);
             double ny = y + qsff::widen(dxp * py * ia);
             double tx = fma(nx, A.inv_h, ox), ty = fma(ny, A.inv_h, oy);
-            AxisBits ax = axis_bits(tx), ay = axis_bits(ty);
+            qsff::AxisBits ax = qsff::axis_bits(tx), ay = qsff::axis_bits(ty);
             // only a particle in the half cells at the walls can have crossed one
             if ((unsigned)(ax.cell - 1) >= (unsigned)(A.N - 1) ||
                 (unsigned)(ay.cell - 1) >= (unsigned)(A.N - 1)) {
@@ -1009,8 +975,8 @@ __device__ void phase_push(const EngineArgs &A, const PS<P> &Q, double *nnext, b
                 reflect(ny, py, A.y_min, A.y_max);
                 tx = fma(nx, A.inv_h, ox);
                 ty = fma(ny, A.inv_h, oy);
-                ax = axis_bits(tx);
-                ay = axis_bits(ty);
+                ax = qsff::axis_bits(tx);
+                ay = qsff::axis_bits(ty);
             }
             Q.x[p] = nx;
             Q.y[p] = ny;

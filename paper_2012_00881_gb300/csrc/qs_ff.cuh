@@ -79,7 +79,9 @@ __device__ __forceinline__ double widen(float f) {
 __device__ __forceinline__ Ff split(double v) {
     const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
     const int e = (int)((hi >> 20) & 0x7ffu) - 1023;
-    if ((unsigned)(e + 70) >= 190u) {  // zero, or beyond what the pair's parts cover
+    if ((unsigned)(e + 70) >= 190u) {
+        if (((hi << 1) | lo) == 0u) return Ff(0.f, 0.f);
+        // beyond what the pair's parts cover
         const float h = (float)v;
         return Ff(h, isfinite(h) ? (float)(v - (double)h) : 0.f);
     }
@@ -92,5 +94,65 @@ __device__ __forceinline__ Ff split(double v) {
 
 // the pair as a float64: one FP64 addition
 __device__ __forceinline__ double join(Ff a) { return widen(a.h) + widen(a.l); }
+
+// Integer part and fraction (as a pair) of 1/2 <= t < 4096 from its bits: a floor,
+// a conversion and a difference would be three FP64-pipe instructions.  With
+// t = s + 1/2 for a position s in cells, `cell` is the right one of the two
+// cell centres around it and f its linear weight.
+struct AxisBits {
+    int cell;
+    Ff f;
+};
+__device__ __forceinline__ AxisBits axis_bits(double t) {
+    const unsigned hi = (unsigned)__double2hiint(t), lo = (unsigned)__double2loint(t);
+    const int e = (int)(hi >> 20) - 1023;
+    AxisBits b;
+    if ((unsigned)(e + 1) > 12u) {  // outside the box (negative, or far beyond it)
+        const double fl = floor(t);
+        b.cell = (int)fl;
+        b.f = split(t - fl);
+        return b;
+    }
+    const unsigned mh = (hi & 0xfffffu) | 0x100000u;
+    b.cell = (int)(mh >> (20 - e));
+    // the fraction as 64 bits: shift the integer part out at the top
+    const int sh = 12 + e;
+    const unsigned fh = __funnelshift_l(lo, mh, sh), fl = lo << sh;
+    const float h = (float)(fh & 0xffffff00u);
+    const float l = (float)((fh << 24) | (fl >> 8));
+    b.f = quick(h * 0x1p-32f, l * 0x1p-56f);
+    return b;
+}
+
+// square root of a > 0: one Newton step from float32
+__device__ __forceinline__ Ff sqrt_pair(Ff a) {
+    const float r = rsqrtf(a.h), y = __fmul_rn(a.h, r);
+    const Ff y2 = two_prod(y, y);
+    const float e = __fadd_rn(__fsub_rn(__fsub_rn(a.h, y2.h), y2.l), a.l);  // a - y^2
+    return quick(y, __fmul_rn(__fmul_rn(e, 0.5f), r));
+}
+
+// sine and cosine of |r| <= pi / 4 by their Taylor series: pairs for the terms
+// above 2^-24 of the sum, float32 for the rest (truncated below 2^-52)
+__device__ __forceinline__ void sincos_pair(Ff r, Ff &s, Ff &c) {
+    constexpr double f3 = 6, f4 = 24, f5 = 120, f6 = 720, f7 = 5040, f8 = 40320, f9 = 362880,
+                     f10 = 3628800, f11 = 39916800, f12 = 479001600, f13 = 6227020800,
+                     f14 = 87178291200, f15 = 1307674368000, f16 = 20922789888000;
+    const Ff z = r * r;
+    const float zf = z.h;
+    const float st = fmaf(zf, fmaf(zf, (float)(-1 / f15), (float)(1 / f13)), (float)(-1 / f11));
+    const float ct = fmaf(zf, fmaf(zf, (float)(1 / f16), (float)(-1 / f14)), (float)(1 / f12));
+    Ff p = Ff(1 / f9) + Ff(zf * st, 0.f);
+    p = Ff(-1 / f7) + z * p;
+    p = Ff(1 / f5) + z * p;
+    p = Ff(-1 / f3) + z * p;
+    s = r + (r * z) * p;
+    Ff q = Ff(-1 / f10) + Ff(zf * ct, 0.f);
+    q = Ff(1 / f8) + z * q;
+    q = Ff(-1 / f6) + z * q;
+    q = Ff(1 / f4) + z * q;
+    q = Ff(-0.5) + z * q;
+    c = Ff(1.f, 0.f) + z * q;
+}
 
 }  // namespace qsff
