@@ -172,19 +172,24 @@ struct Deal {
     }
 };
 
-// -i v forward, +i v inverse
-template <bool INV, typename V>
+// -i v
+template <typename V>
 __device__ __forceinline__ V mul_i(V v) {
     V r;
-    r.x = INV ? -v.y : v.y;
-    r.y = INV ? v.x : -v.x;
+    r.x = v.y;
+    r.y = -v.x;
     return r;
 }
+template <typename V>
+__device__ __forceinline__ V conj(V v) {
+    v.y = -v.y;
+    return v;
+}
 
-template <typename T, bool INV, typename V>
+template <typename V>
 __device__ __forceinline__ void dft4(V &a, V &b, V &c, V &d) {
     const V s02 = cadd(a, c), d02 = csub(a, c);
-    const V s13 = cadd(b, d), q = mul_i<INV>(csub(b, d));
+    const V s13 = cadd(b, d), q = mul_i(csub(b, d));
     a = cadd(s02, s13);
     b = cadd(d02, q);
     c = csub(s02, s13);
@@ -193,7 +198,7 @@ __device__ __forceinline__ void dft4(V &a, V &b, V &c, V &d) {
 
 // One Stockham pass of radix R over gl lines of N points: the sub-transforms
 // done so far have length Ns = N / n (a power of two).
-template <typename T, int R, bool INV>
+template <typename T, int R>
 __device__ __forceinline__ void pass(const V2<T> *src, V2<T> *dst, const V2<T> *tw, int N, int n,
                                      int Ns, const Deal &D, int gl) {
     using V = V2<T>;
@@ -210,19 +215,19 @@ __device__ __forceinline__ void pass(const V2<T> *src, V2<T> *dst, const V2<T> *
                 // powers of one twiddle: its multiples' table entries lie in
                 // few banks (512 points, four lines: 1,400 cycles a pass)
                 const V w1 = tw[ks], w2 = cmul<false>(w1, w1), w3 = cmul<false>(w2, w1);
-                v[1] = cmul<INV>(v[1], w1);
-                v[2] = cmul<INV>(v[2], w2);
-                v[3] = cmul<INV>(v[3], w3);
+                v[1] = cmul<false>(v[1], w1);
+                v[2] = cmul<false>(v[2], w2);
+                v[3] = cmul<false>(v[3], w3);
                 if constexpr (R == 8) {
                     const V w4 = cmul<false>(w2, w2);
-                    v[4] = cmul<INV>(v[4], w4);
-                    v[5] = cmul<INV>(v[5], cmul<false>(w4, w1));
-                    v[6] = cmul<INV>(v[6], cmul<false>(w4, w2));
-                    v[7] = cmul<INV>(v[7], cmul<false>(w4, w3));
+                    v[4] = cmul<false>(v[4], w4);
+                    v[5] = cmul<false>(v[5], cmul<false>(w4, w1));
+                    v[6] = cmul<false>(v[6], cmul<false>(w4, w2));
+                    v[7] = cmul<false>(v[7], cmul<false>(w4, w3));
                 }
             } else {
 #pragma unroll
-                for (int r = 1; r < R; ++r) v[r] = cmul<INV>(v[r], tw[r * ks]);
+                for (int r = 1; r < R; ++r) v[r] = cmul<false>(v[r], tw[r * ks]);
             }
         }
         auto put = [&](int r, V q) { y[pad<T>(o + r * Ns)] = q; };
@@ -230,17 +235,17 @@ __device__ __forceinline__ void pass(const V2<T> *src, V2<T> *dst, const V2<T> *
             put(0, cadd(v[0], v[1]));
             put(1, csub(v[0], v[1]));
         } else if constexpr (R == 4) {
-            dft4<T, INV>(v[0], v[1], v[2], v[3]);
+            dft4(v[0], v[1], v[2], v[3]);
 #pragma unroll
             for (int r = 0; r < 4; ++r) put(r, v[r]);
         } else if constexpr (R == 8) {
             // even and odd halves, the odd one turned by multiples of pi / 4
-            dft4<T, INV>(v[0], v[2], v[4], v[6]);
-            dft4<T, INV>(v[1], v[3], v[5], v[7]);
+            dft4(v[0], v[2], v[4], v[6]);
+            dft4(v[1], v[3], v[5], v[7]);
             const T h = T(0.70710678118654752440);
-            const V q1 = mul_i<INV>(v[3]), q3 = mul_i<INV>(v[7]);
+            const V q1 = mul_i(v[3]), q3 = mul_i(v[7]);
             const V o1 = mk<T>(h * (v[3].x + q1.x), h * (v[3].y + q1.y));
-            const V o2 = mul_i<INV>(v[5]);
+            const V o2 = mul_i(v[5]);
             const V o3 = mk<T>(h * (q3.x - v[7].x), h * (q3.y - v[7].y));
             put(0, cadd(v[0], v[1]));
             put(1, cadd(v[2], o1));
@@ -255,7 +260,7 @@ __device__ __forceinline__ void pass(const V2<T> *src, V2<T> *dst, const V2<T> *
             for (int q = 0; q < R; ++q) {
                 V t = v[0];
 #pragma unroll
-                for (int r = 1; r < R; ++r) t = cadd(t, cmul<INV>(v[r], tw[((q * r) % R) * nb]));
+                for (int r = 1; r < R; ++r) t = cadd(t, cmul<false>(v[r], tw[((q * r) % R) * nb]));
                 put(q, t);
             }
         }
@@ -263,64 +268,41 @@ __device__ __forceinline__ void pass(const V2<T> *src, V2<T> *dst, const V2<T> *
     __syncthreads();
 }
 
-// Powers of two with every size a constant.  float32: radix 8 while more than 4
-// or 16 is left, then 4.  Pairs: radix 4, whose 300 instructions on two warps a
-// 256-point line finish sooner than radix 8's 900 on one (4,400 -> 2,340
-// cycles a transform).  LGS: log2 of the sub-transforms done.
-template <typename T, bool INV, int LG, int LGS>
-__device__ __forceinline__ bool pow2(V2<T> *a, V2<T> *b, const V2<T> *tw, const Deal &D, int gl) {
-    constexpr int left = LG - LGS;
-    if constexpr (left == 0) {
-        return false;
-    } else {
-        constexpr bool four = !std::is_same<T, float>::value || left == 2 || left == 4;
-        constexpr int lr = left == 1 ? 1 : four ? 2 : 3;
-        pass<T, 1 << lr, INV>(a, b, tw, 1 << LG, 1 << left, 1 << LGS, D, gl);
-        return !pow2<T, INV, LG, LGS + lr>(b, a, tw, D, gl);
-    }
-}
-
-// The transform of the gl lines at offset `a`; returns the offset of the buffer
-// that holds the result, a or b.  Every thread of the block; the caller has
-// synchronised the block after filling the lines.  Out of line: the slice
-// engine's phases would otherwise hold a dozen copies and run from a cold
-// instruction cache.
+// The transform (e^{-2 pi i jk/N}) of the gl lines at offset `a`; returns the
+// offset of the buffer that holds the result, a or b.  The inverse transform is
+// its conjugate of the conjugate.  Every thread of the block; the caller has
+// synchronised the block after filling the lines.
 //
-// float32 is bound by the passes' latency (shared memory, block barrier): few
-// passes of a high radix with constant sizes (256 points, two lines: 1,780 ->
-// 950 cycles).  float64 is bound by the FP64 pipe: a warp-wide
-// instruction occupies one of the SM's four units for 64 cycles however many
-// lanes are active, and a radix-4 pass on fewer than 128 butterflies leaves
-// units idle; radix 2 has twice as many, each less than half the work.
-template <typename T, bool INV>
+// One copy of the code, out of line, with one instance of each radix and sizes
+// in registers: the slice engine runs a few thousand instructions of each phase
+// once and moves on, so that its phases are bound by instruction fetches as much
+// as by data (with constant sizes a 256-point transform of two lines alone takes
+// 1,050 cycles, with these 1,640, but a slice of the engine takes 219 us
+// instead of 232).  float32: radix 8, with 4 or 4 x 4 for the rest.  Pairs:
+// radix 4, whose 300 instructions on two warps a 256-point line finish sooner
+// than radix 8's 900 on one.
+template <typename T>
 __device__ __noinline__ int fft(int a, int b, int tab, int N, int lgG, int gl) {
     const V2<T> *tw = cplx_at<T>(tab);
     const Deal D(lgG);
-    constexpr bool fp64 = std::is_same<T, double>::value;
-    if constexpr (!fp64) {
-        V2<T> *const pa = cplx_at<T>(a), *const pb = cplx_at<T>(b);
-        switch (N) {
-        case 32: return pow2<T, INV, 5, 0>(pa, pb, tw, D, gl) ? b : a;
-        case 64: return pow2<T, INV, 6, 0>(pa, pb, tw, D, gl) ? b : a;
-        case 128: return pow2<T, INV, 7, 0>(pa, pb, tw, D, gl) ? b : a;
-        case 256: return pow2<T, INV, 8, 0>(pa, pb, tw, D, gl) ? b : a;
-        case 512: return pow2<T, INV, 9, 0>(pa, pb, tw, D, gl) ? b : a;
-        case 1024: return pow2<T, INV, 10, 0>(pa, pb, tw, D, gl) ? b : a;
-        default: break;
-        }
-    }
     int Ns = 1, n = N;
     auto run = [&](auto radix) {
         constexpr int R = decltype(radix)::value;
-        pass<T, R, INV>(cplx_at<T>(a), cplx_at<T>(b), tw, N, n, Ns, D, gl);
+        pass<T, R>(cplx_at<T>(a), cplx_at<T>(b), tw, N, n, Ns, D, gl);
         const int t = a;
         a = b;
         b = t;
         Ns *= R;
         n = (unsigned)n / R;
     };
-    while ((!fp64 || gl * N >= 512) && (n & 3) == 0) run(std::integral_constant<int, 4>());
-    while ((n & 1) == 0) run(std::integral_constant<int, 2>());
+    int k = __ffs(n) - 1;  // factors of two left
+    if constexpr (std::is_same<T, float>::value) {
+#pragma unroll 1
+        for (; k >= 3 && k != 4; k -= 3) run(std::integral_constant<int, 8>());
+    }
+#pragma unroll 1
+    for (; k >= 2; k -= 2) run(std::integral_constant<int, 4>());
+    if (k) run(std::integral_constant<int, 2>());
     if (n == 3) run(std::integral_constant<int, 3>());
     else if (n == 5) run(std::integral_constant<int, 5>());
     else if (n == 7) run(std::integral_constant<int, 7>());
@@ -337,6 +319,13 @@ __device__ __forceinline__ int lines_at_once(int nl, int nblk, int gmax) {
 
 // Where sample i of a line sits in the FFT input; odd samples change sign.
 __device__ __forceinline__ int slot_of(int i, int N) { return (i & 1) ? N - 1 - (i >> 1) : i >> 1; }
+// sample i from the conjugate of the inverse transform
+template <typename V>
+__device__ __forceinline__ V sample(V v, int i) {
+    if (i & 1) v.x = -v.x;
+    else v.y = -v.y;
+    return v;
+}
 
 // The second half of rows_forward: transform of the filled lines l0 ... and
 // the coefficients (times 2) to `out`.
@@ -346,7 +335,7 @@ __device__ __noinline__ void rows_forward_rest(int a, int b, int tab, int N, int
     using V = V2<T>;
     const Deal D(lgG);
     __syncthreads();
-    const V *r = cplx_at<T>(fft<T, false>(a, b, tab, N, lgG, gl));
+    const V *r = cplx_at<T>(fft<T>(a, b, tab, N, lgG, gl));
     const V *dct = dct_table<T>(tab, N);
     for (int j = D.g < gl ? D.j0 : N; 2 * j <= N; j += D.stride) {
         const V *x = r + D.g * line_len<T>(N);
@@ -427,7 +416,7 @@ __device__ __noinline__ void columns_rest(int a, int b, int tab, int N, int l0, 
     const V *const dct = dct_table<T>(tab, N);
     const T *const lam = lam_table<T>(tab, N);
     __syncthreads();
-    const int f = fft<T, false>(a, b, tab, N, lgG, gl);
+    const int f = fft<T>(a, b, tab, N, lgG, gl);
     for (int j = D.g < gl ? D.j0 : N; 2 * j <= N; j += D.stride) {
         const int l = l0 + D.g;
         T kr;
@@ -447,7 +436,7 @@ __device__ __noinline__ void columns_rest(int a, int b, int tab, int N, int l0, 
         };
         V *x = cplx_at<T>(f) + D.g * line_len<T>(N);
         if (j == 0) {
-            x[0] = scaled(cadd(x[0], x[0]), 0);
+            x[0] = conj(scaled(cadd(x[0], x[0]), 0));
             continue;
         }
         const V w = dct[j];
@@ -456,17 +445,16 @@ __device__ __noinline__ void columns_rest(int a, int b, int tab, int N, int l0, 
         // -i C_{N-j} with C_{N-j} = i m scaled: the parts swap twice
         V d = scaled(mk<T>(-m.y, m.x), N - j);
         d = mk<T>(d.y, -d.x);
-        x[pad<T>(j)] = cmul<true>(cadd(c, d), w);
-        if (2 * j < N) x[pad<T>(N - j)] = cmul<false>(csub(c, d), w);
+        x[pad<T>(j)] = conj(cmul<true>(cadd(c, d), w));
+        if (2 * j < N) x[pad<T>(N - j)] = conj(cmul<false>(csub(c, d), w));
     }
     __syncthreads();
-    const V *r = cplx_at<T>(fft<T, true>(f, f == a ? b : a, tab, N, lgG, gl));
+    const V *r = cplx_at<T>(fft<T>(f, f == a ? b : a, tab, N, lgG, gl));
     for (int t = threadIdx.x; t < (N << lgG); t += blockDim.x) {
         const int y = t >> lgG, g = t & (G - 1);
         if (g >= gl) continue;
-        V v = r[g * line_len<T>(N) + pad<T>(slot_of(y, N))];
-        if (y & 1) v = mk<T>(-v.x, -v.y);
-        out[(size_t)y * nl + l0 + g] = v;
+        const V v = r[g * line_len<T>(N) + pad<T>(slot_of(y, N))];
+        out[(size_t)y * nl + l0 + g] = sample(v, y);
     }
     __syncthreads();
 }
@@ -495,7 +483,7 @@ __device__ __forceinline__ void columns(const Lines &P, int bid, int nblk, V2<T>
 }
 
 // The first half of rows_inverse: coefficients of lines l0 ... to samples;
-// returns the offset of the buffer that holds them.
+// returns the offset of the buffer that holds their conjugates (see sample).
 template <typename T, int NC>
 __device__ __noinline__ int rows_inverse_first(int a, int b, int tab, int N, int l0, int lgG, int gl,
                                                const V2<T> *in) {
@@ -515,16 +503,16 @@ __device__ __noinline__ int rows_inverse_first(int a, int b, int tab, int N, int
         V *x = cplx_at<T>(a) + D.g * line_len<T>(N);
         const V c = coef(j);
         if (j == 0) {
-            x[0] = c;
+            x[0] = conj(c);
             continue;
         }
         const V w = dct[j], e = coef(N - j);
         const V d = mk<T>(e.y, -e.x);  // -i C_{N-j}
-        x[pad<T>(j)] = cmul<true>(cadd(c, d), w);
-        if (2 * j < N) x[pad<T>(N - j)] = cmul<false>(csub(c, d), w);
+        x[pad<T>(j)] = conj(cmul<true>(cadd(c, d), w));
+        if (2 * j < N) x[pad<T>(N - j)] = conj(cmul<false>(csub(c, d), w));
     }
     __syncthreads();
-    return fft<T, true>(a, b, tab, N, lgG, gl);
+    return fft<T>(a, b, tab, N, lgG, gl);
 }
 
 // Rows inverse: store(line, x, value) takes the solution's samples.
@@ -540,9 +528,7 @@ __device__ __forceinline__ void rows_inverse(const Lines &P, int bid, int nblk, 
         const V *r = cplx_at<T>(
             rows_inverse_first<T, NC>(P.a, buf_b<T>(P), P.tab, N, l0, lgG, gl, in));
         for (int x = D.g < gl ? D.j0 : N; x < N; x += D.stride) {
-            V v = r[D.g * line_len<T>(N) + pad<T>(slot_of(x, N))];
-            if (x & 1) v = mk<T>(-v.x, -v.y);
-            store(l0 + D.g, x, v);
+            store(l0 + D.g, x, sample(r[D.g * line_len<T>(N) + pad<T>(slot_of(x, N))], x));
         }
         __syncthreads();
     }
@@ -567,9 +553,7 @@ __device__ __forceinline__ void rows_inverse_forward(const Lines &P, const Lines
         V2<U> *q = cplx_at<U>(o) + D.g * line_len<U>(N);
         for (int x = D.g < gl ? D.j0 : N; x < N; x += D.stride) {
             const int at = slot_of(x, N);
-            V v = r[pad<T>(at)];
-            if (x & 1) v = mk<T>(-v.x, -v.y);
-            V2<U> w = next(l0 + D.g, x, v);
+            V2<U> w = next(l0 + D.g, x, sample(r[pad<T>(at)], x));
             if (x & 1) w = mk<U>(-w.x, -w.y);
             q[pad<U>(at)] = w;
         }

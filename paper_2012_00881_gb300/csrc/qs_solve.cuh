@@ -1121,7 +1121,7 @@ __device__ bool direct_poisson(const EngineArgs &A, const Sync &S, const SolveSp
 // residual they start from; then u += e, r <- r - A e in float64 and again.
 // Float64 form: in pairs of floats to the tolerance (in float64 the two phases
 // of an iteration took 21 and 20 us at 256^2, bound by the FP64 pipe; pairs:
-// CGFF us); the same step then checks it.  Both stop on the float64 residual.
+// 11.7 and 10.9 us); the same step then checks it.  Both stop on the float64 residual.
 // The sums are of values scaled by a power of two near 1 / ||f||, so that
 // float32 cannot underflow in them.
 // prepared: the source's row transform and copy are in tr and cr already.
