@@ -12,7 +12,7 @@
 //             adjoint of a gather is a deposit), the gather weights' slope
 //             adds to the position cotangent
 //   B_perp    (lap - kappa) mu = dL/dB (the operator is symmetric, so the
-//             transposed solve is the same multigrid solve); then the source
+//             transposed solve is the same solve); then the source
 //             S of Eq. FluxCurr1_A backwards, kappa = n_*/(1+psi), j_z
 //   E_z, B_z  lap nu = dL/dE_z, dL/dB_z; then j_perp backwards through the
 //             central differences of Eqs. EqM_N8_A and Mag_z_A
@@ -24,8 +24,9 @@
 //
 // The sub-step schedule is that of the forward run and the 1+psi guard is
 // treated as inactive where it did not clamp (a clamped value has no
-// derivative).  All arithmetic is float64; the transposed solves use the
-// context's multigrid (refined form: float32 inner cycles, float64 residual).
+// derivative).  Cotangents are float64; the refined form's particle phases
+// evaluate theirs in pairs of floats.  The transposed solves are the forward
+// engine's (qs_solve.cuh).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -34,20 +35,70 @@
 
 namespace {
 
+// Arithmetic of the particle phases: float64, or in the refined form pairs of
+// floats (qs_ff.cuh), with float64 cotangents and sums.  In float64 the three
+// phases issue about 630 FP64-pipe instructions a particle (64 cycles a warp
+// each).  Forward and gradient of a 256^2 window in the refined form: 54.5 ms
+// with float64 particle phases, 47.2 with pairs.  The error of the gradient
+// against float64 is unchanged (median 3.3e-9, that of the forward state).
+using qsff::Ff;
+template <typename R>
+__device__ __forceinline__ R in(double v) {
+    if constexpr (sizeof(R) == 8 && std::is_same<R, double>::value) return v;
+    else return qsff::split(v);
+}
+__device__ __forceinline__ double out(double v) { return v; }
+__device__ __forceinline__ double out(Ff v) { return qsff::join(v); }
+__device__ __forceinline__ double rcp(double v) { return 1.0 / v; }
+__device__ __forceinline__ Ff rcp(Ff v) { return qsff::recip(v); }
+__device__ __forceinline__ bool below(double a, double b) { return a < b; }
+__device__ __forceinline__ bool below(Ff a, Ff b) { return a.h < b.h || (a.h == b.h && a.l < b.l); }
+
 // CIC with the per-axis weights kept, so that the slope of an interpolation
 // in x and y is available: for a gather v = sum_c w_c u_c,
 //   dv/dx = (1/h) (wy0 (u01 - u00) + wy1 (u11 - u10)),
 //   dv/dy = (1/h) (wx0 (u10 - u00) + wx1 (u11 - u01)).
+// Cells and fractions from the bits of s + 1/2 (qsff::axis_bits).
+template <typename R>
 struct CicD {
     int i00, i01, i10, i11;
-    double wx0, wx1, wy0, wy1;
+    R wx0, wx1, wy0, wy1;
+    double fx, fy;  // wx1, wy1 in float64
 };
 
-__device__ __forceinline__ CicD cic_d(double x, double y, const EngineArgs &A) {
+__device__ __forceinline__ void fold_cells(int right, int n, int &a, int &b) {
+    a = right - 1;
+    b = right;
+    if (a < 0) a = -1 - a;
+    if (b > n - 1) b = 2 * n - 1 - b;
+    a = min(max(a, 0), n - 1);
+    b = min(max(b, 0), n - 1);
+}
+
+template <typename R>
+__device__ __forceinline__ CicD<R> cic_d(double x, double y, const EngineArgs &A) {
+    const double tx = fma(x, A.inv_h, fma(-A.x_min, A.inv_h, 0.5));
+    const double ty = fma(y, A.inv_h, fma(-A.y_min, A.inv_h, 0.5));
+    const qsff::AxisBits bx = qsff::axis_bits(tx), by = qsff::axis_bits(ty);
     int ix0, ix1, iy0, iy1;
-    CicD c;
-    cic_axis((x - A.x_min) * A.inv_h, A.N, ix0, ix1, c.wx0, c.wx1);
-    cic_axis((y - A.y_min) * A.inv_h, A.N, iy0, iy1, c.wy0, c.wy1);
+    fold_cells(bx.cell, A.N, ix0, ix1);
+    fold_cells(by.cell, A.N, iy0, iy1);
+    CicD<R> c;
+    // 2^52 + 2^31 + cell is exact: a float64 of the cell without a conversion
+    const double bias = 4503599627370496.0 + 2147483648.0;
+    c.fx = tx - (__hiloint2double(0x43300000, bx.cell ^ 0x80000000) - bias);
+    c.fy = ty - (__hiloint2double(0x43300000, by.cell ^ 0x80000000) - bias);
+    if constexpr (std::is_same<R, double>::value) {
+        c.wx1 = c.fx;
+        c.wy1 = c.fy;
+        c.wx0 = 1.0 - c.fx;
+        c.wy0 = 1.0 - c.fy;
+    } else {
+        c.wx1 = bx.f;
+        c.wy1 = by.f;
+        c.wx0 = Ff(1.f, 0.f) - bx.f;
+        c.wy0 = Ff(1.f, 0.f) - by.f;
+    }
     const int n = A.N;
     c.i00 = iy0 * n + ix0;
     c.i01 = iy0 * n + ix1;
@@ -56,13 +107,16 @@ __device__ __forceinline__ CicD cic_d(double x, double y, const EngineArgs &A) {
     return c;
 }
 
+template <typename R>
 struct GatherD {
-    double v, dx, dy;  // value and slopes (slopes without the 1/h)
+    R v, dx, dy;  // value and slopes (slopes without the 1/h)
 };
 
-__device__ __forceinline__ GatherD gather_d(const double *u, const CicD &c) {
-    const double u00 = u[c.i00], u01 = u[c.i01], u10 = u[c.i10], u11 = u[c.i11];
-    GatherD g;
+template <typename R>
+__device__ __forceinline__ GatherD<R> gather_d(const double *u, const CicD<R> &c) {
+    const R u00 = in<R>(u[c.i00]), u01 = in<R>(u[c.i01]), u10 = in<R>(u[c.i10]),
+            u11 = in<R>(u[c.i11]);
+    GatherD<R> g;
     g.v = c.wy0 * (c.wx0 * u00 + c.wx1 * u01) + c.wy1 * (c.wx0 * u10 + c.wx1 * u11);
     g.dx = c.wy0 * (u01 - u00) + c.wy1 * (u11 - u10);
     g.dy = c.wx0 * (u10 - u00) + c.wx1 * (u11 - u01);
@@ -70,12 +124,15 @@ __device__ __forceinline__ GatherD gather_d(const double *u, const CicD &c) {
 }
 
 // deposit with the same weights (no 1/h^2): the adjoint of gather_d's value
-__device__ __forceinline__ void scatter(double *g, const CicD &c, double q) {
+template <typename R>
+__device__ __forceinline__ void scatter(double *g, const CicD<R> &c, R qr) {
+    const double q = out(qr);
     if (q == 0.0) return;
-    atomicAdd(g + c.i00, q * c.wy0 * c.wx0);
-    atomicAdd(g + c.i01, q * c.wy0 * c.wx1);
-    atomicAdd(g + c.i10, q * c.wy1 * c.wx0);
-    atomicAdd(g + c.i11, q * c.wy1 * c.wx1);
+    const double q1 = q * c.fy, q0 = q - q1, q01 = q0 * c.fx, q11 = q1 * c.fx;
+    atomicAdd(g + c.i00, q0 - q01);
+    atomicAdd(g + c.i01, q01);
+    atomicAdd(g + c.i10, q1 - q11);
+    atomicAdd(g + c.i11, q11);
 }
 
 // central differences: zero ghosts (moment grids) and the transpose of the
@@ -179,36 +236,39 @@ __device__ void adj_prepare(const EngineArgs &A, const AdjArgs &D, const Slice &
 // the Boris-like half kick / rotation / half kick and the drift; specular
 // walls).  On entry l* hold dL/dP_{s+1}; on exit the part of dL/dP_s that
 // flows through the push.  Field cotangents are scattered.
+template <typename R>
 __device__ void adj_push(const EngineArgs &A, const AdjArgs &D, const Slice &S, Thr T) {
-    const double dxi = A.dxi0 / S.m, half = 0.5 * dxi;
-    const double ih = A.inv_h;
+    const double dxi_d = A.dxi0 / S.m;
+    const R dxi = in<R>(dxi_d), half = in<R>(0.5 * dxi_d), ih = in<R>(A.inv_h);
+    const R one = R(1.f), two = R(2.f), hf = R(0.5f), floor_ = in<R>(A.psi_floor);
     for (int64_t p = T.t0; p < A.np; p += T.nt) {
-        const double x = S.x[p], y = S.y[p], px = S.px[p], py = S.py[p];
-        const CicD c = cic_d(x, y, A);
-        const GatherD Gp = gather_d(S.psi, c), Ggx = gather_d(A.dpx, c),
+        const double xd = S.x[p], yd = S.y[p];
+        const R px = in<R>(S.px[p]), py = in<R>(S.py[p]);
+        const CicD<R> c = cic_d<R>(xd, yd, A);
+        const GatherD<R> Gp = gather_d(S.psi, c), Ggx = gather_d(A.dpx, c),
                       Ggy = gather_d(A.dpy, c), Gbx = gather_d(S.bx, c),
                       Gby = gather_d(S.by, c), Gbz = gather_d(S.bz, c);
-        double a = 1.0 + Gp.v;
-        const bool act = a >= A.psi_floor;
-        if (!act) a = A.psi_floor;
-        const double ia = 1.0 / a, ia2 = ia * ia;  // one divide per particle
-        const double gx = Ggx.v, gy = Ggy.v, bx = Gbx.v, by = Gby.v, bz = Gbz.v;
+        R a = one + Gp.v;
+        const bool act = !below(a, floor_);
+        if (!act) a = floor_;
+        const R ia = rcp(a), ia2 = ia * ia;  // one reciprocal per particle
+        const R gx = Ggx.v, gy = Ggy.v, bx = Gbx.v, by = Gby.v, bz = Gbz.v;
         // forward
-        const double gam = (1.0 + px * px + py * py + a * a) * (0.5 * ia);
-        const double pxm = px + half * (gam * gx * ia - by);
-        const double pym = py + half * (gam * gy * ia + bx);
-        const double tau = half * bz * ia;
-        const double pxp = pxm - tau * pym;
-        const double pyp = pym + tau * pxm;
-        const double t2 = 1.0 + tau * tau;
-        const double sr = 2.0 * tau / t2;
-        const double pxr = pxm - sr * pyp;
-        const double pyr = pym + sr * pxp;
-        const double gam2 = (1.0 + pxr * pxr + pyr * pyr + a * a) * (0.5 * ia);
-        const double px2 = pxr + half * (gam2 * gx * ia - by);
-        const double py2 = pyr + half * (gam2 * gy * ia + bx);
-        const double nx0 = x + dxi * px2 * ia;
-        const double ny0 = y + dxi * py2 * ia;
+        const R gam = (one + px * px + py * py + a * a) * (hf * ia);
+        const R pxm = px + half * (gam * gx * ia - by);
+        const R pym = py + half * (gam * gy * ia + bx);
+        const R tau = half * bz * ia;
+        const R pxp = pxm - tau * pym;
+        const R pyp = pym + tau * pxm;
+        const R t2 = one + tau * tau;
+        const R it2 = rcp(t2), sr = two * tau * it2;
+        const R pxr = pxm - sr * pyp;
+        const R pyr = pym + sr * pxp;
+        const R gam2 = (one + pxr * pxr + pyr * pyr + a * a) * (hf * ia);
+        const R px2 = pxr + half * (gam2 * gx * ia - by);
+        const R py2 = pyr + half * (gam2 * gy * ia + bx);
+        const double nx0 = xd + out(dxi * px2 * ia);
+        const double ny0 = yd + out(dxi * py2 * ia);
         int fx = 0, fy = 0;  // reflections at the walls (each flips position and momentum)
         {
             double v = nx0;
@@ -220,16 +280,17 @@ __device__ void adj_push(const EngineArgs &A, const AdjArgs &D, const Slice &S, 
         }
         // reverse
         const double sx = (fx & 1) ? -1.0 : 1.0, sy = (fy & 1) ? -1.0 : 1.0;
-        const double l_nx = sx * D.lx[p], l_ny = sy * D.ly[p];
-        double l_px2 = sx * D.lpx[p], l_py2 = sy * D.lpy[p];
-        double l_x = l_nx, l_y = l_ny;
-        double ab = 0.0, gxb = 0.0, gyb = 0.0, bxb = 0.0, byb = 0.0, bzb = 0.0;
+        const R l_nx = in<R>(sx * D.lx[p]), l_ny = in<R>(sy * D.ly[p]);
+        R l_px2 = in<R>(sx * D.lpx[p]), l_py2 = in<R>(sy * D.lpy[p]);
+        R l_x = l_nx, l_y = l_ny;
+        const R zero = R(0.f);
+        R ab = zero, gxb = zero, gyb = zero, bxb = zero, byb = zero, bzb = zero;
         l_px2 += l_nx * dxi * ia;
         l_py2 += l_ny * dxi * ia;
         ab -= (l_nx * px2 + l_ny * py2) * dxi * ia2;
         // second half kick
-        double l_pxr = l_px2, l_pyr = l_py2;
-        double g2b = half * (l_px2 * gx + l_py2 * gy) * ia;
+        R l_pxr = l_px2, l_pyr = l_py2;
+        R g2b = half * (l_px2 * gx + l_py2 * gy) * ia;
         gxb += l_px2 * half * gam2 * ia;
         gyb += l_py2 * half * gam2 * ia;
         ab -= half * gam2 * (l_px2 * gx + l_py2 * gy) * ia2;
@@ -238,24 +299,24 @@ __device__ void adj_push(const EngineArgs &A, const AdjArgs &D, const Slice &S, 
         // gamma2
         l_pxr += g2b * pxr * ia;
         l_pyr += g2b * pyr * ia;
-        ab += g2b * (0.5 - (1.0 + pxr * pxr + pyr * pyr) * (0.5 * ia2));
+        ab += g2b * (hf - (one + pxr * pxr + pyr * pyr) * (hf * ia2));
         // rotation
-        double l_pxm = l_pxr, l_pym = l_pyr;
-        double srb = -l_pxr * pyp + l_pyr * pxp;
-        const double l_pyp = -l_pxr * sr;
-        const double l_pxp = l_pyr * sr;
+        R l_pxm = l_pxr, l_pym = l_pyr;
+        R srb = l_pyr * pxp - l_pxr * pyp;
+        const R l_pyp = -(l_pxr * sr);
+        const R l_pxp = l_pyr * sr;
         l_pxm += l_pxp;
-        double taub = -l_pxp * pym;
+        R taub = -(l_pxp * pym);
         l_pym -= l_pxp * tau;
         l_pym += l_pyp;
         taub += l_pyp * pxm;
         l_pxm += l_pyp * tau;
-        taub += srb * 2.0 * (1.0 - tau * tau) / (t2 * t2);
+        taub += srb * two * (one - tau * tau) * (it2 * it2);
         bzb += taub * half * ia;
         ab -= taub * tau * ia;
         // first half kick
-        double l_px = l_pxm, l_py = l_pym;
-        const double g1b = half * (l_pxm * gx + l_pym * gy) * ia;
+        R l_px = l_pxm, l_py = l_pym;
+        const R g1b = half * (l_pxm * gx + l_pym * gy) * ia;
         gxb += l_pxm * half * gam * ia;
         gyb += l_pym * half * gam * ia;
         ab -= half * gam * (l_pxm * gx + l_pym * gy) * ia2;
@@ -263,8 +324,8 @@ __device__ void adj_push(const EngineArgs &A, const AdjArgs &D, const Slice &S, 
         bxb += l_pym * half;
         l_px += g1b * px * ia;
         l_py += g1b * py * ia;
-        ab += g1b * (0.5 - (1.0 + px * px + py * py) * (0.5 * ia2));
-        if (!act) ab = 0.0;
+        ab += g1b * (hf - (one + px * px + py * py) * (hf * ia2));
+        if (!act) ab = zero;
         // gathers: slopes into the position cotangent, values scattered
         l_x += (ab * Gp.dx + gxb * Ggx.dx + gyb * Ggy.dx + bxb * Gbx.dx + byb * Gby.dx +
                 bzb * Gbz.dx) * ih;
@@ -276,10 +337,10 @@ __device__ void adj_push(const EngineArgs &A, const AdjArgs &D, const Slice &S, 
         scatter(D.g_bx, c, bxb);
         scatter(D.g_by, c, byb);
         scatter(D.g_bz, c, bzb);
-        D.lx[p] = l_x;
-        D.ly[p] = l_y;
-        D.lpx[p] = l_px;
-        D.lpy[p] = l_py;
+        D.lx[p] = out(l_x);
+        D.ly[p] = out(l_y);
+        D.lpx[p] = out(l_px);
+        D.lpy[p] = out(l_py);
     }
 }
 
@@ -389,38 +450,40 @@ __device__ void adj_jperp(const EngineArgs &A, const AdjArgs &D, Thr T) {
 // P5: reverse of the moment deposits (j = n_* <V>, T = n_* <V V>, G = n_*
 // <gamma>; deposits carry 1/h^2) through V = p/(1+psi_p) and gamma from the
 // constant of motion; 1 + psi_p is a gather of psi.
+template <typename R>
 __device__ void adj_moments(const EngineArgs &A, const AdjArgs &D, const Slice &S, Thr T) {
-    const double ih = A.inv_h, s2 = A.inv_h * A.inv_h;
+    const double s2d = A.inv_h * A.inv_h;
+    const R s2 = in<R>(s2d), ih = in<R>(A.inv_h), one = R(1.f), two = R(2.f), hf = R(0.5f);
+    const R floor_ = in<R>(A.psi_floor);
     for (int64_t p = T.t0; p < A.np; p += T.nt) {
-        const double px = S.px[p], py = S.py[p], w = A.w[p];
-        const CicD c = cic_d(S.x[p], S.y[p], A);
-        const GatherD Gp = gather_d(S.psi, c);
-        double a = 1.0 + Gp.v;
-        const bool act = a >= A.psi_floor;
-        if (!act) a = A.psi_floor;
-        const double ia = 1.0 / a, ia2 = ia * ia;
-        const double vx = px * ia, vy = py * ia;
-        const double gam = (1.0 + px * px + py * py + a * a) * (0.5 * ia);
-        const GatherD Gjx = gather_d(D.g_jx, c), Gjy = gather_d(D.g_jy, c),
-                      Gxx = gather_d(D.g_txx, c), Gxy = gather_d(D.g_txy, c),
-                      Gyy = gather_d(D.g_tyy, c), GG = gather_d(D.g_G, c);
-        // deposited values per unit weight
-        const double qjx = vx, qjy = vy, qxx = vx * vx, qxy = vx * vy, qyy = vy * vy, qG = gam;
-        D.lw[p] += (qjx * Gjx.v + qjy * Gjy.v + qxx * Gxx.v + qxy * Gxy.v + qyy * Gyy.v +
-                    qG * GG.v) * s2;
-        const double vxb = w * s2 * (Gjx.v + 2.0 * vx * Gxx.v + vy * Gxy.v);
-        const double vyb = w * s2 * (Gjy.v + vx * Gxy.v + 2.0 * vy * Gyy.v);
-        const double gb = w * s2 * GG.v;
-        double ab = -(vxb * px + vyb * py) * ia2 +
-                    gb * (0.5 - (1.0 + px * px + py * py) * (0.5 * ia2));
-        if (!act) ab = 0.0;
-        D.lpx[p] += vxb * ia + gb * px * ia;
-        D.lpy[p] += vyb * ia + gb * py * ia;
-        const double wq = w * s2 * ih;
-        D.lx[p] += wq * (qjx * Gjx.dx + qjy * Gjy.dx + qxx * Gxx.dx + qxy * Gxy.dx +
-                         qyy * Gyy.dx + qG * GG.dx) + ab * Gp.dx * ih;
-        D.ly[p] += wq * (qjx * Gjx.dy + qjy * Gjy.dy + qxx * Gxx.dy + qxy * Gxy.dy +
-                         qyy * Gyy.dy + qG * GG.dy) + ab * Gp.dy * ih;
+        const R px = in<R>(S.px[p]), py = in<R>(S.py[p]), w = in<R>(A.w[p]);
+        const CicD<R> c = cic_d<R>(S.x[p], S.y[p], A);
+        const GatherD<R> Gp = gather_d(S.psi, c);
+        R a = one + Gp.v;
+        const bool act = !below(a, floor_);
+        if (!act) a = floor_;
+        const R ia = rcp(a), ia2 = ia * ia;
+        const R vx = px * ia, vy = py * ia, p2 = one + px * px + py * py;
+        const R gam = (p2 + a * a) * (hf * ia);
+        const GatherD<R> Gjx = gather_d(D.g_jx, c), Gjy = gather_d(D.g_jy, c),
+                         Gxx = gather_d(D.g_txx, c), Gxy = gather_d(D.g_txy, c),
+                         Gyy = gather_d(D.g_tyy, c), GG = gather_d(D.g_G, c);
+        // deposited values per unit weight: vx, vy, vx^2, vx vy, vy^2, gamma
+        const R xx = vx * vx, xy = vx * vy, yy = vy * vy;
+        D.lw[p] += out((vx * Gjx.v + vy * Gjy.v + xx * Gxx.v + xy * Gxy.v + yy * Gyy.v +
+                        gam * GG.v) * s2);
+        const R ws = w * s2;
+        const R vxb = ws * (Gjx.v + two * vx * Gxx.v + vy * Gxy.v);
+        const R vyb = ws * (Gjy.v + vx * Gxy.v + two * vy * Gyy.v);
+        const R gb = ws * GG.v;
+        R ab = gb * (hf - p2 * (hf * ia2)) - (vxb * px + vyb * py) * ia2;
+        if (!act) ab = R(0.f);
+        D.lpx[p] += out((vxb + gb * px) * ia);
+        D.lpy[p] += out((vyb + gb * py) * ia);
+        D.lx[p] += out((ws * (vx * Gjx.dx + vy * Gjy.dx + xx * Gxx.dx + xy * Gxy.dx +
+                              yy * Gyy.dx + gam * GG.dx) + ab * Gp.dx) * ih);
+        D.ly[p] += out((ws * (vx * Gjx.dy + vy * Gjy.dy + xx * Gxx.dy + xy * Gxy.dy +
+                              yy * Gyy.dy + gam * GG.dy) + ab * Gp.dy) * ih);
         scatter(D.g_psi, c, ab);
     }
 }
@@ -443,16 +506,17 @@ __device__ void adj_psi_rhs(const EngineArgs &A, const AdjArgs &D, Thr T) {
 
 // P7: reverse of the n_* deposit (Eq. continuity; 1/h^2) with dL/dn_* =
 // g_n + nu_psi; n_ion's cotangent is -nu_psi.
+template <typename R>
 __device__ void adj_density(const EngineArgs &A, const AdjArgs &D, const Slice &S, Thr T) {
     const int nn = A.N * A.N;
-    const double ih = A.inv_h, s2 = A.inv_h * A.inv_h;
+    const R s2 = in<R>(A.inv_h * A.inv_h), ih = in<R>(A.inv_h);
     for (int64_t p = T.t0; p < A.np; p += T.nt) {
-        const CicD c = cic_d(S.x[p], S.y[p], A);
-        const GatherD g1 = gather_d(D.g_n, c), g2 = gather_d(D.nu_psi, c);
-        const double w = A.w[p];
-        D.lw[p] += (g1.v + g2.v) * s2;
-        D.lx[p] += w * s2 * ih * (g1.dx + g2.dx);
-        D.ly[p] += w * s2 * ih * (g1.dy + g2.dy);
+        const CicD<R> c = cic_d<R>(S.x[p], S.y[p], A);
+        const GatherD<R> g1 = gather_d(D.g_n, c), g2 = gather_d(D.nu_psi, c);
+        D.lw[p] += out((g1.v + g2.v) * s2);
+        const R k = in<R>(A.w[p]) * s2 * ih;
+        D.lx[p] += out(k * (g1.dx + g2.dx));
+        D.ly[p] += out(k * (g1.dy + g2.dy));
     }
     for (int i = T.t0; i < nn; i += T.nt) D.d_nion[i] -= D.nu_psi[i];
 }
@@ -460,6 +524,7 @@ __device__ void adj_density(const EngineArgs &A, const AdjArgs &D, const Slice &
 template <bool REF>
 __device__ bool run_adjoint(const EngineArgs &A, const AdjArgs &D, int bid, int nblk,
                             const Sync &S, void *smem, int *s_inv_ready) {
+    using R = typename std::conditional<REF, Ff, double>::type;
     DevScalars *sc = A.sc;
     const Thr T = grid_thr(bid, nblk);
     const bool lead = (bid == 0 && threadIdx.x == 0);
@@ -477,7 +542,7 @@ __device__ bool run_adjoint(const EngineArgs &A, const AdjArgs &D, int bid, int 
         adj_prepare(A, D, Sl, T);
         SYNC(101);
         if (!Sl.last) {
-            adj_push(A, D, Sl, T);
+            adj_push<R>(A, D, Sl, T);
             SYNC(102);
         }
         rhs_norms(A, 2, D.g_bx, D.g_by, T);
@@ -488,12 +553,12 @@ __device__ bool run_adjoint(const EngineArgs &A, const AdjArgs &D, int bid, int 
         if (!mg_solve<REF>(A, S, Veb, slot, bid, nblk, smem, s_inv_ready)) return false;
         adj_jperp(A, D, T);
         SYNC(105);
-        adj_moments(A, D, Sl, T);
+        adj_moments<R>(A, D, Sl, T);
         SYNC(106);
         adj_psi_rhs(A, D, T);
         SYNC(107);
         if (!mg_solve<REF>(A, S, Vpsi, slot, bid, nblk, smem, s_inv_ready)) return false;
-        adj_density(A, D, Sl, T);
+        adj_density<R>(A, D, Sl, T);
         if (lead) {
             sc->slices += 1;
             sc->fnorm[0][0] = sc->fnorm[0][1] = 0.0;
