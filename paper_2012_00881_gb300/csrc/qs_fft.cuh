@@ -562,7 +562,8 @@ __device__ __forceinline__ void rows_inverse_forward(const Lines &P, const Lines
 }
 
 // Sums of 16 values over the block: thread t < 16 returns the sum of v[t].  Each
-// shuffle halves the values a lane holds: 16 shuffles instead of 80.
+// shuffle halves the values a lane holds: 16 shuffles instead of 80.  A block
+// barrier stands between two calls.
 static __device__ float block_sums16(float v[16]) {
     __shared__ float red[32][17];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (int)blockDim.x >> 5;
@@ -583,7 +584,6 @@ static __device__ float block_sums16(float v[16]) {
     float t = 0.f;
     if (threadIdx.x < 16)
         for (int w = 0; w < nw; ++w) t += red[w][threadIdx.x];
-    __syncthreads();  // red is reused by the next call
     return t;
 }
 

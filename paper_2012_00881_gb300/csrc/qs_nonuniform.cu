@@ -923,6 +923,7 @@ __device__ __forceinline__ void column_solve(const NuArgs &A, int n, float mbar,
 // the slots two uses ahead.
 __device__ void nu_reduce(NuScalars *sc, float *v, int count, int use) {
     for (int b = 0; b < count; b += 16) {
+        if (b > 0) __syncthreads();  // the sums' memory
         const float t = qsfft::block_sums16(v + b);
         if (threadIdx.x < 16 && t != 0.f) atomicAdd(&sc->dots[use & 3][b + threadIdx.x], t);
     }

@@ -974,38 +974,55 @@ __device__ void reduce16(DevScalars *sc, float v[16], O *out, int slot, int bid)
     }
 }
 
-// Scalars of an iterative solve, one copy per block (thread 0, or thread c for
-// component c, writes them between block barriers).
+// Scalars of an iterative solve, one copy per block.  Lane c of the first warp
+// writes those of component c; block barriers stand between uses.  They stand
+// on every phase's critical path, and a float64 instruction takes 64 cycles
+// there: what only steers the iteration is float32 (a step size only has to be
+// the same for all vectors).  With the tests in float64 on one thread an
+// iteration at 64^2 took 17.2 us instead of 16.5, a slice of the refined form
+// at 256^2 219 instead of 213.
 struct IterScalars {
     float scale[2];           // powers of two near 1 / ||f|| (sums are of scaled values)
     double thr[2], r0[2];     // stopping bound, residual a round starts from (squared, scaled)
-    // of the last iteration: 1 / (r, z), 1 / alpha, step sizes; ||r||^2 after it,
-    // ||A p||^2 (scaled).  float32: a step size only has to be the same for all
-    // vectors, and a float64 division takes thread 0 a third of a microsecond.
-    float ig[2], ia[2], al[2], be[2], rr[2], ss[2];
-    double kbar;
+    float target[2], fs[2];   // ||r||^2 that ends a round; ||f||^2 (scaled)
+    // of the last iteration: 1 / (r, z), 1 / alpha, step sizes, ||A p||^2 (scaled)
+    float ig[2], ia[2], al[2], be[2], ss[2];
+    float kbar;
     int go;
 };
 
+// `red` times the residual a round starts from, or just below the bound
+__device__ __forceinline__ float round_target(double red, double r0, double thr) {
+    return fmaxf((float)fmax(red * r0, 0.09 * thr), 1e-37f);
+}
+
 // Source scales and stopping bounds; go: whether any component needs work.  A
 // NaN or infinite source keeps scale 1 and fails every stopping test.
-__device__ void iter_begin(const EngineArgs &A, const SolveSpec &V, IterScalars &I) {
+__device__ void iter_begin(const EngineArgs &A, const SolveSpec &V, IterScalars &I, double red) {
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int any = 0;
-        for (int c = 0; c < 2; ++c) {
+    if (threadIdx.x < 32) {
+        const int c = threadIdx.x;
+        bool work = false;
+        if (c < 2) {
             const double fn = c < V.nc ? vload(&A.sc->fnorm[V.kind][c]) : 0.0;
             const int ex = (int)((__double_as_longlong(fn) >> 52) & 0x7ff);
             const int k = ex == 0 || ex == 0x7ff ? 0 : (ex - 1023) / 2;
             const int kc = min(max(k, -120), 120);
             I.scale[c] = __int_as_float((127 - kc) << 23);
-            const double s2 = (double)I.scale[c] * (double)I.scale[c];
-            I.thr[c] = fmax(A.mg_tol * A.mg_tol * fn, A.mg_atol * A.mg_atol) * s2;
-            I.r0[c] = fn * s2;
-            if (!(I.r0[c] <= I.thr[c])) any = 1;
+            const double s2 = __longlong_as_double((long long)(1023 - 2 * kc) << 52);
+            const double thr = fmax(A.mg_tol * A.mg_tol * fn, A.mg_atol * A.mg_atol) * s2;
+            const double r0 = fn * s2;
+            I.thr[c] = thr;
+            I.r0[c] = r0;
+            I.target[c] = round_target(red, r0, thr);
+            I.fs[c] = (float)r0;
+            work = !(r0 <= thr);
         }
-        I.kbar = V.screened ? vload(&A.sc->ksum) / ((double)A.N * (double)A.N) : 0.0;
-        I.go = any;
+        const unsigned any = __ballot_sync(0xffffffffu, work);
+        if (c == 0) {
+            I.kbar = V.screened ? qsff::split(vload(&A.sc->ksum)).h / (float)(A.N * A.N) : 0.f;
+            I.go = any != 0;
+        }
     }
     __syncthreads();
 }
@@ -1013,27 +1030,29 @@ __device__ void iter_begin(const EngineArgs &A, const SolveSpec &V, IterScalars 
 // After u += e and the new residual's norms (rnorm[slot]): converged (1), too
 // slow or out of iterations (0), or another round (-2).
 __device__ int iter_check(const EngineArgs &A, const SolveSpec &V, IterScalars &I, int slot,
-                          int bid, bool last) {
+                          int bid, bool last, double red) {
     DevScalars *sc = A.sc;
-    if (threadIdx.x == 0) {
-        const double fl = 1e-13 * A.lev_inv_h2[0];
-        int conv = 1, slow = 0;
-        double rel = 0.0;
-        for (int c = 0; c < V.nc; ++c) {
+    if (threadIdx.x < 32) {
+        const int c = threadIdx.x;
+        bool open = false, slow = false;
+        float rel = 0.f;
+        if (c < V.nc) {
+            const double fl = 1e-13 * A.lev_inv_h2[0];
             const double rn = vload(&sc->rnorm[slot & 3][c]);
             const double un = vload(&sc->rnorm[slot & 3][2 + c]);
-            if (!(rn <= fmax(I.thr[c], fl * fl * un))) {
-                conv = 0;
-                if (!(rn <= 0.0625 * I.r0[c])) slow = 1;
-            }
+            open = !(rn <= fmax(I.thr[c], fl * fl * un));
+            slow = open && !(rn <= 0.0625 * I.r0[c]);
             I.r0[c] = rn;
-            if (bid == 0) {
-                const double fn = vload(&sc->fnorm[V.kind][c]);
-                if (fn > 0.0) rel = fmax(rel, sqrt(rn / fn) / (double)I.scale[c]);
-            }
+            I.target[c] = round_target(red, rn, I.thr[c]);
+            if (I.fs[c] > 0.f) rel = sqrtf((float)rn / I.fs[c]);
         }
-        if (bid == 0 && conv && rel > sc->max_relres) sc->max_relres = rel;
-        I.go = conv ? 1 : (slow || last) ? 0 : -2;
+        const unsigned nopen = __ballot_sync(0xffffffffu, open);
+        const unsigned nslow = __ballot_sync(0xffffffffu, slow);
+        rel = fmaxf(rel, __shfl_sync(0xffffffffu, rel, 1));
+        if (c == 0) {
+            if (bid == 0 && !nopen && (double)rel > sc->max_relres) sc->max_relres = (double)rel;
+            I.go = !nopen ? 1 : (nslow || last) ? 0 : -2;
+        }
     }
     __syncthreads();
     const int r = I.go;
@@ -1140,12 +1159,13 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
     C *const cz = (C *)A.fft.cz, *const cr = (C *)A.fft.cr, *const cp = (C *)A.fft.cp,
              *const cs = (C *)A.fft.cs, *const ce = (C *)A.fft.ce;
     __shared__ IterScalars I;
-    iter_begin(A, V, I);
+    const double red = REF ? 1e-10 : 1e-26;  // a round's reduction, squared
+    iter_begin(A, V, I, red);
     if (!I.go) {  // both sources are rounding noise or zero
         zero_solution(A, V, bid, nblk);
         return S(50) ? 1 : -1;
     }
-    const T kbar = narrow<T>(I.kbar);
+    const T kbar(I.kbar);
     const float sc0 = I.scale[0], sc1 = I.scale[1];
     auto dk = [&](size_t i) {  // kbar - kappa
         if constexpr (REF) return kbar - A.k32[i];
@@ -1161,7 +1181,6 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
         if (!S(51)) return -1;
     }
     const int cap = min(A.mg_max_vcycles, 48);
-    const double red = REF ? 1e-10 : 1e-26;  // a round's reduction, squared
     int it = 0, result = -2;
     for (int round = 0; result == -2; ++round) {
         float al0 = 0.f, al1 = 0.f, be0 = 0.f, be1 = 0.f;
@@ -1236,48 +1255,44 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
             });
             reduce16(sc, d, sc->cgd[slot & 3], slot, bid);
             if (!S(53)) return -1;
-            if (threadIdx.x < 2) {  // one thread a component
+            if (threadIdx.x < 32) {  // one lane a component
                 const int c = threadIdx.x;
-                const float *g = sc->cgd[slot & 3];
-                const float ga = vload(g + c), de = vload(g + 2 + c);
-                float be = 0.f, al = 0.f, ia = 0.f, ig = 0.f;
-                if (ga != 0.f) {
-                    ig = 1.f / ga;
-                    be = inner > 0 ? ga * I.ig[c] : 0.f;
-                    ia = de * ig - be * (inner > 0 ? I.ia[c] : 0.f);
-                    al = ia != 0.f ? 1.f / ia : 0.f;
+                bool open = false;
+                if (c < 2) {
+                    const float *g = sc->cgd[slot & 3];
+                    const float ga = vload(g + c), de = vload(g + 2 + c);
+                    const float rw = vload(g + 4 + c), rs = vload(g + 6 + c),
+                                ww = vload(g + 8 + c), ws = vload(g + 10 + c),
+                                rr = vload(g + 12 + c);
+                    float be = 0.f, al = 0.f, ia = 0.f, ig = 0.f;
+                    if (ga != 0.f) {
+                        ig = 1.f / ga;
+                        be = inner > 0 ? ga * I.ig[c] : 0.f;
+                        ia = de * ig - be * (inner > 0 ? I.ia[c] : 0.f);
+                        al = ia != 0.f ? 1.f / ia : 0.f;
+                    }
+                    I.ig[c] = ig;
+                    I.ia[c] = ia;
+                    I.al[c] = al;
+                    I.be[c] = be;
+                    // ||r - al s||^2 with s = w + be s_old.  The sums are good to
+                    // about 1e-7 of ||r||^2: no smaller value is believed.
+                    const float so = inner > 0 ? I.ss[c] : 0.f;
+                    const float ss = ww + be * (2.f * ws + be * so);
+                    I.ss[c] = ss;
+                    const float nr = rr - al * (2.f * (rw + be * rs) - al * ss);
+                    open = !((nr < 2e-7f * rr ? 2e-7f * rr : nr) <= I.target[c]);  // a NaN stays
                 }
-                I.ig[c] = ig;
-                I.ia[c] = ia;
-                I.al[c] = al;
-                I.be[c] = be;
-                // ||r - al s||^2 with s = w + be s_old.  The sums are good to
-                // about 1e-7 of ||r||^2: no smaller value is believed.
-                const float a = al, b = be;
-                const float rw = vload(g + 4 + c), rs = vload(g + 6 + c), ww = vload(g + 8 + c),
-                            ws = vload(g + 10 + c);
-                const float so = inner > 0 ? I.ss[c] : 0.f;
-                const float ss = ww + b * (2.f * ws + b * so);
-                const float rr = vload(g + 12 + c);
-                I.ss[c] = ss;
-                const float nr = rr - a * (2.f * (rw + b * rs) - a * ss);
-                I.rr[c] = nr < 2e-7f * rr ? 2e-7f * rr : nr;  // a NaN stays
+                const unsigned nopen = __ballot_sync(0xffffffffu, open);
+                if (c == 0) I.go = nopen != 0;
             }
             ++slot;
             __syncthreads();
-            if (threadIdx.x == 0) {
-                int go = 0;
-                for (int c = 0; c < 2; ++c)
-                    if (!((double)I.rr[c] <= fmax(red * I.r0[c], 0.09 * I.thr[c]))) go = 1;
-                I.go = go;
-            }
             al0 = I.al[0];
             al1 = I.al[1];
             be0 = I.be[0];
             be1 = I.be[1];
-            __syncthreads();
-            const bool go = I.go != 0;
-            __syncthreads();  // rewritten by the next test
+            const bool go = I.go != 0;  // rewritten two grid barriers on
             ++it;
             ++inner;
             if (!go || it >= cap || inner >= 24) break;
@@ -1336,7 +1351,7 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
         });
         reduce16(sc, n, A.sc->rnorm[slot & 3], slot, bid);
         if (!S(55)) return -1;
-        result = iter_check(A, V, I, slot, bid, it >= cap);
+        result = iter_check(A, V, I, slot, bid, it >= cap, red);
         ++slot;
     }
     if (bid == 0 && threadIdx.x == 0) sc->vcycles[V.kind] += it;
