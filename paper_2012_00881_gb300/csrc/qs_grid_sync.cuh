@@ -38,22 +38,24 @@ struct GridBarrier {
         __shared__ int s_ok;
         __syncthreads();
         if (threadIdx.x == 0) {
-            int ok = vload(&sc->err) == 0;
-            if (ok) {
-                const unsigned long long target = (*epoch + 1) * gridDim.x;
-                *epoch += 1;
-                release_add_u64(&sc->bar, 1ull);
-                const long long t0 = clock64();
-                while (acquire_u64(&sc->bar) < target) {
-                    if (vload(&sc->err) != 0) {
-                        ok = 0;
-                        break;
-                    }
-                    if (clock64() - t0 > limit) {
-                        if (atomicCAS(&sc->err, 0, QS_ERR_TIMEOUT) == 0) sc->err_where = where;
-                        ok = 0;
-                        break;
-                    }
+            int ok = 1;
+            const unsigned long long target = (*epoch + 1) * gridDim.x;
+            *epoch += 1;
+            release_add_u64(&sc->bar, 1ull);
+            const long long t0 = clock64();
+            // the error word beside the counter, never in the way of an arrival
+            // or of a poll: a block that gave up does not arrive
+            for (;;) {
+                const int err = vload(&sc->err);
+                if (acquire_u64(&sc->bar) >= target) break;
+                if (err != 0) {
+                    ok = 0;
+                    break;
+                }
+                if (clock64() - t0 > limit) {
+                    if (atomicCAS(&sc->err, 0, QS_ERR_TIMEOUT) == 0) sc->err_where = where;
+                    ok = 0;
+                    break;
                 }
             }
             s_ok = ok;
