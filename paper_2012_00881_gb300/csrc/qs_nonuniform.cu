@@ -47,12 +47,17 @@
 // products with n x n matrices.  GMRES on the residual equation in float32,
 // right-preconditioned with it (Saad and Schultz, SIAM J. Sci. Stat. Comput. 7
 // (1986) 856; the preconditioned vectors are kept, so it need not be exact),
-// to 3e-4 a round, which is what float32 second differences resolve; then
-// u += e and the float64 residual, which is also the stopping test.  The
-// third-order terms and the variation of M leave a perturbation that takes 7
-// iterations in all (M = 0) to 13 (a blowout's M) on the three-region grid
-// and up to 16 on alternating spacings, 20 us each at 255^2, against 12 V-cycles
-// of 180 us.  The V-cycles take over when that does not converge.
+// to 1e-5 a round; then u += e and the float64 residual, which is also the
+// stopping test.  The third-order terms and the variation of M leave a
+// perturbation that takes 7 iterations in all (M = 0) to 13 (a blowout's M) on
+// the three-region grid and up to 16 on alternating spacings, 21 us each for
+// one field at 255^2 and 29 for two, against 12 V-cycles of 180 us.  The
+// V-cycles take over when that does not converge.  An iteration is two grid
+// phases: columns, and rows with the operator, its dot products and the row
+// transform of A z, whose recurrence the column phase applies.  (With a phase
+// each for the rows, the operator, the new vector and its transform, and 3e-4 a
+// round with an update phase of its own, a 255^2 set of three solves took 1,380
+// us; so 1,180.)
 //
 // Every wait is bounded; a timeout sets an error word that ends the kernel at
 // the next barrier.
@@ -111,11 +116,11 @@ struct NuScalars {
     double fnorm[kMaxRhs];
     double relres[kMaxRhs];
     // direct-solve path: |f|^2, |r|^2 of a round (ring), sum of M, dot products
-    // (ring of 4 uses, 4 x kBasis)
+    // (ring of 4 uses, 16 a field)
     double dfnorm[kMaxRhs];
     double dnorm[3][kMaxRhs];
     double msum;
-    float dots[4][32];
+    float dots[4][16 * kMaxRhs];
 };
 
 constexpr int kBasis = 8;  // iterations a round
@@ -127,10 +132,11 @@ struct NuDirect {
     // the eigenbasis, vx[k][x] = Q[x][k] / sqrt(s_x) back; the same along y
     const float *wx, *vx, *wy, *vy;
     const float *lx, *ly;  // eigenvalues of D2
-    float *v;              // [kBasis + 1][nrhs][n n] basis (unnormalised)
+    float *v;              // [kBasis][nrhs][n n] basis (unnormalised)
     float *z;              // [kBasis][nrhs][n n] preconditioned basis
-    float *w;              // [nrhs][n n] A z of the current iteration
-    float *t1, *t2;        // [nrhs][n n] transforms
+    float *t;              // [kBasis][nrhs][n n] row transforms of the basis
+    float *w, *tw;         // [nrhs][n n] A z of the current iteration, its row transform
+    float *t2;             // [nrhs][n n] solved columns
 };
 
 struct NuArgs {
@@ -885,51 +891,6 @@ __device__ __forceinline__ void row_products(int n, int rows, const float *M, L 
     else row_products_g<8>(n, rows, M, load, store);
 }
 
-// Columns of all fields: t2 = Vy diag(1 / (ly + lx + mbar)) Wy t1, times
-// scale[field].
-template <int G>
-__device__ __forceinline__ void column_solve_g(const NuArgs &A, int n, float mbar,
-                                               const float *scale) {
-    const LineSmem S = line_smem(n);
-    const NuDirect &D = A.d;
-    const int groups = (n + G - 1) / G;
-    for (int u = blockIdx.x; u < groups * A.nrhs; u += gridDim.x) {
-        const int c = u / groups, k0 = (u - c * groups) * G, gl = min(G, n - k0);
-        const float *t1 = D.t1 + (size_t)c * n * n + k0;
-        float *t2 = D.t2 + (size_t)c * n * n + k0;
-        for (int q = threadIdx.x; q < G * n; q += blockDim.x) {
-            const int y = q / G, g = q - y * G;
-            S.in[q] = g < gl ? t1[(size_t)y * n + g] : 0.f;
-        }
-        __syncthreads();
-        const float sc = scale[c];
-        line_product<G>(S.in, S.part, D.wy, n, S.kq, [&](int g, int j, float v) {
-            S.mid[j * G + g] = g < gl ? v * sc / (D.ly[j] + D.lx[k0 + g] + mbar) : 0.f;
-        });
-        line_product<G>(S.mid, S.part, D.vy, n, S.kq, [&](int g, int y, float v) {
-            if (g < gl) t2[(size_t)y * n + g] = v;
-        });
-    }
-}
-__device__ __forceinline__ void column_solve(const NuArgs &A, int n, float mbar,
-                                             const float *scale) {
-    const int per = (n * A.nrhs + (int)gridDim.x - 1) / (int)gridDim.x;
-    if (per <= 2) column_solve_g<2>(A, n, mbar, scale);
-    else if (per <= 4) column_solve_g<4>(A, n, mbar, scale);
-    else column_solve_g<8>(A, n, mbar, scale);
-}
-
-// Adds the block's sums v[0 .. count) (count <= 32) to dots[use & 3] and clears
-// the slots two uses ahead.
-__device__ void nu_reduce(NuScalars *sc, float *v, int count, int use) {
-    for (int b = 0; b < count; b += 16) {
-        if (b > 0) __syncthreads();  // the sums' memory
-        const float t = qsfft::block_sums16(v + b);
-        if (threadIdx.x < 16 && t != 0.f) atomicAdd(&sc->dots[use & 3][b + threadIdx.x], t);
-    }
-    if (blockIdx.x == 0 && threadIdx.x < 32) sc->dots[(use + 2) & 3][threadIdx.x] = 0.f;
-}
-
 // Least squares of one field's round: Hessenberg columns reduced by Givens
 // rotations as they come.
 struct NuRound {
@@ -939,12 +900,206 @@ struct NuRound {
     float g[kMaxRhs][kBasis + 1];          // rotated right-hand side
     float y[kMaxRhs][kBasis];
     float coef[kMaxRhs][kBasis];           // (w, v_j) / |v_j|^2
-    float inv[kMaxRhs];                    // 1 / |v_k| of the next basis vector
+    float inv[kMaxRhs];                    // about 1 / |v_k| of the next basis vector
+    float pk[kMaxRhs], gk[kMaxRhs];        // the last column's rotation, to be redone
     double target[kMaxRhs], beta2[kMaxRhs];
     // powers of two near 1 / |J'| and their inverses: float32 vectors are scaled
     double scale[kMaxRhs], unscale[kMaxRhs];
     int go;
 };
+
+// Columns of all fields: t2 = Vy diag(1 / (ly + lx + mbar)) Wy t_k, times
+// inv[field].  t_k, the row transform of the next basis vector, follows from
+// those of w and of the earlier ones as the vector does.
+template <int G>
+__device__ __forceinline__ void column_solve_g(const NuArgs &A, const NuRound &R, int n, int k,
+                                               float mbar) {
+    const LineSmem S = line_smem(n);
+    const NuDirect &D = A.d;
+    const int groups = (n + G - 1) / G, nr = A.nrhs;
+    const size_t nn = (size_t)n * n;
+    for (int u = blockIdx.x; u < groups * nr; u += gridDim.x) {
+        const int c = u / groups, k0 = (u - c * groups) * G, gl = min(G, n - k0);
+        float *t2 = D.t2 + c * nn + k0;
+        for (int q = threadIdx.x; q < G * n; q += blockDim.x) {
+            const int y = q / G, g = q - y * G;
+            float t = 0.f;
+            if (g < gl) {
+                const size_t cp = c * nn + (size_t)y * n + k0 + g;
+                if (k == 0) {
+                    t = D.t[cp];
+                } else {
+                    t = D.tw[cp];
+                    for (int b = 0; b < k; ++b) t = fmaf(-R.coef[c][b], D.t[b * nr * nn + cp], t);
+                    D.t[k * nr * nn + cp] = t;
+                }
+            }
+            S.in[q] = t;
+        }
+        __syncthreads();
+        const float sc = R.inv[c];
+        line_product<G>(S.in, S.part, D.wy, n, S.kq, [&](int g, int j, float v) {
+            S.mid[j * G + g] = g < gl ? v * sc / (D.ly[j] + D.lx[k0 + g] + mbar) : 0.f;
+        });
+        line_product<G>(S.mid, S.part, D.vy, n, S.kq, [&](int g, int y, float v) {
+            if (g < gl) t2[(size_t)y * n + g] = v;
+        });
+    }
+}
+__device__ __forceinline__ void column_solve(const NuArgs &A, const NuRound &R, int n, int k,
+                                             float mbar) {
+    const int per = (n * A.nrhs + (int)gridDim.x - 1) / (int)gridDim.x;
+    if (per <= 2) column_solve_g<2>(A, R, n, k, mbar);
+    else if (per <= 4) column_solve_g<4>(A, R, n, k, mbar);
+    else column_solve_g<8>(A, R, n, k, mbar);
+}
+
+// Rows a block takes at a time: the fewest that leave no second turn.
+__device__ __forceinline__ int rows_owned(int n, int nr) {
+    if ((n + 1) / 2 * nr <= (int)gridDim.x) return 2;
+    return (n + 3) / 4 * nr <= (int)gridDim.x ? 4 : 6;
+}
+
+// Rows of iteration k: z = V t2 (own rows and one on each side, which the
+// stencil needs), the basis vector v_k = w - sum coef v, w = A z, its products
+// with the basis, |v_k|^2 and |w|^2, and the row transform of w.
+template <bool CORR, int OWN>
+__device__ __forceinline__ void apply_rows_g(const NuArgs &A, const NuRound &R, int n, int k,
+                                             int use) {
+    constexpr int G = OWN + 2;
+    const LineSmem S = line_smem(n);
+    const NuDirect &D = A.d;
+    const Level<float> &L = A.h32[0];
+    const int units = (n + OWN - 1) / OWN, nr = A.nrhs;
+    const size_t nn = (size_t)n * n;
+    for (int u = blockIdx.x; u < units * nr; u += gridDim.x) {
+        const int c = u / units, j0 = (u - c * units) * OWN, own = min(OWN, n - j0);
+        for (int q = threadIdx.x; q < G * n; q += blockDim.x) {
+            const int g = q / n, x = q - g * n, j = j0 - 1 + g;
+            S.in[x * G + g] = j >= 0 && j < n ? D.t2[c * nn + (size_t)j * n + x] : 0.f;
+        }
+        __syncthreads();
+        line_product<G>(S.in, S.part, D.vx, n, S.kq, [&](int g, int x, float v) {
+            S.mid[x * G + g] = v;
+            if (g >= 1 && g <= own)
+                D.z[(k * nr + c) * nn + (size_t)(j0 + g - 1) * n + x] = v;
+        });
+        float d[16] = {0.f};
+        for (int q = threadIdx.x; q < OWN * n; q += blockDim.x) {
+            const int g = q / n, x = q - g * n, j = j0 + g;
+            float w = 0.f;
+            if (g < own) {
+                const size_t cp = c * nn + (size_t)j * n + x;
+                float mrow[3], mcol[3], m0, v[3][3];
+                load_m(A.has_m ? L.m : nullptr, n, x, j, mrow, mcol, m0);
+#pragma unroll
+                for (int b = 0; b < 3; ++b)
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) {
+                        const int xx = x + a - 1;
+                        v[b][a] = xx >= 0 && xx < n ? S.mid[xx * G + g + b] : 0.f;
+                    }
+                w = apply_point<CORR>(L.ax[x], L.ay[j], v, mrow, mcol, m0);
+                float vk = k == 0 ? D.v[cp] : D.w[cp];
+#pragma unroll
+                for (int b = 0; b < kBasis; ++b)
+                    if (b < k) {
+                        const float vb = D.v[b * nr * nn + cp];
+                        vk = fmaf(-R.coef[c][b], vb, vk);
+                        d[b] += w * vb;
+                    }
+                if (k > 0) D.v[k * nr * nn + cp] = vk;
+                D.w[cp] = w;
+#pragma unroll
+                for (int b = 0; b < kBasis; ++b)
+                    if (b == k) d[b] += w * vk;
+                d[kBasis] += vk * vk;
+                d[kBasis + 1] += w * w;
+            }
+            S.in[x * OWN + g] = w;
+        }
+        const float t = qsfft::block_sums16(d);
+        if (threadIdx.x < kBasis + 2 && t != 0.f)
+            atomicAdd(&A.sc->dots[use & 3][16 * c + threadIdx.x], t);
+        line_product<OWN>(S.in, S.part, D.wx, n, S.kq, [&](int g, int q, float v) {
+            if (g < own) D.tw[c * nn + (size_t)(j0 + g) * n + q] = v;
+        });
+    }
+    if (blockIdx.x == 0 && threadIdx.x < 16 * kMaxRhs)
+        A.sc->dots[(use + 2) & 3][threadIdx.x] = 0.f;
+}
+template <bool CORR>
+__device__ __forceinline__ void apply_rows(const NuArgs &A, const NuRound &R, int n, int k,
+                                           int use) {
+    const int own = rows_owned(n, A.nrhs);
+    if (own == 2) apply_rows_g<CORR, 2>(A, R, n, k, use);
+    else if (own == 4) apply_rows_g<CORR, 4>(A, R, n, k, use);
+    else apply_rows_g<CORR, 6>(A, R, n, k, use);
+}
+
+// The end of a round: u += e, r <- r - A e in float64 with e = sum y z, |r|^2
+// into rn, and the first basis vector of the next round with its row transform.
+template <bool CORR, int OWN>
+__device__ __forceinline__ void round_rows_g(const NuArgs &A, const NuRound &R, int n, int its,
+                                             double *rn) {
+    constexpr int G = OWN + 2;
+    const LineSmem S = line_smem(n);
+    const NuDirect &D = A.d;
+    const Level<double> &top = A.top;
+    const int units = (n + OWN - 1) / OWN, nr = A.nrhs;
+    const size_t nn = (size_t)n * n;
+    for (int u = blockIdx.x; u < units * nr; u += gridDim.x) {
+        const int c = u / units, j0 = (u - c * units) * OWN, own = min(OWN, n - j0);
+        for (int q = threadIdx.x; q < G * n; q += blockDim.x) {
+            const int g = q / n, x = q - g * n, j = j0 - 1 + g;
+            float e = 0.f;
+            if (j >= 0 && j < n)
+                for (int b = 0; b < its; ++b)
+                    e = fmaf(R.y[c][b], D.z[(b * nr + c) * nn + (size_t)j * n + x], e);
+            S.mid[x * G + g] = e;
+        }
+        __syncthreads();
+        const double us = R.unscale[c], sc = R.scale[c];
+        for (int q = threadIdx.x; q < OWN * n; q += blockDim.x) {
+            const int g = q / n, x = q - g * n, j = j0 + g;
+            float rf = 0.f;
+            if (g < own) {
+                const size_t cp = c * nn + (size_t)j * n + x;
+                double mrow[3], mcol[3], m0, v[3][3];
+                load_m(A.m_in, n, x, j, mrow, mcol, m0);
+#pragma unroll
+                for (int b = 0; b < 3; ++b)
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) {
+                        const int xx = x + a - 1;
+                        v[b][a] = xx >= 0 && xx < n ? qsff::widen(S.mid[xx * G + g + b]) : 0.0;
+                    }
+                top.u[cp] += v[1][1] * us;
+                const double r =
+                    top.f[cp] - us * apply_point<CORR>(top.ax[x], top.ay[j], v, mrow, mcol, m0);
+                top.f[cp] = r;
+#pragma unroll
+                for (int cc = 0; cc < kMaxRhs; ++cc)
+                    if (cc == c) rn[cc] += r * r;
+                rf = (float)(r * sc);
+                D.v[cp] = rf;
+            }
+            S.in[x * OWN + g] = rf;
+        }
+        __syncthreads();
+        line_product<OWN>(S.in, S.part, D.wx, n, S.kq, [&](int g, int q, float v) {
+            if (g < own) D.t[c * nn + (size_t)(j0 + g) * n + q] = v;
+        });
+    }
+}
+template <bool CORR>
+__device__ __forceinline__ void round_rows(const NuArgs &A, const NuRound &R, int n, int its,
+                                           double *rn) {
+    const int own = rows_owned(n, A.nrhs);
+    if (own == 2) round_rows_g<CORR, 2>(A, R, n, its, rn);
+    else if (own == 4) round_rows_g<CORR, 4>(A, R, n, its, rn);
+    else round_rows_g<CORR, 6>(A, R, n, its, rn);
+}
 
 // 1: converged, 0: not (u holds the last iterate), -1: a barrier failed.
 template <bool CORR>
@@ -987,25 +1142,26 @@ __device__ int nu_direct(const NuArgs &A, const GridBarrier &gsync, int &its) {
     }
     __syncthreads();
     const float mbar = A.has_m ? (float)(vload(&sc->msum) / (double)nn) : 0.f;
-    for (int round = 0;; ++round) {
-        double rn[kMaxRhs] = {0, 0, 0, 0};  // float64 residual
-        row_products(n, rows, D.wx,
-                     [&](int row, int i) {
-                         const int c = row / n, j = row - c * n;
-                         const size_t cp = (size_t)c * nn + (size_t)j * n + i;
-                         double mrow[3], mcol[3], m0, v[3][3];
-                         load_m(A.m_in, n, i, j, mrow, mcol, m0);
-                         load_v(top.u + (size_t)c * nn, n, i, j, v);
-                         const double r = top.f[cp] - apply_point<CORR>(top.ax[i], top.ay[j], v,
-                                                                        mrow, mcol, m0);
+    double rn[kMaxRhs] = {0, 0, 0, 0};  // float64 residual, kept in J's memory
+    row_products(n, rows, D.wx,
+                 [&](int row, int i) {
+                     const int c = row / n, j = row - c * n;
+                     const size_t cp = (size_t)c * nn + (size_t)j * n + i;
+                     double mrow[3], mcol[3], m0, v[3][3];
+                     load_m(A.m_in, n, i, j, mrow, mcol, m0);
+                     load_v(top.u + (size_t)c * nn, n, i, j, v);
+                     const double r = top.f[cp] - apply_point<CORR>(top.ax[i], top.ay[j], v, mrow,
+                                                                    mcol, m0);
+                     top.f[cp] = r;
 #pragma unroll
-                         for (int cc = 0; cc < kMaxRhs; ++cc)
-                             if (cc == c) rn[cc] += r * r;
-                         const float rf = (float)(r * R.scale[c]);
-                         D.v[cp] = rf;
-                         return rf;
-                     },
-                     [&](int row, int k, float v) { D.t1[(size_t)row * n + k] = v; });
+                     for (int cc = 0; cc < kMaxRhs; ++cc)
+                         if (cc == c) rn[cc] += r * r;
+                     const float rf = (float)(r * R.scale[c]);
+                     D.v[cp] = rf;
+                     return rf;
+                 },
+                 [&](int row, int k, float v) { D.t[(size_t)row * n + k] = v; });
+    for (int round = 0;; ++round) {
         if (blockIdx.x == 0 && threadIdx.x < kMaxRhs) sc->dnorm[(round + 1) % 3][threadIdx.x] = 0.0;
         qsync::block_sum_add<kThreads>(rn, nr, sc->dnorm[round % 3]);
         if (!gsync(20)) return -1;
@@ -1020,7 +1176,7 @@ __device__ int nu_direct(const NuArgs &A, const GridBarrier &gsync, int &its) {
                 }
                 R.beta2[c] = r2;
                 const double s2 = R.scale[c] * R.scale[c];
-                R.target[c] = fmax(9e-8 * r2, 0.09 * thr) * s2;
+                R.target[c] = fmax(1e-10 * r2, 0.09 * thr) * s2;
                 const float b = f2 > 0.0 && r2 > thr ? (float)sqrt(r2 * s2) : 0.f;
                 R.nu[c][0] = R.g[c][0] = b;
                 R.inv[c] = b > 0.f ? 1.f / b : 0.f;
@@ -1043,79 +1199,48 @@ __device__ int nu_direct(const NuArgs &A, const GridBarrier &gsync, int &its) {
         }
         int k = 0;
         for (;;) {
-            column_solve(A, n, mbar, R.inv);
+            column_solve(A, R, n, k, mbar);
             if (!gsync(21)) return -1;
-            row_products(n, rows, D.vx,
-                         [&](int row, int q) { return D.t2[(size_t)row * n + q]; },
-                         [&](int row, int x, float v) {
-                             D.z[(size_t)k * nr * nn + (size_t)row * n + x] = v;
-                         });
+            apply_rows<CORR>(A, R, n, k, use);
             if (!gsync(22)) return -1;
-            // w = A z and its products with the basis
-            float d[32] = {0.f};
-            for (int p = grid.t; p < nn; p += grid.nt) {
-                const int j = p / n, i = p - j * n;
-                float mrow[3], mcol[3], m0;
-                load_m(A.has_m ? L.m : nullptr, n, i, j, mrow, mcol, m0);
-                for (int c = 0; c < nr; ++c) {
-                    float v[3][3];
-                    load_v(D.z + ((size_t)k * nr + c) * nn, n, i, j, v);
-                    const float w = apply_point<CORR>(L.ax[i], L.ay[j], v, mrow, mcol, m0);
-                    D.w[(size_t)c * nn + p] = w;
-#pragma unroll
-                    for (int b = 0; b < kBasis; ++b)
-                        if (b <= k) {
-                            const float t = w * D.v[((size_t)b * nr + c) * nn + p];
-#pragma unroll
-                            for (int cc = 0; cc < kMaxRhs; ++cc)
-                                if (cc == c) d[cc * kBasis + b] += t;
-                        }
-                }
-            }
-            nu_reduce(sc, d, nr * kBasis, use);
-            if (!gsync(23)) return -1;
             if (threadIdx.x < nr) {
                 const int c = threadIdx.x;
-                for (int b = 0; b <= k; ++b) {
-                    const float dot = vload(&sc->dots[use & 3][c * kBasis + b]), nu = R.nu[c][b];
-                    R.h[c][b][k] = nu > 0.f ? dot / nu : 0.f;
-                    R.coef[c][b] = nu > 0.f ? dot / (nu * nu) : 0.f;
-                }
-            }
-            ++use;
-            __syncthreads();
-            // the next basis vector, its norm and its row transform
-            float nv[16] = {0.f};
-            row_products(n, rows, D.wx,
-                         [&](int row, int x) {
-                             const int c = row / n;
-                             const size_t cp = (size_t)row * n + x;
-                             float w = D.w[cp];
-                             for (int b = 0; b <= k; ++b)
-                                 w = fmaf(-R.coef[c][b], D.v[(size_t)b * nr * nn + cp], w);
-                             D.v[(size_t)(k + 1) * nr * nn + cp] = w;
+                const float *g = &sc->dots[use & 3][16 * c];
+                float d[kBasis];
 #pragma unroll
-                             for (int cc = 0; cc < kMaxRhs; ++cc)
-                                 if (cc == c) nv[cc] += w * w;
-                             return w;
-                         },
-                         [&](int row, int q, float v) { D.t1[(size_t)row * n + q] = v; });
-            nu_reduce(sc, nv, 16, use);
-            if (!gsync(24)) return -1;
-            if (threadIdx.x < nr) {
-                const int c = threadIdx.x;
-                const float nu = sqrtf(vload(&sc->dots[use & 3][c]));
-                R.nu[c][k + 1] = nu;
-                R.inv[c] = nu > 0.f ? 1.f / nu : 0.f;
+                for (int b = 0; b < kBasis; ++b) d[b] = vload(g + b);
+                const float vv = vload(g + kBasis), ww = vload(g + kBasis + 1);
+                if (k > 0) {  // the rotation of the last column with |v_k| as it came out
+                    const float nu = sqrtf(vv), p = R.pk[c], r = sqrtf(p * p + nu * nu);
+                    const float cs = r > 0.f ? p / r : 1.f, sn = r > 0.f ? nu / r : 0.f;
+                    R.nu[c][k] = nu;
+                    R.cs[c][k - 1] = cs;
+                    R.sn[c][k - 1] = sn;
+                    R.h[c][k - 1][k - 1] = r;
+                    R.g[c][k] = -sn * R.gk[c];
+                    R.g[c][k - 1] = cs * R.gk[c];
+                }
+                float rest = ww;
+#pragma unroll
+                for (int b = 0; b < kBasis; ++b)
+                    if (b <= k) {
+                        const float nu = R.nu[c][b], h = nu > 0.f ? d[b] / nu : 0.f;
+                        R.h[c][b][k] = h;
+                        R.coef[c][b] = nu > 0.f ? h / nu : 0.f;
+                        rest -= h * h;
+                    }
                 for (int b = 0; b < k; ++b) {  // earlier rotations on the new column
                     const float p = R.h[c][b][k], q = R.h[c][b + 1][k];
                     R.h[c][b][k] = R.cs[c][b] * p + R.sn[c][b] * q;
                     R.h[c][b + 1][k] = R.cs[c][b] * q - R.sn[c][b] * p;
                 }
+                // |v_{k+1}| by Pythagoras until its sum is there: good to 1e-7 |w|
+                const float nu = sqrtf(rest < 1e-7f * ww ? 1e-7f * ww : rest);
                 const float p = R.h[c][k][k], r = sqrtf(p * p + nu * nu);
                 const float cs = r > 0.f ? p / r : 1.f, sn = r > 0.f ? nu / r : 0.f;
-                R.cs[c][k] = cs;
-                R.sn[c][k] = sn;
+                R.inv[c] = nu > 0.f ? 1.f / nu : 0.f;
+                R.pk[c] = p;
+                R.gk[c] = R.g[c][k];
                 R.h[c][k][k] = r;
                 R.g[c][k + 1] = -sn * R.g[c][k];
                 R.g[c][k] *= cs;
@@ -1146,14 +1271,8 @@ __device__ int nu_direct(const NuArgs &A, const GridBarrier &gsync, int &its) {
             }
         }
         __syncthreads();
-        for (int p = grid.t; p < nn; p += grid.nt)
-            for (int c = 0; c < nr; ++c) {
-                float e = 0.f;
-                for (int b = 0; b < k; ++b)
-                    e = fmaf(R.y[c][b], D.z[((size_t)b * nr + c) * nn + p], e);
-                top.u[(size_t)c * nn + p] += (double)e * R.unscale[c];
-            }
-        if (!gsync(25)) return -1;
+        for (int c = 0; c < kMaxRhs; ++c) rn[c] = 0.0;
+        round_rows<CORR>(A, R, n, k, rn);
     }
 }
 
@@ -1492,13 +1611,13 @@ bool tridiagonal_values(std::vector<double> d, std::vector<double> e, std::vecto
             if (m == l) break;
             if (it == 60) return false;
             double g = (d[l + 1] - d[l]) / (2.0 * e[l]);
-            double r = std::hypot(g, 1.0);
+            double r = std::sqrt(g * g + 1.0);
             g = d[m] - d[l] + e[l] / (g + (g >= 0.0 ? r : -r));
             double s = 1.0, c = 1.0, p = 0.0;
             int i = m - 1;
             for (; i >= l; --i) {
                 const double f = s * e[i], b = c * e[i];
-                r = std::hypot(f, g);
+                r = std::sqrt(f * f + g * g);
                 e[i + 1] = r;
                 if (r == 0.0) {
                     d[i + 1] -= p;
@@ -1563,7 +1682,7 @@ void tridiagonal_vector(const std::vector<double> &d, const std::vector<double> 
     b[n - 1] = c[n - 1] = 0.0;
     // a start with no special symmetry, another for each vector
     for (int i = 0; i < n; ++i) x[i] = 1.0 + 0.37 * ((i * 7919 + k * 104729) % 101) / 101.0;
-    for (int it = 0; it < 3; ++it) {
+    for (int it = 0; it < 2; ++it) {
         for (int i = 0; i < n - 1; ++i) {
             if (swapped[i]) std::swap(x[i], x[i + 1]);
             x[i + 1] -= lo[i] * x[i];
@@ -1579,12 +1698,9 @@ void tridiagonal_vector(const std::vector<double> &d, const std::vector<double> 
         for (int i = 0; i < n; ++i) x[i] /= s;
         for (int j = first; j < k; ++j) {
             const double *y = q_all.data() + (size_t)j * n;
-            double t = 0.0, own = 0.0;
-            for (int i = 0; i < n; ++i) {
-                t += x[i] * y[i];
-                own += y[i] * y[i];
-            }
-            for (int i = 0; i < n; ++i) x[i] -= t / own * y[i];
+            double t = 0.0;
+            for (int i = 0; i < n; ++i) t += x[i] * y[i];
+            for (int i = 0; i < n; ++i) x[i] -= t * y[i];
         }
         double l2 = 0.0;
         for (int i = 0; i < n; ++i) l2 += x[i] * x[i];
@@ -1635,7 +1751,7 @@ void create_direct(qs_nu_solver *s, const std::vector<double> &x, const std::vec
     if (!same && !axis_basis(y, wy, vy, ly)) return;
     const size_t nn = (size_t)n * n, ld = padded(n),
                  mats = (same ? 1 : 2) * (2 * n * ld + ld);
-    const size_t vecs = (2 * kBasis + 4) * kMaxRhs * nn;
+    const size_t vecs = (3 * kBasis + 3) * kMaxRhs * nn;
     if (cudaMalloc(&s->direct, (mats + vecs) * sizeof(float)) != cudaSuccess) {
         cudaGetLastError();
         s->direct = nullptr;
@@ -1658,12 +1774,14 @@ void create_direct(qs_nu_solver *s, const std::vector<double> &x, const std::vec
     D.ly = same ? D.lx : put(ly);
     float *p = base + mats;
     D.v = p;
-    p += (kBasis + 1) * kMaxRhs * nn;
+    p += kBasis * kMaxRhs * nn;
     D.z = p;
+    p += kBasis * kMaxRhs * nn;
+    D.t = p;
     p += kBasis * kMaxRhs * nn;
     D.w = p;
     p += kMaxRhs * nn;
-    D.t1 = p;
+    D.tw = p;
     p += kMaxRhs * nn;
     D.t2 = p;
     if (cudaMemcpyAsync(base, host.data(), host.size() * sizeof(float), cudaMemcpyHostToDevice,
