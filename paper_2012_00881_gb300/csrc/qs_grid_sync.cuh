@@ -89,23 +89,25 @@ __device__ __forceinline__ Team spread_team() {
                 (int)(gridDim.x * blockDim.x)};
 }
 
-// Adds the block's sums of vals[0 .. k) into dst[0 .. k) (one atomic each).
+// Adds the block's sums of vals[0 .. k) into dst[0 .. k), k <= 4 (one atomic
+// each).  A float64 add takes its scheduler 64 cycles: warp c adds the warps'
+// sums of value c in a tree (one thread adding 16 of them took 0.6 us a value).
 template <int kThreadsMax>
 __device__ void block_sum_add(const double *vals, int k, double *dst) {
-    __shared__ double red[kThreadsMax / 32][4];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    __shared__ double red[4][kThreadsMax / 32];
+    static_assert(kThreadsMax <= 1024, "one warp adds the warps' sums");
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (int)blockDim.x / 32;
     for (int c = 0; c < k; ++c) {
         double v = vals[c];
         for (int o = 16; o; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) red[wid][c] = v;
+        if (lane == 0) red[c][wid] = v;
     }
     __syncthreads();
-    if (threadIdx.x == 0)
-        for (int c = 0; c < k; ++c) {
-            double s = 0.0;
-            for (int w = 0; w < (int)(blockDim.x / 32); ++w) s += red[w][c];
-            atomicAdd(&dst[c], s);
-        }
+    for (int c = wid; c < k; c += nw) {
+        double s = lane < nw ? red[c][lane] : 0.0;
+        for (int o = kThreadsMax / 64; o; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (lane == 0) atomicAdd(&dst[c], s);
+    }
     __syncthreads();
 }
 

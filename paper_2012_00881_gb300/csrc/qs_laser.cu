@@ -571,7 +571,7 @@ __device__ int slice_direct(const LzArgs &A, const qsync::GridBarrier<LzScalars>
     const double2 *aj = A.a + (size_t)j * nn;
     const double *chij = A.chi + (size_t)j * nn;
     __shared__ float2 s_al, s_be, s_ig, s_ia;
-    __shared__ float s_ss;
+    __shared__ float s_ss, s_target;  // (scaled) |A p|^2; |r|^2 that ends a round
     __shared__ double s_r0, s_thr;
     __shared__ int s_go;
     its = 0;
@@ -633,6 +633,11 @@ __device__ int slice_direct(const LzArgs &A, const qsync::GridBarrier<LzScalars>
         return gsync(2) ? 1 : -1;
     }
     const int cap = min(4 * A.max_cycles, 48);
+    // float32 for the test on the path of every iteration, set once a round
+    auto set_target = [&] {
+        s_target = fmaxf((float)(fmax(1e-24 * s_r0, 0.09 * s_thr) * scale2), 1e-37f);
+    };
+    if (threadIdx.x == 0) set_target();
     for (int round = 0;; ++round) {
         float2 al = make_float2(0.f, 0.f), be = al;
         int inner = 0;
@@ -723,14 +728,13 @@ __device__ int slice_direct(const LzArgs &A, const qsync::GridBarrier<LzScalars>
                 float nr = rr - 2.f * ars.x + (a.x * a.x + a.y * a.y) * ss;
                 nr = nr < 2e-7f * rr ? 2e-7f * rr : nr;
                 s_ss = ss;
-                s_go = !((double)nr <= fmax(1e-24 * s_r0, 0.09 * s_thr) * scale2);
+                s_go = !(nr <= s_target);
             }
             ++use;
             __syncthreads();
             al = s_al;
             be = s_be;
-            const bool go = s_go != 0;
-            __syncthreads();  // rewritten by the next test
+            const bool go = s_go != 0;  // rewritten two grid barriers on
             ++its;
             ++inner;
             if (!go || its >= cap || inner >= 24) break;
@@ -772,6 +776,7 @@ __device__ int slice_direct(const LzArgs &A, const qsync::GridBarrier<LzScalars>
             const bool slow = !(r2 <= 0.0625 * s_r0);
             s_go = r2 <= s_thr ? 1 : (slow || its >= cap) ? 0 : 2;
             s_r0 = r2;
+            set_target();
             relres = f2 > 0.0 ? sqrt(r2 / f2) : 0.0;
         }
         ++kglob;
