@@ -81,18 +81,46 @@ __device__ __forceinline__ void dep(P *g, const CicP<P> &c, P q) {
     atomicAdd(g + c.i11, q * c.w11);
 }
 
-// Six float32 moments q of a particle into one cell with weight w: two vector
-// reductions of the cell's sector instead of six scalar ones.  The moments
-// phase is bound by them (512^2, nine particles a cell: 247 us with 57 M scalar
-// ones and float64 arithmetic, 121 us with 19 M vector ones and pairs).
-__device__ __forceinline__ void dep6(float4 *m, int i, float w, const float (&q)[6]) {
-    float4 *a = m + 2 * (size_t)i;
-    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(a), "f"(q[0] * w),
-                 "f"(q[1] * w), "f"(q[2] * w), "f"(q[3] * w)
-                 : "memory");
-    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(a + 1), "f"(q[4] * w),
-                 "f"(q[5] * w)
-                 : "memory");
+// Six float32 moments of a lane's particle, times the weights, to its four
+// cells of the interleaved grid (two float4 a cell: six moments and two zeros).
+// A pair of lanes does the even lane's particle and then the odd one's, the even
+// lane the first float4 of every cell and the odd lane the second: a request
+// then covers whole 32-byte sectors, half as many of them, which is what the
+// reductions are bound by.  The moments phase at 512^2, nine particles a cell:
+// 97 us, with each lane on its own particle 120, with six scalar reductions and
+// float64 arithmetic 247; at 256^2, four a cell: 14.0 and 18.6.  All 32 lanes call.
+__device__ __forceinline__ void dep6_pairs(float4 *g, const CicP<float> &c, const float q[6]) {
+    const bool odd = (threadIdx.x & 1) != 0;
+    const float own[4] = {odd ? q[4] : q[0], odd ? q[5] : q[1], odd ? 0.f : q[2],
+                          odd ? 0.f : q[3]};
+    auto swap = [](auto v) { return __shfl_xor_sync(0xffffffffu, v, 1); };
+    const float got[4] = {swap(odd ? q[0] : q[4]), swap(odd ? q[1] : q[5]),
+                          swap(odd ? q[2] : 0.f), swap(odd ? q[3] : 0.f)};
+    const int i[4] = {c.i00, c.i01, c.i10, c.i11};
+    const float w[4] = {c.w00, c.w01, c.w10, c.w11};
+    int j[4];
+    float v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        j[k] = swap(i[k]);
+        v[k] = swap(w[k]);
+    }
+    g += odd;
+#pragma unroll
+    for (int turn = 0; turn < 2; ++turn) {
+        const bool mine = odd == (turn == 1);
+        float d[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) d[k] = mine ? own[k] : got[k];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float wk = mine ? w[k] : v[k];
+            asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(
+                             g + 2 * (size_t)(mine ? i[k] : j[k])),
+                         "f"(d[0] * wk), "f"(d[1] * wk), "f"(d[2] * wk), "f"(d[3] * wk)
+                         : "memory");
+        }
+    }
 }
 
 // 1 / a in float64 for a >= psi_floor > 0 by Newton's iteration for the
@@ -392,14 +420,19 @@ __device__ void phase_moments(const EngineArgs &A, const PS<P> &Q, Thr T, int bi
         using qsff::Ff;
         const Ff fl = qsff::split(A.psi_floor);
         const double ox = fma(-A.x_min, A.inv_h, 0.5), oy = fma(-A.y_min, A.inv_h, 0.5);
-        for (int64_t p = p0; p < p1; p += pst) {
+        const int lane = threadIdx.x & 31;
+        for (int64_t pw = p0 - lane; pw < p1; pw += pst) {  // whole warps
+            const bool in = pw + lane < p1;
+            const int64_t p = in ? pw + lane : p1 - 1;
+            unsigned hit = 0;
             const CicF cf = cic_pairs(fma(Q.x[p], A.inv_h, ox), fma(Q.y[p], A.inv_h, oy), A.N);
             const CicP<P> c = cf.single();
-            const Ff a = one_plus_psi(gather_pairs(A.psi2, cf), fl, hits);
+            const Ff a = one_plus_psi(gather_pairs(A.psi2, cf), fl, hit);
+            if (in) hits += hit;
             const P px = Q.px[p], py = Q.py[p];
             const Ff ia = qsff::recip(a);
             const P vx = px * ia.h, vy = py * ia.h;
-            const P wq = Q.w[p] * s;
+            const P wq = in ? Q.w[p] * s : P(0);
             // gamma - 1 = (p^2 + psi^2 + |A|^2 / 2) / (2 (1 + psi))
             const Ff am1 = a + Ff(-1.f, 0.f);
             Ff g = qsff::two_prod(px, px) + qsff::two_prod(py, py) + am1 * am1;
@@ -410,12 +443,9 @@ __device__ void phase_moments(const EngineArgs &A, const PS<P> &Q, Thr T, int bi
             if (banded) {
 #pragma unroll
                 for (int k = 0; k < 6; ++k)
-                    dep_band<ST>(Q.m[k], sb + k * cells, lo, hi, c, q[k]);
+                    if (in) dep_band<ST>(Q.m[k], sb + k * cells, lo, hi, c, q[k]);
             } else {
-                dep6(A.mom32, c.i00, c.w00, q);
-                dep6(A.mom32, c.i01, c.w01, q);
-                dep6(A.mom32, c.i10, c.w10, q);
-                dep6(A.mom32, c.i11, c.w11, q);
+                dep6_pairs(A.mom32, c, q);
             }
         }
     }
