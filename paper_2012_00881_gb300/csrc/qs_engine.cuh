@@ -123,18 +123,6 @@ __device__ __forceinline__ void dep6_pairs(float4 *g, const CicP<float> &c, cons
     }
 }
 
-// 1 / a in float64 for a >= psi_floor > 0 by Newton's iteration for the
-// reciprocal, r <- r (2 - a r), from the float32 reciprocal: each step doubles
-// the correct bits (24, 48, then float64 rounding).  Four float64 operations
-// and two conversions instead of a float64 divide, a long instruction
-// sequence on GB300's 1/64-rate float64 pipe.
-__device__ __forceinline__ double rcp_newton(double a) {
-    double r = (double)__frcp_rn((float)a);
-    r = r * fma(-a, r, 2.0);
-    r = r * fma(-a, r, 2.0);
-    return r;
-}
-
 // ---------------------------------------------------------------------------
 // Privatised deposits.  With the plasma sorted by cell, a block that takes a
 // contiguous chunk of the particle array finds its CIC stencils in a narrow

@@ -42,10 +42,6 @@ struct Cplx {
     using type = float2;
 };
 template <>
-struct Cplx<double> {
-    using type = double2;
-};
-template <>
 struct Cplx<Ff> {
     using type = Ff2;
 };
@@ -391,15 +387,7 @@ __device__ __forceinline__ void rows_forward(const Lines &P, int bid, int nblk, 
 }
 
 using qsff::recip;
-// 1 / d for d != 0: float32 directly, float64 by two Newton steps from the
-// float32 reciprocal (a float64 divide is a long sequence on the FP64 pipe)
 __device__ __forceinline__ float recip(float d) { return 1.f / d; }
-__device__ __forceinline__ double recip(double d) {
-    double r = (double)(1.f / (float)d);
-    r = r * fma(-d, r, 2.0);
-    r = r * fma(-d, r, 2.0);
-    return r;
-}
 
 // The rest of `columns` after its lines are filled: forward, times
 // 1 / (4 N^2 (lam_x + lam_y - kbar)), inverse, and the store.  kbar: a real
