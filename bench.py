@@ -18,6 +18,7 @@ from __future__ import annotations
 import argparse
 import atexit
 import json
+import math
 import os
 import signal
 import statistics
@@ -189,7 +190,7 @@ FP64_PEAK_SOURCE = ("nominal: 152 SMs x 2.07 GHz x 2 FP64 FMA/clk/SM x 2 flop/FM
 
 # ---------------------------------------------------------------- ncu traffic
 ENGINE_SOURCES = ("qs_engine.cuh", "qs_engine_fp64.cu", "qs_engine_fp32r.cu", "qs_solve.cuh",
-                  "qs_mg.cuh", "qs_tile.cuh", "qs_internal.cuh")
+                  "qs_mg.cuh", "qs_tile.cuh", "qs_internal.cuh", "qs_fft.cuh", "qs_ff.cuh")
 
 
 def engine_source_hash(sources=ENGINE_SOURCES) -> str:
@@ -241,7 +242,13 @@ def cycle_sweeps(form: str, over=None) -> int:
     return pre + over.get("post_sweeps", 2)
 
 
-def algorithmic_bytes(stats, wl, form: str, n_xi: int, sweeps: int = None) -> float:
+def direct_solves(n: int) -> bool:
+    """Whether a grid of side n takes the direct solves (the library's rule)."""
+    return n % 2 == 0 and 8 <= n <= 2048
+
+
+def algorithmic_bytes(stats, wl, form: str, n_xi: int, sweeps: int = None,
+                      direct: bool = False) -> float:
     """Bytes one slice-engine launch must move at minimum (the byte model).
 
     b = 8 (float64 form) or 4 (refined form: float32 momenta, weights, moment
@@ -272,6 +279,9 @@ def algorithmic_bytes(stats, wl, form: str, n_xi: int, sweeps: int = None) -> fl
     grid = ((21 * b + 29 * 8) * slices + 10 * 8 * n_xi) * nn
     v = stats["vcycles"]
     comp_cycles = v[0] + 2 * v[1] + 2 * v[2]
+    if direct:
+        mg = ((v[0] + 2 * v[1]) * 48 + v[2] * (18 * 2 * b + b) + slices * (5 * 2 * b + 40)) * nn
+        return float(part + grid + mg)
     nu = sweeps if sweeps is not None else cycle_sweeps(form)
     fine = 3 * nu * b + 4.5 * b
     mg = (comp_cycles * (fine + 2 * b + fine / 3) + v[2] * 8 * b) * nn
@@ -419,7 +429,7 @@ def run_native(args):
             pushes += st["pushes"]
             vc = [a + b for a, b in zip(vc, st["vcycles"])]
             max_m = max(max_m, st["max_m"])
-            bytes_alg += algorithmic_bytes(st, wl, form, wl.n_xi)
+            bytes_alg += algorithmic_bytes(st, wl, form, wl.n_xi, direct=direct_solves(wl.n))
         clocks = sampler.stop()
         total_ms = max_over_ranks(sum(times), dev)
         # end to end through the public API with host buffers: each step copies
@@ -657,7 +667,8 @@ def run_batched(args):
             slices += s_["slices"]
             pushes += s_["pushes"]
             bytes_alg += algorithmic_bytes(s_, wl, "fp32r", wl.n_xi,
-                                           sweeps=cycle_sweeps("fp32r", AT.apply(wl, tuned)))
+                                           sweeps=cycle_sweeps("fp32r", AT.apply(wl, tuned)),
+                                           direct=direct_solves(wl.n))
     clocks = sampler.stop()
     total_ms = max_over_ranks(sum(times), dev)
     # end to end: beams from pinned host memory each step, read back after
@@ -723,12 +734,32 @@ def run_batched(args):
 # ---------------------------------------------------------------- oracle timing
 # ---------------------------------------------------------------- nonuniform grid
 NONUNI = "nonuni255"
-NONUNI_SOURCES = ("qs_nonuniform.cu", "qs_grid_sync.cuh")
+NONUNI_SOURCES = ("qs_nonuniform.cu", "qs_grid_sync.cuh", "qs_ff.cuh", "qs_fft.cuh")
 # FP64 flops per finest node, field and V-cycle: four Gauss-Seidel sweeps of
 # the 9-point corrected operator (65 flops a node), one residual (63) and the
 # grid transfers (13), times 4/3 for the coarse levels, plus the residual of
 # the convergence test (63).
 NONUNI_FLOPS_PER_NODE_CYCLE = 4.0 / 3.0 * (4 * 65 + 63 + 13) + 63
+# the nominal float32 peak, for the solves in float32 and in pairs of floats
+FP32_PEAK = 80550.0
+FP32_PEAK_SOURCE = ("nominal: 152 SMs x 2.07 GHz x 128 FP32 FMA/clk/SM x 2 flop/FMA "
+                    "= 80.55 TFLOP/s")
+
+
+def nonuni_direct(form: str, n: int) -> bool:
+    """Whether a nonuniform solver takes GMRES with the direct-solve
+    preconditioner (the library's rule)."""
+    return form == "fp32r" and 15 <= n <= 511
+
+
+def nonuni_flops(form: str, n: int, fields: int, cycles) -> float:
+    """Flops of a solve that reports `cycles`.  The direct path reports a
+    quarter of its iterations, rounded up: at least 4 cycles - 3 iterations of
+    four n x n matrix products a field."""
+    if nonuni_direct(form, n):
+        return max(0.0, 4 * cycles - 3) * 8.0 * n ** 3 * fields
+    return NONUNI_FLOPS_PER_NODE_CYCLE * n * n * fields * cycles
+
 # The five solves of one slice, grouped as the slice advance groups them:
 # psi; E_z and B_z (one Poisson pair); B_x and B_y (one screened pair).
 NONUNI_GROUPS = ((("psi",), False), (("ez", "bz"), False), (("bx", "by"), True))
@@ -812,7 +843,7 @@ def run_nonuniform(args):
             clocks = sampler.stop()
         ms = max_over_ranks(t0.elapsed_time(t1), f"cuda:{local}") / args.steps
         dur = sum(a.elapsed_time(b) for a, b, _, _ in launches) / 1e3
-        flops = sum(NONUNI_FLOPS_PER_NODE_CYCLE * wl.n * wl.n * nr * cyc
+        flops = sum(nonuni_flops(form, wl.n, nr, cyc)
                     for _, _, nr, cyc in launches)
         results[form] = dict(solver=solver, ms=ms, clocks=clocks,
                              value=job_rate(args.steps, world, ms * args.steps / 1e3),
@@ -821,10 +852,12 @@ def run_nonuniform(args):
     main = "fp32r" if "fp32r" in results else forms[0]
     r = results[main]
     solver = r["solver"]
-    # dominant kernel: the solve launch; FP64-equivalent flops counted from
-    # the cycles it ran (the refined form's float32 cycles are counted the
-    # same way, so its fraction is of the float64 peak)
+    # dominant kernel: the solve launch; flops counted from the cycles it ran
+    # (float32 matrix products in the refined form, float64 V-cycles otherwise)
     achieved = r["flops_per_s"] / 1e9
+    direct = nonuni_direct(main, wl.n)
+    if direct:
+        fp64_peak = FP32_PEAK
     traffic = measured_traffic("nu_solve_kernel", NONUNI, main,
                                source_hash=engine_source_hash(NONUNI_SOURCES))
 
@@ -865,9 +898,9 @@ def run_nonuniform(args):
                    "v_cycles": r["cycles"], "l2": "working set (about 12 MB) is L2-resident; "
                    "every step restarts the solves from zero"},
         "roofline": {"bound": "alu", "achieved": achieved, "peak": fp64_peak,
-                     "unit": "GFLOP/s (FP64-equivalent, nominal FP64 peak)",
+                     "unit": "GFLOP/s (%s, nominal peak)" % ("FP32" if direct else "FP64"),
                      "frac": achieved / fp64_peak, "traffic": traffic,
-                     "peak_source": FP64_PEAK_SOURCE},
+                     "peak_source": FP32_PEAK_SOURCE if direct else FP64_PEAK_SOURCE},
         "e2e": {"value": job_rate(args.steps, world, e2e_ms * args.steps / 1e3),
                 "unit": "slice field sets/s", "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": d2h},
@@ -905,12 +938,23 @@ def nonuni_cpu_baseline(wl, seconds: float):
 
 # ---------------------------------------------------------------- laser envelope
 LASER = "laser256"
-LASER_SOURCES = ("qs_laser.cu", "qs_grid_sync.cuh")
+LASER_SOURCES = ("qs_laser.cu", "qs_grid_sync.cuh", "qs_ff.cuh", "qs_fft.cuh")
 # FP64 flops per cell and V-cycle of the complex solve: four red-black sweeps
 # at 30 flops a cell (complex 5-point Laplacian, kappa u, the update), one
 # residual (22) and the transfers (10), times 4/3 for the coarse levels, plus
 # the residual of the stopping test (22).
 LASER_FLOPS_PER_CELL_CYCLE = 4.0 / 3.0 * (4 * 30 + 22 + 10) + 22
+# direct path (even sides): it reports a quarter of its iterations, rounded up.
+# An iteration transforms every line four times (5 log2 n operations a point)
+# and does about 80 more operations a point, in pairs of floats, ten float32
+# flops each at least
+
+
+def laser_flops(n: int, cycles, slices) -> float:
+    if n % 2 == 0 and 8 <= n <= 2048:
+        return max(0.0, 4 * cycles - 3 * slices) * (20 * math.log2(n) + 80) * 10 * n * n
+    return LASER_FLOPS_PER_CELL_CYCLE * n * n * cycles
+
 
 
 def _laser_desc(wl):
@@ -965,9 +1009,10 @@ def run_laser(args):
     ms = max_over_ranks(sum(x.elapsed_time(y) for x, y in evs), f"cuda:{local}") / args.steps
     slices = wl.n_xi * args.steps
     value = job_rate(slices, world, ms * args.steps / 1e3)
-    flops = LASER_FLOPS_PER_CELL_CYCLE * wl.n * wl.n * cycles
+    flops = laser_flops(wl.n, cycles, slices)
     achieved = flops / (ms * args.steps / 1e3) / 1e9
-    fp64_peak = 1250.0
+    direct = wl.n % 2 == 0 and 8 <= wl.n <= 2048
+    fp64_peak = FP32_PEAK if direct else 1250.0
     traffic = measured_traffic("laser_kernel", LASER, "fp64",
                                source_hash=engine_source_hash(LASER_SOURCES))
     # end to end: envelope and susceptibility from pinned host memory, the
@@ -995,8 +1040,9 @@ def run_laser(args):
                    "l2": "working set (about 190 MB: envelope and susceptibility of every "
                          "slice) exceeds L2"},
         "roofline": {"bound": "alu", "achieved": achieved, "peak": fp64_peak,
-                     "unit": "GFLOP/s (FP64, nominal peak)", "frac": achieved / fp64_peak,
-                     "traffic": traffic, "peak_source": FP64_PEAK_SOURCE},
+                     "unit": "GFLOP/s (%s, nominal peak)" % ("FP32" if direct else "FP64"),
+                     "frac": achieved / fp64_peak, "traffic": traffic,
+                     "peak_source": FP32_PEAK_SOURCE if direct else FP64_PEAK_SOURCE},
         "e2e": {"value": job_rate(slices, world, e2e_ms * args.steps / 1e3),
                 "unit": "laser slices/s", "h2d_bytes_per_step": a_host.numel() * 16 +
                 chi_host.numel() * 8, "d2h_bytes_per_step": a_host.numel() * 16},
@@ -1199,7 +1245,12 @@ def run_nupic(args):
     total_s = max_over_ranks(ms_dev / 1e3, dev)
     value = job_rate(slices, world, total_s)
     n_nodes = len(ax) - 2
-    nu_flops = NONUNI_FLOPS_PER_NODE_CYCLE * n_nodes * n_nodes * (vc[0] + 2 * vc[1] + 2 * vc[2])
+    # cycles summed over the slices: a solve's rounding goes with each of them
+    n_solves = 0 if not nonuni_direct(form, n_nodes) else slices
+    nu_flops = sum(NONUNI_FLOPS_PER_NODE_CYCLE * n_nodes * n_nodes * k * v if not n_solves else
+                   max(0.0, 4 * v - 3 * n_solves) * 8.0 * n_nodes ** 3 * k
+                   for k, v in zip((1, 2, 2), vc))
+    nu_peak = FP32_PEAK if n_solves else 1250.0
     # end to end: the driver current in from pinned host memory, the wake out
     jz_host = torch.tensor(jzb_np).pin_memory()
     hist_host = torch.empty((5,) + tuple(jzb_np.shape), dtype=torch.float64).pin_memory()
@@ -1246,10 +1297,10 @@ def run_nupic(args):
            # also holds the particle and assembly phases: a lower bound for
            # the solve kernel
            "roofline": {"bound": "alu", "kernel": "nu_solve_kernel",
-                        "achieved": nu_flops / (ms_dev / 1e3) / 1e9, "peak": 1250.0,
-                        "unit": "GFLOP/s (FP64-equivalent, nominal FP64 peak)",
-                        "frac": nu_flops / (ms_dev / 1e3) / 1e9 / 1250.0, "traffic": None,
-                        "peak_source": FP64_PEAK_SOURCE,
+                        "achieved": nu_flops / (ms_dev / 1e3) / 1e9, "peak": nu_peak,
+                        "unit": "GFLOP/s (%s, nominal peak)" % ("FP32" if n_solves else "FP64"),
+                        "frac": nu_flops / (ms_dev / 1e3) / 1e9 / nu_peak, "traffic": None,
+                        "peak_source": FP32_PEAK_SOURCE if n_solves else FP64_PEAK_SOURCE,
                         "time": "the whole step's device time"},
            # per computed slice: deposit, psi source, three solves (one
            # persistent launch each), moments, two assemblies, push (none
@@ -1366,9 +1417,11 @@ def run_dla(args):
            "config": {"workload": f"{DLA}: 200,000 witness electrons (gamma 20), one laser "
                                   f"time step of {lw.dt} in {DLA_NSUB} sub-steps, in the wake "
                                   f"and envelopes of one laserwake256 step"},
-           "roofline": {"bound": "alu", "achieved": achieved, "peak": 1250.0,
-                        "unit": "GFLOP/s (FP64)", "frac": achieved / 1250.0, "traffic": None,
-                        "peak_source": FP64_PEAK_SOURCE},
+           # the push's operations are in pairs of floats: ten float32 flops each
+           # at least (a product is 6 instructions, a sum 11)
+           "roofline": {"bound": "alu", "achieved": 10 * achieved, "peak": FP32_PEAK,
+                        "unit": "GFLOP/s (FP32)", "frac": 10 * achieved / FP32_PEAK,
+                        "traffic": None, "peak_source": FP32_PEAK_SOURCE},
            "e2e": {"value": subs * args.steps / e2e_s, "unit": "particle sub-steps/s",
                    "h2d_bytes_per_step": 7 * 8 * spec.n_particles,
                    "d2h_bytes_per_step": 7 * 8 * spec.n_particles},
@@ -1474,7 +1527,7 @@ def run_laserwake(args):
             wake_ms += st["gpu_ms"]
             slices += st["slices"]
             env_cycles += st["env_cycles"]
-            bytes_alg += algorithmic_bytes(st, wl, form, wl.n_xi)
+            bytes_alg += algorithmic_bytes(st, wl, form, wl.n_xi, direct=direct_solves(wl.n))
         clocks = sampler.stop()
         total_ms = max_over_ranks(sum(times), dev)
         # end to end: the envelope from pinned host memory and back every step

@@ -41,7 +41,7 @@ extern "C" {
 #define QS_ERR_ARG (-1)            /* invalid argument or configuration      */
 #define QS_ERR_CUDA (-2)           /* a CUDA runtime call failed             */
 #define QS_ERR_OOM (-3)            /* device allocation failed               */
-#define QS_ERR_NOT_CONVERGED (-4)  /* a multigrid solve hit mg_max_vcycles;   */
+#define QS_ERR_NOT_CONVERGED (-4)  /* a field solve hit mg_max_vcycles;       */
                                    /* fields hold the last iterate            */
 #define QS_ERR_PSI_FLOOR (-5)      /* 1+psi fell below psi_floor more often   */
                                    /* than max_psi_guard_hits allows          */
@@ -50,10 +50,13 @@ extern "C" {
                                    /* the kernel returned early               */
 
 /* ---- arithmetic forms -------------------------------------------------- */
-#define QS_FP64 0          /* every step in float64                          */
-#define QS_FP32_REFINED 1  /* float32 particles, smoothing and grid transfers; */
-                           /* float64 residuals, defect correction, coarsest */
-                           /* solve and gamma reconstruction                  */
+#define QS_FP64 0          /* float64 particles, sources and stopping tests;  */
+                           /* direct and conjugate-gradient solves in pairs   */
+                           /* of floats (47 bits), V-cycles in float64        */
+#define QS_FP32_REFINED 1  /* float32 momenta, moments and inner iterations;  */
+                           /* float64 positions, n_*, residuals and defect    */
+                           /* correction; gathers, gamma, sources and the     */
+                           /* direct solves in pairs of floats                */
 
 /* ---- field selection for qs_fields (order of the output blocks) -------- */
 #define QS_FIELD_PSI 1  /* wake potential psi = phi - A_z (Eq. EqM_N8_AA)  */
@@ -78,8 +81,15 @@ typedef struct {
     int refine_k;               /* smallest sub-step is dxi0 / refine_k         */
                                 /* (refinement level k of Sec. 5.1), >= 1       */
     int precision;              /* QS_FP64 or QS_FP32_REFINED                   */
+                                /* Fields: even N, 8 <= N <= 2048, are solved   */
+                                /* directly by sine transforms (psi, E_z, B_z)  */
+                                /* and by conjugate gradients preconditioned    */
+                                /* with them (B_perp); other N, an explicit     */
+                                /* cluster_size of 8 or 16 and a solve that the */
+                                /* iterations don't bring to mg_tol by V-cycles */
     double mg_tol;              /* stop when ||f - A u||_2 <= mg_tol ||f||_2    */
-    int mg_max_vcycles;         /* per solve; exceeding it -> NOT_CONVERGED     */
+    int mg_max_vcycles;         /* per solve, iterations and then V-cycles;     */
+                                /* exceeding it -> NOT_CONVERGED                */
     double psi_floor;           /* 1+psi is clamped to >= psi_floor             */
     int64_t max_psi_guard_hits; /* -1: unlimited                                */
     int sort_every;             /* > 0: every this many base slices the slice   */
@@ -87,6 +97,7 @@ typedef struct {
                                 /* order of qs_cell_sort (not in steps that     */
                                 /* store checkpoints for the adjoint); 0 = the  */
                                 /* lattice order throughout                     */
+                                /* of the V-cycles (and the settings below):    */
     int pre_sweeps, post_sweeps;/* red-black Gauss-Seidel sweeps per level      */
                                 /* (0 .. 8, not both 0); pre_sweeps -1 = the    */
                                 /* form's default (3 refined, 2 QS_FP64)        */
@@ -95,7 +106,7 @@ typedef struct {
                                 /* 0 = default (16 for QS_FP64, 32 for refined) */
     int trace_capacity;         /* > 0: record up to this many phase timestamps */
                                 /* per step (see qs_phase_trace); 0 = off        */
-    int warm_start_order;       /* initial guess of each solve: 0 = previous    */
+    int warm_start_order;       /* initial guess of V-cycle solves: 0 = previous */
                                 /* slice's solution (Sec. 7.1); 1, 2 = that     */
                                 /* history extrapolated in xi, linear/quadratic */
     int tile_x, tile_y;         /* output tile of the grid-wide multigrid      */
@@ -125,10 +136,9 @@ typedef struct {
                                 /* rest of the slice loop on every block:       */
                                 /* QS_FP64 solves of grids N <= 128, the float32 */
                                 /* inner cycles of QS_FP32_REFINED up to 256;   */
-                                /* 0 = automatic (float64: 16 for N <= 64      */
-                                /* dividing by 32, 8 dividing by 16; refined:   */
-                                /* off, its grid-wide cycles being faster), 1 = */
-                                /* off                                           */
+                                /* 0 and 1 = off (the direct solves are faster: */
+                                /* a float64 wake at 64^2 19 ms, clusters of 16 */
+                                /* blocks 101 ms)                               */
     int deposit_band_rows;      /* privatised deposits of the moments and n_*:  */
                                 /* each block adds its contiguous chunk of the  */
                                 /* (cell-sorted) plasma into a band of at most  */
@@ -157,7 +167,7 @@ typedef struct {
     int64_t slices;          /* computed slices including sub-steps          */
     int64_t substeps;        /* computed slices that are not base slices     */
     int64_t pushes;          /* plasma macroparticle pushes                  */
-    int64_t vcycles[3];      /* V-cycles (or outer refinement iterations):   */
+    int64_t vcycles[3];      /* direct solves, iterations or V-cycles:       */
                              /* [0] psi, [1] (E_z, B_z), [2] (B_x, B_y)       */
     int64_t psi_guard_hits;  /* clamps of 1+psi (particles and grid points)  */
     int64_t sorts;           /* cell sorts performed                          */

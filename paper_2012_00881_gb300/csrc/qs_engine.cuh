@@ -4,7 +4,11 @@
 // barrier whose waits are bounded in time; a timed-out wait records
 // QS_ERR_TIMEOUT and every block leaves the kernel at its next barrier.
 //
-// The solves (qs_solve.cuh) are red-black Gauss-Seidel V(nu1, nu2) cycles
+// The solves (qs_solve.cuh) are direct, by sine transforms, and for B_perp
+// conjugate gradients preconditioned with them; sources are formed where their
+// row transforms read them.  Grid sides without the transforms (odd, below 8 or
+// above 2048, clusters on request) and solves that the iterations do not finish
+// take red-black Gauss-Seidel V(nu1, nu2) cycles
 // with 4-cell-average restriction, bilinear prolongation and rediscretised
 // coarse operators (kappa averaged).  Levels of side <= block_level_n are
 // solved redundantly by every block in its shared memory, down to a coarsest

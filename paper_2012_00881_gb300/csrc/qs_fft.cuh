@@ -16,9 +16,9 @@
 //
 // A direct solve is three grid phases: rows forward, columns forward - divide -
 // inverse, rows inverse, each a read and a write of the grid through L2.  What
-// bounds them: in float64 the FP64 pipe (two FMA a clock and SM; about 8,500
-// instructions a 256-point complex line), in float32 the two L2 round trips and
-// the grid barrier of each phase.
+// bounds them, in float32 and in pairs of floats: instruction fetches, the two
+// L2 round trips and the grid barrier of each phase (256^2, two fields: 8 to 10 us
+// a phase; in float64, bound by its pipe, 12).
 #pragma once
 
 #include <cuda_runtime.h>

@@ -1,7 +1,7 @@
 // Device machinery shared by the slice engine and the adjoint engine: the
-// bounded grid barrier, block reductions, and the multigrid solves (float64
-// V-cycles; refined form: float64 residual, float32 staged V-cycles, float64
-// correction).  Everything is in an unnamed namespace: each translation unit
+// bounded grid barrier, block reductions, the direct and conjugate-gradient
+// solves by sine transforms, and the multigrid solves (float64 V-cycles; refined
+// form: float64 residual, float32 staged V-cycles, float64 correction).  Everything is in an unnamed namespace: each translation unit
 // that includes this header gets its own copy.
 #pragma once
 
@@ -49,7 +49,7 @@ __device__ __forceinline__ void red_release_add_u64(unsigned long long *p, unsig
 // error word is read beside the counter, never before the arrival or between
 // two polls, where its trip to L2 would lie on every phase's path: a block that
 // gave up does not arrive, so the others are still polling when they see it.
-// A refined slice at 256^2 (31 barriers) took 213 us with both in the way, 204
+// A refined slice at 256^2 (23 barriers) took 213 us with both in the way, 204
 // without.
 struct Sync {
     DevScalars *sc;             // the instance's scalars (error word, trace count)
