@@ -415,10 +415,16 @@ int create_impl(qs_ctx *c) {
         need = (need + 255) & ~(size_t)255;
         const size_t tabs = (size_t)c->N * (ref ? 36 : 24) + (size_t)(c->N / 2 + 1) * (ref ? 24 : 16);
         if (need + tabs <= 220 * 1024) {
+            const size_t smem = c->engine_smem;
             f.tab_off = (int)need;
             c->engine_smem = need + tabs;
             const int r = create_fft(c);
-            if (r != QS_OK) return r;
+            if (r == QS_ERR_OOM) {  // the V-cycles need none of its grids
+                f = FftArgs{};
+                c->engine_smem = smem;
+            } else if (r != QS_OK) {
+                return r;
+            }
         }
     }
     if (c->engine_smem > 220 * 1024)
