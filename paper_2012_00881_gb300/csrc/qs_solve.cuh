@@ -1390,6 +1390,10 @@ __device__ bool mg_solve(const EngineArgs &A, const Sync &S, const SolveSpec &V,
         const int r = cg_screened<REF>(A, S, V, slot, bid, nblk, prepared);
         if (r != 0) return r > 0;
         screened_diagonal(A, grid_thr(bid, nblk));
+        // The cycles move `slot` on without clearing the dot products' ring: the
+        // next slice's iterations would add to what these left in it.
+        if (bid == 0 && threadIdx.x < 64)
+            sc->cgd[threadIdx.x >> 4][threadIdx.x & 15] = 0.f;
         SYNC(56);
     }
     // shared memory: [coarsest inverses][coarse levels + work][staged tile]
