@@ -739,7 +739,7 @@ __device__ void rows_eb_bp(const EngineArgs &A, const PS<P> &Q, const double *nc
     using C = qsfft::V2<T>;
     const int n = A.N;
     const double inv2h = 0.5 * A.inv_h;
-    float sums[16] = {0.f};
+    double sx2 = 0.0, sy2 = 0.0;
     const Ff fl = qsff::split(A.psi_floor), i2h = qsff::split(inv2h);
     C *const cr = (C *)A.fft.cr;
     qsfft::rows_inverse_forward<Ff, T, 2>(
@@ -816,13 +816,11 @@ __device__ void rows_eb_bp(const EngineArgs &A, const PS<P> &Q, const double *nc
             A.f_bx[i] = fx;
             A.f_by[i] = fy;
             cr[i] = r;
-            const float hx = head(r.x), hy = head(r.y);
-            sums[0] += hx * hx;
-            sums[1] += hy * hy;
+            sx2 += fx * fx;
+            sy2 += fy * fy;
             return r;
         });
-    const float t = qsfft::block_sums16(sums);
-    if (threadIdx.x < 2) atomicAdd(&A.sc->fnorm[2][threadIdx.x], (double)t);
+    block_sum_wide(sx2, sy2, A.sc->fnorm[2]);
 }
 
 // (double)i for 0 <= i < 2^31 without a conversion: 2^52 + i is exact

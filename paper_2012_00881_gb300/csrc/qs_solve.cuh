@@ -173,6 +173,51 @@ __device__ void block_sum4f(float v[4]) {
     __syncthreads();  // red4 is reused by the next call
 }
 
+// Adds the block's sums of a and b (>= 0; squares) to dst[0] and dst[1].  The
+// values keep float64's range and the sums float32's precision, each warp's
+// with a power of two of its own: a norm may be of 1e-30 or of 1e+30, which
+// squares in float32 are not.  (A float64 sum is 10 additions of 64 cycles a
+// warp and value.)
+__device__ void block_sum_wide(double a, double b, double *dst) {
+    __shared__ float sm[2][32];
+    __shared__ int se[2][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = ((int)blockDim.x + 31) >> 5;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const double v = c ? b : a;
+        const unsigned hi = (unsigned)__double2hiint(v);
+        const int e = (int)(hi >> 20) & 0x7ff, E = __reduce_max_sync(0xffffffffu, e);
+        float m = 0.f;
+        if (e == 0x7ff) m = (float)v;  // infinite or NaN
+        else if (e > 0 && E - e <= 60)
+            m = qsff::split(__hiloint2double((int)(hi + ((unsigned)(1023 - E) << 20)),
+                                             __double2loint(v))).h;
+        for (int o = 16; o; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
+        if (lane == 0) {
+            sm[c][wid] = m;
+            se[c][wid] = E;
+        }
+    }
+    __syncthreads();
+    for (int c = wid; c < 2; c += nw) {
+        const int e = lane < nw ? se[c][lane] : 0, E = __reduce_max_sync(0xffffffffu, e);
+        float m = lane < nw ? sm[c][lane] : 0.f;
+        if (E - e > 60) m = 0.f;
+        else m *= __int_as_float((127 + e - E) << 23);
+        for (int o = 16; o; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
+        if (lane == 0 && m != 0.f) {
+            const double w = qsff::widen(m);
+            const int x = ((__double2hiint(w) >> 20) & 0x7ff) + E - 1023;
+            double t = w;  // not finite
+            if (E != 0x7ff)
+                t = x >= 0x7ff ? __longlong_as_double(0x7ff0000000000000LL)
+                               : __hiloint2double((__double2hiint(w) & 0xfffff) | (x << 20),
+                                                  __double2loint(w));
+            atomicAdd(dst + c, t);
+        }
+    }
+}
+
 __device__ float block_max(float v) {
     __shared__ float redf[32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -706,13 +751,13 @@ __device__ __noinline__ void mg_solve_cluster64(const EngineArgs &A, const Solve
                 const double f2 = fn[comp];
                 double thr = fmax(A.mg_tol * A.mg_tol * f2, A.mg_atol * A.mg_atol);
                 thr = fmax(thr, fl * fl * s_tot[1]);
-                s_conv = f2 == 0.0 || s_tot[0] <= thr;
+                s_conv = f2 == 0.0 ? 1 : !(s_tot[0] <= 1.7e308) ? 2 : s_tot[0] <= thr;
                 s_rel = f2 > 0.0 ? sqrt(s_tot[0] / f2) : 0.0;
             }
             __syncthreads();
-            conv = s_conv != 0;
+            conv = s_conv == 1;
             mk(70);
-            if (conv || it >= A.mg_max_vcycles) break;
+            if (s_conv || it >= A.mg_max_vcycles) break;
         }
         cluster_vcycle<double>(A, cl, cv, ci, it == 0, mk);
         ++it;
@@ -848,7 +893,7 @@ __device__ __noinline__ bool mg_solve_ref_cluster(const EngineArgs &A, const Syn
     for (;;) {
         if (threadIdx.x == 0) {
             const double fl = 1e-13 * A.lev_inv_h2[0];
-            int cv = 1;
+            int cv = 1, stop = 0;
             rel = 0.0;
             for (int c = 0; c < V.nc; ++c) {
                 const double fn = s_fn[c];
@@ -857,16 +902,18 @@ __device__ __noinline__ bool mg_solve_ref_cluster(const EngineArgs &A, const Syn
                 const double un = vload(&sc->rnorm[slot & 3][2 + c]);
                 double thr = fmax(A.mg_tol * A.mg_tol * fn, A.mg_atol * A.mg_atol);
                 thr = fmax(thr, fl * fl * un);
-                if (rn > thr) cv = 0;
+                if (!(rn <= thr)) cv = 0;
+                if (!(rn <= 1.7e308)) stop = 1;
                 rel = fmax(rel, sqrt(rn / fn));
             }
-            s_conv = cv;
+            s_conv = stop ? 2 : cv;
         }
         __syncthreads();
-        conv = s_conv != 0;
+        const int sv = s_conv;
         __syncthreads();
+        conv = sv == 1;
         ++slot;
-        if (conv || it >= A.mg_max_vcycles) break;
+        if (sv || it >= A.mg_max_vcycles) break;
         cluster_inner_cycle(A, V, bid, smem_base, ci, it == 0);
         SYNC(24);
         if (V.nc == 1) update_from_e<1>(A, V, T, sc->rnorm[slot & 3]);
@@ -990,6 +1037,7 @@ struct IterScalars {
     float ig[2], ia[2], al[2], be[2], ss[2];
     float kbar;
     int go;
+    int bad;  // the last residual is not finite
 };
 
 // `red` times the residual a round starts from, or just below the bound
@@ -997,18 +1045,20 @@ __device__ __forceinline__ float round_target(double red, double r0, double thr)
     return fmaxf((float)fmax(red * r0, 0.09 * thr), 1e-37f);
 }
 
-// Source scales and stopping bounds; go: whether any component needs work.  A
-// NaN or infinite source keeps scale 1 and fails every stopping test.
+// Source scales and stopping bounds; go: 1 if any component needs work, 0 if
+// none does, 2 if a source is beyond what the iterations' float32 exponents hold
+// (||f|| above 2^100: N^2 times it passes through the transforms) or not finite.
 __device__ void iter_begin(const EngineArgs &A, const SolveSpec &V, IterScalars &I, double red) {
     __syncthreads();
     if (threadIdx.x < 32) {
         const int c = threadIdx.x;
-        bool work = false;
+        bool work = false, beyond = false;
         if (c < 2) {
             const double fn = c < V.nc ? vload(&A.sc->fnorm[V.kind][c]) : 0.0;
             const int ex = (int)((__double_as_longlong(fn) >> 52) & 0x7ff);
             const int k = ex == 0 || ex == 0x7ff ? 0 : (ex - 1023) / 2;
             const int kc = min(max(k, -120), 120);
+            beyond = ex == 0x7ff || k > 100;
             I.scale[c] = __int_as_float((127 - kc) << 23);
             const double s2 = __longlong_as_double((long long)(1023 - 2 * kc) << 52);
             const double thr = fmax(A.mg_tol * A.mg_tol * fn, A.mg_atol * A.mg_atol) * s2;
@@ -1020,9 +1070,10 @@ __device__ void iter_begin(const EngineArgs &A, const SolveSpec &V, IterScalars 
             work = !(r0 <= thr);
         }
         const unsigned any = __ballot_sync(0xffffffffu, work);
+        const unsigned out = __ballot_sync(0xffffffffu, beyond);
         if (c == 0) {
             I.kbar = V.screened ? qsff::split(vload(&A.sc->ksum)).h / (float)(A.N * A.N) : 0.f;
-            I.go = any != 0;
+            I.go = out ? 2 : any != 0;
         }
     }
     __syncthreads();
@@ -1035,7 +1086,7 @@ __device__ int iter_check(const EngineArgs &A, const SolveSpec &V, IterScalars &
     DevScalars *sc = A.sc;
     if (threadIdx.x < 32) {
         const int c = threadIdx.x;
-        bool open = false, slow = false;
+        bool open = false, slow = false, bad = false;
         float rel = 0.f;
         if (c < V.nc) {
             const double fl = 1e-13 * A.lev_inv_h2[0];
@@ -1043,16 +1094,19 @@ __device__ int iter_check(const EngineArgs &A, const SolveSpec &V, IterScalars &
             const double un = vload(&sc->rnorm[slot & 3][2 + c]);
             open = !(rn <= fmax(I.thr[c], fl * fl * un));
             slow = open && !(rn <= 0.0625 * I.r0[c]);
+            bad = !(rn <= 1.7e308);
             I.r0[c] = rn;
             I.target[c] = round_target(red, rn, I.thr[c]);
             if (I.fs[c] > 0.f) rel = sqrtf((float)rn / I.fs[c]);
         }
         const unsigned nopen = __ballot_sync(0xffffffffu, open);
         const unsigned nslow = __ballot_sync(0xffffffffu, slow);
+        const unsigned nbad = __ballot_sync(0xffffffffu, bad);
         rel = fmaxf(rel, __shfl_sync(0xffffffffu, rel, 1));
         if (c == 0) {
             if (bid == 0 && !nopen && (double)rel > sc->max_relres) sc->max_relres = (double)rel;
             I.go = !nopen ? 1 : (nslow || last) ? 0 : -2;
+            I.bad = nbad != 0;
         }
     }
     __syncthreads();
@@ -1162,6 +1216,7 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
     __shared__ IterScalars I;
     const double red = REF ? 1e-10 : 1e-26;  // a round's reduction, squared
     iter_begin(A, V, I, red);
+    if (I.go == 2) return 0;
     if (!I.go) {  // both sources are rounding noise or zero
         zero_solution(A, V, bid, nblk);
         return S(50) ? 1 : -1;
@@ -1266,11 +1321,13 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
                                 ww = vload(g + 8 + c), ws = vload(g + 10 + c),
                                 rr = vload(g + 12 + c);
                     float be = 0.f, al = 0.f, ia = 0.f, ig = 0.f;
-                    if (ga != 0.f) {
+                    // a component that is solved to float32's smallest numbers
+                    // stands still (1 / ga would be infinite)
+                    if (fabsf(ga) >= 1e-36f) {
                         ig = 1.f / ga;
                         be = inner > 0 ? ga * I.ig[c] : 0.f;
                         ia = de * ig - be * (inner > 0 ? I.ia[c] : 0.f);
-                        al = ia != 0.f ? 1.f / ia : 0.f;
+                        al = fabsf(ia) >= 1e-30f ? 1.f / ia : 0.f;
                     }
                     I.ig[c] = ig;
                     I.ia[c] = ia;
@@ -1282,7 +1339,8 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
                     const float ss = ww + be * (2.f * ws + be * so);
                     I.ss[c] = ss;
                     const float nr = rr - al * (2.f * (rw + be * rs) - al * ss);
-                    open = !((nr < 2e-7f * rr ? 2e-7f * rr : nr) <= I.target[c]);  // a NaN stays
+                    // a NaN ends the round: its float64 residual decides
+                    open = (nr < 2e-7f * rr ? 2e-7f * rr : nr) > I.target[c];
                 }
                 const unsigned nopen = __ballot_sync(0xffffffffu, open);
                 if (c == 0) I.go = nopen != 0;
@@ -1356,6 +1414,8 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
         ++slot;
     }
     if (bid == 0 && threadIdx.x == 0) sc->vcycles[V.kind] += it;
+    // nothing for the cycles to go on from
+    if (result == 0 && I.bad) zero_solution(A, V, bid, nblk);
     return result;
 }
 
@@ -1476,7 +1536,9 @@ __device__ bool mg_solve(const EngineArgs &A, const Sync &S, const SolveSpec &V,
             }
             if (threadIdx.x == 0) {
                 const double fl = 1e-13 * A.lev_inv_h2[0];
-                int cv = 1;
+                // a residual that is not finite is not below any bound, and
+                // further cycles don't mend it
+                int cv = 1, stop = 0;
                 rel = 0.0;
                 for (int c = 0; c < V.nc; ++c) {
                     const double fn = s_fn[c];
@@ -1485,16 +1547,18 @@ __device__ bool mg_solve(const EngineArgs &A, const Sync &S, const SolveSpec &V,
                     const double un = vload(&sc->rnorm[slot & 3][2 + c]);
                     double thr = fmax(A.mg_tol * A.mg_tol * fn, A.mg_atol * A.mg_atol);
                     thr = fmax(thr, fl * fl * un);
-                    if (rn > thr) cv = 0;
+                    if (!(rn <= thr)) cv = 0;
+                    if (!(rn <= 1.7e308)) stop = 1;
                     rel = fmax(rel, sqrt(rn / fn));
                 }
-                s_conv = cv;
+                s_conv = stop ? 2 : cv;
             }
             __syncthreads();
-            conv = s_conv != 0;
+            const int sv = s_conv;
             __syncthreads();  // s_conv is rewritten by the next test
+            conv = sv == 1;
             ++slot;
-            if (conv || it >= A.mg_max_vcycles) break;
+            if (sv || it >= A.mg_max_vcycles) break;
         }
         bool ok;
         norms_ready = false;

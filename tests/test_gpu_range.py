@@ -1,0 +1,49 @@
+"""Sources at the ends of the number range and values that are not numbers (GPU).
+
+The first slice is linear in the driver: a driver 2^k times as strong has 2^k
+times the fields, to the solver's tolerance (1e-12 of the source, tens of times
+that in the solution).  2^83 squares beyond float32's range; 2^116 is beyond what
+the iterations hold, so that the V-cycles solve it (float64 form; the refined
+form's own cycles are float32).  A source with a NaN has no solution: the call
+says so."""
+import numpy as np
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def _context(qs, form, n_xi=1, scale=1.0, cluster=0, n=32):
+    wl = W.Workload(name="r", n=n, half_width=3.0, n_xi=n_xi, xi_len=1.0 * n_xi, ppc=4,
+                    beams=(W.BeamSpec(amplitude=1.0, sigma_x=0.7, sigma_y=0.5, sigma_z=0.6,
+                                      xi_c=0.3, n_particles=3000, seed=3, x_c=0.3),))
+    beam = W.sample_beam(wl.beams[0])
+    beam["w"] = beam["w"] * scale
+    ctx = qs.Context(qs.config_from_workload(wl, precision=form, mg_tol=1e-12,
+                                             cluster_size=cluster))
+    ctx.init_plasma(wl.ppc)
+    return ctx, qs.Beam(beam)
+
+
+@pytest.mark.parametrize("form,k", [("fp64", 83), ("fp64", 116), ("fp32r", 83)])
+def test_first_slice_is_linear_in_the_driver(qs, form, k):
+    got = []
+    for s in (1.0, 2.0 ** k):
+        ctx, beam = _context(qs, form, scale=s)
+        ctx.step3d([beam])
+        got.append(ctx.fields(qs.FIELD_BX | qs.FIELD_BY, device=False).numpy() / s)
+        ctx.close()
+    assert np.linalg.norm(got[0]) > 0.0
+    assert np.linalg.norm(got[1] - got[0]) < 1e-9 * np.linalg.norm(got[0])
+
+
+@pytest.mark.parametrize("form,cluster", [("fp64", 0), ("fp32r", 0), ("fp64", 8), ("fp32r", 8)])
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_no_solution_is_reported(qs, form, cluster, bad):
+    ctx, beam = _context(qs, form, n_xi=3, cluster=cluster)
+    beam.t["w"][7] = bad
+    with pytest.raises(qs.QsError) as e:
+        ctx.step3d([beam])
+    assert e.value.status == qs.QS_ERR_NOT_CONVERGED
+    ctx.close()
