@@ -61,6 +61,7 @@ constexpr int kLocalN = 8;             // levels this small run in block 0
 constexpr int kNu = 2;                 // pre- and post-sweeps, V(2, 2)
 constexpr int kTileX = 32, kTileY = 16;  // largest staged output tile
 constexpr int kCoarseSweeps = 20;
+constexpr double kFinite = 1.7e308;     // a norm above it, or NaN, is below no bound
 constexpr size_t kScalarBytes = 1024;     // room for LzScalars ahead of the grids
 constexpr long long kBarrierLimit = 4000000000LL;  // clock cycles, ~2 s
 
@@ -560,8 +561,8 @@ __device__ void lz_reduce(LzScalars *sc, float v[16], int use) {
 
 // The change of slice j's envelope into A.dlt.  On entry A.dlt is the previous
 // slice's change (added to the caller's array here).  Returns 1 (converged),
-// 0 (not: A.u = A^n + the change so far, for the V-cycles), -1 (a barrier
-// failed).  its: iterations; relres: the final relative residual (thread 0).
+// 0 (not: A.u = A^n + the change so far, for the V-cycles), 3 (not finite), -1
+// (a barrier failed).  its: iterations; relres: the final relative residual (thread 0).
 __device__ int slice_direct(const LzArgs &A, const qsync::GridBarrier<LzScalars> &gsync, int j,
                             long long g, long long &kglob, int &use, int &its, double &relres) {
     LzScalars *sc = A.sc;
@@ -612,7 +613,7 @@ __device__ int slice_direct(const LzArgs &A, const qsync::GridBarrier<LzScalars>
         const double f2 = qsync::vload(&sc->fnorm[g % 3]);
         s_r0 = qsync::vload(&sc->start[g % 3][0]);
         s_thr = A.tol * A.tol * f2;
-        s_go = s_r0 <= s_thr;
+        s_go = s_r0 <= s_thr && s_r0 <= kFinite;
         relres = f2 > 0.0 ? sqrt(s_r0 / f2) : 0.0;
     }
     __syncthreads();
@@ -703,7 +704,8 @@ __device__ int slice_direct(const LzArgs &A, const qsync::GridBarrier<LzScalars>
                 const float2 ga = make_float2(v[0], v[1]), de = make_float2(v[2], v[3]);
                 const float2 zero = make_float2(0.f, 0.f);
                 float2 b = zero, a = zero, ia = zero, ig = zero;
-                if (ga.x != 0.f || ga.y != 0.f) {
+                // solved to float32's smallest numbers: stands still
+                if (fmaxf(fabsf(ga.x), fabsf(ga.y)) >= 1e-36f) {
                     ig = finv(ga);
                     if (inner > 0) b = fmul(ga, s_ig);
                     ia = fmul(de, ig);
@@ -711,7 +713,7 @@ __device__ int slice_direct(const LzArgs &A, const qsync::GridBarrier<LzScalars>
                         const float2 t = fmul(b, s_ia);
                         ia = make_float2(ia.x - t.x, ia.y - t.y);
                     }
-                    if (ia.x != 0.f || ia.y != 0.f) a = finv(ia);
+                    if (fmaxf(fabsf(ia.x), fabsf(ia.y)) >= 1e-30f) a = finv(ia);
                 }
                 s_ig = ig;
                 s_ia = ia;
@@ -728,7 +730,7 @@ __device__ int slice_direct(const LzArgs &A, const qsync::GridBarrier<LzScalars>
                 float nr = rr - 2.f * ars.x + (a.x * a.x + a.y * a.y) * ss;
                 nr = nr < 2e-7f * rr ? 2e-7f * rr : nr;
                 s_ss = ss;
-                s_go = !(nr <= s_target);
+                s_go = nr > s_target;  // a NaN ends the round
             }
             ++use;
             __syncthreads();
@@ -774,7 +776,7 @@ __device__ int slice_direct(const LzArgs &A, const qsync::GridBarrier<LzScalars>
             const double r2 = qsync::vload(&sc->norm[kglob % 3]);
             const double f2 = qsync::vload(&sc->fnorm[g % 3]);
             const bool slow = !(r2 <= 0.0625 * s_r0);
-            s_go = r2 <= s_thr ? 1 : (slow || its >= cap) ? 0 : 2;
+            s_go = !(r2 <= kFinite) ? 3 : r2 <= s_thr ? 1 : (slow || its >= cap) ? 0 : 2;
             s_r0 = r2;
             set_target();
             relres = f2 > 0.0 ? sqrt(r2 / f2) : 0.0;
@@ -839,16 +841,18 @@ __global__ void __launch_bounds__(kThreads, 1) laser_kernel(const __grid_constan
                 double rel = 0.0;
                 const int r = slice_direct(A, gsync, j, g, kglob, use, its, rel);
                 if (r < 0) return;
-                if (r > 0) {
+                if (r == 1) {
                     if (blockIdx.x == 0 && threadIdx.x == 0) {
                         sc->cycles += (its + 3) / 4;  // the work of a V-cycle, at least
                         if (rel > sc->max_relres) sc->max_relres = rel;
                     }
                     continue;
                 }
-                // the V-cycles go on from its iterate
-                for (int p = grid.t; p < nn; p += grid.nt)
+                // the V-cycles go on from its iterate, or start from A^n
+                for (int p = grid.t; p < nn; p += grid.nt) {
                     L0.kap[p] = make_double2(chij[p] - A.c.x, -A.c.y);
+                    if (r == 3) U[p] = aj[p];
+                }
             } else {
                 // right-hand side, warm start, kappa and 1/diag of level 0; the
                 // previous slice's new envelope goes to the caller's array
@@ -905,8 +909,9 @@ __global__ void __launch_bounds__(kThreads, 1) laser_kernel(const __grid_constan
                 const double r2 = qsync::vload(&sc->norm[kglob % 3]);
                 const double f2 = qsync::vload(&sc->fnorm[g % 3]);
                 ++kglob;
-                const bool conv = r2 <= A.tol * A.tol * f2;
-                if (conv || cyc >= A.max_cycles) {
+                const bool bad = !(r2 <= kFinite);  // more cycles don't mend it
+                const bool conv = !bad && r2 <= A.tol * A.tol * f2;
+                if (conv || bad || cyc >= A.max_cycles) {
                     if (blockIdx.x == 0 && threadIdx.x == 0) {
                         sc->cycles += cyc;
                         const double rel = f2 > 0.0 ? sqrt(r2 / f2) : 0.0;

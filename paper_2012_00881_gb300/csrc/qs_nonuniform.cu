@@ -124,6 +124,7 @@ struct NuScalars {
 };
 
 constexpr int kBasis = 8;  // iterations a round
+constexpr double kFinite = 1.7e308;
 
 // Arrays of the direct-solve preconditioner.
 struct NuDirect {
@@ -1167,10 +1168,12 @@ __device__ int nu_direct(const NuArgs &A, const GridBarrier &gsync, int &its) {
         if (!gsync(20)) return -1;
         if (threadIdx.x == 0) {
             int conv = 1, slow = 0;
+            bool bad = false;  // a residual that is not finite is below no bound
             for (int c = 0; c < nr; ++c) {
                 const double f2 = vload(&sc->dfnorm[c]), r2 = vload(&sc->dnorm[round % 3][c]);
                 const double thr = A.tol * A.tol * f2;
-                if (f2 > 0.0 && !(r2 <= thr)) {
+                bad = bad || !(r2 <= kFinite);
+                if (f2 != 0.0 && !(r2 <= thr && r2 <= kFinite)) {
                     conv = 0;
                     if (round > 0 && !(r2 <= 0.0625 * R.beta2[c])) slow = 1;
                 }
@@ -1181,10 +1184,14 @@ __device__ int nu_direct(const NuArgs &A, const GridBarrier &gsync, int &its) {
                 R.nu[c][0] = R.g[c][0] = b;
                 R.inv[c] = b > 0.f ? 1.f / b : 0.f;
             }
-            s_result = conv ? 1 : (slow || round >= 12) ? 0 : 2;
+            s_result = conv ? 1 : bad ? 3 : (slow || round >= 12) ? 0 : 2;
         }
         __syncthreads();
         result = s_result;
+        if (result == 3) {  // nothing for the cycles to go on from
+            for (int p = grid.t; p < nn * nr; p += grid.nt) top.u[p] = 0.0;
+            return gsync(23) ? 0 : -1;
+        }
         if (result != 2) {
             if (blockIdx.x == 0 && threadIdx.x == 0)
                 for (int c = 0; c < nr; ++c) {
@@ -1368,18 +1375,20 @@ __global__ void __launch_bounds__(kThreads, 1) nu_solve_kernel(const __grid_cons
     for (int cyc = 0;; ++cyc) {
         // convergence test on the float64 residual left by the previous
         // cycle (slot cyc % 3)
-        bool conv = true;
+        bool conv = true, bad = false;
         for (int c = 0; c < nr; ++c) {
             const double rn = vload(&sc->norm[cyc % 3][c]);
-            if (fn2[c] > 0.0 && rn > A.tol * A.tol * fn2[c]) conv = false;
+            if (fn2[c] != 0.0 && !(rn <= A.tol * A.tol * fn2[c])) conv = false;
+            if (!(rn <= kFinite)) bad = true;  // more cycles don't mend it
         }
-        if (conv || cyc >= A.max_cycles) {
+        if (bad) conv = false;
+        if (conv || bad || cyc >= A.max_cycles) {
             if (blockIdx.x == 0 && threadIdx.x == 0) {
                 sc->cycles = cyc;
                 sc->converged = conv ? 1 : 0;
                 for (int c = 0; c < nr; ++c)
                     sc->relres[c] =
-                        fn2[c] > 0.0 ? sqrt(vload(&sc->norm[cyc % 3][c]) / fn2[c]) : 0.0;
+                        fn2[c] != 0.0 ? sqrt(vload(&sc->norm[cyc % 3][c]) / fn2[c]) : 0.0;
             }
             // a field whose source is zero has the solution zero
             for (int c = 0; c < nr; ++c)

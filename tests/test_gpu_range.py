@@ -47,3 +47,30 @@ def test_no_solution_is_reported(qs, form, cluster, bad):
         ctx.step3d([beam])
     assert e.value.status == qs.QS_ERR_NOT_CONVERGED
     ctx.close()
+
+
+@pytest.mark.parametrize("form", ["fp64", "fp32r"])
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_nonuniform_solve_reports_no_solution(qs, form, bad):
+    import torch
+    x = np.linspace(-3.0, 3.0, 33)
+    j = torch.zeros((2, 31, 31), dtype=torch.float64, device="cuda")
+    j[0, 10, 12] = 1.0
+    j[1, 10, 12] = bad
+    s = qs.NonuniformSolver(x, x, precision=form)
+    s.solve(j, max_cycles=20, raise_on_error=False)
+    assert s.status == qs.QS_ERR_NOT_CONVERGED
+    u, _, relres = s.solve(j[:1].contiguous(), max_cycles=40)  # the solver is fine after it
+    assert relres[0] <= 1e-10 and bool(torch.isfinite(u).all())
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_envelope_reports_no_solution(qs, bad):
+    import torch
+    n, n_xi = 16, 3
+    a = torch.ones((n_xi, n, n), dtype=torch.complex128, device="cuda")
+    a[1, 3, 4] = bad
+    chi = torch.zeros((n_xi, n, n), dtype=torch.float64, device="cuda")
+    lz = qs.LaserEnvelope(n, 8.0, n_xi, 5.0, 1.0, 0.2)
+    lz.advance(chi, a, raise_on_error=False)
+    assert lz.status == qs.QS_ERR_NOT_CONVERGED
