@@ -659,6 +659,15 @@ __device__ __forceinline__ double driver_jz(const double *J0, const double *J1, 
     return q == 0 ? J0[i] : (1.0 - frac) * J0[i] + frac * (J1 ? J1[i] : 0.0);
 }
 
+// source of E_z (c = 0) or B_z (c = 1) at a cell from the refined form's moments
+__device__ __forceinline__ Ff eb_source(const EngineArgs &A, int c, int n, int ix, int iy, Ff i2h) {
+    const float *const m = (const float *)A.mom32 + 8 * (size_t)(iy * n + ix);
+    auto j = [&](bool in, int k, int comp) { return in ? m[8 * k + comp] : 0.f; };
+    const Ff a = qsff::two_sum(j(ix < n - 1, 1, c), -j(ix > 0, -1, c)),
+             b = qsff::two_sum(j(iy < n - 1, n, 1 - c), -j(iy > 0, -n, 1 - c));
+    return (c ? a - b : -(a + b)) * i2h;
+}
+
 // sources of E_z, B_z; j_z, kappa and its sum, grad psi.  The refined form
 // keeps j_z and grad psi as pairs of floats in the float64 grids' memory.
 template <typename P>
@@ -671,14 +680,19 @@ __device__ void rows_eb(const EngineArgs &A, const PS<P> &Q, const double *ncur,
     unsigned hits = 0;
     float sums[16] = {0.f};
     const Ff fl = qsff::split(A.psi_floor), i2h = qsff::split(inv2h);
-    poisson_rows<2>(A, bid, nblk, [&](int iy, int ix) {
-        const int i = iy * n + ix;
+    poisson_rows<2>(A, bid, nblk, [&](int l, int ix) {
+        const int iy = l, c = l & 1, i = iy * n + ix;  // this line's own row of the two
         const double nv = ncur[i];
         double kap;
         Ff2 f;
         if constexpr (sizeof(P) == 8) {
-            f.x = qsff::split(-(dx0(Q.m[M_JX], n, ix, i, inv2h) + dy0(Q.m[M_JY], n, iy, i, inv2h)));
-            f.y = qsff::split(dx0(Q.m[M_JY], n, ix, i, inv2h) - dy0(Q.m[M_JX], n, iy, i, inv2h));
+            auto src = [&](int y) {
+                const int k = y * n + ix;
+                const double a = dx0(Q.m[c ? M_JY : M_JX], n, ix, k, inv2h),
+                             b = dy0(Q.m[c ? M_JX : M_JY], n, y, k, inv2h);
+                return qsff::split(c ? a - b : -(a + b));
+            };
+            f = qsfft::mk<Ff>(src(l & ~1), src(l | 1));
             const double a = guard(1.0 + A.psi[i], A.psi_floor, hits), ia = 1.0 / a;
             A.jz[i] = Q.m[M_G][i] * ia - nv + driver_jz(J0, J1, i, q, frac);
             kap = nv * ia;
@@ -687,14 +701,7 @@ __device__ void rows_eb(const EngineArgs &A, const PS<P> &Q, const double *ncur,
             A.dpx[i] = dxo(A.psi, n, ix, i, inv2h);
             A.dpy[i] = dyo(A.psi, n, iy, i, inv2h);
         } else {
-            auto jj = [&](bool in, int k) {
-                const float2 *m = (const float2 *)(A.mom32 + 2 * (size_t)k);
-                return in ? *m : make_float2(0.f, 0.f);
-            };
-            const float2 e = jj(ix < n - 1, i + 1), w = jj(ix > 0, i - 1),
-                         s = jj(iy < n - 1, i + n), u = jj(iy > 0, i - n);
-            f.x = -((qsff::two_sum(e.x, -w.x) + qsff::two_sum(s.y, -u.y)) * i2h);
-            f.y = (qsff::two_sum(e.y, -w.y) - qsff::two_sum(s.x, -u.x)) * i2h;
+            f = qsfft::mk<Ff>(eb_source(A, c, n, ix, l & ~1, i2h), eb_source(A, c, n, ix, l | 1, i2h));
             auto psi = [&](int k) {
                 const float2 v = A.psi2[k];
                 return Ff(v.x, v.y);
@@ -733,8 +740,8 @@ __device__ void rows_eb(const EngineArgs &A, const PS<P> &Q, const double *ncur,
 // from them, the right-hand side -e_z x S = (S_y, -S_x) of Eq. Main_Eq_A with
 // its norms, and its row transform: what cg_screened starts from.
 template <typename P>
-__device__ void rows_eb_bp(const EngineArgs &A, const PS<P> &Q, const double *ncur, int bid,
-                           int nblk) {
+__device__ bool rows_eb_bp(const EngineArgs &A, const Sync &S, const PS<P> &Q, const double *ncur,
+                           int bid, int nblk) {
     using T = typename std::conditional<sizeof(P) == 4, float, Ff>::type;
     using C = qsfft::V2<T>;
     const int n = A.N;
@@ -742,85 +749,101 @@ __device__ void rows_eb_bp(const EngineArgs &A, const PS<P> &Q, const double *nc
     double sx2 = 0.0, sy2 = 0.0;
     const Ff fl = qsff::split(A.psi_floor), i2h = qsff::split(inv2h);
     C *const cr = (C *)A.fft.cr;
-    qsfft::rows_inverse_forward<Ff, T, 2>(
-        fft_lines<Ff>(A), fft_lines<T>(A), bid, nblk, (const Ff2 *)A.fft.t2, (C *)A.fft.t1,
-        [&](int iy, int ix, Ff2 v) {
-            const int i = iy * n + ix;
-            const double ezd = qsff::join(v.x), bzd = qsff::join(v.y);
-            A.ez[i] = ezd;
-            A.bz[i] = bzd;
-            double fx, fy;  // S_y, -S_x
-            C r;
-            if constexpr (sizeof(P) == 8) {
-                double a = 1.0 + A.psi[i];
-                if (a < A.psi_floor) a = A.psi_floor;
-                const double jx = Q.m[M_JX][i], jy = Q.m[M_JY][i], txx = Q.m[M_TXX][i],
-                             txy = Q.m[M_TXY][i], tyy = Q.m[M_TYY][i], G = Q.m[M_G][i];
-                const double gx = A.dpx[i], gy = A.dpy[i];
-                const double ia = 1.0 / a, Gia2 = G * ia * ia;
-                double sx = dx0(A.jz, n, ix, i, inv2h) - dx0(Q.m[M_TXX], n, ix, i, inv2h) -
-                            dy0(Q.m[M_TXY], n, iy, i, inv2h) + Gia2 * gx -
-                            (jy * bzd + jx * ezd + txx * gx + txy * gy) * ia;
-                double sy = dy0(A.jz, n, iy, i, inv2h) - dx0(Q.m[M_TXY], n, ix, i, inv2h) -
-                            dy0(Q.m[M_TYY], n, iy, i, inv2h) + Gia2 * gy +
-                            (jx * bzd - jy * ezd - txy * gx - tyy * gy) * ia;
-                if (A.a2_base) {  // -n_* grad(|A|^2/4) / (1+psi)^2
-                    const double nia2 = ncur[i] * ia * ia;
-                    sx -= nia2 * A.pondx[i];
-                    sy -= nia2 * A.pondy[i];
-                }
-                fx = sy;
-                fy = -sx;
-                r = qsfft::mk<T>(qsff::split(fx), qsff::split(fy));
-            } else {
-                A.bz32[i] = v.y.h;  // B_z is final here
-                // T_xx, T_xy, T_yy of a neighbour
-                auto tt = [&](bool in, int k) {
-                    const float4 *m = A.mom32 + 2 * (size_t)k;
-                    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (!in) return z;
-                    const float2 d = *(const float2 *)m, b = *((const float2 *)m + 1);
-                    return make_float4(b.x, b.y, ((const float *)m)[4], d.x);
-                };
-                auto pair = [](const void *g, int k) {
-                    const float2 u = ((const float2 *)g)[k];
-                    return Ff(u.x, u.y);
-                };
-                const Ff zero(0.f, 0.f);
-                const float4 te = tt(ix < n - 1, i + 1), tw = tt(ix > 0, i - 1),
-                             ts = tt(iy < n - 1, i + n), tn = tt(iy > 0, i - n);
-                const Ff dx = (ix < n - 1 ? pair(A.jz, i + 1) : zero) -
-                              (ix > 0 ? pair(A.jz, i - 1) : zero) - qsff::two_sum(te.x, -tw.x) -
-                              qsff::two_sum(ts.y, -tn.y);
-                const Ff dy = (iy < n - 1 ? pair(A.jz, i + n) : zero) -
-                              (iy > 0 ? pair(A.jz, i - n) : zero) - qsff::two_sum(te.y, -tw.y) -
-                              qsff::two_sum(ts.z, -tn.z);
-                const float4 m0 = A.mom32[2 * (size_t)i], m1 = A.mom32[2 * (size_t)i + 1];
-                unsigned dummy = 0;
-                const Ff ia = qsff::recip(one_plus_psi(pair(A.psi2, i), fl, dummy));
-                const Ff nf = qsff::split(ncur[i]), gx = pair(A.dpx, i), gy = pair(A.dpy, i);
-                const Ff Gia = (nf + Ff(m1.y, 0.f)) * ia;
-                // the products with 1 / (1 + psi) taken out
-                Ff px = Gia * gx - (v.y * m0.y + v.x * m0.x + gx * m0.z + gy * m0.w);
-                Ff py = Gia * gy + (v.y * m0.x - v.x * m0.y - gx * m0.w - gy * m1.x);
-                if (A.a2_base) {
-                    const Ff nia = nf * ia;
-                    px -= nia * qsff::split(A.pondx[i]);
-                    py -= nia * qsff::split(A.pondy[i]);
-                }
-                const Ff sx = dx * i2h + px * ia, sy = dy * i2h + py * ia;
-                fx = qsff::join(sy);
-                fy = -qsff::join(sx);
-                r = make_float2(sy.h, -sx.h);
+    auto next = [&](int iy, int ix, Ff2 v) {
+        const int i = iy * n + ix;
+        const double ezd = qsff::join(v.x), bzd = qsff::join(v.y);
+        A.ez[i] = ezd;
+        A.bz[i] = bzd;
+        double fx, fy;  // S_y, -S_x
+        C r;
+        if constexpr (sizeof(P) == 8) {
+            double a = 1.0 + A.psi[i];
+            if (a < A.psi_floor) a = A.psi_floor;
+            const double jx = Q.m[M_JX][i], jy = Q.m[M_JY][i], txx = Q.m[M_TXX][i],
+                         txy = Q.m[M_TXY][i], tyy = Q.m[M_TYY][i], G = Q.m[M_G][i];
+            const double gx = A.dpx[i], gy = A.dpy[i];
+            const double ia = 1.0 / a, Gia2 = G * ia * ia;
+            double sx = dx0(A.jz, n, ix, i, inv2h) - dx0(Q.m[M_TXX], n, ix, i, inv2h) -
+                        dy0(Q.m[M_TXY], n, iy, i, inv2h) + Gia2 * gx -
+                        (jy * bzd + jx * ezd + txx * gx + txy * gy) * ia;
+            double sy = dy0(A.jz, n, iy, i, inv2h) - dx0(Q.m[M_TXY], n, ix, i, inv2h) -
+                        dy0(Q.m[M_TYY], n, iy, i, inv2h) + Gia2 * gy +
+                        (jx * bzd - jy * ezd - txy * gx - tyy * gy) * ia;
+            if (A.a2_base) {  // -n_* grad(|A|^2/4) / (1+psi)^2
+                const double nia2 = ncur[i] * ia * ia;
+                sx -= nia2 * A.pondx[i];
+                sy -= nia2 * A.pondy[i];
             }
-            A.f_bx[i] = fx;
-            A.f_by[i] = fy;
-            cr[i] = r;
-            sx2 += fx * fx;
-            sy2 += fy * fy;
-            return r;
+            fx = sy;
+            fy = -sx;
+            r = qsfft::mk<T>(qsff::split(fx), qsff::split(fy));
+        } else {
+            A.bz32[i] = v.y.h;  // B_z is final here
+            // T_xx, T_xy, T_yy of a neighbour
+            auto tt = [&](bool in, int k) {
+                const float4 *m = A.mom32 + 2 * (size_t)k;
+                const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (!in) return z;
+                const float2 d = *(const float2 *)m, b = *((const float2 *)m + 1);
+                return make_float4(b.x, b.y, ((const float *)m)[4], d.x);
+            };
+            auto pair = [](const void *g, int k) {
+                const float2 u = ((const float2 *)g)[k];
+                return Ff(u.x, u.y);
+            };
+            const Ff zero(0.f, 0.f);
+            const float4 te = tt(ix < n - 1, i + 1), tw = tt(ix > 0, i - 1),
+                         ts = tt(iy < n - 1, i + n), tn = tt(iy > 0, i - n);
+            const Ff dx = (ix < n - 1 ? pair(A.jz, i + 1) : zero) -
+                          (ix > 0 ? pair(A.jz, i - 1) : zero) - qsff::two_sum(te.x, -tw.x) -
+                          qsff::two_sum(ts.y, -tn.y);
+            const Ff dy = (iy < n - 1 ? pair(A.jz, i + n) : zero) -
+                          (iy > 0 ? pair(A.jz, i - n) : zero) - qsff::two_sum(te.y, -tw.y) -
+                          qsff::two_sum(ts.z, -tn.z);
+            const float4 m0 = A.mom32[2 * (size_t)i], m1 = A.mom32[2 * (size_t)i + 1];
+            unsigned dummy = 0;
+            const Ff ia = qsff::recip(one_plus_psi(pair(A.psi2, i), fl, dummy));
+            const Ff nf = qsff::split(ncur[i]), gx = pair(A.dpx, i), gy = pair(A.dpy, i);
+            const Ff Gia = (nf + Ff(m1.y, 0.f)) * ia;
+            // the products with 1 / (1 + psi) taken out
+            Ff px = Gia * gx - (v.y * m0.y + v.x * m0.x + gx * m0.z + gy * m0.w);
+            Ff py = Gia * gy + (v.y * m0.x - v.x * m0.y - gx * m0.w - gy * m1.x);
+            if (A.a2_base) {
+                const Ff nia = nf * ia;
+                px -= nia * qsff::split(A.pondx[i]);
+                py -= nia * qsff::split(A.pondy[i]);
+            }
+            const Ff sx = dx * i2h + px * ia, sy = dy * i2h + py * ia;
+            fx = qsff::join(sy);
+            fy = -qsff::join(sx);
+            r = make_float2(sy.h, -sx.h);
+        }
+        A.f_bx[i] = fx;
+        A.f_by[i] = fy;
+        cr[i] = r;
+        sx2 += fx * fx;
+        sy2 += fy * fy;
+        return r;
+    };
+    const qsfft::Lines PF = fft_lines<Ff>(A), PT = fft_lines<T>(A);
+    if (PF.gmax >= 2) {
+        qsfft::rows_inverse_forward<Ff, T, 2>(PF, PT, bid, nblk, (const Ff2 *)A.fft.t2,
+                                              (C *)A.fft.t1, next);
+    } else {  // one line a block (sides above 1078): the fields first
+        poisson_inverse<2>(A, bid, nblk, [&](int l, int x, Ff2 v) {
+            double *const u = l & 1 ? A.bz : A.ez;
+            const int i = (l & ~1) * n + x;
+            u[i] = qsff::join(v.x);
+            u[i + n] = qsff::join(v.y);
         });
+        SYNC(34);
+        qsfft::rows_forward<T, 2>(PT, bid, nblk, (C *)A.fft.t1, [&](int iy, int ix) {
+            const int i = iy * n + ix;
+            return next(iy, ix, qsfft::mk<Ff>(qsff::split(A.ez[i]), qsff::split(A.bz[i])));
+        });
+    }
     block_sum_wide(sx2, sy2, A.sc->fnorm[2]);
+    return true;
 }
 
 // (double)i for 0 <= i < 2^31 without a conversion: 2^52 + i is exact
@@ -1265,7 +1288,7 @@ __device__ bool run_step(const EngineArgs &A, int bid, int nblk, const Sync &S, 
                 SYNC(4);
                 poisson_columns<2>(A, bid, nblk);
                 SYNC(29);
-                rows_eb_bp<P>(A, Q, ncur, bid, nblk);
+                if (!rows_eb_bp<P>(A, S, Q, ncur, bid, nblk)) return false;
                 SYNC(5);
                 if (!mg_solve<REF>(A, S, Vbp, slot, bid, nblk, smem, s_inv_ready, true))
                     return false;

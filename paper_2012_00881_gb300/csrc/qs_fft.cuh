@@ -305,6 +305,29 @@ __device__ __noinline__ int fft(int a, int b, int tab, int N, int lgG, int gl) {
     return a;
 }
 
+// Lines of real fields: one field (S = 1), whose line p is rows (in the column
+// phase, columns) 2p and 2p + 1, or two (S = 2), each with lines of its own, so
+// that a small field keeps its own relative accuracy beside a large one (as the
+// two parts of one complex line the larger one's rounding reaches the other).
+// Their lines lie one after the other, field c's rows at c N^2; row line 2p + c
+// is line p of field c, column line c N / 2 + p likewise.
+template <int S>
+__device__ __forceinline__ size_t row_base(int line, int N) {
+    if constexpr (S == 1) return (size_t)(2 * line) * N;
+    return ((size_t)(line & 1) * N + (line & ~1)) * N;
+}
+// row y of column line `line`, in complex numbers
+template <int S>
+__device__ __forceinline__ size_t column_at(int y, int line, int N) {
+    const size_t at = (size_t)y * (N / 2) + line;
+    return S == 2 && line >= N / 2 ? at + (size_t)(N - 1) * (N / 2) : at;
+}
+template <int NC, int S>
+__device__ __forceinline__ int lines_of(int N) {
+    static_assert(NC == 1 || S == 1, "stacked fields are real");
+    return NC == 2 || S == 2 ? N : N / 2;
+}
+
 // log2 of the lines a block takes at a time: as few as spread nl lines over nblk
 // blocks in one round, at most gmax.
 __device__ __forceinline__ int lines_at_once(int nl, int nblk, int gmax) {
@@ -325,7 +348,7 @@ __device__ __forceinline__ V sample(V v, int i) {
 
 // The second half of rows_forward: transform of the filled lines l0 ... and
 // the coefficients (times 2) to `out`.
-template <typename T, int NC>
+template <typename T, int NC, int S>
 __device__ __noinline__ void rows_forward_rest(int a, int b, int tab, int N, int l0, int lgG, int gl,
                                                V2<T> *out) {
     using V = V2<T>;
@@ -352,7 +375,7 @@ __device__ __noinline__ void rows_forward_rest(int a, int b, int tab, int N, int
             o[j] = c;
             if (two) o[N - j] = d;
         } else {
-            T *o = (T *)out + (size_t)(2 * (l0 + D.g)) * N;
+            T *o = (T *)out + row_base<S>(l0 + D.g, N);
             o[j] = c.x;
             o[N + j] = c.y;
             if (two) {
@@ -367,11 +390,11 @@ __device__ __noinline__ void rows_forward_rest(int a, int b, int tab, int N, int
 // Rows forward.  Two components (NC = 2): line y is the complex row of both.
 // One component: line p is rows 2p (real part) and 2p + 1.  load(line, x) gives
 // the samples; the coefficients go to `out`, complex [y][j] or real [y][j].
-template <typename T, int NC, typename F>
+template <typename T, int NC, int S = 1, typename F>
 __device__ __forceinline__ void rows_forward(const Lines &P, int bid, int nblk, V2<T> *out,
                                              F load) {
     using V = V2<T>;
-    const int N = P.N, nl = NC == 2 ? N : N / 2;
+    const int N = P.N, nl = lines_of<NC, S>(N);
     const int lgG = lines_at_once(nl, nblk, P.gmax), G = 1 << lgG;
     const Deal D(lgG);
     V *const a = cplx_at<T>(P.a);
@@ -382,7 +405,7 @@ __device__ __forceinline__ void rows_forward(const Lines &P, int bid, int nblk, 
             if (x & 1) v = mk<T>(-v.x, -v.y);
             a[D.g * line_len<T>(N) + pad<T>(slot_of(x, N))] = v;
         }
-        rows_forward_rest<T, NC>(P.a, buf_b<T>(P), P.tab, N, l0, lgG, gl, out);
+        rows_forward_rest<T, NC, S>(P.a, buf_b<T>(P), P.tab, N, l0, lgG, gl, out);
     }
 }
 
@@ -392,13 +415,13 @@ __device__ __forceinline__ float recip(float d) { return 1.f / d; }
 // The rest of `columns` after its lines are filled: forward, times
 // 1 / (4 N^2 (lam_x + lam_y - kbar)), inverse, and the store.  kbar: a real
 // number, or a complex one (two components as one complex field).
-template <typename T, int NC, typename K>
+template <typename T, int NC, int S, typename K>
 __device__ __noinline__ void columns_rest(int a, int b, int tab, int N, int l0, int lgG, int gl,
                                           V2<T> *out, K kbar) {
     constexpr bool cplx = !std::is_same<K, T>::value;
     static_assert(!cplx || NC == 2, "a complex shift needs a complex field");
     using V = V2<T>;
-    const int nl = NC == 2 ? N : N / 2, G = 1 << lgG;
+    const int G = 1 << lgG;
     const Deal D(lgG);
     const T c4 = recip(T(4 * N * N));
     const V *const dct = dct_table<T>(tab, N);
@@ -406,7 +429,8 @@ __device__ __noinline__ void columns_rest(int a, int b, int tab, int N, int l0, 
     __syncthreads();
     const int f = fft<T>(a, b, tab, N, lgG, gl);
     for (int j = D.g < gl ? D.j0 : N; 2 * j <= N; j += D.stride) {
-        const int l = l0 + D.g;
+        int l = l0 + D.g;
+        if (S == 2 && l >= N / 2) l -= N / 2;
         T kr;
         if constexpr (cplx) kr = kbar.x;
         else kr = kbar;
@@ -442,7 +466,7 @@ __device__ __noinline__ void columns_rest(int a, int b, int tab, int N, int l0, 
         const int y = t >> lgG, g = t & (G - 1);
         if (g >= gl) continue;
         const V v = r[g * line_len<T>(N) + pad<T>(slot_of(y, N))];
-        out[(size_t)y * nl + l0 + g] = sample(v, y);
+        out[NC == 2 ? (size_t)y * N + l0 + g : column_at<S>(y, l0 + g, N)] = sample(v, y);
     }
     __syncthreads();
 }
@@ -450,11 +474,11 @@ __device__ __noinline__ void columns_rest(int a, int b, int tab, int N, int l0, 
 // Columns: load(y, line) gives the row coefficients; the solution's row
 // coefficients go to `out`.  The one-component array seen as complex pairs puts
 // columns 2p and 2p + 1 into line p.
-template <typename T, int NC, typename K, typename F>
+template <typename T, int NC, int S = 1, typename K, typename F>
 __device__ __forceinline__ void columns(const Lines &P, int bid, int nblk, V2<T> *out, K kbar,
                                         F load) {
     using V = V2<T>;
-    const int N = P.N, nl = NC == 2 ? N : N / 2;
+    const int N = P.N, nl = lines_of<NC, S>(N);
     const int lgG = lines_at_once(nl, nblk, P.gmax), G = 1 << lgG;
     V *const a = cplx_at<T>(P.a);
     for (int l0 = bid * G; l0 < nl; l0 += nblk * G) {
@@ -466,13 +490,13 @@ __device__ __forceinline__ void columns(const Lines &P, int bid, int nblk, V2<T>
             if (y & 1) v = mk<T>(-v.x, -v.y);
             a[g * line_len<T>(N) + pad<T>(slot_of(y, N))] = v;
         }
-        columns_rest<T, NC, K>(P.a, buf_b<T>(P), P.tab, N, l0, lgG, gl, out, kbar);
+        columns_rest<T, NC, S, K>(P.a, buf_b<T>(P), P.tab, N, l0, lgG, gl, out, kbar);
     }
 }
 
 // The first half of rows_inverse: coefficients of lines l0 ... to samples;
 // returns the offset of the buffer that holds their conjugates (see sample).
-template <typename T, int NC>
+template <typename T, int NC, int S>
 __device__ __noinline__ int rows_inverse_first(int a, int b, int tab, int N, int l0, int lgG, int gl,
                                                const V2<T> *in) {
     using V = V2<T>;
@@ -484,7 +508,7 @@ __device__ __noinline__ int rows_inverse_first(int a, int b, int tab, int N, int
             if constexpr (NC == 2) {
                 return in[(size_t)l * N + jj];
             } else {
-                const T *o = (const T *)in + (size_t)(2 * l) * N;
+                const T *o = (const T *)in + row_base<S>(l, N);
                 return mk<T>(o[jj], o[N + jj]);
             }
         };
@@ -504,17 +528,17 @@ __device__ __noinline__ int rows_inverse_first(int a, int b, int tab, int N, int
 }
 
 // Rows inverse: store(line, x, value) takes the solution's samples.
-template <typename T, int NC, typename F>
+template <typename T, int NC, int S = 1, typename F>
 __device__ __forceinline__ void rows_inverse(const Lines &P, int bid, int nblk, const V2<T> *in,
                                              F store) {
     using V = V2<T>;
-    const int N = P.N, nl = NC == 2 ? N : N / 2;
+    const int N = P.N, nl = lines_of<NC, S>(N);
     const int lgG = lines_at_once(nl, nblk, P.gmax), G = 1 << lgG;
     const Deal D(lgG);
     for (int l0 = bid * G; l0 < nl; l0 += nblk * G) {
         const int gl = min(G, nl - l0);
         const V *r = cplx_at<T>(
-            rows_inverse_first<T, NC>(P.a, buf_b<T>(P), P.tab, N, l0, lgG, gl, in));
+            rows_inverse_first<T, NC, S>(P.a, buf_b<T>(P), P.tab, N, l0, lgG, gl, in));
         for (int x = D.g < gl ? D.j0 : N; x < N; x += D.stride) {
             store(l0 + D.g, x, sample(r[D.g * line_len<T>(N) + pad<T>(slot_of(x, N))], x));
         }
@@ -522,30 +546,36 @@ __device__ __forceinline__ void rows_inverse(const Lines &P, int bid, int nblk, 
     }
 }
 
-// Rows inverse and, of what next(line, x, value) makes of the samples, rows
-// forward again, in another storage type if asked.  Two components only when
-// the types differ.
-template <typename T, typename U, int NC, typename F>
+// Rows inverse and, of what next(row, x, value) makes of the samples of two
+// fields, rows forward of two components again, in another storage type if asked.
+// The fields are the parts of complex rows (S = 1) or stacked (S = 2: a block
+// takes pairs of lines, rows 2p and 2p + 1 of both fields; needs P.gmax >= 2).
+template <typename T, typename U, int S, typename F>
 __device__ __forceinline__ void rows_inverse_forward(const Lines &P, const Lines &PU, int bid,
                                                      int nblk, const V2<T> *in, V2<U> *out,
                                                      F next) {
     using V = V2<T>;
-    const int N = P.N, nl = NC == 2 ? N : N / 2, b = buf_b<T>(P);
-    const int lgG = lines_at_once(nl, nblk, P.gmax), G = 1 << lgG;
+    const int N = P.N, b = buf_b<T>(P);
+    const int lgG = max(S - 1, lines_at_once(N, nblk, P.gmax)), G = 1 << lgG;
     const Deal D(lgG);
-    for (int l0 = bid * G; l0 < nl; l0 += nblk * G) {
-        const int gl = min(G, nl - l0);
-        const int f = rows_inverse_first<T, NC>(P.a, b, P.tab, N, l0, lgG, gl, in);
+    for (int l0 = bid * G; l0 < N; l0 += nblk * G) {
+        const int gl = min(G, N - l0);
+        const int f = rows_inverse_first<T, 3 - S, S>(P.a, b, P.tab, N, l0, lgG, gl, in);
         const int o = f == P.a ? b : P.a;  // the free buffer: no smaller than U needs
-        const V *r = cplx_at<T>(f) + D.g * line_len<T>(N);
+        const V *r = cplx_at<T>(f) + (S == 2 ? D.g & ~1 : D.g) * line_len<T>(N);
         V2<U> *q = cplx_at<U>(o) + D.g * line_len<U>(N);
         for (int x = D.g < gl ? D.j0 : N; x < N; x += D.stride) {
             const int at = slot_of(x, N);
-            V2<U> w = next(l0 + D.g, x, sample(r[pad<T>(at)], x));
+            V v = sample(r[pad<T>(at)], x);
+            if constexpr (S == 2) {
+                const V c = sample(r[line_len<T>(N) + pad<T>(at)], x);
+                v = D.g & 1 ? mk<T>(v.y, c.y) : mk<T>(v.x, c.x);
+            }
+            V2<U> w = next(l0 + D.g, x, v);
             if (x & 1) w = mk<U>(-w.x, -w.y);
             q[pad<U>(at)] = w;
         }
-        rows_forward_rest<U, NC>(o, f, PU.tab, N, l0, lgG, gl, out);
+        rows_forward_rest<U, 2, 1>(o, f, PU.tab, N, l0, lgG, gl, out);
     }
 }
 

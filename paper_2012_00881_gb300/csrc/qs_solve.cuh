@@ -1124,49 +1124,53 @@ __device__ void zero_solution(const EngineArgs &A, const SolveSpec &V, int bid, 
         }
 }
 
-// lap_h u = f for one field, or two at once as the parts of a complex one, in
-// three grid phases, in pairs of floats: their 47 bits leave a residual of
-// 1e-13.  (In float64 the phases are bound by the FP64 pipe: two fields at
-// 256^2 37 us, pairs 28; at 512^2 96 and 57.)  load(line, x) gives the source at
-// a line's point (two fields, or rows 2 line and 2 line + 1 of one field) and
-// store(line, x, value) takes the solution.
+// lap_h u = f for one field, or two at once, in three grid phases, in pairs of
+// floats: their 47 bits leave a residual of 1e-13.  (In float64 the phases are bound
+// by the FP64 pipe: two fields at 256^2 37 us, pairs 28; at 512^2 96 and 57.)  Two
+// fields keep lines of their own: B_z is often orders of magnitude below E_z, and as
+// the imaginary part beside it its residual was 4e-10 of its source on a 64^2
+// linear wake, 3e-8 on a 256^2 blowout.  load(line, x) gives rows 2p and 2p + 1 of a
+// field at the line's point and store(line, x, value) takes the solution.
 template <int NC, typename L>
 __device__ __forceinline__ void poisson_rows(const EngineArgs &A, int bid, int nblk, L load) {
-    qsfft::rows_forward<qsff::Ff, NC>(fft_lines<qsff::Ff>(A), bid, nblk, (qsfft::Ff2 *)A.fft.t1,
-                                      load);
+    qsfft::rows_forward<qsff::Ff, 1, NC>(fft_lines<qsff::Ff>(A), bid, nblk,
+                                         (qsfft::Ff2 *)A.fft.t1, load);
 }
 template <int NC>
 __device__ __noinline__ void poisson_columns(const EngineArgs &A, int bid, int nblk) {
     const qsfft::Ff2 *const t1 = (const qsfft::Ff2 *)A.fft.t1;
-    const int nl = NC == 2 ? A.N : A.N / 2;
-    qsfft::columns<qsff::Ff, NC>(fft_lines<qsff::Ff>(A), bid, nblk, (qsfft::Ff2 *)A.fft.t2,
-                                 qsff::Ff(0.f, 0.f),
-                                 [&](int y, int l) { return t1[(size_t)y * nl + l]; });
+    const int N = A.N;
+    qsfft::columns<qsff::Ff, 1, NC>(
+        fft_lines<qsff::Ff>(A), bid, nblk, (qsfft::Ff2 *)A.fft.t2, qsff::Ff(0.f, 0.f),
+        [&](int y, int l) { return t1[qsfft::column_at<NC>(y, l, N)]; });
     if (bid == 0 && threadIdx.x == 0) A.sc->vcycles[NC - 1] += 1;
 }
 template <int NC, typename F>
 __device__ __forceinline__ void poisson_inverse(const EngineArgs &A, int bid, int nblk, F store) {
-    qsfft::rows_inverse<qsff::Ff, NC>(fft_lines<qsff::Ff>(A), bid, nblk,
-                                      (const qsfft::Ff2 *)A.fft.t2, store);
+    qsfft::rows_inverse<qsff::Ff, 1, NC>(fft_lines<qsff::Ff>(A), bid, nblk,
+                                         (const qsfft::Ff2 *)A.fft.t2, store);
 }
 
 template <int NC>
 __device__ bool direct_poisson(const EngineArgs &A, const Sync &S, const SolveSpec &V, int bid,
                                int nblk) {
-    const int N = A.N, ld = NC == 2 ? N : 2 * N;
-    const double *const f0 = V.f[0], *const f1 = NC == 2 ? V.f[1] : V.f[0] + N;
-    double *const u0 = V.u[0], *const u1 = NC == 2 ? V.u[1] : V.u[0] + N;
+    const int N = A.N;
+    // field and first row of a line
+    auto field = [](int l) { return NC == 2 ? l & 1 : 0; };
+    auto row = [](int l) { return NC == 2 ? l & ~1 : 2 * l; };
     poisson_rows<NC>(A, bid, nblk, [&](int l, int x) {
-        const size_t i = (size_t)l * ld + x;
-        return qsfft::mk<qsff::Ff>(qsff::split(f0[i]), qsff::split(f1[i]));
+        const double *const f = V.f[field(l)];
+        const size_t i = (size_t)row(l) * N + x;
+        return qsfft::mk<qsff::Ff>(qsff::split(f[i]), qsff::split(f[i + N]));
     });
     SYNC(26);
     poisson_columns<NC>(A, bid, nblk);
     SYNC(27);
     poisson_inverse<NC>(A, bid, nblk, [&](int l, int x, qsfft::Ff2 v) {
-        const size_t i = (size_t)l * ld + x;
-        u0[i] = qsff::join(v.x);
-        u1[i] = qsff::join(v.y);
+        double *const u = V.u[field(l)];
+        const size_t i = (size_t)row(l) * N + x;
+        u[i] = qsff::join(v.x);
+        u[i + N] = qsff::join(v.y);
     });
     SYNC(28);
     return true;
@@ -1261,7 +1265,7 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
             });
             if (!S(52)) return -1;
             float d[16] = {0.f};
-            qsfft::rows_inverse_forward<T, T, 2>(P, P, bid, nblk, t2, tz, [&](int y, int x, C z) {
+            qsfft::rows_inverse_forward<T, T, 1>(P, P, bid, nblk, t2, tz, [&](int y, int x, C z) {
                 const size_t i = (size_t)y * N + x;
                 const T k = dk(i);
                 C r = cr[i], s = qsfft::mk<T>(T(0.f), T(0.f));
