@@ -657,7 +657,7 @@ __device__ int slice_direct(const LzArgs &A, const qsync::GridBarrier<LzScalars>
             });
             if (!gsync(7)) return -1;
             float d[16] = {0.f};
-            qsfft::rows_inverse_forward<Ff, Ff, 2>(
+            qsfft::rows_inverse_forward<Ff, Ff, 1>(
                 P, P, blockIdx.x, gridDim.x, A.t2, A.tz, [&](int y, int x, Ff2 z) {
                     const int p = y * n + x;
                     const Ff k = dk(p);
