@@ -539,6 +539,7 @@ __device__ bool run_adjoint(const EngineArgs &A, const AdjArgs &D, int bid, int 
     int q = (j == A.n_xi - 1) ? 0 : m - 1;
     for (int s = D.n_sub - 1; s >= 0; --s) {
         const Slice Sl = slice_at(A, s, j, q, m);
+        if (A.fft.on && bid == nblk - 1) poisson_test(A);  // of the slice before
         adj_prepare(A, D, Sl, T);
         SYNC(101);
         if (!Sl.last) {
@@ -552,6 +553,7 @@ __device__ bool run_adjoint(const EngineArgs &A, const AdjArgs &D, int bid, int 
         SYNC(104);
         if (!mg_solve<REF>(A, S, Veb, slot, bid, nblk, smem, s_inv_ready)) return false;
         adj_jperp(A, D, T);
+        if (A.fft.on) poisson_sums<2>(A, Veb, T);
         SYNC(105);
         adj_moments<R>(A, D, Sl, T);
         SYNC(106);
@@ -559,6 +561,7 @@ __device__ bool run_adjoint(const EngineArgs &A, const AdjArgs &D, int bid, int 
         SYNC(107);
         if (!mg_solve<REF>(A, S, Vpsi, slot, bid, nblk, smem, s_inv_ready)) return false;
         adj_density<R>(A, D, Sl, T);
+        if (A.fft.on) poisson_sums<1>(A, Vpsi, T);
         if (lead) {
             sc->slices += 1;
             sc->fnorm[0][0] = sc->fnorm[0][1] = 0.0;
@@ -578,6 +581,7 @@ __device__ bool run_adjoint(const EngineArgs &A, const AdjArgs &D, int bid, int 
             }
         }
     }
+    if (A.fft.on && bid == nblk - 1) poisson_test(A);
     return true;
 }
 

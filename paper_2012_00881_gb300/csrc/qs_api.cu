@@ -411,6 +411,9 @@ int create_impl(qs_ctx *c) {
         f.gmax = 1;
         while (f.gmax < 8 && 4 * f.gmax * line <= 76 * 1024) f.gmax *= 2;
         size_t need = c->block_offset + 2 * f.gmax * line;
+        // (and, over them, a thread's nine sums of the residuals)
+        const size_t sums = c->block_offset + 9 * sizeof(double) * QS_ENGINE_THREADS;
+        if (need < sums) need = sums;
         if (need < c->engine_smem) need = c->engine_smem;
         need = (need + 255) & ~(size_t)255;
         const size_t tabs = (size_t)c->N * (ref ? 36 : 24) + (size_t)(c->N / 2 + 1) * (ref ? 24 : 16);
@@ -823,6 +826,9 @@ static int step_finish(qs_ctx *c, qs_step_stats *stats, double gpu_ms) {
     DevScalars hs;
     CK(cudaMemcpy(&hs, c->sc, sizeof(hs), cudaMemcpyDeviceToHost), "copy scalars");
     c->have_step = true;
+    for (int k = 0; k < 3; ++k)  // the direct solves' largest residuals
+        if (hs.pworst[k][1] > 0.0)
+            hs.max_relres = std::max(hs.max_relres, std::sqrt(hs.pworst[k][0] / hs.pworst[k][1]));
     int status = QS_OK;
     if (hs.err != 0) {
         status = hs.err;
@@ -832,7 +838,8 @@ static int step_finish(qs_ctx *c, qs_step_stats *stats, double gpu_ms) {
         else
             fail(c, status, "device wait timed out at phase %d", hs.err_where);
     } else if (hs.not_converged) {
-        status = fail(c, QS_ERR_NOT_CONVERGED, "a multigrid solve reached %d V-cycles (relres %g)",
+        status = fail(c, QS_ERR_NOT_CONVERGED,
+                      "a field solve did not converge (%d V-cycles at most, relres %g)",
                       g.mg_max_vcycles, hs.max_relres);
     } else if (g.max_psi_guard_hits >= 0 && (int64_t)hs.guard_hits > g.max_psi_guard_hits) {
         status = fail(c, QS_ERR_PSI_FLOOR, "1+psi clamped %llu times", hs.guard_hits);
@@ -1080,7 +1087,8 @@ int read_scalars(qs_ctx *c, DevScalars &hs, const char *what) {
     if (hs.err != 0) return fail(c, hs.err, "%s: device wait timed out at phase %d", what,
                                  hs.err_where);
     if (hs.not_converged)
-        return fail(c, QS_ERR_NOT_CONVERGED, "%s: a multigrid solve reached %d V-cycles", what,
+        return fail(c, QS_ERR_NOT_CONVERGED,
+                    "%s: a field solve did not converge (%d V-cycles at most)", what,
                     c->cfg.mg_max_vcycles);
     return QS_OK;
 }

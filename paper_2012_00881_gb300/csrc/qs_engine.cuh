@@ -746,7 +746,7 @@ __device__ bool rows_eb_bp(const EngineArgs &A, const Sync &S, const PS<P> &Q, c
     using C = qsfft::V2<T>;
     const int n = A.N;
     const double inv2h = 0.5 * A.inv_h;
-    double sx2 = 0.0, sy2 = 0.0;
+    double s2[2] = {0.0, 0.0};
     const Ff fl = qsff::split(A.psi_floor), i2h = qsff::split(inv2h);
     C *const cr = (C *)A.fft.cr;
     auto next = [&](int iy, int ix, Ff2 v) {
@@ -821,8 +821,8 @@ __device__ bool rows_eb_bp(const EngineArgs &A, const Sync &S, const PS<P> &Q, c
         A.f_bx[i] = fx;
         A.f_by[i] = fy;
         cr[i] = r;
-        sx2 += fx * fx;
-        sy2 += fy * fy;
+        s2[0] += fx * fx;
+        s2[1] += fy * fy;
         return r;
     };
     const qsfft::Lines PF = fft_lines<Ff>(A), PT = fft_lines<T>(A);
@@ -842,9 +842,85 @@ __device__ bool rows_eb_bp(const EngineArgs &A, const Sync &S, const PS<P> &Q, c
             return next(iy, ix, qsfft::mk<Ff>(qsff::split(A.ez[i]), qsff::split(A.bz[i])));
         });
     }
-    block_sum_wide(sx2, sy2, A.sc->fnorm[2]);
+    block_sum_wide(s2, A.sc->fnorm[2]);
     return true;
 }
+
+// The sums of poisson_test: residuals of psi, E_z and B_z with their sources
+// formed anew, at cells q0 ... q1.  Bound by the FP64 pipe, 27 instructions a cell.
+// acc: a thread's sums of the parts before (not the first) and after (not the last).
+template <typename P>
+__device__ __noinline__ void poisson_residuals(const EngineArgs &A, const PS<P> &Q,
+                                               const double *ncur, int q0, int q1, Thr T,
+                                               double *acc, bool first, bool last) {
+    const int n = A.N;
+    const double ih2 = A.lev_inv_h2[0], inv2h = 0.5 * A.inv_h;
+    const Ff i2h = qsff::split(inv2h);
+    double s[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) s[k] = first ? 0.0 : acc[k];
+    for (qsmg::Walk w(q0 + T.t0, T.nt, n); w.q < q1; w.next()) {
+        const int i = w.q, ix = w.col, iy = w.row;
+        double f[2];
+        if constexpr (sizeof(P) == 8) {
+            f[0] = -(dx0(Q.m[M_JX], n, ix, i, inv2h) + dy0(Q.m[M_JY], n, iy, i, inv2h));
+            f[1] = dx0(Q.m[M_JY], n, ix, i, inv2h) - dy0(Q.m[M_JX], n, iy, i, inv2h);
+        } else {
+            f[0] = qsff::join(eb_source(A, 0, n, ix, iy, i2h));
+            f[1] = qsff::join(eb_source(A, 1, n, ix, iy, i2h));
+        }
+        poisson_point(A.psi, ncur[i] - A.n_ion[i], n, ix, iy, i, ih2, s, 0);
+        poisson_point(A.ez, f[0], n, ix, iy, i, ih2, s, 1);
+        poisson_point(A.bz, f[1], n, ix, iy, i, ih2, s, 2);
+    }
+    if (last) {
+        block_sum_wide(s, &A.sc->pchk[0][0]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 9; ++k) acc[k] = s[k];
+    }
+}
+
+// These residuals beside the B_perp solve.  Its phases leave blocks without a line
+// (G lines a block, a power of two: 24 of 152 at 128^2 to 512^2): they do a part of
+// the cells in each phase, of 2 N cells a block, which takes less than the others'
+// transforms do.  By all blocks in one phase the residuals took 8.3 us of a 256^2
+// slice, in this way less than one (refined wake 32.4 ms without, 32.1 with; 512^2
+// channel 80.4 and 81.1).  Where no block is idle all do them in the first phase.
+template <typename P>
+struct PoissonCheck {
+    const EngineArgs &A;
+    const PS<P> &Q;
+    const double *ncur;
+    int rank, cnt, part, parts;
+    __device__ PoissonCheck(const EngineArgs &A_, const PS<P> &Q_, const double *ncur_, int bid,
+                            int nblk)
+        : A(A_), Q(Q_), ncur(ncur_), rank(bid), cnt(nblk), part(0), parts(1) {
+        const int n = A.N, G = 1 << qsfft::lines_at_once(n, nblk, A.fft.gmax);
+        const int busy = (n + G - 1) / G;
+        if (busy < nblk) {
+            rank = bid - busy;
+            cnt = nblk - busy;
+            const int per = cnt * max(2 * n, 256);
+            parts = (n * n + per - 1) / per;
+            if (rank < 0) part = parts;
+        }
+    }
+    __device__ void operator()() {
+        if (part == parts) return;
+        const int nn = A.N * A.N, len = (nn + parts - 1) / parts;
+        // the sums between the parts: over the line buffers, which an idle block
+        // does not use
+        double *const acc =
+            (double *)(qsfft::dyn_smem() + A.block_smem_offset) + 9 * (int)threadIdx.x;
+        poisson_residuals<P>(A, Q, ncur, part * len, min(nn, (part + 1) * len),
+                             grid_thr(rank, cnt), acc, part == 0, part + 1 == parts);
+        ++part;
+    }
+    __device__ void rest() {
+        while (part < parts) (*this)();
+    }
+};
 
 // (double)i for 0 <= i < 2^31 without a conversion: 2^52 + i is exact
 __device__ __forceinline__ double whole(int i) {
@@ -1276,6 +1352,7 @@ __device__ bool run_step(const EngineArgs &A, int bid, int nblk, const Sync &S, 
             const Guess g = s_ctl.g;
             const double frac = s_ctl.frac;
             if (A.fft.on) {
+                if (bid == nblk - 1) poisson_test(A);  // of the slice before
                 rows_psi<P>(A, Q, ncur, nnext, base, j, q, frac, bid, nblk);
                 SYNC(2);
                 poisson_columns<1>(A, bid, nblk);
@@ -1290,12 +1367,14 @@ __device__ bool run_step(const EngineArgs &A, int bid, int nblk, const Sync &S, 
                 SYNC(29);
                 if (!rows_eb_bp<P>(A, S, Q, ncur, bid, nblk)) return false;
                 SYNC(5);
-                if (!mg_solve<REF>(A, S, Vbp, slot, bid, nblk, smem, s_inv_ready, true))
+                PoissonCheck<P> check(A, Q, ncur, bid, nblk);
+                if (!mg_solve<REF>(A, S, Vbp, slot, bid, nblk, smem, s_inv_ready, true, check))
                     return false;
+                check.rest();
             } else {
                 phase_psi_rhs<P>(A, Q, ncur, nnext, base, j, q, frac, T, g);
                 if (!S(2)) return false;
-                if (!mg_solve<REF>(A, S, Vpsi, slot, bid, nblk, smem, s_inv_ready)) return false;
+                if (!mg_cycles<REF>(A, S, Vpsi, slot, bid, nblk, smem, s_inv_ready)) return false;
                 if (REF) {  // psi as pairs, for the gathers
                     for (int i = T.t0; i < A.N * A.N; i += T.nt) {
                         const qsff::Ff v = qsff::split(A.psi[i]);
@@ -1307,10 +1386,10 @@ __device__ bool run_step(const EngineArgs &A, int bid, int nblk, const Sync &S, 
                 if (!S(3)) return false;
                 phase_assemble1<P>(A, Q, ncur, j, q, frac, T, g);
                 if (!S(4)) return false;
-                if (!mg_solve<REF>(A, S, Veb, slot, bid, nblk, smem, s_inv_ready)) return false;
+                if (!mg_cycles<REF>(A, S, Veb, slot, bid, nblk, smem, s_inv_ready)) return false;
                 phase_assemble2<P>(A, Q, ncur, T, g);
                 if (!S(5)) return false;
-                if (!mg_solve<REF>(A, S, Vbp, slot, bid, nblk, smem, s_inv_ready)) return false;
+                if (!mg_cycles<REF>(A, S, Vbp, slot, bid, nblk, smem, s_inv_ready)) return false;
             }
             phase_push<P>(A, Q, nnext, base, last, j, dxi, pk, sub, T, bid, nblk, smem);
             ++sub;
@@ -1359,6 +1438,7 @@ __device__ bool run_step(const EngineArgs &A, int bid, int nblk, const Sync &S, 
         __syncthreads();
         m = s_ctl.m;
     }
+    if (A.fft.on && bid == nblk - 1) poisson_test(A);
     return true;
 }
 

@@ -22,6 +22,10 @@ struct DevScalars {
     double fnorm[3][2];            // ||f||^2 of the psi / (Ez,Bz) / (Bx,By) solves
     float cgd[4][16];              // conjugate gradients: dot products per component, ring of 4
     double ksum;                   // sum of kappa over the cells of this slice
+    // direct Poisson solves (psi, E_z, B_z): ||r||^2, ||u||^2, ||f||^2 of this slice,
+    // and the ||r||^2, ||f||^2 of the slice whose ratio is the largest
+    double pchk[3][3];
+    double pworst[3][2];
     unsigned long long vmax_bits[2];  // V_max of a push (bits of a double >= 0)
     unsigned long long guard_hits;
     long long vcycles[3];

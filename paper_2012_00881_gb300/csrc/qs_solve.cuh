@@ -173,25 +173,26 @@ __device__ void block_sum4f(float v[4]) {
     __syncthreads();  // red4 is reused by the next call
 }
 
-// Adds the block's sums of a and b (>= 0; squares) to dst[0] and dst[1].  The
+// Adds the block's sums of v[0 .. K) (>= 0; squares) to dst[0 .. K).  The
 // values keep float64's range and the sums float32's precision, each warp's
 // with a power of two of its own: a norm may be of 1e-30 or of 1e+30, which
 // squares in float32 are not.  (A float64 sum is 10 additions of 64 cycles a
 // warp and value.)
-__device__ void block_sum_wide(double a, double b, double *dst) {
-    __shared__ float sm[2][32];
-    __shared__ int se[2][32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = ((int)blockDim.x + 31) >> 5;
+template <int K>
+__device__ void block_sum_wide(const double (&v)[K], double *dst) {
+    constexpr int nw = QS_ENGINE_THREADS / 32;
+    __shared__ float sm[K][nw];
+    __shared__ int se[K][nw];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
-        const double v = c ? b : a;
-        const unsigned hi = (unsigned)__double2hiint(v);
+    for (int c = 0; c < K; ++c) {
+        const unsigned hi = (unsigned)__double2hiint(v[c]);
         const int e = (int)(hi >> 20) & 0x7ff, E = __reduce_max_sync(0xffffffffu, e);
         float m = 0.f;
-        if (e == 0x7ff) m = (float)v;  // infinite or NaN
+        if (e == 0x7ff) m = (float)v[c];  // infinite or NaN
         else if (e > 0 && E - e <= 60)
             m = qsff::split(__hiloint2double((int)(hi + ((unsigned)(1023 - E) << 20)),
-                                             __double2loint(v))).h;
+                                             __double2loint(v[c]))).h;
         for (int o = 16; o; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
         if (lane == 0) {
             sm[c][wid] = m;
@@ -199,7 +200,7 @@ __device__ void block_sum_wide(double a, double b, double *dst) {
         }
     }
     __syncthreads();
-    for (int c = wid; c < 2; c += nw) {
+    for (int c = wid; c < K; c += nw) {
         const int e = lane < nw ? se[c][lane] : 0, E = __reduce_max_sync(0xffffffffu, e);
         float m = lane < nw ? sm[c][lane] : 0.f;
         if (E - e > 60) m = 0.f;
@@ -1124,10 +1125,44 @@ __device__ void zero_solution(const EngineArgs &A, const SolveSpec &V, int bid, 
         }
 }
 
+// Adds |r|^2, |u|^2, |f|^2 of lap_h u = f at a cell to s[3 k ...]: r in float64.
+__device__ __forceinline__ void poisson_point(const double *u, double f, int n, int ix, int iy,
+                                              int i, double ih2, double (&s)[9], int k) {
+    const int nw = qsmg::walls(ix, iy, n);
+    const double d = nw == 0 ? 4.0 : nw == 1 ? 5.0 : 6.0, c = u[i];
+    const double w = ix > 0 ? u[i - 1] : 0.0, e = ix < n - 1 ? u[i + 1] : 0.0;
+    const double a = iy > 0 ? u[i - n] : 0.0, b = iy < n - 1 ? u[i + n] : 0.0;
+    const double r = fma(-ih2, fma(-d, c, (w + e) + (a + b)), f);
+    s[3 * k] += r * r;
+    s[3 * k + 1] += c * c;
+    s[3 * k + 2] += f * f;
+}
+
+// The direct solves' stopping test, after the fact, from the sums of the slice
+// before (cleared here): they leave a residual of 2 to 3e-14 ||u|| / h^2 (26 sides from
+// 8 to 2048; smooth, dipole, noisy and mixed sources; of ||f|| that is 1e-14 to
+// 2e-9), under the bound that the V-cycles stop at.  What fails it is not finite or
+// beyond float32's exponents.  One block, a barrier after the sums.
+__device__ void poisson_test(const EngineArgs &A) {
+    DevScalars *sc = A.sc;
+    const int k = threadIdx.x;
+    if (k >= 3) return;
+    const double rn = vload(&sc->pchk[k][0]), un = vload(&sc->pchk[k][1]),
+                 fn = vload(&sc->pchk[k][2]);
+    sc->pchk[k][0] = sc->pchk[k][1] = sc->pchk[k][2] = 0.0;
+    if (fn == 0.0) return;
+    const double fl = 1e-13 * A.lev_inv_h2[0];
+    const double thr = fmax(fmax(A.mg_tol * A.mg_tol * fn, A.mg_atol * A.mg_atol), fl * fl * un);
+    if (!(rn <= thr && rn <= 1.7e308)) sc->not_converged = 1;
+    if (sc->pworst[k][1] == 0.0 || rn * sc->pworst[k][1] > sc->pworst[k][0] * fn) {
+        sc->pworst[k][0] = rn;
+        sc->pworst[k][1] = fn;
+    }
+}
+
 // lap_h u = f for one field, or two at once, in three grid phases, in pairs of
-// floats: their 47 bits leave a residual of 1e-13.  (In float64 the phases are bound
-// by the FP64 pipe: two fields at 256^2 37 us, pairs 28; at 512^2 96 and 57.)  Two
-// fields keep lines of their own: B_z is often orders of magnitude below E_z, and as
+// floats.  (In float64 the phases are bound by the FP64 pipe: two fields at 256^2
+// 37 us, pairs 28; at 512^2 96 and 57.)  Two fields keep lines of their own: B_z is often orders of magnitude below E_z, and as
 // the imaginary part beside it its residual was 4e-10 of its source on a 64^2
 // linear wake, 3e-8 on a 256^2 blowout.  load(line, x) gives rows 2p and 2p + 1 of a
 // field at the line's point and store(line, x, value) takes the solution.
@@ -1203,11 +1238,12 @@ __device__ bool direct_poisson(const EngineArgs &A, const Sync &S, const SolveSp
 // The sums are of values scaled by a power of two near 1 / ||f||, so that
 // float32 cannot underflow in them.
 // prepared: the source's row transform and copy are in tr and cr already.
+// side(): work besides the solve, called before the barriers of its phases.
 // Returns 1 (converged), 0 (not within its cap: u holds the last iterate and
 // the V-cycles take over), -1 (a barrier failed).
-template <bool REF>
+template <bool REF, typename X>
 __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &V, int &slot,
-                           int bid, int nblk, bool prepared) {
+                           int bid, int nblk, bool prepared, X &side) {
     using T = typename std::conditional<REF, float, qsff::Ff>::type;
     using C = qsfft::V2<T>;
     DevScalars *sc = A.sc;
@@ -1263,6 +1299,7 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
                 }
                 return r;
             });
+            side();
             if (!S(52)) return -1;
             float d[16] = {0.f};
             qsfft::rows_inverse_forward<T, T, 1>(P, P, bid, nblk, t2, tz, [&](int y, int x, C z) {
@@ -1314,6 +1351,7 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
                 return w;
             });
             reduce16(sc, d, sc->cgd[slot & 3], slot, bid);
+            side();
             if (!S(53)) return -1;
             if (threadIdx.x < 32) {  // one lane a component
                 const int c = threadIdx.x;
@@ -1423,6 +1461,24 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
     return result;
 }
 
+// The sums of poisson_test for a solve of mg_solve's.
+template <int NC>
+__device__ void poisson_sums(const EngineArgs &A, const SolveSpec &V, Thr T) {
+    const double ih2 = A.lev_inv_h2[0];
+    double s[9] = {0.0};
+    for (qsmg::Walk w(T.t0, T.nt, A.N); w.q < A.N * A.N; w.next())
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+            poisson_point(V.u[c], V.f[c][w.q], A.N, w.col, w.row, w.q, ih2, s, c);
+    if constexpr (NC == 1) {
+        const double t[3] = {s[0], s[1], s[2]};
+        block_sum_wide(t, A.sc->pchk[0]);
+    } else {
+        const double t[6] = {s[0], s[1], s[2], s[3], s[4], s[5]};
+        block_sum_wide(t, A.sc->pchk[1]);
+    }
+}
+
 // The screened smoother's inverse diagonal, needed only when the V-cycles
 // take over from the conjugate gradients.
 __device__ void screened_diagonal(const EngineArgs &A, Thr T) {
@@ -1436,6 +1492,10 @@ __device__ void screened_diagonal(const EngineArgs &A, Thr T) {
     }
 }
 
+struct Nothing {
+    __device__ void operator()() const {}
+};
+
 // Iterate until, for every component,
 //   ||f - A u|| <= max(tol ||f||, 1e-13 ||u|| / h^2, atol)
 // (the second bound is a small multiple of the rounding level of the
@@ -1443,23 +1503,9 @@ __device__ void screened_diagonal(const EngineArgs &A, Thr T) {
 // Float64 form: V-cycles on u.  Refined form: float64 residual, float32
 // V-cycle on the correction, float64 update (iterative refinement).
 template <bool REF>
-__device__ bool mg_solve(const EngineArgs &A, const Sync &S, const SolveSpec &V, int &slot,
-                         int bid, int nblk, void *smem_base, int *inv_ready,
-                         bool prepared = false) {
+__device__ __noinline__ bool mg_cycles(const EngineArgs &A, const Sync &S, const SolveSpec &V, int &slot,
+                          int bid, int nblk, void *smem_base, int *inv_ready) {
     DevScalars *sc = A.sc;
-    if (A.fft.on) {
-        if (!V.screened)
-            return V.nc == 1 ? direct_poisson<1>(A, S, V, bid, nblk)
-                             : direct_poisson<2>(A, S, V, bid, nblk);
-        const int r = cg_screened<REF>(A, S, V, slot, bid, nblk, prepared);
-        if (r != 0) return r > 0;
-        screened_diagonal(A, grid_thr(bid, nblk));
-        // The cycles move `slot` on without clearing the dot products' ring: the
-        // next slice's iterations would add to what these left in it.
-        if (bid == 0 && threadIdx.x < 64)
-            sc->cgd[threadIdx.x >> 4][threadIdx.x & 15] = 0.f;
-        SYNC(56);
-    }
     // shared memory: [coarsest inverses][coarse levels + work][staged tile]
     void *smem = (char *)smem_base + A.block_smem_offset;
     const int mc = A.lev_n[A.nlev - 1] * A.lev_n[A.nlev - 1];
@@ -1615,6 +1661,27 @@ __device__ bool mg_solve(const EngineArgs &A, const Sync &S, const SolveSpec &V,
         SYNC(23);
     }
     return true;
+}
+
+// A field solve: by transforms and iterations, else by V-cycles.
+template <bool REF, typename X = const Nothing>
+__device__ bool mg_solve(const EngineArgs &A, const Sync &S, const SolveSpec &V, int &slot,
+                         int bid, int nblk, void *smem_base, int *inv_ready,
+                         bool prepared = false, X &side = Nothing()) {
+    if (A.fft.on) {
+        if (!V.screened)
+            return V.nc == 1 ? direct_poisson<1>(A, S, V, bid, nblk)
+                             : direct_poisson<2>(A, S, V, bid, nblk);
+        const int r = cg_screened<REF>(A, S, V, slot, bid, nblk, prepared, side);
+        if (r != 0) return r > 0;
+        screened_diagonal(A, grid_thr(bid, nblk));
+        // The cycles move `slot` on without clearing the dot products' ring: the
+        // next slice's iterations would add to what these left in it.
+        if (bid == 0 && threadIdx.x < 64)
+            A.sc->cgd[threadIdx.x >> 4][threadIdx.x & 15] = 0.f;
+        SYNC(56);
+    }
+    return mg_cycles<REF>(A, S, V, slot, bid, nblk, smem_base, inv_ready);
 }
 
 __device__ __forceinline__ double guard(double a, double floor_, unsigned &hits) {
