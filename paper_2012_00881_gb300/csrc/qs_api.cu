@@ -417,7 +417,8 @@ int create_impl(qs_ctx *c) {
         if (need < c->engine_smem) need = c->engine_smem;
         need = (need + 255) & ~(size_t)255;
         const size_t tabs = (size_t)c->N * (ref ? 36 : 24) + (size_t)(c->N / 2 + 1) * (ref ? 24 : 16);
-        if (need + tabs <= 220 * 1024) {
+        const size_t limit = std::min<size_t>(220 * 1024, qs_engine_smem_limit(g.precision));
+        if (need + tabs <= limit) {
             const size_t smem = c->engine_smem;
             f.tab_off = (int)need;
             c->engine_smem = need + tabs;

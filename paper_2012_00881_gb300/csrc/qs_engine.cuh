@@ -1149,7 +1149,7 @@ __device__ void phase_push(const EngineArgs &A, const PS<P> &Q, double *nnext, b
 // exclusive scan of v over the block (any blockDim.x <= 1024); returns the
 // prefix of this thread and the block total in *total
 __device__ int block_exscan(int v, int *total) {
-    __shared__ int ws[32];
+    int *const ws = (int *)qsfft::sum_scratch();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int x = v;
     for (int o = 1; o < 32; o <<= 1) {

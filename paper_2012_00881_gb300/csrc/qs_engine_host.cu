@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include "qs_cluster.cuh"
+#include "qs_launch.cuh"
 #include "qs_tile.cuh"
 
 const void *qs_kernel_engine(int precision) {
@@ -18,9 +19,7 @@ const void *qs_kernel_engine_batched(int precision) {
 int qs_engine_max_blocks(int device, int precision, size_t smem_bytes, int *blocks, int cluster) {
     const void *fn = qs_kernel_engine(precision);
     int per_sm = 0, sms = 0;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes) !=
-        cudaSuccess)
-        return -1;
+    if (qs_raise_smem_limit(fn) != cudaSuccess) return -1;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, QS_ENGINE_THREADS,
                                                       smem_bytes) != cudaSuccess)
         return -1;
@@ -48,6 +47,17 @@ int qs_engine_max_blocks(int device, int precision, size_t smem_bytes, int *bloc
         if (nc * cluster < *blocks) *blocks = nc * cluster;
     }
     return 0;
+}
+
+size_t qs_engine_smem_limit(int precision) {
+    size_t least = 0;
+    for (const void *fn : {qs_kernel_engine(precision), qs_kernel_engine_batched(precision),
+                           qs_kernel_adjoint(precision)}) {
+        size_t l = 0;
+        if (qs_raise_smem_limit(fn, &l) != cudaSuccess) return 0;
+        if (least == 0 || l < least) least = l;
+    }
+    return least;
 }
 
 size_t qs_cluster_smem_bytes(const int *lev_n, int nlev, int cluster, int tsize) {
@@ -78,9 +88,6 @@ cudaError_t qs_launch_engine_batched(cudaStream_t st, const EngineArgs *list, in
                                      size_t smem_bytes) {
     void *args[] = {(void *)&list, &n_inst, &team, &bs};
     const void *fn = qs_kernel_engine_batched(precision);
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes) !=
-        cudaSuccess)
-        return cudaGetLastError();
     return cudaLaunchCooperativeKernel(fn, dim3(team * teams), dim3(QS_ENGINE_THREADS), args,
                                        smem_bytes, st);
 }
@@ -88,9 +95,7 @@ cudaError_t qs_launch_engine_batched(cudaStream_t st, const EngineArgs *list, in
 int qs_engine_batched_max_blocks(int device, int precision, size_t smem_bytes, int *blocks) {
     const void *fn = qs_kernel_engine_batched(precision);
     int per_sm = 0, sms = 0;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes) !=
-        cudaSuccess)
-        return -1;
+    if (qs_raise_smem_limit(fn) != cudaSuccess) return -1;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, QS_ENGINE_THREADS,
                                                       smem_bytes) != cudaSuccess)
         return -1;
@@ -105,11 +110,7 @@ cudaError_t qs_launch_engine(cudaStream_t st, const EngineArgs &a, int grid_bloc
     EngineArgs copy = a;
     void *args[] = {&copy};
     const void *fn = qs_kernel_engine(a.precision);
-    // the limit is a property of the kernel, shared by every context: set it
-    // for this launch (another context may have set a smaller one)
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem_bytes);
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
     if (a.cl_size <= 1)
         return cudaLaunchCooperativeKernel(fn, dim3(grid_blocks), dim3(QS_ENGINE_THREADS), args,
                                            smem_bytes, st);

@@ -579,11 +579,18 @@ __device__ __forceinline__ void rows_inverse_forward(const Lines &P, const Lines
     }
 }
 
+// Shared scratch of the block's sums (up to 16 warps); a block barrier stands
+// between two uses.
+constexpr int kSumWarps = 16;
+static __device__ __forceinline__ float *sum_scratch() {
+    __shared__ __align__(16) float scratch[18 * kSumWarps];
+    return scratch;
+}
+
 // Sums of 16 values over the block: thread t < 16 returns the sum of v[t].  Each
-// shuffle halves the values a lane holds: 16 shuffles instead of 80.  A block
-// barrier stands between two calls.
+// shuffle halves the values a lane holds: 16 shuffles instead of 80.
 static __device__ float block_sums16(float v[16]) {
-    __shared__ float red[32][17];
+    float (*const red)[17] = (float (*)[17])sum_scratch();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (int)blockDim.x >> 5;
 #pragma unroll
     for (int o = 16; o >= 2; o >>= 1) {

@@ -377,6 +377,8 @@ cudaError_t qs_launch_adjoint(cudaStream_t st, const EngineArgs &a, const AdjArg
 int qs_adjoint_max_blocks(int device, int precision, size_t smem_bytes, int *blocks);
 int qs_engine_max_blocks(int device, int precision, size_t smem_bytes, int *blocks,
                          int cluster = 1);
+// dynamic shared memory that every launch of the form's kernels can have
+size_t qs_engine_smem_limit(int precision);
 size_t qs_cluster_smem_bytes(const int *lev_n, int nlev, int cluster, int tsize);
 size_t qs_engine_smem_bytes(const int *lev_n, int nlev, int block_level_n, int precision,
                             int tile_x, int tile_y, int nu, int nu2, size_t *block_offset,

@@ -49,6 +49,7 @@
 #include "qs.h"
 #include "qs_fft.cuh"
 #include "qs_grid_sync.cuh"
+#include "qs_launch.cuh"
 
 namespace {
 
@@ -1119,9 +1120,7 @@ extern "C" int qs_laser_create(int n, double width, int n_xi, double k0, double 
     st = cuda_status(cudaGetDevice(&dev));
     if (st == QS_OK) st = cuda_status(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     if (st == QS_OK)
-        st = cuda_status(cudaFuncSetAttribute((const void *)laser_kernel,
-                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)s->smem));
+        st = cuda_status(qs_raise_smem_limit((const void *)laser_kernel));
     if (st == QS_OK)
         st = cuda_status(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, laser_kernel, kThreads,
                                                                        s->smem));
@@ -1154,12 +1153,6 @@ extern "C" int qs_laser_advance(qs_laser *s, const double *d_chi, double *d_a, i
     int st = cuda_status(cudaMemsetAsync(A.sc, 0, sizeof(LzScalars), s->stream));
     if (st != QS_OK) return st;
     void *params[] = {&A};
-    // the limit belongs to the kernel, which every envelope object shares
-    if (st == QS_OK)
-        st = cuda_status(cudaFuncSetAttribute((const void *)laser_kernel,
-                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)s->smem));
-    if (st != QS_OK) return st;
     st = cuda_status(cudaLaunchCooperativeKernel((const void *)laser_kernel, dim3(s->grid_blocks),
                                                  dim3(kThreads), params, s->smem, s->stream));
     if (st != QS_OK) return st;

@@ -135,7 +135,7 @@ __device__ __forceinline__ Thr grid_thr(int bid, int nblk) {
 
 // sum over the block; valid in thread 0
 __device__ double block_sum(double v) {
-    __shared__ double red[32];
+    double *const red = (double *)qsfft::sum_scratch();
     for (int o = 16; o; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     __syncthreads();
@@ -152,7 +152,7 @@ __device__ double block_sum(double v) {
 // four float32 sums over the block in one pass (one block barrier); valid in
 // thread 0
 __device__ void block_sum4f(float v[4]) {
-    __shared__ float red4[32][4];
+    float (*const red4)[4] = (float (*)[4])qsfft::sum_scratch();
 #pragma unroll
     for (int k = 0; k < 4; ++k)
         for (int o = 16; o; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
@@ -181,9 +181,11 @@ __device__ void block_sum4f(float v[4]) {
 template <int K>
 __device__ void block_sum_wide(const double (&v)[K], double *dst) {
     constexpr int nw = QS_ENGINE_THREADS / 32;
-    __shared__ float sm[K][nw];
-    __shared__ int se[K][nw];
+    static_assert(K <= 9 && nw <= qsfft::kSumWarps, "scratch");
+    float (*const sm)[nw] = (float (*)[nw])qsfft::sum_scratch();
+    int (*const se)[nw] = (int (*)[nw])(qsfft::sum_scratch() + K * nw);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    __syncthreads();  // the scratch may still be read
 #pragma unroll
     for (int c = 0; c < K; ++c) {
         const unsigned hi = (unsigned)__double2hiint(v[c]);
@@ -220,7 +222,7 @@ __device__ void block_sum_wide(const double (&v)[K], double *dst) {
 }
 
 __device__ float block_max(float v) {
-    __shared__ float redf[32];
+    float *const redf = qsfft::sum_scratch();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int o = 16; o; o >>= 1) v = fmaxf(v, __shfl_down_sync(0xffffffffu, v, o));
     __syncthreads();
@@ -234,7 +236,7 @@ __device__ float block_max(float v) {
     return t;
 }
 __device__ double block_max(double v) {
-    __shared__ double red[32];
+    double *const red = (double *)qsfft::sum_scratch();
     for (int o = 16; o; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
     int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     __syncthreads();
@@ -1560,8 +1562,12 @@ __device__ __noinline__ bool mg_cycles(const EngineArgs &A, const Sync &S, const
     if (REF && A.cl_size > 1)
         return mg_solve_ref_cluster(A, S, V, slot, bid, nblk, smem_base, ci, s_fn);
 #endif
-    __shared__ Hier<double> H64;
-    __shared__ Hier<float> H32;
+    // one of the two, by the form
+    __shared__ __align__(16) unsigned char
+        hier_mem[sizeof(Hier<double>) > sizeof(Hier<float>) ? sizeof(Hier<double>)
+                                                            : sizeof(Hier<float>)];
+    Hier<double> &H64 = *(Hier<double> *)hier_mem;
+    Hier<float> &H32 = *(Hier<float> *)hier_mem;
     __syncthreads();
     if (REF) hier32(A, V, H32);
     else hier64(A, V, H64);
