@@ -277,7 +277,9 @@ int create_fft(qs_ctx *c) {
         grid(c->r64[0], sizeof(double));
         grid(c->r64[1], sizeof(double));
     }
-    CK(cudaMemcpy(base, host.data(), tabs, cudaMemcpyHostToDevice), "tables");
+    // on the context's stream, which may not wait for the default one
+    CK(cudaMemcpyAsync(base, host.data(), tabs, cudaMemcpyHostToDevice, c->st), "tables");
+    CK(cudaStreamSynchronize(c->st), "tables");
     f.on = 1;
     return QS_OK;
 }

@@ -1086,8 +1086,14 @@ extern "C" int qs_laser_create(int n, double width, int n_xi, double k0, double 
         }
         A.tables = reinterpret_cast<const qsfft::Ff *>(p);
         std::vector<qsfft::Ff> tab = qsfft::host_tables(n, width / n);
-        st = cuda_status(cudaMemcpy(p, tab.data(), tab.size() * sizeof(qsfft::Ff),
-                                    cudaMemcpyHostToDevice));
+        // on the object's stream, which may not wait for the default one
+        st = cuda_status(cudaMemcpyAsync(p, tab.data(), tab.size() * sizeof(qsfft::Ff),
+                                         cudaMemcpyHostToDevice, s->stream));
+        if (st == QS_OK) st = cuda_status(cudaStreamSynchronize(s->stream));
+        if (st != QS_OK) {
+            qs_laser_destroy(s);
+            return st;
+        }
         p += (tab_pairs + 1) / 2;
         A.gmax = 1;
         while (A.gmax < 8 && 4 * A.gmax * line <= 76 * 1024) A.gmax *= 2;

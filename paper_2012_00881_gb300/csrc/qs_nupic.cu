@@ -373,9 +373,11 @@ extern "C" int qs_nu_pic_create(int n, const double *x_nodes, const double *y_no
         r = nalloc(s, &d[a][0], (size_t)n + 2);
         for (int k = 1; k < 4 && r == QS_OK; ++k) r = nalloc(s, &d[a][k], (size_t)n);
         for (int k = 0; k < 4 && r == QS_OK; ++k)
-            r = cuda_ok(cudaMemcpy(d[a][k], hv[a][k].data(), hv[a][k].size() * sizeof(double),
-                                   cudaMemcpyHostToDevice));
+            r = cuda_ok(cudaMemcpyAsync(d[a][k], hv[a][k].data(),
+                                        hv[a][k].size() * sizeof(double),
+                                        cudaMemcpyHostToDevice, s->st));
     }
+    if (r == QS_OK) r = cuda_ok(cudaStreamSynchronize(s->st));
     const size_t nn = (size_t)n * n;
     double **grids[] = {&s->n_ion, &s->nstar, &s->f_psi, &s->psi, &s->jx,  &s->jy,
                         &s->txx,   &s->txy,   &s->tyy,   &s->G,   &s->jz,  &s->kap,

@@ -1,7 +1,9 @@
 """Host side of the launches, by the sources (CPU): a kernel's limit of dynamic shared
 memory belongs to the kernel, not to a launch, so that a limit of an object's own size
 would refuse another thread's larger launch.  It is set to one value per kernel, where
-objects are made."""
+objects are made.  And what a kernel reads is copied on the object's own stream: one
+that does not wait for the default stream could launch before a copy there has landed
+(from pageable memory such a copy returns when it is staged)."""
 import os
 import re
 
@@ -20,3 +22,9 @@ def test_shared_memory_limits_are_one_value_per_kernel():
         for m in re.finditer(r"cudaFuncAttributeMaxDynamicSharedMemorySize,\s*([^;]*?)\)+;", s):
             value = re.sub(r"\(int\)|[()\s]", "", m.group(1))
             assert value in ("most", "kStageSmemMax"), (f, m.group(0))
+
+
+def test_nothing_is_copied_to_the_device_on_the_default_stream():
+    for f, s in _sources():
+        for m in re.finditer(r"cudaMemcpy\([^;]*;", s):
+            assert "HostToDevice" not in m.group(0), (f, m.group(0))
