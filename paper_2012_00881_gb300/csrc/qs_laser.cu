@@ -1057,13 +1057,17 @@ extern "C" int qs_laser_create(int n, double width, int n_xi, double k0, double 
     int odd = n;
     while (odd % 2 == 0) odd /= 2;
     const size_t line = (size_t)(n + n / 8 + 1) * sizeof(qsfft::Ff2);  // padded
-    const bool fft = n % 2 == 0 && n >= 8 && n <= 2048 && odd <= 7;
+    bool fft = n % 2 == 0 && n >= 8 && n <= 2048 && odd <= 7;
     size_t elems = 2 * (size_t)n * n;  // u, dlt
     const size_t tab_pairs = 3 * (size_t)n + 2 * (size_t)(n / 2 + 1);
-    if (fft) elems += 10 * (size_t)n * n + (tab_pairs + 1) / 2;
     for (int l = 0; l < levels; ++l) elems += 5 * (size_t)sides[l] * sides[l];
-    const size_t bytes = kScalarBytes + elems * sizeof(double2);
-    int st = cuda_status(cudaMalloc(&s->dev, bytes));
+    const size_t extra = fft ? 10 * (size_t)n * n + (tab_pairs + 1) / 2 : 0;
+    int st = cuda_status(cudaMalloc(&s->dev, kScalarBytes + (elems + extra) * sizeof(double2)));
+    if (st == QS_ERR_OOM && fft) {  // the V-cycles need none of the transforms' grids
+        fft = false;
+        s->dev = nullptr;
+        st = cuda_status(cudaMalloc(&s->dev, kScalarBytes + elems * sizeof(double2)));
+    }
     if (st == QS_OK) st = cuda_status(cudaMallocHost(&s->pinned, sizeof(LzScalars)));
     if (st != QS_OK) {
         qs_laser_destroy(s);
