@@ -220,11 +220,11 @@ __device__ void adj_prepare(const EngineArgs &A, const AdjArgs &D, const Slice &
         }
         A.dpx[i] = cdxo(S.psi, n, ix, i) * inv2h;
         A.dpy[i] = cdyo(S.psi, n, iy, i) * inv2h;
-        D.g_psi[i] = dh ? dh[i] : 0.0;
-        D.g_ez[i] = dh ? dh[fs + i] : 0.0;
-        D.g_bz[i] = dh ? dh[2 * fs + i] : 0.0;
-        D.g_bx[i] = dh ? dh[3 * fs + i] : 0.0;
-        D.g_by[i] = dh ? dh[4 * fs + i] : 0.0;
+        D.g_psi[i] = dh ? D.scale * dh[i] : 0.0;
+        D.g_ez[i] = dh ? D.scale * dh[fs + i] : 0.0;
+        D.g_bz[i] = dh ? D.scale * dh[2 * fs + i] : 0.0;
+        D.g_bx[i] = dh ? D.scale * dh[3 * fs + i] : 0.0;
+        D.g_by[i] = dh ? D.scale * dh[4 * fs + i] : 0.0;
         D.g_dpx[i] = 0.0;
         D.g_dpy[i] = 0.0;
     }

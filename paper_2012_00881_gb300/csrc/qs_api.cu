@@ -1205,6 +1205,19 @@ int qs_step3d_adjoint(qs_ctx *c, const double *d_hist, int checkpoint_every, dou
                      &d.mu_x,  &d.mu_y, &d.nu_ez, &d.nu_bz, &d.nu_psi, &d.f_nu_psi};
     for (int k = 0; k < 20; ++k) *gp[k] = grd + (size_t)k * nn;
     d.d_hist = d_hist;
+    // The solves and the refined form's particles hold cotangents in pairs of
+    // floats: a history cotangent whose largest value is outside 2^-60 ... 2^60 is
+    // taken times a power of two, and the results by its inverse.
+    d.scale = 1.0;
+    if (d_hist) {
+        int *d_e = nullptr, e = 0;
+        AL(B.list, d_e, 1);
+        CK(cudaMemsetAsync(d_e, 0, sizeof(int), st), "memset");
+        CK(qs_launch_max_exponent(st, d_hist, (int64_t)5 * nxi * nn, d_e), "max exponent");
+        CK(cudaMemcpyAsync(&e, d_e, sizeof(int), cudaMemcpyDeviceToHost, st), "copy exponent");
+        CK(cudaStreamSynchronize(st), "max exponent");
+        if (e > 0 && std::abs(e - 1023) > 60) d.scale = std::ldexp(1.0, std::min(1023 - e, 1000));
+    }
     d.d_jzb = d_jzb;
     d.d_nion = d_nion;
     int64_t slices = 0, vc[3] = {0, 0, 0};
@@ -1248,6 +1261,12 @@ int qs_step3d_adjoint(qs_ctx *c, const double *d_hist, int checkpoint_every, dou
         if (r != QS_OK) return r;
         slices += hs.slices;
         for (int q = 0; q < 3; ++q) vc[q] += hs.vcycles[q];
+    }
+    if (d.scale != 1.0) {
+        CK(qs_launch_scale(st, d_jzb, (int64_t)nxi * nn, 1.0 / d.scale), "scale");
+        CK(qs_launch_scale(st, d_w, np, 1.0 / d.scale), "scale");
+        CK(qs_launch_scale(st, d_nion, (int64_t)nn, 1.0 / d.scale), "scale");
+        CK(cudaStreamSynchronize(st), "scale");
     }
     if (stats) {
         std::memset(stats, 0, sizeof(*stats));

@@ -214,6 +214,7 @@ struct AdjArgs {
     double *mu_x, *mu_y, *nu_ez, *nu_bz, *nu_psi, *f_nu_psi;
     // inputs / outputs
     const double *d_hist;  // [5][n_xi][N*N] dL/d(stored fields) or nullptr
+    double scale;          // power of two that the cotangents are held times
     double *d_jzb;         // [n_xi][N*N] dL/d(j_z of the bunches), accumulated
     double *d_nion;        // [N*N] dL/d(n_ion), accumulated
 };
@@ -332,6 +333,9 @@ cudaError_t qs_launch_beam_push_dla(cudaStream_t st, const qs_beam &b, int n, do
                                     int n_xi, double xi_min, double dxi0, const double *hist,
                                     const double *env_n, const double *env_np1, double k0,
                                     double dt, int n_sub);
+// max over the finite v[0 .. n) of their biased exponents into *e (device; zeroed before)
+cudaError_t qs_launch_max_exponent(cudaStream_t st, const double *v, int64_t n, int *e);
+cudaError_t qs_launch_scale(cudaStream_t st, double *v, int64_t n, double s);
 cudaError_t qs_launch_convert(cudaStream_t st, const double *src, float *dst, int64_t n);
 // |a|^2 of n interleaved complex128 values
 cudaError_t qs_launch_abs2(cudaStream_t st, const double *a, double *out, int64_t n);

@@ -74,3 +74,20 @@ def test_envelope_reports_no_solution(qs, bad):
     lz = qs.LaserEnvelope(n, 8.0, n_xi, 5.0, 1.0, 0.2)
     lz.advance(chi, a, raise_on_error=False)
     assert lz.status == qs.QS_ERR_NOT_CONVERGED
+
+
+@pytest.mark.parametrize("form", ["fp64", "fp32r"])
+@pytest.mark.parametrize("k", [-300, -110, 120, 300])
+def test_gradients_scale_with_the_cotangent(qs, form, k):
+    import torch
+    ctx, beam = _context(qs, form, n_xi=4)
+    ctx.step3d([beam])
+    g = torch.Generator(device="cuda").manual_seed(1)
+    d = torch.randn((5, 4, 32, 32), dtype=torch.float64, device="cuda", generator=g)
+    ref = ctx.step3d_adjoint(d)
+    got = ctx.step3d_adjoint(d * 2.0 ** k)
+    ctx.close()
+    # two runs of one form: the order of the reductions, the solves' tolerance
+    tol = 1e-9 if form == "fp64" else 1e-7
+    for a, b in zip(got[:3], ref[:3]):
+        assert float((a / 2.0 ** k - b).norm()) <= tol * float(b.norm()) and float(b.norm()) > 0
