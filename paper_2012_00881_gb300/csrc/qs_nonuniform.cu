@@ -47,17 +47,20 @@
 // products with n x n matrices.  GMRES on the residual equation in float32,
 // right-preconditioned with it (Saad and Schultz, SIAM J. Sci. Stat. Comput. 7
 // (1986) 856; the preconditioned vectors are kept, so it need not be exact),
-// to 1e-5 a round; then u += e and the float64 residual, which is also the
-// stopping test.  The third-order terms and the variation of M leave a
-// perturbation that takes 7 iterations in all (M = 0) to 13 (a blowout's M) on
-// the three-region grid and up to 16 on alternating spacings, 21 us each for
+// to 1e-6 a round; then u += e and the float64 residual, which is also the
+// stopping test: its bound is the tolerance, its aim a hundredth of it (stopped at
+// 0.3 of the tolerance the fields' errors were up to 70 times the V-cycles', 5e-11 at
+// 255^2 and 5e-10 on alternating spacings; now 1e-12, as the V-cycles').  The
+// third-order terms and the variation of M leave a
+// perturbation that takes 10 iterations in all (M = 0) to 18 (a blowout's M) on
+// the three-region grid and up to 32 on alternating spacings, 21 us each for
 // one field at 255^2 and 29 for two, against 12 V-cycles of 180 us.  The
 // V-cycles take over when that does not converge.  An iteration is two grid
 // phases: columns, and rows with the operator, its dot products and the row
 // transform of A z, whose recurrence the column phase applies.  (With a phase
 // each for the rows, the operator, the new vector and its transform, and 3e-4 a
 // round with an update phase of its own, a 255^2 set of three solves took 1,380
-// us; so 1,180.)
+// us; so 1,180; with the aim 1,450.)
 //
 // Every wait is bounded; a timeout sets an error word that ends the kernel at
 // the next barrier.
@@ -1167,24 +1170,30 @@ __device__ int nu_direct(const NuArgs &A, const GridBarrier &gsync, int &its) {
         qsync::block_sum_add<kThreads>(rn, nr, sc->dnorm[round % 3]);
         if (!gsync(20)) return -1;
         if (threadIdx.x == 0) {
-            int conv = 1, slow = 0;
+            int open = 0, slow = 0;
             bool bad = false;  // a residual that is not finite is below no bound
             for (int c = 0; c < nr; ++c) {
                 const double f2 = vload(&sc->dfnorm[c]), r2 = vload(&sc->dnorm[round % 3][c]);
-                const double thr = A.tol * A.tol * f2;
-                bad = bad || !(r2 <= kFinite);
-                if (f2 != 0.0 && !(r2 <= thr && r2 <= kFinite)) {
-                    conv = 0;
-                    if (round > 0 && !(r2 <= 0.0625 * R.beta2[c])) slow = 1;
+                // The tolerance is the bound, a hundredth of it (not below 1e-12) the
+                // aim: the residual of V-cycles that just meet a tolerance is
+                // of short waves and the field's error far smaller, that of
+                // this iteration is not.
+                const double thr = A.tol * A.tol * f2, aim = fmax(1e-4 * thr, fmin(thr, 1e-24 * f2));
+                const bool stalled = round > 0 && !(r2 <= 0.0625 * R.beta2[c]);
+                const bool done = f2 == 0.0 || r2 <= aim || (r2 <= thr && (stalled || round >= 12));
+                bad = bad || !(r2 <= kFinite) || !(f2 <= kFinite);
+                if (!done) {
+                    open = 1;
+                    if (stalled) slow = 1;
                 }
                 R.beta2[c] = r2;
                 const double s2 = R.scale[c] * R.scale[c];
-                R.target[c] = fmax(1e-10 * r2, 0.09 * thr) * s2;
-                const float b = f2 > 0.0 && r2 > thr ? (float)sqrt(r2 * s2) : 0.f;
+                R.target[c] = fmax(1e-12 * r2, 0.25 * aim) * s2;
+                const float b = done ? 0.f : (float)sqrt(r2 * s2);
                 R.nu[c][0] = R.g[c][0] = b;
                 R.inv[c] = b > 0.f ? 1.f / b : 0.f;
             }
-            s_result = conv ? 1 : bad ? 3 : (slow || round >= 12) ? 0 : 2;
+            s_result = bad ? 3 : !open ? 1 : (slow || round >= 12) ? 0 : 2;
         }
         __syncthreads();
         result = s_result;
