@@ -1158,8 +1158,9 @@ extern "C" int qs_laser_advance(qs_laser *s, const double *d_chi, double *d_a, i
     A.steps = steps;
     A.tol = tol;
     A.max_cycles = max_cycles;
-    // a cap of a few V-cycles keeps its meaning: V-cycles
-    if (max_cycles < 4) A.fft = 0;
+    // a cap of a few V-cycles keeps its meaning: V-cycles; so does a tolerance below the
+    // rounding of A, to which the iterations' residual (of A's change) is blind
+    if (max_cycles < 4 || tol < 0x1p-52) A.fft = 0;
     int st = cuda_status(cudaMemsetAsync(A.sc, 0, sizeof(LzScalars), s->stream));
     if (st != QS_OK) return st;
     void *params[] = {&A};

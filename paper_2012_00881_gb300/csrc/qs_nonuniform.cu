@@ -141,6 +141,7 @@ struct NuDirect {
     float *t;              // [kBasis][nrhs][n n] row transforms of the basis
     float *w, *tw;         // [nrhs][n n] A z of the current iteration, its row transform
     float *t2;             // [nrhs][n n] solved columns
+    double *u2;            // [nrhs][n n] the solution's other buffer
 };
 
 struct NuArgs {
@@ -1041,11 +1042,14 @@ __device__ __forceinline__ void apply_rows(const NuArgs &A, const NuRound &R, in
     else apply_rows_g<CORR, 6>(A, R, n, k, use);
 }
 
-// The end of a round: u += e, r <- r - A e in float64 with e = sum y z, |r|^2
-// into rn, and the first basis vector of the next round with its row transform.
+// The end of a round: un = uo + e and the residual J' - A un in float64 with e = sum
+// y z, |r|^2 into rn, and the first basis vector of the next round with its row
+// transform.  Two buffers of u: neighbours' rows of the old one are read.  (The
+// residual is formed anew: updated as r - A e it went below any tolerance, while
+// that of the rounded solution stood still.)
 template <bool CORR, int OWN>
 __device__ __forceinline__ void round_rows_g(const NuArgs &A, const NuRound &R, int n, int its,
-                                             double *rn) {
+                                             const double *uo, double *un, double *rn) {
     constexpr int G = OWN + 2;
     const LineSmem S = line_smem(n);
     const NuDirect &D = A.d;
@@ -1076,12 +1080,15 @@ __device__ __forceinline__ void round_rows_g(const NuArgs &A, const NuRound &R, 
 #pragma unroll
                     for (int a = 0; a < 3; ++a) {
                         const int xx = x + a - 1;
-                        v[b][a] = xx >= 0 && xx < n ? qsff::widen(S.mid[xx * G + g + b]) : 0.0;
+                        const bool in = xx >= 0 && xx < n && (b != 0 || j > 0) &&
+                                        (b != 2 || j < n - 1);
+                        v[b][a] = in ? fma(us, qsff::widen(S.mid[xx * G + g + b]),
+                                           uo[cp + (b - 1) * n + (a - 1)])
+                                     : 0.0;
                     }
-                top.u[cp] += v[1][1] * us;
+                un[cp] = v[1][1];
                 const double r =
-                    top.f[cp] - us * apply_point<CORR>(top.ax[x], top.ay[j], v, mrow, mcol, m0);
-                top.f[cp] = r;
+                    top.f[cp] - apply_point<CORR>(top.ax[x], top.ay[j], v, mrow, mcol, m0);
 #pragma unroll
                 for (int cc = 0; cc < kMaxRhs; ++cc)
                     if (cc == c) rn[cc] += r * r;
@@ -1098,11 +1105,11 @@ __device__ __forceinline__ void round_rows_g(const NuArgs &A, const NuRound &R, 
 }
 template <bool CORR>
 __device__ __forceinline__ void round_rows(const NuArgs &A, const NuRound &R, int n, int its,
-                                           double *rn) {
+                                           const double *u, double *un, double *rn) {
     const int own = rows_owned(n, A.nrhs);
-    if (own == 2) round_rows_g<CORR, 2>(A, R, n, its, rn);
-    else if (own == 4) round_rows_g<CORR, 4>(A, R, n, its, rn);
-    else round_rows_g<CORR, 6>(A, R, n, its, rn);
+    if (own == 2) round_rows_g<CORR, 2>(A, R, n, its, u, un, rn);
+    else if (own == 4) round_rows_g<CORR, 4>(A, R, n, its, u, un, rn);
+    else round_rows_g<CORR, 6>(A, R, n, its, u, un, rn);
 }
 
 // 1: converged, 0: not (u holds the last iterate), -1: a barrier failed.
@@ -1146,7 +1153,8 @@ __device__ int nu_direct(const NuArgs &A, const GridBarrier &gsync, int &its) {
     }
     __syncthreads();
     const float mbar = A.has_m ? (float)(vload(&sc->msum) / (double)nn) : 0.f;
-    double rn[kMaxRhs] = {0, 0, 0, 0};  // float64 residual, kept in J's memory
+    double rn[kMaxRhs] = {0, 0, 0, 0};  // float64 residual
+    double *u = top.u, *un = D.u2;      // the solution so far, and its next buffer
     row_products(n, rows, D.wx,
                  [&](int row, int i) {
                      const int c = row / n, j = row - c * n;
@@ -1156,7 +1164,6 @@ __device__ int nu_direct(const NuArgs &A, const GridBarrier &gsync, int &its) {
                      load_v(top.u + (size_t)c * nn, n, i, j, v);
                      const double r = top.f[cp] - apply_point<CORR>(top.ax[i], top.ay[j], v, mrow,
                                                                     mcol, m0);
-                     top.f[cp] = r;
 #pragma unroll
                      for (int cc = 0; cc < kMaxRhs; ++cc)
                          if (cc == c) rn[cc] += r * r;
@@ -1202,15 +1209,19 @@ __device__ int nu_direct(const NuArgs &A, const GridBarrier &gsync, int &its) {
             return gsync(23) ? 0 : -1;
         }
         if (result != 2) {
+            // to the caller's array; a field whose source is zero has the solution zero
+            for (int c = 0; c < nr; ++c) {
+                const bool zero = result == 1 && vload(&sc->dfnorm[c]) == 0.0;
+                if (zero || u != top.u)
+                    for (int p = grid.t; p < nn; p += grid.nt)
+                        top.u[(size_t)c * nn + p] = zero ? 0.0 : u[(size_t)c * nn + p];
+            }
+            if (result == 0 && u != top.u && !gsync(24)) return -1;
             if (blockIdx.x == 0 && threadIdx.x == 0)
                 for (int c = 0; c < nr; ++c) {
                     const double f2 = vload(&sc->dfnorm[c]);
                     sc->relres[c] = f2 > 0.0 ? sqrt(R.beta2[c] / f2) : 0.0;
                 }
-            if (result == 1)  // a field whose source is zero has the solution zero
-                for (int c = 0; c < nr; ++c)
-                    if (vload(&sc->dfnorm[c]) == 0.0)
-                        for (int p = grid.t; p < nn; p += grid.nt) top.u[(size_t)c * nn + p] = 0.0;
             return result;
         }
         int k = 0;
@@ -1288,7 +1299,10 @@ __device__ int nu_direct(const NuArgs &A, const GridBarrier &gsync, int &its) {
         }
         __syncthreads();
         for (int c = 0; c < kMaxRhs; ++c) rn[c] = 0.0;
-        round_rows<CORR>(A, R, n, k, rn);
+        round_rows<CORR>(A, R, n, k, u, un, rn);
+        double *const t = u;
+        u = un;
+        un = t;
     }
 }
 
@@ -1769,8 +1783,9 @@ void create_direct(qs_nu_solver *s, const std::vector<double> &x, const std::vec
     if (!same && !axis_basis(y, wy, vy, ly)) return;
     const size_t nn = (size_t)n * n, ld = padded(n),
                  mats = (same ? 1 : 2) * (2 * n * ld + ld);
-    const size_t vecs = (3 * kBasis + 3) * kMaxRhs * nn;
-    if (cudaMalloc(&s->direct, (mats + vecs) * sizeof(float)) != cudaSuccess) {
+    const size_t vecs = (3 * kBasis + 3) * kMaxRhs * nn, u2 = kMaxRhs * nn * sizeof(double);
+    // [u2][matrices][vectors]
+    if (cudaMalloc(&s->direct, u2 + (mats + vecs) * sizeof(float)) != cudaSuccess) {
         cudaGetLastError();
         s->direct = nullptr;
         return;
@@ -1778,7 +1793,8 @@ void create_direct(qs_nu_solver *s, const std::vector<double> &x, const std::vec
     std::vector<float> host;
     host.reserve(mats);
     NuDirect &D = s->args.d;
-    float *const base = static_cast<float *>(s->direct);
+    D.u2 = static_cast<double *>(s->direct);
+    float *const base = reinterpret_cast<float *>(D.u2 + kMaxRhs * nn);
     auto put = [&](const std::vector<float> &v) {
         const float *p = base + host.size();
         host.insert(host.end(), v.begin(), v.end());

@@ -91,3 +91,32 @@ def test_gradients_scale_with_the_cotangent(qs, form, k):
     tol = 1e-9 if form == "fp64" else 1e-7
     for a, b in zip(got[:3], ref[:3]):
         assert float((a / 2.0 ** k - b).norm()) <= tol * float(b.norm()) and float(b.norm()) > 0
+
+
+@pytest.mark.parametrize("form", ["fp64", "fp32r"])
+def test_nonuniform_residual_is_that_of_the_solution(qs, form):
+    import torch
+    from workloads.nonuniform import three_region_axis
+    x = three_region_axis(255, 12.5)
+    j = torch.randn((2, 255, 255), dtype=torch.float64, device="cuda",
+                    generator=torch.Generator(device="cuda").manual_seed(2))
+    s = qs.NonuniformSolver(x, x, precision=form)
+    # below the rounding of the residual of a rounded solution, some 1e-14 here
+    u, _, relres = s.solve(j, tol=1e-18, max_cycles=9, raise_on_error=False)
+    assert s.status == qs.QS_ERR_NOT_CONVERGED
+    for c in range(2):
+        f = s.source(j[c].contiguous())
+        r = float((f - s.apply(u[c].contiguous())).norm() / f.norm())
+        # two evaluations of one residual at its rounding: within a factor
+        assert r / 4 <= relres[c] <= 4 * r
+
+
+def test_envelope_tolerance_below_rounding_is_not_met(qs):
+    import torch
+    n, n_xi = 32, 2
+    a = torch.randn((n_xi, n, n), dtype=torch.complex128, device="cuda",
+                    generator=torch.Generator(device="cuda").manual_seed(2))
+    chi = torch.full((n_xi, n, n), 0.5, dtype=torch.float64, device="cuda")
+    lz = qs.LaserEnvelope(n, 8.0, n_xi, 5.0, 1.0, 0.2)
+    lz.advance(chi, a, tol=1e-19, max_cycles=9, raise_on_error=False)
+    assert lz.status == qs.QS_ERR_NOT_CONVERGED
