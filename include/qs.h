@@ -171,7 +171,8 @@ typedef struct {
                              /* [0] psi, [1] (E_z, B_z), [2] (B_x, B_y)       */
     int64_t psi_guard_hits;  /* clamps of 1+psi (particles and grid points)  */
     int64_t sorts;           /* cell sorts performed                          */
-    double max_relres;       /* largest final relative residual of any solve */
+    double max_relres;       /* largest final relative residual of any solve  */
+                             /* (of psi, E_z, B_z as of B_perp)               */
     double vmax;             /* largest V_max of any push                     */
     int32_t max_m;           /* largest sub-step count of any base interval   */
     int32_t status;          /* same as the return value                      */
@@ -186,7 +187,10 @@ void qs_config_default(qs_config *cfg);
 
 /* Create a context on the current CUDA device; `cuda_stream` is a
  * cudaStream_t (NULL = legacy default stream).  Allocates the grids, the
- * multigrid hierarchy and the base-slice history (6 * n_xi * N^2 float64).
+ * multigrid hierarchy, the base-slice history (6 * n_xi * N^2 float64) and the
+ * transforms' grids (88 N^2 bytes in the refined form, 160 N^2 in QS_FP64; a
+ * context for which these do not fit is made without them and solves by
+ * V-cycles).
  * Errors: QS_ERR_ARG (bad config), QS_ERR_OOM, QS_ERR_CUDA. */
 int qs_create(const qs_config *cfg, void *cuda_stream, qs_ctx **out);
 
@@ -468,7 +472,14 @@ int qs_cell_sort_noalloc(int n, double x_min, double y_min, double h, const doub
  * physical coordinates, restriction its dual-length-weighted transpose (also
  * applied to M), the smoother four-colour Gauss-Seidel over-relaxed by 1.3,
  * the 3 x 3 level is solved exactly.  The paper cites the transfer weights without giving
- * them; these are the readings. */
+ * them; these are the readings.
+ *
+ * The refined form of 15 <= n <= 511 solves by GMRES on the residual equation,
+ * preconditioned with a direct solve of the separable part, and leaves to the
+ * V-cycles what that does not bring to tol.  Four of its iterations count as
+ * one cycle; at most 4 max_cycles (and 96) are made.  A cap max_cycles < 8,
+ * too few iterations to be of use, and a cycle of the caller's own
+ * (qs_nu_set_cycle) mean V-cycles alone. */
 typedef struct qs_nu_solver qs_nu_solver;
 
 /* Build the hierarchy for n interior nodes per side, n = 2^k - 1 with
@@ -481,7 +492,8 @@ typedef struct qs_nu_solver qs_nu_solver;
  * float64).  cuda_stream: the cudaStream_t every call of this solver queues
  * on (NULL = legacy default stream).  The solver owns its device memory
  * (about 14 * 4/3 * n^2 elements of its precision, plus 5 n^2 float64 for
- * the refined form) until qs_nu_destroy.  Argument checks come before any
+ * the refined form and, for GMRES, 464 n^2 bytes and four n x n float32
+ * matrices; without room for these it keeps the V-cycles) until qs_nu_destroy.  Argument checks come before any
  * CUDA call.  Errors: QS_ERR_ARG (n not 2^k - 1, axes not increasing, bad
  * flag), QS_ERR_OOM, QS_ERR_CUDA. */
 int qs_nu_create(int n, const double *x_nodes, const double *y_nodes, int correction,
@@ -495,8 +507,10 @@ int qs_nu_create(int n, const double *x_nodes, const double *y_nodes, int correc
  *      iterate when the cycle cap is hit).  Caller-owned, written in place.
  * Stops when every field has ||J' - A u||_2 <= tol ||J'||_2 (a field with
  * J' = 0 gets u = 0), or after max_cycles V-cycles.  cycles (HOST, may be
- * NULL) receives the V-cycles done; relres (HOST, nrhs, may be NULL) the
- * final relative residuals.  Synchronises the solver's stream.
+ * NULL) receives the cycles done: V-cycles, and a quarter of the iterations
+ * before them, rounded up (so that it may exceed max_cycles); relres (HOST,
+ * nrhs, may be NULL) the final relative residuals.  A source that is not
+ * finite is not solved: QS_ERR_NOT_CONVERGED.  Synchronises the solver's stream.
  * Errors: QS_ERR_ARG, QS_ERR_NOT_CONVERGED (cap hit), QS_ERR_TIMEOUT (a grid
  * barrier wait ran out; the kernel returned), QS_ERR_CUDA. */
 int qs_nu_solve(qs_nu_solver *s, const double *d_m, int nrhs, const double *d_j, double *d_u,
@@ -569,7 +583,7 @@ int qs_nu_pic_init_plasma(qs_nu_pic *s, int ppc);
  * xi at sub-steps).  d_hist: DEVICE float64 [5][n_xi][n][n], OVERWRITTEN with
  * psi, E_z, B_z, B_x, B_y at the base slices.  Each solve stops at relative
  * residual tol or max_cycles V-cycles.  stats (may be NULL): slices,
- * pushes, V-cycles per solve kind, max_m, gpu_ms.  Synchronises.  Errors:
+ * pushes, cycles per solve kind as qs_nu_solve counts them, max_m, gpu_ms.  Synchronises.  Errors:
  * QS_ERR_STATE (no plasma), QS_ERR_ARG, QS_ERR_NOT_CONVERGED (a solve hit
  * max_cycles; the step still completed), QS_ERR_TIMEOUT, QS_ERR_CUDA. */
 int qs_nu_pic_step3d(qs_nu_pic *s, const double *d_jzb, double *d_hist, double tol,
@@ -593,8 +607,11 @@ void qs_nu_pic_destroy(qs_nu_pic *s);
  * complex screened-Poisson equation
  *   (lap - chi_j + c) A^{n+1}_j = (c + chi_j - lap) A^n_j - q (A^{n+1}_{j-1} - A^n_{j-1}),
  *   c = 4 (i k0 - 1/dxi) / dt,  q = 4 / (dt dxi)
- * solved by complex multigrid (red-black Gauss-Seidel V(2,2), warm-started
- * from A^n_j as the paper does).  chi is held at t_n; A = 0 ahead of the
+ * solved, for even n from 8 to 2048 with an odd factor of at most 7, by
+ * conjugate gradients for the complex symmetric operator, preconditioned with
+ * sine transforms; otherwise, and where that does not converge, by complex
+ * multigrid (red-black Gauss-Seidel V(2,2), warm-started from A^n_j as the
+ * paper does).  chi is held at t_n; A = 0 ahead of the
  * window and on the walls.  The grid is the slice advance's: n x n cells on a
  * square box of side `width`, cell-centred, 5-point Laplacian with odd
  * ghosts; multigrid coarsens while the side is even and above 4, so n should
@@ -604,8 +621,9 @@ typedef struct qs_laser qs_laser;
 /* n cells per side (2 .. 8192), width > 0 (k_p^-1), n_xi >= 1 slices, k0 =
  * omega_0 / omega_p > 0, dt > 0 (1/omega_p), dxi > 0 the slice spacing, or
  * +inf for no xi coupling (q = 0).  cuda_stream: the cudaStream_t of every
- * call (NULL = legacy default).  The object owns about (4 + 5 * 4/3) n^2
- * complex128 of device memory until qs_laser_destroy.  Argument checks come
+ * call (NULL = legacy default).  The object owns about (2 + 5 * 4/3) n^2
+ * complex128 of device memory until qs_laser_destroy, and 10 n^2 for the
+ * transforms (without room for these it keeps the V-cycles).  Argument checks come
  * before any CUDA call.  Errors: QS_ERR_ARG, QS_ERR_OOM, QS_ERR_CUDA. */
 int qs_laser_create(int n, double width, int n_xi, double k0, double dt, double dxi,
                     void *cuda_stream, qs_laser **out);
@@ -614,8 +632,9 @@ int qs_laser_create(int n, double width, int n_xi, double k0, double dt, double 
  * d_chi: DEVICE float64 [n_xi][n][n]; d_a: DEVICE complex128 [n_xi][n][n]
  * (interleaved re, im), A^n in, A^{n+steps} out, caller-owned, written in
  * place.  Each slice's solve stops at ||f - A u||_2 <= tol ||f||_2 or after
- * max_cycles V-cycles.  cycles (HOST, may be NULL): V-cycles over all slices
- * and steps; max_relres (HOST, may be NULL): the largest final relative
+ * max_cycles V-cycles, after at most 4 max_cycles (and 48) iterations; a cap
+ * max_cycles < 4 means V-cycles alone.  cycles (HOST, may be NULL): V-cycles, and
+ * a quarter of a slice's iterations, rounded up, over all slices and steps; max_relres (HOST, may be NULL): the largest final relative
  * residual of a slice.  Synchronises the stream.  Errors: QS_ERR_ARG,
  * QS_ERR_NOT_CONVERGED (some slice hit max_cycles; the advance still
  * completed), QS_ERR_TIMEOUT, QS_ERR_CUDA. */
@@ -636,7 +655,7 @@ void qs_laser_destroy(qs_laser *s);
  * spacing (QS_ERR_ARG otherwise).  The context allocates, on first use, two
  * float64 arrays of n_xi * N^2 (|A|^2 and chi), kept until qs_destroy.
  * stats: the slice loop's counters; env_cycles, env_relres (HOST, may be
- * NULL): the envelope advance's V-cycles and largest final relative
+ * NULL): the envelope advance's cycles and largest final relative
  * residual.  Synchronises.  Errors: those of qs_step3d_laser and
  * qs_laser_advance, QS_ERR_OOM. */
 int qs_laser_step3d(qs_ctx *ctx, qs_laser *laser, const qs_beam *beams, int n_beams,

@@ -837,14 +837,16 @@ __global__ void __launch_bounds__(kThreads, 1) laser_kernel(const __grid_constan
             const double2 *aj = A.a + (size_t)j * nn;
             const double *chij = A.chi + (size_t)j * nn;
             const bool direct = A.fft != 0;
+            int before = 0;  // what the iterations count as
             if (direct) {
                 int its = 0;
                 double rel = 0.0;
                 const int r = slice_direct(A, gsync, j, g, kglob, use, its, rel);
                 if (r < 0) return;
+                before = (its + 3) / 4;
                 if (r == 1) {
                     if (blockIdx.x == 0 && threadIdx.x == 0) {
-                        sc->cycles += (its + 3) / 4;  // the work of a V-cycle, at least
+                        sc->cycles += before;
                         if (rel > sc->max_relres) sc->max_relres = rel;
                     }
                     continue;
@@ -914,7 +916,7 @@ __global__ void __launch_bounds__(kThreads, 1) laser_kernel(const __grid_constan
                 const bool conv = !bad && r2 <= A.tol * A.tol * f2;
                 if (conv || bad || cyc >= A.max_cycles) {
                     if (blockIdx.x == 0 && threadIdx.x == 0) {
-                        sc->cycles += cyc;
+                        sc->cycles += before + cyc;
                         const double rel = f2 > 0.0 ? sqrt(r2 / f2) : 0.0;
                         if (rel > sc->max_relres) sc->max_relres = rel;
                         if (!conv) sc->fail = 1;

@@ -1124,6 +1124,8 @@ __device__ int nu_direct(const NuArgs &A, const GridBarrier &gsync, int &its) {
     __shared__ NuRound R;
     __shared__ int s_result;
     its = 0;
+    // four iterations count as one V-cycle, which takes longer
+    const int cap = min(4 * A.max_cycles, 96);
     int use = 0, result = 2;
     {  // J' and its norm; M in float32 and its sum
         double fn[kMaxRhs] = {0, 0, 0, 0}, ms = 0.0;
@@ -1187,7 +1189,7 @@ __device__ int nu_direct(const NuArgs &A, const GridBarrier &gsync, int &its) {
                 // this iteration is not.
                 const double thr = A.tol * A.tol * f2, aim = fmax(1e-4 * thr, fmin(thr, 1e-24 * f2));
                 const bool stalled = round > 0 && !(r2 <= 0.0625 * R.beta2[c]);
-                const bool done = f2 == 0.0 || r2 <= aim || (r2 <= thr && (stalled || round >= 12));
+                const bool done = f2 == 0.0 || r2 <= aim || (r2 <= thr && (stalled || its >= cap));
                 bad = bad || !(r2 <= kFinite) || !(f2 <= kFinite);
                 if (!done) {
                     open = 1;
@@ -1200,7 +1202,7 @@ __device__ int nu_direct(const NuArgs &A, const GridBarrier &gsync, int &its) {
                 R.nu[c][0] = R.g[c][0] = b;
                 R.inv[c] = b > 0.f ? 1.f / b : 0.f;
             }
-            s_result = bad ? 3 : !open ? 1 : (slow || round >= 12) ? 0 : 2;
+            s_result = bad ? 3 : !open ? 1 : (slow || its >= cap) ? 0 : 2;
         }
         __syncthreads();
         result = s_result;
@@ -1285,7 +1287,7 @@ __device__ int nu_direct(const NuArgs &A, const GridBarrier &gsync, int &its) {
             __syncthreads();
             ++k;
             ++its;
-            if (!R.go || k == kBasis) break;
+            if (!R.go || k == kBasis || its >= cap) break;
         }
         // y from the triangular factor; u += sum_k y_k z_k / |v_k|: the column
         // phase has the 1 / |v_k| in z already
@@ -1331,14 +1333,16 @@ __global__ void __launch_bounds__(kThreads, 1) nu_solve_kernel(const __grid_cons
     int loc = 0;
     while (loc < Lc && H[loc].n > A.local_n) ++loc;
 
+    int before = 0;  // what the iterations count as
     if constexpr (REF) {
         if (A.d.on) {
             int its = 0;
             const int r = nu_direct<CORR>(A, gsync, its);
             if (r < 0) return;
+            before = (its + 3) / 4;
             if (r > 0) {
                 if (blockIdx.x == 0 && threadIdx.x == 0) {
-                    sc->cycles = (its + 3) / 4;  // no more work than so many V-cycles
+                    sc->cycles = before;
                     sc->converged = 1;
                 }
                 return;
@@ -1407,7 +1411,7 @@ __global__ void __launch_bounds__(kThreads, 1) nu_solve_kernel(const __grid_cons
         if (bad) conv = false;
         if (conv || bad || cyc >= A.max_cycles) {
             if (blockIdx.x == 0 && threadIdx.x == 0) {
-                sc->cycles = cyc;
+                sc->cycles = before + cyc;
                 sc->converged = conv ? 1 : 0;
                 for (int c = 0; c < nr; ++c)
                     sc->relres[c] =

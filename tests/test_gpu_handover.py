@@ -41,3 +41,15 @@ def test_cycles_finish_capped_iterations(qs, form, n):
     # a cycle takes off about as much as an iteration: what the cap cuts off a
     # solve comes back as a cycle or two, not as another full set of them
     assert counts[4] <= counts[60] + 2 * ref.slices
+
+
+def test_nonuniform_counts_the_iterations_too(qs):
+    import torch
+    x = np.linspace(-3.0, 3.0, 33)
+    j = torch.randn((31, 31), dtype=torch.float64, device="cuda",
+                    generator=torch.Generator(device="cuda").manual_seed(2))
+    s = qs.NonuniformSolver(x, x, precision="fp32r")
+    # below the rounding of the residual: the iterations stall, the cycles reach the cap
+    _, cycles, relres = s.solve(j, tol=1e-18, max_cycles=9, raise_on_error=False)
+    assert s.status == qs.QS_ERR_NOT_CONVERGED and relres[0] < 1e-12
+    assert 9 < cycles <= 18  # the quarter of 36 iterations at most
