@@ -53,3 +53,39 @@ def test_nonuniform_counts_the_iterations_too(qs):
     _, cycles, relres = s.solve(j, tol=1e-18, max_cycles=9, raise_on_error=False)
     assert s.status == qs.QS_ERR_NOT_CONVERGED and relres[0] < 1e-12
     assert 9 < cycles <= 18  # the quarter of 36 iterations at most
+
+
+@pytest.mark.parametrize("scale,power", [(1e4, 3), (1e5, 6)])
+def test_envelope_cycles_finish_stalled_iterations(qs, scale, power):
+    """A susceptibility so rough that the iterations make 48 steps (the first) or
+    stall in a round of 24 (the second): 12 and 6 cycles' worth, then V-cycles, for
+    every slice, each of which starts afresh."""
+    import torch
+    from oracle import qs_laser as QL
+    from oracle.qs_oracle import Grid
+    n, n_xi, width = 64, 3, 8.0
+    rng = np.random.default_rng(int(power))
+    a0 = rng.standard_normal((n_xi, n, n)) + 1j * rng.standard_normal((n_xi, n, n))
+    chi = scale * rng.uniform(0.0, 1.0, (n_xi, n, n)) ** power
+    ref = QL.envelope_advance(Grid.square(n, width / 2), a0, chi, 5.0, 1.0, 0.2, 1)
+    a = torch.tensor(a0, device="cuda")
+    _, cycles, relres = qs.LaserEnvelope(n, width, n_xi, 5.0, 1.0, 0.2).advance(
+        torch.tensor(chi, device="cuda"), a, tol=1e-12, max_cycles=60)
+    assert relres <= 1e-12 and cycles >= 7 * n_xi
+    assert np.linalg.norm(a.cpu().numpy() - ref) < 1e-9 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("scale,power", [(1e4, 3), (1e5, 6)])
+def test_nonuniform_cycles_finish_stalled_iterations(qs, scale, power):
+    """The same for GMRES: rounds of 8, so at least 2 cycles' worth before it gives up;
+    the float64 form's V-cycles are the reference."""
+    import torch
+    n = 63
+    x = np.linspace(-4.0, 4.0, n + 2)
+    rng = np.random.default_rng(int(power))
+    j = torch.tensor(rng.standard_normal((2, n, n)), device="cuda")
+    m = torch.tensor(-scale * rng.uniform(0.0, 1.0, (n, n)) ** power, device="cuda")
+    ref, alone, _ = qs.NonuniformSolver(x, x, precision="fp64").solve(j, m=m, max_cycles=60)
+    u, cycles, relres = qs.NonuniformSolver(x, x, precision="fp32r").solve(j, m=m, max_cycles=60)
+    assert max(relres) <= 1e-10 and cycles > 2
+    assert float((u - ref).norm()) <= 1e-8 * float(ref.norm())
