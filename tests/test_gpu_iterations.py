@@ -35,3 +35,23 @@ def test_nonuniform_iterations_converge(qs, n):
     s = qs.NonuniformSolver(x, x, precision="fp32r")
     _, cycles, relres = s.solve(j, m=m)
     assert relres[0] <= 1e-10 and cycles <= 5
+
+
+@pytest.mark.parametrize("kind", ["mirrored", "twin", "slanted", "two axes"])
+def test_bases_of_other_axes(qs, kind):
+    """The preconditioner's bases: of an axis that is its own mirror image (halved),
+    with two fine regions whose eigenvalues agree to rounding, of one that is not, and
+    of two different axes.  A basis that lacks a vector would leave GMRES stalled."""
+    import torch
+    n = 127
+    t = np.linspace(-1.0, 1.0, n + 2)
+    twin = t - 0.12 * np.sin(2 * np.pi * t) * np.abs(np.sin(np.pi * t))
+    x = {"mirrored": t + 0.4 * t ** 3, "twin": twin, "slanted": t + 0.2 * t ** 2,
+         "two axes": t + 0.4 * t ** 3}[kind]
+    x, y = 6.0 * x, 6.0 * (t + 0.2 * t ** 2 if kind == "two axes" else x)
+    X, Y = np.meshgrid(x[1:-1], y[1:-1])
+    j = torch.tensor(np.exp(-((X - 0.3) ** 2 + Y ** 2)), device="cuda")
+    u, cycles, relres = qs.NonuniformSolver(x, y, precision="fp32r").solve(j)
+    ref, _, _ = qs.NonuniformSolver(x, y, precision="fp64").solve(j, tol=1e-11)
+    assert relres[0] <= 1e-10 and cycles <= 6
+    assert float((u - ref).norm()) <= 1e-9 * float(ref.norm())
