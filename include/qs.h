@@ -81,7 +81,9 @@ typedef struct {
     int refine_k;               /* smallest sub-step is dxi0 / refine_k         */
                                 /* (refinement level k of Sec. 5.1), >= 1       */
     int precision;              /* QS_FP64 or QS_FP32_REFINED                   */
-                                /* Fields: even N, 8 <= N <= 2048, are solved   */
+                                /* Fields: even N, 8 <= N <= 2048 (QS_FP64 1024, */
+                                /* where the tables fit beside the default       */
+                                /* tiles), are solved                           */
                                 /* directly by sine transforms (psi, E_z, B_z)  */
                                 /* and by conjugate gradients preconditioned    */
                                 /* with them (B_perp); other N, an explicit     */

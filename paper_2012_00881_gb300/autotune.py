@@ -13,6 +13,10 @@ keeps the fastest:
 and, for the whole batch, the number of thread blocks per team
 (tune_team).
 
+These are settings of the V-cycles.  Sides that the library solves directly take
+V-cycles only where its iterations do not converge: candidates that differ in
+nothing else would be told apart by noise, and only one is timed, without them.
+
 Every candidate solves to the same residual tolerance, so the choice changes
 only the time, not the result.  A candidate is timed on a batch of the
 instances of that size with the xi window truncated to a few slices, through
@@ -39,6 +43,27 @@ def candidates(tiles=DEFAULT_TILES, sweeps=DEFAULT_SWEEPS, coarse=DEFAULT_COARSE
     return [dict(tile_x=t[0], tile_y=t[1], pre_sweeps=s[0], post_sweeps=s[1], coarse_block_n=c,
                  omega_pct=o)
             for t, s, c, o in itertools.product(tiles, sweeps, coarse, omegas)]
+
+
+VCYCLE_SETTINGS = ("tile_x", "tile_y", "pre_sweeps", "post_sweeps", "coarse_pre_sweeps",
+                   "coarse_block_n", "omega_pct", "warm_start_order")
+
+
+def direct_solves(n: int, precision: str) -> bool:
+    """Whether the library solves a grid of side n directly (its rule, with the
+    default tiles: the tables of larger float64 grids do not fit beside them)."""
+    return n % 2 == 0 and 8 <= n <= (2048 if precision == "fp32r" else 1024)
+
+
+def distinct(cands: Sequence[Dict], n: int, precision: str) -> List[Dict]:
+    """The candidates that a grid of side n can tell apart."""
+    out: List[Dict] = []
+    for c in cands:
+        if direct_solves(n, precision) and c.get("cluster_size", 0) < 2:
+            c = {k: v for k, v in c.items() if k not in VCYCLE_SETTINGS}
+        if c not in out:
+            out.append(c)
+    return out
 
 
 def _truncated(wl, n_slices: int):
@@ -96,7 +121,7 @@ def tune(wls: Sequence, precision: str = "fp32r", n_slices: int = 16,
     for n, group in sorted(by_size.items()):
         group = group[:max_per_size]
         scored = []
-        for cand in cands:
+        for cand in distinct(cands, n, precision):
             t = time_candidate(group, cand, n_slices, precision, beams_cache)
             scored.append((t, cand))
             if verbose:
