@@ -89,3 +89,52 @@ def test_nonuniform_cycles_finish_stalled_iterations(qs, scale, power):
     u, cycles, relres = qs.NonuniformSolver(x, x, precision="fp32r").solve(j, m=m, max_cycles=60)
     assert max(relres) <= 1e-10 and cycles > 2
     assert float((u - ref).norm()) <= 1e-8 * float(ref.norm())
+
+
+@pytest.mark.parametrize("form", ["fp64", "fp32r"])
+@pytest.mark.parametrize("settings", [dict(tile_x=16, tile_y=8, coarse_block_n=16),
+                                      dict(tile_x=32, tile_y=32, pre_sweeps=2, post_sweeps=1),
+                                      dict(coarse_block_n=32), dict(omega_pct=100)])
+def test_settings_of_the_cycles_that_finish(qs, form, settings):
+    """The multigrid's settings, on a side that takes it only after capped iterations:
+    staged tiles of other shapes, other sweeps, more levels in one block, no
+    over-relaxation."""
+    n = 64
+    wl = W.Workload(name="h", n=n, half_width=3.0, n_xi=6, xi_len=1.2, ppc=4,
+                    beams=(W.BeamSpec(amplitude=1.5, sigma_x=0.7, sigma_y=0.5, sigma_z=0.6,
+                                      xi_c=0.6, n_particles=3000, seed=n, x_c=0.3),))
+    beams = [W.sample_beam(b) for b in wl.beams]
+    pl, n_ion = O.plasma_from_workload(wl)
+    ref = O.step3d(O.config_from_workload(wl), pl, n_ion, beams)
+    ctx = qs.Context(qs.config_from_workload(wl, precision=form, mg_tol=1e-10, mg_max_vcycles=4,
+                                             **settings))
+    ctx.init_plasma(wl.ppc)
+    st = ctx.step3d([qs.Beam(b) for b in beams], schedule=list(ref.m))
+    got = ctx.fields(qs.FIELD_ALL, device=False).numpy()
+    ctx.close()
+    assert st["vcycles"][2] > 4 * ref.slices  # more than the iterations alone
+    scale = np.linalg.norm(ref.history[0])
+    for i in range(5):
+        err = np.linalg.norm(got[i] - ref.history[i])
+        assert err < TOL[form] * max(np.linalg.norm(ref.history[i]), scale), i
+
+
+@pytest.mark.parametrize("form", ["fp64", "fp32r"])
+def test_warm_starts_of_clustered_cycles_agree(qs, form):
+    """Clusters on request keep the V-cycles, whose initial guesses the warm-start order
+    sets: the same fields from each, from fewer cycles the higher the order."""
+    wl = W.Workload(name="w", n=64, half_width=3.0, n_xi=16, xi_len=1.6, ppc=4,
+                    beams=(W.BeamSpec(amplitude=0.5, sigma_x=0.7, sigma_y=0.5, sigma_z=0.6,
+                                      xi_c=0.8, n_particles=3000, seed=1),))
+    got, cycles = [], []
+    for order in (0, 1, 2):
+        ctx = qs.Context(qs.config_from_workload(wl, precision=form, mg_tol=1e-10, cluster_size=8,
+                                                 warm_start_order=order))
+        ctx.init_plasma(wl.ppc)
+        st = ctx.step3d([qs.Beam(W.sample_beam(b)) for b in wl.beams])
+        got.append(ctx.fields(qs.FIELD_ALL, device=False).numpy())
+        cycles.append(st["vcycles"][0])
+        ctx.close()
+    assert cycles[0] > cycles[2] > 2 * 16  # V-cycles: a direct solve counts one a slice
+    for g in got[1:]:
+        assert np.linalg.norm(g - got[0]) < TOL[form] * np.linalg.norm(got[0])
