@@ -1370,7 +1370,6 @@ __device__ bool run_step(const EngineArgs &A, int bid, int nblk, const Sync &S, 
                 PoissonCheck<P> check(A, Q, ncur, bid, nblk);
                 if (!mg_solve<REF>(A, S, Vbp, slot, bid, nblk, smem, s_inv_ready, true, check))
                     return false;
-                check.rest();
             } else {
                 phase_psi_rhs<P>(A, Q, ncur, nnext, base, j, q, frac, T, g);
                 if (!S(2)) return false;

@@ -1240,7 +1240,8 @@ __device__ bool direct_poisson(const EngineArgs &A, const Sync &S, const SolveSp
 // The sums are of values scaled by a power of two near 1 / ||f||, so that
 // float32 cannot underflow in them.
 // prepared: the source's row transform and copy are in tr and cr already.
-// side(): work besides the solve, called before the barriers of its phases.
+// side(): work besides the solve, called before the barriers of its phases (and
+// side.rest() by the caller after it).
 // Returns 1 (converged), 0 (not within its cap: u holds the last iterate and
 // the V-cycles take over), -1 (a barrier failed).
 template <bool REF, typename X>
@@ -1496,6 +1497,7 @@ __device__ void screened_diagonal(const EngineArgs &A, Thr T) {
 
 struct Nothing {
     __device__ void operator()() const {}
+    __device__ void rest() const {}
 };
 
 // Iterate until, for every component,
@@ -1679,7 +1681,9 @@ __device__ bool mg_solve(const EngineArgs &A, const Sync &S, const SolveSpec &V,
             return V.nc == 1 ? direct_poisson<1>(A, S, V, bid, nblk)
                              : direct_poisson<2>(A, S, V, bid, nblk);
         const int r = cg_screened<REF>(A, S, V, slot, bid, nblk, prepared, side);
-        if (r != 0) return r > 0;
+        if (r < 0) return false;
+        side.rest();  // before the cycles take the shared memory
+        if (r > 0) return true;
         screened_diagonal(A, grid_thr(bid, nblk));
         // The cycles move `slot` on without clearing the dot products' ring: the
         // next slice's iterations would add to what these left in it.

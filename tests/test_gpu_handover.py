@@ -138,3 +138,18 @@ def test_warm_starts_of_clustered_cycles_agree(qs, form):
     assert cycles[0] > cycles[2] > 2 * 16  # V-cycles: a direct solve counts one a slice
     for g in got[1:]:
         assert np.linalg.norm(g - got[0]) < TOL[form] * np.linalg.norm(got[0])
+
+
+@pytest.mark.parametrize("form", ["fp64", "fp32r"])
+def test_residuals_are_complete_before_the_cycles(qs, form):
+    """Two iterations are four phases, fewer than the parts in which idle blocks form
+    the residuals of psi, E_z and B_z at 256^2; their partial sums lie where the cycles
+    that follow put their tiles.  A wrong sum would be reported as not converged."""
+    wl = W.Workload(name="p", n=256, half_width=4.0, n_xi=4, xi_len=0.8, ppc=1,
+                    beams=(W.BeamSpec(amplitude=1.0, sigma_x=0.7, sigma_y=0.5, sigma_z=0.6,
+                                      xi_c=0.3, n_particles=3000, seed=2),))
+    ctx = qs.Context(qs.config_from_workload(wl, precision=form, mg_tol=1e-6, mg_max_vcycles=2))
+    ctx.init_plasma(wl.ppc)
+    st = ctx.step3d([qs.Beam(W.sample_beam(wl.beams[0]))])
+    ctx.close()
+    assert st["vcycles"][2] > 2 * st["slices"] and st["max_relres"] <= 1e-6
