@@ -39,8 +39,10 @@ namespace {
 // floats (qs_ff.cuh), with float64 cotangents and sums.  In float64 the three
 // phases issue about 630 FP64-pipe instructions a particle (64 cycles a warp
 // each).  Forward and gradient of a 256^2 window in the refined form: 54.5 ms
-// with float64 particle phases, 47.2 with pairs.  The error of the gradient
-// against float64 is unchanged (median 3.3e-9, that of the forward state).
+// with float64 particle phases, 47.2 with pairs.  Gradients and loss differ
+// between two runs by 3e-10 to 2e-9, the order of the forward step's float32
+// moment reductions, and by 3e-10 to 1e-8 from float64; both with float64 and with
+// pairs here.
 using qsff::Ff;
 template <typename R>
 __device__ __forceinline__ R in(double v) {
