@@ -834,6 +834,14 @@ def run_nonuniform(args):
                 torch.distributed.barrier()
             sampler = ClockSampler(local)
             sampler.start()
+            # A step is a few host-paced calls of half a millisecond: timed while the
+            # sampler's process starts it takes a third longer (598 sets/s where
+            # the end-to-end loop after it gave 836), and a few steps are over
+            # before the first sample.
+            began = time.perf_counter()
+            while time.perf_counter() - began < 0.6:
+                step(False)
+            stream.synchronize()
             t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
             t0.record(stream)
             for _ in range(args.steps):
