@@ -883,42 +883,53 @@ __device__ __noinline__ void poisson_residuals(const EngineArgs &A, const PS<P> 
 
 // These residuals beside the B_perp solve.  Its phases leave blocks without a line
 // (G lines a block, a power of two: 24 of 152 at 128^2 to 512^2): they do a part of
-// the cells in each phase, of 2 N cells a block, which takes less than the others'
-// transforms do.  By all blocks in one phase the residuals took 8.3 us of a 256^2
-// slice, in this way less than one (refined wake 32.4 ms without, 32.1 with; 512^2
-// channel 80.4 and 81.1).  Where no block is idle all do them in the first phase.
+// the cells in each iteration, of 3 N cells a block, which takes about as long as the
+// others' two phases; what is left at the end all blocks do.  Refined blowout at
+// 256^2, a slice without the residuals 197 us: all blocks in one phase +8.3 us, idle
+// blocks with a part in each phase (2 N, N, N / 2 cells) +8, +6, +10, a part in each
+// iteration (N, 2 N, 3 N, 4 N, 6 N) +9, +5, +4, +5, +12.  Where no block
+// is idle all do them in the first phase.
 template <typename P>
 struct PoissonCheck {
     const EngineArgs &A;
     const PS<P> &Q;
     const double *ncur;
-    int rank, cnt, part, parts;
-    __device__ PoissonCheck(const EngineArgs &A_, const PS<P> &Q_, const double *ncur_, int bid,
-                            int nblk)
-        : A(A_), Q(Q_), ncur(ncur_), rank(bid), cnt(nblk), part(0), parts(1) {
+    int bid, nblk, rank, cnt, part, parts;
+    __device__ PoissonCheck(const EngineArgs &A_, const PS<P> &Q_, const double *ncur_, int bid_,
+                            int nblk_)
+        : A(A_), Q(Q_), ncur(ncur_), bid(bid_), nblk(nblk_), rank(bid_), cnt(nblk_), part(0),
+          parts(1) {
         const int n = A.N, G = 1 << qsfft::lines_at_once(n, nblk, A.fft.gmax);
         const int busy = (n + G - 1) / G;
         if (busy < nblk) {
             rank = bid - busy;
             cnt = nblk - busy;
-            const int per = cnt * max(2 * n, 256);
+            const int per = cnt * max(3 * n, 128);
             parts = (n * n + per - 1) / per;
-            if (rank < 0) part = parts;
         }
     }
+    __device__ __forceinline__ int begin(int k) const {
+        const int nn = A.N * A.N, len = (nn + parts - 1) / parts;
+        return min(nn, k * len);
+    }
+    // the sums between the parts: over the line buffers, which an idle block does
+    // not use
+    __device__ __forceinline__ double *acc() const {
+        return (double *)(qsfft::dyn_smem() + A.block_smem_offset) + 9 * (int)threadIdx.x;
+    }
+    __device__ bool idle() const { return cnt < nblk && rank >= 0; }
     __device__ void operator()() {
         if (part == parts) return;
-        const int nn = A.N * A.N, len = (nn + parts - 1) / parts;
-        // the sums between the parts: over the line buffers, which an idle block
-        // does not use
-        double *const acc =
-            (double *)(qsfft::dyn_smem() + A.block_smem_offset) + 9 * (int)threadIdx.x;
-        poisson_residuals<P>(A, Q, ncur, part * len, min(nn, (part + 1) * len),
-                             grid_thr(rank, cnt), acc, part == 0, part + 1 == parts);
+        if (rank >= 0)
+            poisson_residuals<P>(A, Q, ncur, begin(part), begin(part + 1), grid_thr(rank, cnt),
+                                 acc(), part == 0, part + 1 == parts);
         ++part;
     }
     __device__ void rest() {
-        while (part < parts) (*this)();
+        if (part == parts) return;
+        poisson_residuals<P>(A, Q, ncur, begin(part), A.N * A.N, grid_thr(bid, nblk), acc(),
+                             part == 0 || rank < 0, true);
+        part = parts;
     }
 };
 

@@ -62,6 +62,15 @@ struct Sync {
     bool tracer;                // this block records the phase trace
     int cl = 1;                 // cluster size of the launch (> 1: clusters run
                                 // the multigrid cycles, see qs_cluster.cuh)
+    // Arrival without the wait, of a block that neither reads what the others wrote
+    // before this barrier nor writes before the next one, where it waits.
+    __device__ void arrive() const {
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            *epoch += 1;
+            red_release_add_u64(bar, 1ull);
+        }
+    }
     __device__ bool operator()(int where) const {
         __shared__ int s_ok;
         __syncthreads();
@@ -1240,8 +1249,9 @@ __device__ bool direct_poisson(const EngineArgs &A, const Sync &S, const SolveSp
 // The sums are of values scaled by a power of two near 1 / ||f||, so that
 // float32 cannot underflow in them.
 // prepared: the source's row transform and copy are in tr and cr already.
-// side(): work besides the solve, called before the barriers of its phases (and
-// side.rest() by the caller after it).
+// side(): work besides the solve, once an iteration (and side.rest() by the caller
+// after it); side.idle(): this block has no line, so that it need not wait for the
+// columns and has both phases of the iteration for that work.
 // Returns 1 (converged), 0 (not within its cap: u holds the last iterate and
 // the V-cycles take over), -1 (a barrier failed).
 template <bool REF, typename X>
@@ -1302,8 +1312,8 @@ __device__ int cg_screened(const EngineArgs &A, const Sync &S, const SolveSpec &
                 }
                 return r;
             });
-            side();
-            if (!S(52)) return -1;
+            if (side.idle()) S.arrive();
+            else if (!S(52)) return -1;
             float d[16] = {0.f};
             qsfft::rows_inverse_forward<T, T, 1>(P, P, bid, nblk, t2, tz, [&](int y, int x, C z) {
                 const size_t i = (size_t)y * N + x;
@@ -1496,6 +1506,7 @@ __device__ void screened_diagonal(const EngineArgs &A, Thr T) {
 }
 
 struct Nothing {
+    __device__ bool idle() const { return false; }
     __device__ void operator()() const {}
     __device__ void rest() const {}
 };
