@@ -127,6 +127,44 @@ __device__ __forceinline__ void dep6_pairs(float4 *g, const CicP<float> &c, cons
     }
 }
 
+// Whether the refined form sums its moments in float64, in the grids of the float64
+// form, and rounds the sums: in steps that a gradient is taken of.  The order in
+// which float32 reductions arrive made two losses of one input differ by 3e-10 to
+// 2e-9 at 256^2, which a line search or a difference quotient sees; with float64
+// sums 2e-13 to 4e-11, nearer to the float64 form's.  The moments phase takes 40 us
+// instead of 14 there (a gradient 43.6 -> 44.9 ms).  Privatised deposits keep theirs.
+__device__ __forceinline__ bool sums64(const EngineArgs &A) {
+    return A.precision == QS_FP32_REFINED && (A.ckpt || A.seg_g) && A.band_rows == 0;
+}
+
+__device__ __forceinline__ void dep6_float64(const EngineArgs &A, const CicP<float> &c,
+                                             const float q[6]) {
+    double *const g[6] = {A.jx, A.jy, A.txx, A.txy, A.tyy, A.G};
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        atomicAdd(g[k] + c.i00, qsff::widen(q[k] * c.w00));
+        atomicAdd(g[k] + c.i01, qsff::widen(q[k] * c.w01));
+        atomicAdd(g[k] + c.i10, qsff::widen(q[k] * c.w10));
+        atomicAdd(g[k] + c.i11, qsff::widen(q[k] * c.w11));
+    }
+}
+
+// a cell's accumulators before the deposit
+__device__ __forceinline__ void clear_moments(const EngineArgs &A, int i) {
+    if (sums64(A)) A.jx[i] = A.jy[i] = A.txx[i] = A.txy[i] = A.tyy[i] = A.G[i] = 0.0;
+    else
+        A.mom32[2 * (size_t)i] = A.mom32[2 * (size_t)i + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
+// the rounded sums to the refined form's cells
+__device__ __noinline__ void round_moments(const EngineArgs &A, Thr T) {
+    auto f = [](double v) { return qsff::split(v).h; };
+    for (int i = T.t0; i < A.N * A.N; i += T.nt) {
+        A.mom32[2 * (size_t)i] = make_float4(f(A.jx[i]), f(A.jy[i]), f(A.txx[i]), f(A.txy[i]));
+        A.mom32[2 * (size_t)i + 1] = make_float4(f(A.tyy[i]), f(A.G[i]), 0.f, 0.f);
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Privatised deposits.  With the plasma sorted by cell, a block that takes a
 // contiguous chunk of the particle array finds its CIC stencils in a narrow
@@ -284,7 +322,7 @@ __device__ void phase_psi_rhs(const EngineArgs &A, const PS<P> &Q, const double 
 #pragma unroll
             for (int k = 0; k < 6; ++k) Q.m[k][i] = 0.0;
         } else {
-            A.mom32[2 * (size_t)i] = A.mom32[2 * (size_t)i + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
+            clear_moments(A, i);
         }
         nnext[i] = 0.0;
     }
@@ -366,6 +404,7 @@ __device__ void phase_moments(const EngineArgs &A, const PS<P> &Q, Thr T, int bi
     const P s = (P)(A.inv_h * A.inv_h);
     constexpr int ST = PS<P>::stride;
     unsigned hits = 0;
+    const bool sums = sums64(A);
     // privatised: this block's chunk into the six bands of sb
     const bool banded = A.band_rows > 0;
     int64_t p0 = T.t0, p1 = A.np, pst = T.nt;
@@ -436,6 +475,8 @@ __device__ void phase_moments(const EngineArgs &A, const PS<P> &Q, Thr T, int bi
 #pragma unroll
                 for (int k = 0; k < 6; ++k)
                     if (in) dep_band<ST>(Q.m[k], sb + k * cells, lo, hi, c, q[k]);
+            } else if (sums) {
+                if (in) dep6_float64(A, c, q);
             } else {
                 dep6_pairs(A.mom32, c, q);
             }
@@ -610,7 +651,7 @@ __device__ void rows_psi(const EngineArgs &A, const PS<P> &Q, const double *ncur
 #pragma unroll
             for (int k = 0; k < 6; ++k) Q.m[k][i] = 0.0;
         } else {
-            A.mom32[2 * (size_t)i] = A.mom32[2 * (size_t)i + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
+            clear_moments(A, i);
         }
         nnext[i] = 0.0;
         return qsff::split(nv - A.n_ion[i]);
@@ -1372,6 +1413,10 @@ __device__ bool run_step(const EngineArgs &A, int bid, int nblk, const Sync &S, 
                 SYNC(28);
                 phase_moments<P>(A, Q, T, bid, nblk, smem);
                 SYNC(3);
+                if (sums64(A)) {
+                    round_moments(A, T);
+                    SYNC(33);
+                }
                 rows_eb<P>(A, Q, ncur, j, q, frac, bid, nblk);
                 SYNC(4);
                 poisson_columns<2>(A, bid, nblk);
@@ -1394,6 +1439,10 @@ __device__ bool run_step(const EngineArgs &A, int bid, int nblk, const Sync &S, 
                 }
                 phase_moments<P>(A, Q, T, bid, nblk, smem);
                 if (!S(3)) return false;
+                if (sums64(A)) {
+                    round_moments(A, T);
+                    if (!S(33)) return false;
+                }
                 phase_assemble1<P>(A, Q, ncur, j, q, frac, T, g);
                 if (!S(4)) return false;
                 if (!mg_cycles<REF>(A, S, Veb, slot, bid, nblk, smem, s_inv_ready)) return false;
